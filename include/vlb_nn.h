@@ -48,12 +48,14 @@ int vlb_nn_set_params(vlb_nn *net, const float *host);
  * Keeps what the backward pass needs. With bfloat16 storage, a 3x3 layer
  * whose Co is a power of two in [16, 256], whose grid has a multiple of 128
  * cells and whose Ci is a multiple of 8 runs on the tensor cores (tcgen05:
- * an implicit GEMM with FP32 accumulators in tensor memory); the others,
- * the FP32 storage and the backward pass run on the CUDA cores. VLB_ECUDA if
- * a tensor-core layer gave up waiting (one second) for its MMAs. */
+ * an implicit GEMM with FP32 accumulators in tensor memory), and so does its
+ * backward pass where its rows are a multiple of 8 and at most 256 cells long
+ * (Ci a multiple of 16 below the first layer); the others and the FP32
+ * storage run on the CUDA cores. VLB_ECUDA if a tensor-core layer gave up
+ * waiting (one second) for its MMAs. */
 int vlb_nn_forward(vlb_nn *net, const float *d_x, float *d_y, int32_t batch);
-/* Whether bfloat16 forward passes may use the tensor cores (default 1); 0
- * runs every layer on the CUDA cores (for comparison). */
+/* Whether bfloat16 passes may use the tensor cores (default 1); 0 runs every
+ * layer on the CUDA cores (for comparison). */
 int vlb_nn_set_tensor_cores(vlb_nn *net, int32_t enable);
 /* Mean-square loss over all outputs against d_target and its gradient with
  * respect to y, written to d_dy (may alias nothing else); loss is returned in
@@ -61,7 +63,8 @@ int vlb_nn_set_tensor_cores(vlb_nn *net, int32_t enable);
 int vlb_nn_mse(vlb_nn *net, const float *d_y, const float *d_target, float *d_dy, int32_t batch,
                double *loss);
 /* Gradients of the parameters for dL/dy = d_dy, through the activations of the
- * last forward call (replaces any previous gradients). */
+ * last forward call (replaces any previous gradients). Gradients are FP32; on
+ * the tensor cores each is the exact sum of three bfloat16 operands. */
 int vlb_nn_backward(vlb_nn *net, const float *d_dy, int32_t batch);
 int vlb_nn_get_grads(const vlb_nn *net, float *host);
 /* One Adam step (step index t >= 1) on the FP32 master parameters; the

@@ -3,13 +3,14 @@
 // stored in FP32 or bfloat16 and every product is accumulated in FP32; the
 // optimizer (Adam) works on an FP32 master copy of the parameters.
 //
-// Kernels: a tiled direct convolution (3x3 or 1x1, zero padding) that also
+// Kernels: a tiled direct convolution (3x3, zero padding) that also
 // serves the backward pass with respect to its input (with transposed,
 // flipped weights), a tiled weight-gradient reduction with fixed-order
 // split sums (deterministic), 2x2 average pooling, 2x nearest upsampling,
-// ReLU masks, bias gradients, the mean-square loss and Adam. Activations
-// are NCHW with a batch stride, so a channel concatenation is a view into
-// one buffer.
+// the 1x1 head, ReLU masks, bias gradients, the mean-square loss and Adam.
+// With bfloat16 storage the 3x3 layers run on the tensor cores, forward and
+// backward, where they fit (vlb_nn_tc.cuh). Activations are NCHW with a
+// batch stride, so a channel concatenation is a view into one buffer.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -23,6 +24,7 @@
 
 #include "../../include/vlb.h"
 #include "../../include/vlb_nn.h"
+#include "vlb_nn_tc.cuh"
 
 namespace vlb {
 int set_error(int code, const char *fmt, ...);
@@ -113,196 +115,6 @@ __global__ void __launch_bounds__(kThreads) k_conv(const TI *__restrict__ in, in
     if (RELU) v = fmaxf(v, 0.0f);
     ob[(int64_t)(co0 + o) * HW] = st<TO>(v);
   }
-}
-
-// ------------------------------------------------- tensor-core convolution
-// The 3x3 forward convolution of bfloat16 activations and weights as an
-// implicit GEMM on the fifth-generation tensor cores (tcgen05, sm_100 and
-// later): for the 128 output pixels p of a tile and kk = ci * 9 + tap,
-//   D[p][co] = sum_kk A[p][kk] B[co][kk],  A = the input patches (gathered
-//   on the fly), B = w[co][ci][tap] (K-contiguous as stored),
-// one MMA of M = 128, N = Co, K = 16 per step, FP32 accumulators in tensor
-// memory. The operands go through two shared-memory stages in the
-// no-swizzle K-major layout of 8-row x 16-byte core matrices (core (r/8,
-// k/8) at (r/8) * 256 + (k/8) * 128 bytes), each stage guarded by an mbarrier
-// that the MMA's commit arrives on. Every wait is bounded in time; a block
-// that gives up sets *err, waits (bounded) for its own MMAs and frees its
-// tensor memory.
-constexpr int kTcM = 128;   // output pixels per tile (MMA M)
-constexpr uint64_t kTcWaitNs = 1000000000ull;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// shared-memory matrix descriptor: start address, leading (K-direction)
-// byte offset 128 and stride (M/N-direction) byte offset 256, all >> 4; the
-// descriptor version bit (46); no swizzle
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
-         ((uint64_t)1 << 46);
-}
-__device__ __forceinline__ int core_off(int r, int k) {
-  return (r >> 3) * 256 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
-// wait until the mbarrier has completed the phase of the given parity, at
-// most until t0 + kTcWaitNs; returns whether it did
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_t t0) {
-  uint32_t done = 0;
-  while (true) {
-    asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
-                 : "=r"(done)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    if (done) return true;
-    if (gtimer() - t0 > kTcWaitNs) return false;
-  }
-}
-__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi) {
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
-// out[b][co][p] = act(bias[co] + sum_ci sum_tap w[co][ci][tap] in[b][ci][p + off_tap])
-// for Co = N output channels; grid (H * W / 128, B), block 128 (thread t
-// gathers the patch of pixel p0 + t and, in the epilogue, reads TMEM lane t).
-// Needs H * W a multiple of 128, Ci a multiple of 8 (16-byte weight pieces)
-// and 16-byte aligned weights.
-template <int N, bool RELU>
-__global__ void __launch_bounds__(kTcM) k_conv3_tc(const __nv_bfloat16 *__restrict__ in, int64_t ibs,
-                                                  const __nv_bfloat16 *__restrict__ w, const float *__restrict__ bias,
-                                                  __nv_bfloat16 *__restrict__ out, int64_t obs, int Ci, int H, int W,
-                                                  int *err) {
-  static_assert(N % 16 == 0 && N >= 16 && N <= 256, "MMA N for M = 128");
-  constexpr int TCOLS = N < 32 ? 32 : N;   // tensor-memory columns: a power of two, at least 32
-  static_assert((TCOLS & (TCOLS - 1)) == 0, "N must be a power of two");
-  __shared__ __align__(1024) unsigned char sA[2][kTcM * 32];
-  __shared__ __align__(1024) unsigned char sB[2][N * 32];
-  __shared__ __align__(8) uint64_t bar[2];
-  __shared__ uint32_t tslot;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int HW = H * W, p = blockIdx.x * kTcM + tid, b = blockIdx.y;
-  const int y = p / W, x = p - y * W;
-  const int K9 = Ci * 9, nch = (K9 + 15) / 16;
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[0])));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar[1])));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tslot)),
-                 "r"(TCOLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = tslot;
-  // instruction descriptor: FP32 accumulators, bfloat16 A and B, both
-  // K-major, N >> 3 at bit 17, M >> 4 at bit 24
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTcM >> 4) << 24);
-  const __nv_bfloat16 *inb = in + (int64_t)b * ibs;
-  // the operands of step j in registers: this pixel's 16 patch values as
-  // bfloat16 pairs, and this thread's 16-byte weight pieces; they are loaded
-  // one step ahead, so that their latency overlaps the previous MMA
-  constexpr int NQ = (2 * N + kTcM - 1) / kTcM;   // weight pieces per thread
-  uint32_t pa[8];
-  uint4 pb[NQ];
-  auto load_step = [&](int j) {
-#pragma unroll
-    for (int e = 0; e < 16; e += 2) {
-      __nv_bfloat16 v2[2];
-#pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const int kk = j * 16 + e + u;
-        __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
-        if (kk < K9) {
-          const int ci = kk / 9, tap = kk - ci * 9;
-          const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-          if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = inb[(int64_t)ci * HW + yy * W + xx];
-        }
-        v2[u] = v;
-      }
-      pa[e / 2] = pack_bf16(v2[0], v2[1]);
-    }
-    // (a piece lies wholly inside or wholly past the row end: 9 Ci is a
-    // multiple of 8)
-#pragma unroll
-    for (int i = 0; i < NQ; i++) {
-      const int q = tid + i * kTcM, kk0 = j * 16 + (q & 1) * 8;
-      pb[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (q < 2 * N && kk0 < K9) pb[i] = *reinterpret_cast<const uint4 *>(w + (int64_t)(q >> 1) * K9 + kk0);
-    }
-  };
-  const uint64_t t0 = gtimer();
-  bool ok = true;
-  int issued = 0;
-  load_step(0);
-  for (int j = 0; j < nch; j++) {
-    const int s = j & 1;
-    // the MMA of step j - 2 read this stage
-    bool late = false;
-    if (j >= 2) late = !mbar_wait(smem_u32(&bar[s]), ((j - 2) >> 1) & 1, t0);
-    if (__syncthreads_or(late)) {
-      ok = false;
-      break;
-    }
-    // A: two 16-byte pieces of this pixel's row; B: this thread's weight pieces
-    *reinterpret_cast<uint4 *>(&sA[s][core_off(tid, 0)]) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
-    *reinterpret_cast<uint4 *>(&sA[s][core_off(tid, 8)]) = make_uint4(pa[4], pa[5], pa[6], pa[7]);
-#pragma unroll
-    for (int i = 0; i < NQ; i++) {
-      const int q = tid + i * kTcM;
-      if (q < 2 * N) *reinterpret_cast<uint4 *>(&sB[s][core_off(q >> 1, (q & 1) * 8)]) = pb[i];
-    }
-    // the stores above are read by the tensor cores (the async proxy)
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      asm volatile(
-          "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-          "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-          "l"(umma_desc(smem_u32(&sA[s][0]))), "l"(umma_desc(smem_u32(&sB[s][0]))), "r"(idesc), "r"(j > 0 ? 1 : 0));
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       smem_u32(&bar[s]))
-                   : "memory");
-    }
-    issued = j + 1;
-    if (j + 1 < nch) load_step(j + 1);
-  }
-  // the last MMA done (its commit also covers every earlier one)
-  bool late = false;
-  if (issued > 0) late = !mbar_wait(smem_u32(&bar[(issued - 1) & 1]), ((issued - 1) >> 1) & 1, gtimer());
-  if (__syncthreads_or(late)) ok = false;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (ok && issued == nch) {
-    // epilogue: warp w reads TMEM lanes 32w.. (pixels), 16 channels at a time
-    __nv_bfloat16 *ob = out + (int64_t)b * obs + p;
-#pragma unroll 1
-    for (int c0 = 0; c0 < N; c0 += 16) {
-      uint32_t r[16];
-      const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(ta));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-      for (int u = 0; u < 16; u++) {
-        float v = __uint_as_float(r[u]) + (bias ? bias[c0 + u] : 0.0f);
-        if (RELU) v = fmaxf(v, 0.0f);
-        ob[(int64_t)(c0 + u) * HW] = __float2bfloat16_rn(v);
-      }
-    }
-  } else if (tid == 0) {
-    atomicOr(err, 1);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
 }
 
 // wt[ci][co][k'] = w[co][ci][K*K - 1 - k'] (FP32): the weights of the
@@ -399,19 +211,36 @@ __global__ void k_relu_mask(float *__restrict__ g, int64_t gbs, const TA *__rest
   if (!(ld(act + b * abs_ + r) > 0.0f)) g[b * gbs + r] = 0.0f;
 }
 
-// 2x2 average pool: out [C][H/2][W/2] from in [C][H][W]
+// two neighbouring values of type T (the first at an even element offset)
 template <typename T>
-__global__ void k_pool(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int C, int H, int W,
-                       int B) {
-  const int Ho = H / 2, Wo = W / 2;
-  const int64_t n = (int64_t)B * C * Ho * Wo;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int x = (int)(i % Wo), y = (int)((i / Wo) % Ho), c = (int)((i / ((int64_t)Wo * Ho)) % C);
-  const int64_t b = i / ((int64_t)Wo * Ho * C);
-  const T *p = in + b * ibs + (int64_t)c * H * W + (int64_t)(2 * y) * W + 2 * x;
-  const float v = 0.25f * (ld(p) + ld(p + 1) + ld(p + W) + ld(p + W + 1));
-  out[b * obs + (int64_t)c * Ho * Wo + (int64_t)y * Wo + x] = st<T>(v);
+struct Pair;
+template <>
+struct Pair<float> {
+  using V = float2;
+  static __device__ __forceinline__ float2 f(V v) { return v; }
+  static __device__ __forceinline__ V both(float x) { return make_float2(x, x); }
+};
+template <>
+struct Pair<__nv_bfloat16> {
+  using V = __nv_bfloat162;
+  static __device__ __forceinline__ float2 f(V v) { return __bfloat1622float2(v); }
+  static __device__ __forceinline__ V both(__nv_bfloat16 x) { return __nv_bfloat162(x, x); }
+};
+
+// 2x2 average pool: out [C][H/2][W/2] from in [C][H][W]; a block per channel
+// and sample, so that no thread divides 64-bit indices (k_up likewise: 44 us
+// -> 6 us for 16 MB written at width 64, 32 x 64, batch 32). Grid (C, B).
+template <typename T>
+__global__ void k_pool(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int H, int W) {
+  const int Ho = H / 2, Wo = W / 2, c = blockIdx.x, b = blockIdx.y;
+  const T *p = in + (int64_t)b * ibs + (int64_t)c * H * W;
+  T *o = out + (int64_t)b * obs + (int64_t)c * Ho * Wo;
+  for (int i = threadIdx.x; i < Ho * Wo; i += blockDim.x) {
+    const int y = i / Wo, x = i - y * Wo;
+    const typename Pair<T>::V *q = reinterpret_cast<const typename Pair<T>::V *>(p + 2 * y * W + 2 * x);
+    const float2 u = Pair<T>::f(q[0]), v = Pair<T>::f(q[W / 2]);
+    o[i] = st<T>(0.25f * (u.x + u.y + v.x + v.y));
+  }
 }
 
 // gradient of the pool: gin[..] += gout / 4 (gin FP32)
@@ -426,17 +255,52 @@ __global__ void k_pool_bwd(const float *__restrict__ gout, int64_t gobs, float *
       0.25f * gout[b * gobs + (int64_t)c * (H / 2) * (W / 2) + (int64_t)(y / 2) * (W / 2) + x / 2];
 }
 
-// 2x nearest upsampling: out [C][2h][2w] from in [C][h][w]
+// 2x nearest upsampling: out [C][2h][2w] from in [C][h][w], a pair of equal
+// values per store. Grid (C, B).
 template <typename T>
-__global__ void k_up(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int C, int h, int w,
-                     int B) {
-  const int64_t n = (int64_t)B * C * 4 * h * w;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int W2 = 2 * w, H2 = 2 * h;
-  const int x = (int)(i % W2), y = (int)((i / W2) % H2), c = (int)((i / ((int64_t)W2 * H2)) % C);
-  const int64_t b = i / ((int64_t)W2 * H2 * C);
-  out[b * obs + (int64_t)c * H2 * W2 + (int64_t)y * W2 + x] = in[b * ibs + (int64_t)c * h * w + (int64_t)(y / 2) * w + x / 2];
+__global__ void k_up(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int h, int w) {
+  const int c = blockIdx.x, b = blockIdx.y;
+  const T *p = in + (int64_t)b * ibs + (int64_t)c * h * w;
+  typename Pair<T>::V *o = reinterpret_cast<typename Pair<T>::V *>(out + (int64_t)b * obs + (int64_t)c * 4 * h * w);
+  for (int i = threadIdx.x; i < h * w; i += blockDim.x) {
+    const int y = i / w, x = i - y * w;
+    const typename Pair<T>::V v = Pair<T>::both(p[i]);
+    o[2 * y * w + x] = v;
+    o[(2 * y + 1) * w + x] = v;
+  }
+}
+
+// The 1x1 head: out[b][co][p] = bias[co] + sum_c w[co][c] in[b][c][p], FP32 out,
+// the channels in order for every output. Bounded by reading the input
+// once; a thread takes two pixels and NCO outputs. grid (ceil(HW / 256), B,
+// ceil(Co / NCO)), block 128; HW even.
+template <typename T, typename TW, int NCO>
+__global__ void __launch_bounds__(128) k_head(const T *__restrict__ in, int64_t ibs, const TW *__restrict__ w,
+                                              const float *__restrict__ bias, float *__restrict__ out, int64_t obs,
+                                              int C, int Co, int HW) {
+  const int b = blockIdx.y, o0 = blockIdx.z * NCO, p = (blockIdx.x * 128 + threadIdx.x) * 2;
+  if (p >= HW) return;
+  const T *ib = in + (int64_t)b * ibs + p;
+  float2 acc[NCO];
+#pragma unroll
+  for (int o = 0; o < NCO; o++) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll 8
+  for (int c = 0; c < C; c++) {
+    const float2 v = Pair<T>::f(*reinterpret_cast<const typename Pair<T>::V *>(ib + (int64_t)c * HW));
+#pragma unroll
+    for (int o = 0; o < NCO; o++) {
+      const float wv = o0 + o < Co ? ld(w + (int64_t)(o0 + o) * C + c) : 0.0f;
+      acc[o].x = fmaf(v.x, wv, acc[o].x);
+      acc[o].y = fmaf(v.y, wv, acc[o].y);
+    }
+  }
+#pragma unroll
+  for (int o = 0; o < NCO; o++) {
+    if (o0 + o >= Co) break;
+    float *q = out + (int64_t)b * obs + (int64_t)(o0 + o) * HW + p;
+    q[0] = acc[o].x + bias[o0 + o];
+    q[1] = acc[o].y + bias[o0 + o];
+  }
 }
 
 // gradient of the upsampling: gin[c][y][x] = sum of the four children (assigns)
@@ -465,15 +329,6 @@ __global__ void k_convert_into(const float *__restrict__ src, int64_t sbs, TO *_
   if (i >= CHW * B) return;
   const int64_t b = i / CHW, r = i % CHW;
   dst[b * dbs + r] = st<TO>(src[b * sbs + r]);
-}
-
-// dst[b][r] += src[b][r] for a channel block (between views)
-__global__ void k_add_into(const float *__restrict__ src, int64_t sbs, float *__restrict__ dst, int64_t dbs, int64_t CHW,
-                           int B) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= CHW * B) return;
-  const int64_t b = i / CHW, r = i % CHW;
-  dst[b * dbs + r] += src[b * sbs + r];
 }
 
 // mean-square loss: partial sums per block and dy = 2 (y - t) / n
@@ -548,8 +403,17 @@ struct vlb_nn {
   double *lossp = nullptr;
   int64_t act_n = 0, wt_n = 0, dwp_n = 0;
   int nsplit = 16;
-  int *d_err = nullptr;      // set by a tensor-core convolution that gave up waiting
-  int tc = 1;                // 3x3 forward convolutions in bfloat16 on the tensor cores where they fit
+  int *d_err = nullptr;      // set by a tensor-core kernel that gave up waiting
+  int tc = 1;                // bfloat16 3x3 convolutions on the tensor cores where they fit
+  // tensor-core layers: packed weights (forward and backward offsets per
+  // layer, -1 where the layer does not fit), the planes of one layer's output
+  // gradient and the bias and head gradients' partial sums
+  nn::bf16 *wp = nullptr;
+  nn::bf16 *planes = nullptr;
+  float *bsum = nullptr, *hp = nullptr;
+  int64_t wp_n = 0, planes_n = 0;
+  int64_t fwd_off[11], bwd_off[11];
+  int nsm = 152;
   // activation views (offsets in act / gr), per sample sizes
   View x_in, e1, c1, s1, p1, e2, c2, s2, p2, e3, b3, d2, t2, d1, t1;
 };
@@ -565,40 +429,103 @@ namespace {
   } while (0)
 
 // the tensor-core form of a 3x3 layer (bfloat16 storage): Co a power of two
-// in [16, 256], H * W a multiple of 128, Ci a multiple of 8 and the layer's
-// weights 16-byte aligned
-inline bool tc_fits(const vlb_nn *n, const NNLayer &l) {
+// in [16, 256], H * W a multiple of 128 (whole tiles of MMA rows; it also
+// puts every view of the level on a multiple of 8 elements) and Ci a
+// multiple of 8
+inline bool tc_shape(const vlb_nn *n, const NNLayer &l) {
   const bool pow2 = l.cout >= 16 && l.cout <= 256 && (l.cout & (l.cout - 1)) == 0;
-  // (16-byte weight pieces: the layer's weights start on a multiple of 8 elements)
-  return n->tc && n->storage == VLB_NN_BF16 && l.k == 3 && pow2 && ((int64_t)l.h * l.w) % nn::kTcM == 0 &&
-         l.cin % 8 == 0 && l.woff % 8 == 0;
+  return n->storage == VLB_NN_BF16 && l.k == 3 && pow2 && ((int64_t)l.h * l.w) % nn::kTcM == 0 && l.cin % 8 == 0;
+}
+// its backward pass: pixel groups of 8 within a row, the positions a tap
+// reaches within a block's shared memory, positions in 32 bits
+inline bool tc_bwd_shape(const vlb_nn *n, const NNLayer &l) {
+  return tc_shape(n, l) && l.w % 8 == 0 && l.w <= 256 &&
+         (int64_t)n->maxb * (l.h + 1) * (l.w + 1) < ((int64_t)1 << 30);
 }
 
-template <int N>
-void launch_tc(const vlb_nn *n, const NNLayer &l, const __nv_bfloat16 *in, int64_t ibs, const __nv_bfloat16 *w,
-               const float *bias, __nv_bfloat16 *out, int64_t obs, bool relu, int B) {
-  const dim3 grid((unsigned)((int64_t)l.h * l.w / nn::kTcM), (unsigned)B);
-  if (relu)
-    nn::k_conv3_tc<N, true><<<grid, nn::kTcM>>>(in, ibs, w, bias, out, obs, l.cin, l.h, l.w, n->d_err);
-  else
-    nn::k_conv3_tc<N, false><<<grid, nn::kTcM>>>(in, ibs, w, bias, out, obs, l.cin, l.h, l.w, n->d_err);
+// Rows of the weight operand per block: the patch matrix is formed once per
+// block, so as many as fit, but fewer where that leaves SMs without a block
+// (coarse grids, small batches)
+inline int pick_nb(const vlb_nn *n, int co, int64_t tiles, int most) {
+  const int cand[5] = {128, 64, 48, 32, 16};
+  int nb = 16;
+  for (int c : cand)
+    if (c <= most && co % c == 0) {
+      nb = c;
+      if (tiles * (co / c) >= n->nsm * 2 / 3) break;
+    }
+  return nb;
+}
+
+template <int NB, bool RELU, bool EVENW>
+cudaError_t launch_conv_mma(const vlb_nn *n, const NNLayer &l, const nn::bf16 *in, int64_t ibs, const nn::bf16 *wp,
+                            const float *bias, nn::bf16 *out, int64_t obs, int B) {
+  constexpr int smem = 2 * nn::kTcABytes + 2 * nn::kTcKG * NB * 16;
+  auto kern = nn::k_conv3_mma<NB, RELU, EVENW>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((int64_t)l.h * l.w / nn::kTcM), (unsigned)(l.cout / NB), (unsigned)B);
+  kern<<<grid, 128, smem>>>(in, ibs, l.cin, wp, l.cout, bias, out, obs, l.h, l.w, n->d_err);
+  return cudaGetLastError();
+}
+template <bool RELU>
+cudaError_t conv_mma(const vlb_nn *n, const NNLayer &l, const nn::bf16 *in, int64_t ibs, const nn::bf16 *wp,
+                     const float *bias, nn::bf16 *out, int64_t obs, int B) {
+  auto go = [&](auto nb, auto even) {
+    return launch_conv_mma<decltype(nb)::value, RELU, decltype(even)::value>(n, l, in, ibs, wp, bias, out, obs, B);
+  };
+  const std::true_type even;
+  if (l.w % 2) return go(std::integral_constant<int, 16>(), std::false_type());   // rows of odd width: 16-bit gathers
+  switch (pick_nb(n, l.cout, (int64_t)l.h * l.w / nn::kTcM * B, 128)) {
+    case 128: return go(std::integral_constant<int, 128>(), even);
+    case 64: return go(std::integral_constant<int, 64>(), even);
+    case 32: return go(std::integral_constant<int, 32>(), even);
+    default: return go(std::integral_constant<int, 16>(), even);
+  }
+}
+
+template <int NB>
+cudaError_t launch_dgrad(const vlb_nn *n, const NNLayer &l, int64_t plane, int64_t npos, const nn::bf16 *wp, float *out,
+                         int64_t obs, int B, int tiles) {
+  const int stage = nn::dg_stage_bytes(NB, l.w);
+  // two blocks per SM where two stages of each fit
+  int nst = 112 * 1024 / stage;
+  nst = nst < 2 ? 2 : nst > nn::kDgMaxStages ? nn::kDgMaxStages : nst;
+  auto kern = nn::k_dgrad_mma<NB>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, nst * stage);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3((unsigned)tiles, (unsigned)(l.cin / NB)), 192, nst * stage>>>(n->planes, plane, npos, l.cout, wp, l.cin,
+                                                                            out, obs, l.h, l.w, B, nst, n->d_err);
+  return cudaGetLastError();
+}
+
+template <int CB, int NBK>
+cudaError_t launch_wgrad_t(const NNLayer &l, const nn::bf16 *in, int64_t ibs, const nn::bf16 *g, int64_t npos,
+                           int64_t plane, float *dwp, int ngrp, int nsplit, int B, int *err) {
+  constexpr int smem = 2 * (nn::wg_sets(CB) * nn::kWgA + NBK * nn::kWgB);
+  auto kern = nn::k_wgrad_mma<CB, NBK>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)(l.cout / CB * ngrp), (unsigned)nsplit);
+  kern<<<grid, 256, smem>>>(in, ibs, l.cin, g, npos, plane, l.cout, dwp, l.h, l.w, B, ngrp, err);
+  return cudaGetLastError();
+}
+template <int CB>
+cudaError_t launch_wgrad(const NNLayer &l, const nn::bf16 *in, int64_t ibs, const nn::bf16 *g, int64_t npos,
+                         int64_t plane, float *dwp, int nb, int ngrp, int nsplit, int B, int *err) {
+  return nb == 2 ? launch_wgrad_t<CB, 2>(l, in, ibs, g, npos, plane, dwp, ngrp, nsplit, B, err)
+                 : launch_wgrad_t<CB, 1>(l, in, ibs, g, npos, plane, dwp, ngrp, nsplit, B, err);
 }
 
 template <typename T>
 int conv(const vlb_nn *n, const NNLayer &l, const T *in, int64_t ibs, const void *w, const float *bias, void *out,
-         int64_t obs, bool relu, bool out_f32, int B) {
+         int64_t obs, bool relu, int B) {
   if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-    if (tc_fits(n, l)) {
-      const __nv_bfloat16 *wb = static_cast<const __nv_bfloat16 *>(w);
-      __nv_bfloat16 *ob = static_cast<__nv_bfloat16 *>(out);
-      switch (l.cout) {
-        case 16: launch_tc<16>(n, l, in, ibs, wb, bias, ob, obs, relu, B); break;
-        case 32: launch_tc<32>(n, l, in, ibs, wb, bias, ob, obs, relu, B); break;
-        case 64: launch_tc<64>(n, l, in, ibs, wb, bias, ob, obs, relu, B); break;
-        case 128: launch_tc<128>(n, l, in, ibs, wb, bias, ob, obs, relu, B); break;
-        default: launch_tc<256>(n, l, in, ibs, wb, bias, ob, obs, relu, B); break;
-      }
-      NN_CU(cudaGetLastError());
+    const int64_t wo = n->fwd_off[&l - n->L.data()];
+    if (n->tc && wo >= 0) {
+      T *ob = static_cast<T *>(out);
+      NN_CU(relu ? conv_mma<true>(n, l, in, ibs, n->wp + wo, bias, ob, obs, B)
+                 : conv_mma<false>(n, l, in, ibs, n->wp + wo, bias, ob, obs, B));
       return VLB_OK;
     }
   }
@@ -623,14 +550,15 @@ int conv(const vlb_nn *n, const NNLayer &l, const T *in, int64_t ibs, const void
     }
   } else {
     // the 1x1 head writes FP32 outputs
+    constexpr int NCO = 4;
+    const int HW = l.h * l.w;
+    const dim3 hg((unsigned)((HW + 255) / 256), (unsigned)B, (unsigned)((l.cout + NCO - 1) / NCO));
     if (bf)
-      nn::k_conv<1, T, __nv_bfloat16, float, false><<<grid, nn::kThreads>>>(
-          in, ibs, (const __nv_bfloat16 *)w, bias, (float *)out, obs, l.cin, l.cout, l.h, l.w);
+      nn::k_head<T, __nv_bfloat16, NCO><<<hg, 128>>>(in, ibs, (const __nv_bfloat16 *)w, bias, (float *)out, obs, l.cin,
+                                                    l.cout, HW);
     else
-      nn::k_conv<1, T, float, float, false><<<grid, nn::kThreads>>>(in, ibs, (const float *)w, bias, (float *)out,
-                                                                   obs, l.cin, l.cout, l.h, l.w);
+      nn::k_head<T, float, NCO><<<hg, 128>>>(in, ibs, (const float *)w, bias, (float *)out, obs, l.cin, l.cout, HW);
   }
-  (void)out_f32;
   NN_CU(cudaGetLastError());
   return VLB_OK;
 }
@@ -689,6 +617,17 @@ int relu_mask(float *g, int64_t gbs, const T *act, int64_t abs_, int C, int H, i
     if (rc_) return rc_;   \
   } while (0)
 
+// wait for the stream and report a tensor-core kernel that gave up waiting
+int finish(vlb_nn *n, const char *what) {
+  int err = 0;
+  NN_CU(cudaMemcpy(&err, n->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (err) {
+    cudaMemset(n->d_err, 0, sizeof(int));
+    return vlb::set_error(VLB_ECUDA, "%s: a tensor-core convolution gave up waiting for its MMAs", what);
+  }
+  return VLB_OK;
+}
+
 template <typename T>
 int forward_t(vlb_nn *n, const float *d_x, float *d_y, int B) {
   T *A = static_cast<T *>(n->act);
@@ -703,113 +642,188 @@ int forward_t(vlb_nn *n, const float *d_x, float *d_y, int B) {
   const int64_t chw = (int64_t)n->ci * H * W;
   nn::k_convert_into<T><<<nn::nblk(chw * B), 256>>>(d_x, chw, A + n->x_in.off, n->x_in.bs, chw, B);
   NN_CU(cudaGetLastError());
-  NN_TRY(conv<T>(n, L[0], A + n->x_in.off, n->x_in.bs, wp(L[0]), n->p + L[0].boff, A + n->e1.off, n->e1.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[1], A + n->e1.off, n->e1.bs, wp(L[1]), n->p + L[1].boff, A + n->s1.off, n->s1.bs, true, false, B));
-  nn::k_pool<T><<<nn::nblk((int64_t)B * w * H2 * W2), 256>>>(A + n->s1.off, n->s1.bs, A + n->p1.off, n->p1.bs, w, H, W, B);
+  NN_TRY(conv<T>(n, L[0], A + n->x_in.off, n->x_in.bs, wp(L[0]), n->p + L[0].boff, A + n->e1.off, n->e1.bs, true, B));
+  NN_TRY(conv<T>(n, L[1], A + n->e1.off, n->e1.bs, wp(L[1]), n->p + L[1].boff, A + n->s1.off, n->s1.bs, true, B));
+  nn::k_pool<T><<<dim3((unsigned)w, (unsigned)B), 256>>>(A + n->s1.off, n->s1.bs, A + n->p1.off, n->p1.bs, H, W);
   NN_CU(cudaGetLastError());
-  NN_TRY(conv<T>(n, L[2], A + n->p1.off, n->p1.bs, wp(L[2]), n->p + L[2].boff, A + n->e2.off, n->e2.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[3], A + n->e2.off, n->e2.bs, wp(L[3]), n->p + L[3].boff, A + n->s2.off, n->s2.bs, true, false, B));
-  nn::k_pool<T><<<nn::nblk((int64_t)B * 2 * w * H4 * W4), 256>>>(A + n->s2.off, n->s2.bs, A + n->p2.off, n->p2.bs, 2 * w,
-                                                                  H2, W2, B);
+  NN_TRY(conv<T>(n, L[2], A + n->p1.off, n->p1.bs, wp(L[2]), n->p + L[2].boff, A + n->e2.off, n->e2.bs, true, B));
+  NN_TRY(conv<T>(n, L[3], A + n->e2.off, n->e2.bs, wp(L[3]), n->p + L[3].boff, A + n->s2.off, n->s2.bs, true, B));
+  nn::k_pool<T><<<dim3((unsigned)(2 * w), (unsigned)B), 128>>>(A + n->s2.off, n->s2.bs, A + n->p2.off, n->p2.bs, H2, W2);
   NN_CU(cudaGetLastError());
-  NN_TRY(conv<T>(n, L[4], A + n->p2.off, n->p2.bs, wp(L[4]), n->p + L[4].boff, A + n->e3.off, n->e3.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[5], A + n->e3.off, n->e3.bs, wp(L[5]), n->p + L[5].boff, A + n->b3.off, n->b3.bs, true, false, B));
+  NN_TRY(conv<T>(n, L[4], A + n->p2.off, n->p2.bs, wp(L[4]), n->p + L[4].boff, A + n->e3.off, n->e3.bs, true, B));
+  NN_TRY(conv<T>(n, L[5], A + n->e3.off, n->e3.bs, wp(L[5]), n->p + L[5].boff, A + n->b3.off, n->b3.bs, true, B));
   // c2 = [up(b3), s2]: s2 already sits in its slice
-  nn::k_up<T><<<nn::nblk((int64_t)B * 4 * w * H2 * W2), 256>>>(A + n->b3.off, n->b3.bs, A + n->c2.off, n->c2.bs, 4 * w,
-                                                                H4, W4, B);
+  nn::k_up<T><<<dim3((unsigned)(4 * w), (unsigned)B), 128>>>(A + n->b3.off, n->b3.bs, A + n->c2.off, n->c2.bs, H4, W4);
   NN_CU(cudaGetLastError());
-  NN_TRY(conv<T>(n, L[6], A + n->c2.off, n->c2.bs, wp(L[6]), n->p + L[6].boff, A + n->d2.off, n->d2.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[7], A + n->d2.off, n->d2.bs, wp(L[7]), n->p + L[7].boff, A + n->t2.off, n->t2.bs, true, false, B));
-  nn::k_up<T><<<nn::nblk((int64_t)B * 2 * w * H * W), 256>>>(A + n->t2.off, n->t2.bs, A + n->c1.off, n->c1.bs, 2 * w, H2,
-                                                              W2, B);
+  NN_TRY(conv<T>(n, L[6], A + n->c2.off, n->c2.bs, wp(L[6]), n->p + L[6].boff, A + n->d2.off, n->d2.bs, true, B));
+  NN_TRY(conv<T>(n, L[7], A + n->d2.off, n->d2.bs, wp(L[7]), n->p + L[7].boff, A + n->t2.off, n->t2.bs, true, B));
+  nn::k_up<T><<<dim3((unsigned)(2 * w), (unsigned)B), 256>>>(A + n->t2.off, n->t2.bs, A + n->c1.off, n->c1.bs, H2, W2);
   NN_CU(cudaGetLastError());
-  NN_TRY(conv<T>(n, L[8], A + n->c1.off, n->c1.bs, wp(L[8]), n->p + L[8].boff, A + n->d1.off, n->d1.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[9], A + n->d1.off, n->d1.bs, wp(L[9]), n->p + L[9].boff, A + n->t1.off, n->t1.bs, true, false, B));
-  NN_TRY(conv<T>(n, L[10], A + n->t1.off, n->t1.bs, wp(L[10]), n->p + L[10].boff, d_y, (int64_t)n->co * H * W, false,
-                 true, B));
-  NN_CU(cudaDeviceSynchronize());
-  int err = 0;
-  NN_CU(cudaMemcpy(&err, n->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
-    cudaMemset(n->d_err, 0, sizeof(int));
-    return vlb::set_error(VLB_ECUDA, "vlb_nn_forward: a tensor-core convolution gave up waiting for its MMAs");
+  NN_TRY(conv<T>(n, L[8], A + n->c1.off, n->c1.bs, wp(L[8]), n->p + L[8].boff, A + n->d1.off, n->d1.bs, true, B));
+  NN_TRY(conv<T>(n, L[9], A + n->d1.off, n->d1.bs, wp(L[9]), n->p + L[9].boff, A + n->t1.off, n->t1.bs, true, B));
+  NN_TRY(conv<T>(n, L[10], A + n->t1.off, n->t1.bs, wp(L[10]), n->p + L[10].boff, d_y, (int64_t)n->co * H * W, false, B));
+  return finish(n, "vlb_nn_forward");
+}
+
+// Where the gradient of a layer's output comes from: its own slot of the
+// gradient buffer (mode 0), the four children of g below an upsampling
+// (mode 1; h x w of the layer's own grid), or its slot plus the gradient gp
+// of its 2x2 pool (mode 2)
+struct GradSrc {
+  int mode;
+  View g, gp;
+};
+
+// blocks of the kernels that form a layer's planes, per 8 channels: about
+// eight per SM over all of them (their partial sums are added one after another)
+inline int plane_blocks(const vlb_nn *n, int c, int64_t npos) {
+  const int64_t want = std::max<int64_t>(1, (int64_t)n->nsm * 8 / (c / 8));
+  return (int)std::min<int64_t>(want, (npos + 127) / 128);
+}
+
+// Backward pass of one 3x3 layer: its weight and bias gradients and, unless
+// gin is NULL, the gradient of its input. out: its output (activation and
+// gradient slot). split: its output's gradient planes and bias sums are
+// there already (from the head).
+template <typename T>
+int layer_backward(vlb_nn *n, int li, View in, View out, const GradSrc &src, const View *gin, bool split, int B) {
+  const NNLayer &l = n->L[li];
+  const T *A = static_cast<const T *>(n->act);
+  float *G = n->gr;
+  const int64_t hw = (int64_t)l.h * l.w;
+  if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+    if (n->tc && n->bwd_off[li] >= 0) {
+      const nn::Padded pad{l.h, l.w, B};
+      const int64_t npos = pad.positions(), plane = npos * l.cout;
+      const int blocks = plane_blocks(n, l.cout, npos);
+      if (!split) {
+        const dim3 grid((unsigned)blocks, (unsigned)(l.cout / 8));
+        const T *act = A + out.off;
+        auto launch = [&](auto kern) {
+          kern<<<grid, 128>>>(G + src.g.off, src.g.bs, G + src.gp.off, src.gp.bs, act, out.bs, n->planes, plane,
+                              (int)npos, n->bsum, l.h, l.w, B);
+        };
+        if (src.mode == 0)
+          launch(nn::k_mask_split<0>);
+        else if (src.mode == 1)
+          launch(nn::k_mask_split<1>);
+        else
+          launch(nn::k_mask_split<2>);
+        NN_CU(cudaGetLastError());
+      }
+      // weights: groups of 32 or 16 input channels per block (the gradient rows
+      // are read once per group), splits to fill the SMs
+      const int cb = l.cout < 128 ? l.cout : 128, nci = (l.cin + 15) / 16;
+      const int nb = nci % 2 == 0 ? 2 : 1, ngrp = nci / nb;
+      const int64_t nw = (int64_t)l.cin * l.cout * 9, tiles = (int64_t)(l.cout / cb) * ngrp;
+      int64_t nsplit = std::min<int64_t>(n->nsm / tiles, (int64_t)B * (hw / 64));
+      nsplit = std::max<int64_t>(1, std::min<int64_t>(nsplit, n->dwp_n / (nw * nn::wg_groups(cb))));
+      const T *x = A + in.off;
+      const int nbk = nb, ng = ngrp, ns = (int)nsplit;
+      switch (cb) {
+        case 16: NN_CU(launch_wgrad<16>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
+        case 32: NN_CU(launch_wgrad<32>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
+        case 64: NN_CU(launch_wgrad<64>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
+        default: NN_CU(launch_wgrad<128>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
+      }
+      nn::k_sum_parts<<<nn::nblk(nw + l.cout), 256>>>(n->dwp, ns * nn::wg_groups(cb), nw, n->bsum, blocks, l.cout,
+                                                      n->g + l.woff);
+      NN_CU(cudaGetLastError());
+      if (gin) {
+        float *o = G + gin->off;
+        const nn::bf16 *wt = n->wp + n->bwd_off[li];
+        const int tiles = pad.tiles();
+        switch (pick_nb(n, l.cin, tiles, 64)) {
+          case 64: NN_CU(launch_dgrad<64>(n, l, plane, npos, wt, o, gin->bs, B, tiles)); break;
+          case 48: NN_CU(launch_dgrad<48>(n, l, plane, npos, wt, o, gin->bs, B, tiles)); break;
+          case 32: NN_CU(launch_dgrad<32>(n, l, plane, npos, wt, o, gin->bs, B, tiles)); break;
+          default: NN_CU(launch_dgrad<16>(n, l, plane, npos, wt, o, gin->bs, B, tiles)); break;
+        }
+      }
+      return VLB_OK;
+    }
   }
+  if (src.mode == 1)
+    nn::k_up_bwd<<<nn::nblk((int64_t)B * l.cout * hw), 256>>>(G + src.g.off, src.g.bs, G + out.off, out.bs, l.cout, l.h,
+                                                              l.w, B);
+  if (src.mode == 2)
+    nn::k_pool_bwd<<<nn::nblk((int64_t)B * l.cout * hw), 256>>>(G + src.gp.off, src.gp.bs, G + out.off, out.bs, l.cout,
+                                                                l.h, l.w, B);
+  NN_CU(cudaGetLastError());
+  NN_TRY(relu_mask<T>(G + out.off, out.bs, A + out.off, out.bs, l.cout, l.h, l.w, B));
+  NN_TRY(conv_bwd_weight<T>(n, l, A + in.off, in.bs, G + out.off, out.bs, B));
+  if (gin) NN_TRY(conv_bwd_data(n, l, G + out.off, out.bs, G + gin->off, gin->bs, B));
   return VLB_OK;
+}
+
+template <int NCO>
+void launch_head_bwd(vlb_nn *n, const float *d_dy, int64_t ybs, int B) {
+  const NNLayer &l = n->L[10];
+  const int64_t npos = nn::Padded{l.h, l.w, B}.positions();
+  nn::k_head_bwd<NCO><<<dim3((unsigned)plane_blocks(n, l.cin, npos), (unsigned)(l.cin / 8)), 128>>>(
+      d_dy, ybs, (const __nv_bfloat16 *)n->pc + l.woff, (const __nv_bfloat16 *)n->act + n->t1.off, n->t1.bs, n->planes,
+      npos * l.cin, (int)npos, n->bsum, n->hp, l.h, l.w, B);
 }
 
 template <typename T>
 int backward_t(vlb_nn *n, const float *d_dy, int B) {
   const T *A = static_cast<const T *>(n->act);
   float *G = n->gr;
-  const int w = n->width, H = n->H, W = n->W, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
   const auto &L = n->L;
-  const int64_t ybs = (int64_t)n->co * H * W;
-  NN_CU(cudaMemset(G, 0, sizeof(float) * n->act_n));
-  // head
-  NN_TRY(conv_bwd_weight<T>(n, L[10], A + n->t1.off, n->t1.bs, d_dy, ybs, B));
-  NN_TRY(conv_bwd_data(n, L[10], d_dy, ybs, G + n->t1.off, n->t1.bs, B));
-  // t1 = relu(conv(d1))
-  NN_TRY(relu_mask<T>(G + n->t1.off, n->t1.bs, A + n->t1.off, n->t1.bs, w, H, W, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[9], A + n->d1.off, n->d1.bs, G + n->t1.off, n->t1.bs, B));
-  NN_TRY(conv_bwd_data(n, L[9], G + n->t1.off, n->t1.bs, G + n->d1.off, n->d1.bs, B));
-  // d1 = relu(conv(c1))
-  NN_TRY(relu_mask<T>(G + n->d1.off, n->d1.bs, A + n->d1.off, n->d1.bs, w, H, W, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[8], A + n->c1.off, n->c1.bs, G + n->d1.off, n->d1.bs, B));
-  NN_TRY(conv_bwd_data(n, L[8], G + n->d1.off, n->d1.bs, G + n->c1.off, n->c1.bs, B));
+  const int64_t ybs = (int64_t)n->co * n->H * n->W;
+  // the head: every gradient slot below is written before it is read
+  const bool head = n->tc && n->bwd_off[9] >= 0 && n->co <= 4;
+  if (head) {
+    switch (n->co) {
+      case 1: launch_head_bwd<1>(n, d_dy, ybs, B); break;
+      case 2: launch_head_bwd<2>(n, d_dy, ybs, B); break;
+      case 3: launch_head_bwd<3>(n, d_dy, ybs, B); break;
+      default: launch_head_bwd<4>(n, d_dy, ybs, B);
+    }
+    NN_CU(cudaGetLastError());
+    const int64_t nw = (int64_t)n->co * L[10].cin + n->co;
+    nn::k_sum_parts<<<nn::nblk(nw), 256>>>(n->hp, plane_blocks(n, L[10].cin, nn::Padded{n->H, n->W, B}.positions()), nw,
+                                           nullptr, 0, 0, n->g + L[10].woff);
+    NN_CU(cudaGetLastError());
+  } else {
+    NN_TRY(conv_bwd_weight<T>(n, L[10], A + n->t1.off, n->t1.bs, d_dy, ybs, B));
+    NN_TRY(conv_bwd_data(n, L[10], d_dy, ybs, G + n->t1.off, n->t1.bs, B));
+  }
+  auto own = [](View v) { return GradSrc{0, v, v}; };
+  // t1 = relu(conv(d1)), d1 = relu(conv(c1))
+  NN_TRY(layer_backward<T>(n, 9, n->d1, n->t1, own(n->t1), &n->d1, head, B));
+  NN_TRY(layer_backward<T>(n, 8, n->c1, n->d1, own(n->d1), &n->c1, false, B));
   // c1 = [up(t2), s1]: gradient of t2 from the first 2w channels; s1's part stays in its slice
-  nn::k_up_bwd<<<nn::nblk((int64_t)B * 2 * w * H2 * W2), 256>>>(G + n->c1.off, n->c1.bs, G + n->t2.off, n->t2.bs, 2 * w,
-                                                                 H2, W2, B);
-  NN_CU(cudaGetLastError());
-  // t2 = relu(conv(d2))
-  NN_TRY(relu_mask<T>(G + n->t2.off, n->t2.bs, A + n->t2.off, n->t2.bs, 2 * w, H2, W2, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[7], A + n->d2.off, n->d2.bs, G + n->t2.off, n->t2.bs, B));
-  NN_TRY(conv_bwd_data(n, L[7], G + n->t2.off, n->t2.bs, G + n->d2.off, n->d2.bs, B));
-  // d2 = relu(conv(c2))
-  NN_TRY(relu_mask<T>(G + n->d2.off, n->d2.bs, A + n->d2.off, n->d2.bs, 2 * w, H2, W2, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[6], A + n->c2.off, n->c2.bs, G + n->d2.off, n->d2.bs, B));
-  NN_TRY(conv_bwd_data(n, L[6], G + n->d2.off, n->d2.bs, G + n->c2.off, n->c2.bs, B));
+  NN_TRY(layer_backward<T>(n, 7, n->d2, n->t2, GradSrc{1, n->c1, n->c1}, &n->d2, false, B));
+  NN_TRY(layer_backward<T>(n, 6, n->c2, n->d2, own(n->d2), &n->c2, false, B));
   // c2 = [up(b3), s2]
-  nn::k_up_bwd<<<nn::nblk((int64_t)B * 4 * w * H4 * W4), 256>>>(G + n->c2.off, n->c2.bs, G + n->b3.off, n->b3.bs, 4 * w,
-                                                                 H4, W4, B);
-  NN_CU(cudaGetLastError());
-  // b3 = relu(conv(e3))
-  NN_TRY(relu_mask<T>(G + n->b3.off, n->b3.bs, A + n->b3.off, n->b3.bs, 4 * w, H4, W4, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[5], A + n->e3.off, n->e3.bs, G + n->b3.off, n->b3.bs, B));
-  NN_TRY(conv_bwd_data(n, L[5], G + n->b3.off, n->b3.bs, G + n->e3.off, n->e3.bs, B));
-  // e3 = relu(conv(p2))
-  NN_TRY(relu_mask<T>(G + n->e3.off, n->e3.bs, A + n->e3.off, n->e3.bs, 4 * w, H4, W4, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[4], A + n->p2.off, n->p2.bs, G + n->e3.off, n->e3.bs, B));
-  NN_TRY(conv_bwd_data(n, L[4], G + n->e3.off, n->e3.bs, G + n->p2.off, n->p2.bs, B));
-  // p2 = pool(s2): add into s2's gradient (its slice of c2)
-  nn::k_pool_bwd<<<nn::nblk((int64_t)B * 2 * w * H2 * W2), 256>>>(G + n->p2.off, n->p2.bs, G + n->s2.off, n->s2.bs,
-                                                                   2 * w, H2, W2, B);
-  NN_CU(cudaGetLastError());
-  // s2 = relu(conv(e2))
-  NN_TRY(relu_mask<T>(G + n->s2.off, n->s2.bs, A + n->s2.off, n->s2.bs, 2 * w, H2, W2, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[3], A + n->e2.off, n->e2.bs, G + n->s2.off, n->s2.bs, B));
-  NN_TRY(conv_bwd_data(n, L[3], G + n->s2.off, n->s2.bs, G + n->e2.off, n->e2.bs, B));
-  // e2 = relu(conv(p1))
-  NN_TRY(relu_mask<T>(G + n->e2.off, n->e2.bs, A + n->e2.off, n->e2.bs, 2 * w, H2, W2, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[2], A + n->p1.off, n->p1.bs, G + n->e2.off, n->e2.bs, B));
-  NN_TRY(conv_bwd_data(n, L[2], G + n->e2.off, n->e2.bs, G + n->p1.off, n->p1.bs, B));
+  NN_TRY(layer_backward<T>(n, 5, n->e3, n->b3, GradSrc{1, n->c2, n->c2}, &n->e3, false, B));
+  NN_TRY(layer_backward<T>(n, 4, n->p2, n->e3, own(n->e3), &n->p2, false, B));
+  // p2 = pool(s2): adds to s2's gradient (its slice of c2)
+  NN_TRY(layer_backward<T>(n, 3, n->e2, n->s2, GradSrc{2, n->s2, n->p2}, &n->e2, false, B));
+  NN_TRY(layer_backward<T>(n, 2, n->p1, n->e2, own(n->e2), &n->p1, false, B));
   // p1 = pool(s1)
-  nn::k_pool_bwd<<<nn::nblk((int64_t)B * w * H * W), 256>>>(G + n->p1.off, n->p1.bs, G + n->s1.off, n->s1.bs, w, H, W, B);
-  NN_CU(cudaGetLastError());
-  // s1 = relu(conv(e1))
-  NN_TRY(relu_mask<T>(G + n->s1.off, n->s1.bs, A + n->s1.off, n->s1.bs, w, H, W, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[1], A + n->e1.off, n->e1.bs, G + n->s1.off, n->s1.bs, B));
-  NN_TRY(conv_bwd_data(n, L[1], G + n->s1.off, n->s1.bs, G + n->e1.off, n->e1.bs, B));
-  // e1 = relu(conv(x))
-  NN_TRY(relu_mask<T>(G + n->e1.off, n->e1.bs, A + n->e1.off, n->e1.bs, w, H, W, B));
-  NN_TRY(conv_bwd_weight<T>(n, L[0], A + n->x_in.off, n->x_in.bs, G + n->e1.off, n->e1.bs, B));
-  NN_CU(cudaDeviceSynchronize());
-  return VLB_OK;
+  NN_TRY(layer_backward<T>(n, 1, n->e1, n->s1, GradSrc{2, n->s1, n->p1}, &n->e1, false, B));
+  NN_TRY(layer_backward<T>(n, 0, n->x_in, n->e1, own(n->e1), nullptr, false, B));
+  return finish(n, "vlb_nn_backward");
 }
 
 int refresh_compute_copy(vlb_nn *n) {
   if (n->storage != VLB_NN_BF16) return VLB_OK;
   nn::k_convert<__nv_bfloat16><<<nn::nblk(n->np), 256>>>(n->p, (__nv_bfloat16 *)n->pc, n->np);
   NN_CU(cudaGetLastError());
+  if (n->wp) {
+    nn::PackTable t;
+    t.n = 10;
+    int most = 1;
+    for (int i = 0; i < 10; i++) {
+      const NNLayer &l = n->L[i];
+      t.l[i] = nn::PackLayer{l.cin, l.cout, l.woff, n->fwd_off[i], n->bwd_off[i]};
+      most = std::max(most, (std::max(l.cin, l.cout) + 15) / 16);
+    }
+    nn::k_pack_weights<<<dim3((unsigned)(most * 16), 20), 256>>>(n->p, n->wp, t);
+    NN_CU(cudaGetLastError());
+  }
   return VLB_OK;
 }
 
@@ -883,7 +897,35 @@ int vlb_nn_create(int32_t in_ch, int32_t out_ch, int32_t width, int32_t H, int32
   n->wt_n = wmax;
   n->dwp_n = dwmax * n->nsplit;
   const size_t es = storage == VLB_NN_BF16 ? 2 : 4;
+  // tensor-core layers: packed weights and the largest layer's gradient planes
+  auto steps = [](int c) { return (int64_t)((c + nn::kTcCh - 1) / nn::kTcCh) * nn::kTcKG * 8; };
+  for (int i = 0; i < 11; i++) {
+    const NNLayer &l = n->L[i];
+    n->fwd_off[i] = n->bwd_off[i] = -1;
+    if (tc_shape(n, l)) {
+      n->fwd_off[i] = n->wp_n;
+      n->wp_n += steps(l.cin) * l.cout;
+    }
+    // (the first layer's input gradient is not needed; its packed rows, 8 input
+    // channels, would not fill an MMA, and its offset only marks the fit)
+    if (tc_bwd_shape(n, l) && (i == 0 || l.cin % 16 == 0)) {
+      n->bwd_off[i] = n->wp_n;
+      n->wp_n += steps(l.cout) * l.cin;
+      n->planes_n = std::max<int64_t>(n->planes_n, 3 * l.cout * nn::Padded{l.h, l.w, max_batch}.positions());
+    }
+  }
+  int dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n->nsm, cudaDevAttrMultiProcessorCount, dev);
+  // partial sums: at most 64 nsm channels x blocks, and the blocks' head parts
+  const int64_t bs_n = std::max<int64_t>(64 * (int64_t)n->nsm, 256),
+                hp_n = std::max<int64_t>(1, (int64_t)n->nsm * 8 / std::max(1, w / 8)) * ((int64_t)out_ch * w + out_ch);
   cudaError_t e = cudaMalloc(&n->p, sizeof(float) * n->np);
+  if (e == cudaSuccess && n->wp_n) e = cudaMalloc(&n->wp, sizeof(nn::bf16) * n->wp_n);
+  if (e == cudaSuccess && n->planes_n) e = cudaMalloc(&n->planes, sizeof(nn::bf16) * n->planes_n);
+  if (e == cudaSuccess && n->planes_n) e = cudaMalloc(&n->bsum, sizeof(float) * bs_n);
+  if (e == cudaSuccess && n->planes_n)
+    e = cudaMalloc(&n->hp, sizeof(float) * hp_n);
   if (e == cudaSuccess) e = cudaMalloc(&n->g, sizeof(float) * n->np);
   if (e == cudaSuccess) e = cudaMalloc(&n->m, sizeof(float) * n->np);
   if (e == cudaSuccess) e = cudaMalloc(&n->v, sizeof(float) * n->np);
@@ -1006,6 +1048,10 @@ void vlb_nn_destroy(vlb_nn *n) {
   cudaFree(n->dwp);
   cudaFree(n->lossp);
   if (n->d_err) cudaFree(n->d_err);
+  if (n->wp) cudaFree(n->wp);
+  if (n->planes) cudaFree(n->planes);
+  if (n->bsum) cudaFree(n->bsum);
+  if (n->hp) cudaFree(n->hp);
   delete n;
 }
 
