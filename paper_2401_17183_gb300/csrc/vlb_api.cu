@@ -339,17 +339,27 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
   using L19 = vlb::CoefLayout<19>;
   s->nc = q == 9    ? (plane ? L9::stride<float, true>() : L9::stride<float, false>())
           : q == 19 ? (plane ? L19::stride<float, true>() : L19::stride<float, false>())
-                    : 0;  // D3Q39: no records, the kernels read the mesh geometry
+                    : 0;  // D3Q39: below
   if (q == VLB_D3Q39) {
-    // D3Q39: no records; per cell the chord data of its force map (q39_prepare)
-    s->nc = 12;
+    // D3Q39: per cell the record of its force map (q39_prepare)
+    s->nc = vlb::kRec39;
     s->ncoef = mesh->ncell;
   }
   const size_t es = f64 ? 8 : 4;
   // 16 bytes of padding: a 16-bit population is read as the aligned 32-bit
   // word that contains it
   cudaError_t e = cudaMalloc(&s->d_f, vlb::storage_bytes(params->precision) * q * mesh->ncell + 16);
-  if (e == cudaSuccess && s->ncoef > 0) e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
+  if (e == cudaSuccess && q == VLB_D3Q39) {
+    e = cudaMalloc(&s->d_coef, vlb::q39_record_bytes(mesh->ncell));
+    if (e == cudaErrorMemoryAllocation) {
+      // no room for the records: the chord data alone, and the map direction by direction
+      cudaGetLastError();
+      s->nc = vlb::kChord39;
+      e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
+    }
+  } else if (e == cudaSuccess) {
+    e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&s->d_err, sizeof(int));
   if (e != cudaSuccess) {
     vlb_destroy(s);

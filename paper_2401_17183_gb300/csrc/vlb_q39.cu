@@ -1,16 +1,26 @@
 // vlb_q39.cu -- the time step, initialisation, moments and state access for the
 // 6th-order isotropic D3Q39 velocity set (vlb_q39.cuh) on periodic meshes, in
-// FP64. The reduced force map of the D3Q19/D2Q9 kernels relies on velocity
-// components in {-1, 0, 1}; here every relation of section 2.2 is evaluated
-// pair of opposite directions by pair instead:
-//   f = N / J, rho and U (Eqs. 14, 15, 17); a fixed point on F (Eq. 27), each
-//   evaluation forming U~ = U + F / (2 rho), f^eq (Eq. 33 with T0 = 2/3),
-//   deltaPi (Eq. 30), deltaN (Eq. 31), Omega = -(N - J f^eq) / tau (Eq. 20)
-//   and N' = N + Omega + deltaN (Eq. 12); the converged N' is advected one to
-//   one (Eq. 22) in place with the A-A pattern of the other kernels (even
-//   steps: slot a of q in, slot abar of q out; odd steps: slot abar of q - c_a
-//   in, slot a of q + c_a out), with neighbours wrapped periodically on every
-//   axis (each axis at least 3 cells long, speeds at most 3).
+// FP64. Streaming is in place with the A-A pattern of the other kernels (even
+// steps: slot a of q in, slot abar of q out; odd steps: slot abar of q - c_a
+// in, slot a of q + c_a out), with neighbours wrapped periodically on every
+// axis (each axis at least 3 cells long, speeds at most 3).
+//
+// The collision (section 2.2) takes directions in pairs (p, pbar = p + 19) with
+// c_pbar = -c_p and writes the force map of Eq. 27 as a polynomial in U~ with
+// coefficients of the cell's geometry and tau alone (Rec39, build_record39), as the
+// D3Q19 kernel does: one chord step costs about 75 FP64 operations instead of a
+// pass over the 39 directions, and N' is formed once, at the converged force.
+// With Phi = J F, m = sum N, s_p = N_p + N_pbar, t_p = N_p - N_pbar, M_p = K_p +
+// K_pbar, D_p = K_p - K_pbar, f^eq = rho w (1 + xe +- xo) (Eq. 33) and
+// P = J deltaPi (Eq. 30), linear in the xo_p,
+//   Phi_new = m G + sum_p (am M_p s_p + ad D_p t_p) - m/(2 tau) sum_p w_p M_p
+//             - m/2 sum_p {w_p M_p xe_p / tau + Ao_p xo_p} - 1/2 TT Phi,
+//   am = -(2 - 1/tau)/4, ad = 1/(4 tau),
+//   Ao^i_p = w_p [D^i_p / tau - (1 - 1/(2 tau)) c_p.R^i.M_p],
+//   R^i_kl = sum_p w_p M^i_p (c^k c^l / T0 - delta_kl) / T0,  TT^i_j = sum_p w_p D^i_p c^j_p / T0,
+// and xe is linear in B = (g - delta) T0 + U~U~, xo in U and the symmetric C^jkl of Eq. 33.
+// Where the records do not fit into device memory, every relation is evaluated
+// direction pair by pair instead, with 12 values per cell (collide39).
 // The link coefficients K^i_a = sum_j c^j_a Theta^i_j(q + c_a, q) (Eq. 11)
 // come from the mesh's FP64 geometry, so the relations of Eqs. 27 and 30 read
 //   sum_j c^j_a Theta^i_j(q - c_a, q) = -K^i_abar.
@@ -44,7 +54,9 @@ struct Q39Args {
   int64_t ncell;
   int64_t n[3];
   const double *J, *gl, *gu, *ginv, *K;
-  // per cell: the chord matrix H = (I - dG/dF)^-1 of the force map at the
+  // records of the polynomial force map (Rec39), or NULL
+  const double *rec;
+  // without them, per cell: the chord matrix H = (I - dG/dF)^-1 of the force map at the
   // rest state (row-major) and the rest state's force at rho = 1, 12 values;
   // NULL before q39_prepare has filled them
   const double *chord;
@@ -227,8 +239,9 @@ __device__ void eval39(const double N[kQ39], double J, double rho, const double 
 // tol max(rho, |F|); N' at the converged F (to within that change). False if
 // max_iter is reached.
 __device__ bool collide39(const double N[kQ39], double J, const double gd[3][3], const double G[3],
-                          const double *K, const double *ch, double tau, double tol, int max_iter,
+                          const double *K, const double *chord, int64_t c, double tau, double tol, int max_iter,
                           double Np[kQ39], double &rho, double U[3], double F[3]) {
+  const double *ch = chord ? chord + c * 12 : nullptr;
   rho = 0.0;
   for (int a = 0; a < kQ39; a++) rho += N[a] / J;
   for (int i = 0; i < 3; i++) {
@@ -319,6 +332,473 @@ __global__ void __launch_bounds__(kQ39Threads) k_prep39(const Q39Args A, double 
   }
 }
 
+// ------------------------------------------------- the polynomial force map
+// Record of one cell: value k of cell c at ((c / 32) NR + k) 32 + c % 32, so that a
+// warp reads 256 consecutive bytes per value.
+struct Rec39 {
+  static constexpr int GD = 0;              // g^ij - delta^ij, packed (6)
+  static constexpr int BC = GD + 6;         // terms of the map proportional to m (3)
+  static constexpr int PO1 = BC + 3;        // coefficient of U, row-major (9)
+  static constexpr int HM = PO1 + 9;        // chord matrix (9)
+  static constexpr int QM = HM + 9;         // H times the coefficients of the 6 + 10 monomials (3 x 16)
+  static constexpr int FR = QM + 48;        // F of the rest state at rho = 1 (3)
+  static constexpr int IJ = FR + 3;         // 1 / J
+  static constexpr int LK = IJ + 1;         // per pair: am M_p (3), ad D_p (3)
+  static constexpr int NR = LK + 6 * kH39;
+};
+static_assert(Rec39::NR == kRec39, "record size");
+__device__ __forceinline__ int64_t rec39(int64_t c) { return (c >> 5) * (Rec39::NR * 32) + (c & 31); }
+
+// the distinct components of a symmetric third-rank tensor
+__host__ __device__ constexpr int sym3(int i, int j, int k) {
+  const int a = i < j ? (i < k ? i : k) : (j < k ? j : k), c = i > j ? (i > k ? i : k) : (j > k ? j : k);
+  const int b = i + j + k - a - c;
+  // 000 001 002 011 012 022 111 112 122 222
+  return a == 0 ? (b == 0 ? c : b == 1 ? 2 + c : 5) : a == 1 ? (b == 1 ? 5 + c : 8) : 9;
+}
+__host__ __device__ constexpr int q39_len(int p) {   // largest |c| component of pair p
+  const int x = Lat<39>::c(p, 0), y = Lat<39>::c(p, 1), z = Lat<39>::c(p, 2);
+  const int ax = x < 0 ? -x : x, ay = y < 0 ? -y : y, az = z < 0 ? -z : z;
+  return ax > ay ? (ax > az ? ax : az) : (ay > az ? ay : az);
+}
+__host__ __device__ constexpr int q39_nnz(int p) {
+  return (Lat<39>::c(p, 0) != 0) + (Lat<39>::c(p, 1) != 0) + (Lat<39>::c(p, 2) != 0);
+}
+
+// polynomial part of a chord step: a^i = sum_k QM[i][k] monomial_k(U~)
+template <typename LD>
+__device__ __forceinline__ void map39(const double Ut[3], LD ld, double a[3]) {
+  const double x = Ut[0], y = Ut[1], z = Ut[2];
+  const double xx = x * x, yy = y * y, zz = z * z;
+  const double mono[16] = {xx, x * y, x * z, yy, y * z, zz,
+                           xx * x, xx * y, xx * z, x * yy, (x * y) * z, x * zz, yy * y, yy * z, y * zz, zz * z};
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 16; k++) v = fma(ld(Rec39::QM + 16 * i + k), mono[k], v);
+    a[i] = v;
+  }
+}
+
+// Fills the record of every cell from its geometry (see the top of the file):
+//   PE = R / (2 tau),  S^i_jkl = 1/(6 T0^3) sum_p Ao^i_p h^jkl_p,
+//   h = ccc - T0 (c delta + cyclic),  PO1 = sum_p Ao_p c / T0,
+//   LO^i_l = 3 T0 sum_jk (g - delta)_jk S^i_jkl,  LD^i_l = 3 T0 sum_j S^i_jjl,
+// so that Phi_new = Pb - m/2 {PE : U~U~ + S : U~U~U~ + LO U~} - (TT + LD/2) Phi / 2 and, with
+// U~ = U + Phi / (2m), A = LO/4 + (TT + LD/2)/2 and H = (I + A)^-1, the chord step is
+// Phi <- H (Pc - m/2 Q(U~)), Pc = m BC + sum_p (am M s + ad D t) - m/2 (PO1 + LO) U.
+__global__ void __launch_bounds__(kQ39Threads) k_prep39_rec(const Q39Args A, double *out) {
+  const double T0 = kT0_39, itau = 1.0 / A.tau, am = -0.25 * (2.0 - itau), ad = 0.25 * itau;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < A.ncell;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    double *o = out + rec39(c);
+    const double *K = A.K + c * kQ39 * 3;
+    double gd[3][3], G[3];
+    cell_metric(A, c, gd, G);
+    const double J = A.J[c];
+    double R[3][6], TT[3][3], KW[3];
+    for (int i = 0; i < 3; i++) {
+      KW[i] = 0.0;
+      for (int k = 0; k < 6; k++) R[i][k] = 0.0;
+      for (int j = 0; j < 3; j++) TT[i][j] = 0.0;
+    }
+#pragma unroll 1
+    for (int p = 1; p <= kH39; p++) {
+      const double cv[3] = {kT39.c[p][0], kT39.c[p][1], kT39.c[p][2]}, w = kT39.w[p];
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const double M = K[p * 3 + i] + K[(p + kH39) * 3 + i], D = K[p * 3 + i] - K[(p + kH39) * 3 + i];
+        o[(Rec39::LK + 6 * (p - 1) + i) * 32] = am * M;
+        o[(Rec39::LK + 6 * (p - 1) + 3 + i) * 32] = ad * D;
+        KW[i] += w * M;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+          TT[i][k] += w * D * cv[k] / T0;
+#pragma unroll
+          for (int l = k; l < 3; l++) R[i][sym<3>(k, l)] += w * M * (cv[k] * cv[l] / T0 - (k == l ? 1.0 : 0.0)) / T0;
+        }
+      }
+    }
+    double S[3][10], PO1[3][3];
+    for (int i = 0; i < 3; i++) {
+      for (int k = 0; k < 10; k++) S[i][k] = 0.0;
+      for (int k = 0; k < 3; k++) PO1[i][k] = 0.0;
+    }
+#pragma unroll 1
+    for (int p = 1; p <= kH39; p++) {
+      const double cv[3] = {kT39.c[p][0], kT39.c[p][1], kT39.c[p][2]}, w = kT39.w[p];
+      double M[3];
+#pragma unroll
+      for (int i = 0; i < 3; i++) M[i] = K[p * 3 + i] + K[(p + kH39) * 3 + i];
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        double cRM = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+#pragma unroll
+          for (int l = 0; l < 3; l++) cRM += cv[k] * R[i][sym<3>(k, l)] * M[l];
+        const double D = K[p * 3 + i] - K[(p + kH39) * 3 + i];
+        const double Ao = w * (itau * D - (1.0 - 0.5 * itau) * cRM);
+#pragma unroll
+        for (int l = 0; l < 3; l++) PO1[i][l] += Ao * cv[l] / T0;
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+#pragma unroll
+          for (int k = j; k < 3; k++)
+#pragma unroll
+            for (int l = k; l < 3; l++) {
+              const double h = cv[j] * cv[k] * cv[l] - T0 * ((k == l ? cv[j] : 0.0) + (j == l ? cv[k] : 0.0) +
+                                                             (j == k ? cv[l] : 0.0));
+              S[i][sym3(j, k, l)] += Ao * h / (6.0 * T0 * T0 * T0);
+            }
+      }
+    }
+    double Am[3][3], LO[3][3], BC[3];
+    for (int i = 0; i < 3; i++) {
+      double ce = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int l = 0; l < 3; l++) ce += T0 * 0.5 * itau * R[i][sym<3>(k, l)] * gd[k][l];
+      BC[i] = G[i] - 0.5 * itau * KW[i] - 0.5 * ce;
+#pragma unroll
+      for (int l = 0; l < 3; l++) {
+        double lo = 0.0, ld = 0.0;
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+          ld += 3.0 * T0 * S[i][sym3(j, j, l)];
+#pragma unroll
+          for (int k = 0; k < 3; k++) lo += 3.0 * T0 * gd[j][k] * S[i][sym3(j, k, l)];
+        }
+        LO[i][l] = lo;
+        Am[i][l] = (i == l ? 1.0 : 0.0) + 0.25 * lo + 0.5 * (TT[i][l] + 0.5 * ld);
+      }
+    }
+    double Hm[3][3];
+    {
+      double C[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+          const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+          C[i][j] = Am[i1][j1] * Am[i2][j2] - Am[i1][j2] * Am[i2][j1];
+        }
+      const double det = Am[0][0] * C[0][0] + Am[0][1] * C[0][1] + Am[0][2] * C[0][2];
+#pragma unroll
+      for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) Hm[i][j] = C[j][i] / det;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int j = i; j < 3; j++) o[(Rec39::GD + sym<3>(i, j)) * 32] = gd[i][j];
+    double QM[3][16];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      o[(Rec39::BC + i) * 32] = BC[i];
+#pragma unroll
+      for (int l = 0; l < 3; l++) {
+        o[(Rec39::PO1 + 3 * i + l) * 32] = PO1[i][l] + LO[i][l];
+        o[(Rec39::HM + 3 * i + l) * 32] = Hm[i][l];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int l = k; l < 3; l++) {
+          double v = 0.0;
+#pragma unroll
+          for (int j = 0; j < 3; j++) v += Hm[i][j] * R[j][sym<3>(k, l)];
+          QM[i][sym<3>(k, l)] = (k == l ? 0.5 : 1.0) * itau * v;
+        }
+#pragma unroll
+      for (int j = 0; j < 3; j++)
+#pragma unroll
+        for (int k = j; k < 3; k++)
+#pragma unroll
+          for (int l = k; l < 3; l++) {
+            double v = 0.0;
+#pragma unroll
+            for (int q = 0; q < 3; q++) v += Hm[i][q] * S[q][sym3(j, k, l)];
+            QM[i][6 + sym3(j, k, l)] = (j == l ? 1.0 : j == k || k == l ? 3.0 : 6.0) * v;
+          }
+#pragma unroll
+      for (int k = 0; k < 16; k++) o[(Rec39::QM + 16 * i + k) * 32] = QM[i][k];
+    }
+    o[Rec39::IJ * 32] = 1.0 / J;
+    // the rest state (rho = 1, U = 0): N = J w (1 + xe) with B = (g - delta) T0, m = J
+    double Pc[3], Pt[3], Phi[3] = {0.0, 0.0, 0.0}, trg = gd[0][0] + gd[1][1] + gd[2][2];
+    for (int i = 0; i < 3; i++) Pc[i] = J * BC[i];
+#pragma unroll 1
+    for (int p = 1; p <= kH39; p++) {
+      const double x = kT39.c[p][0], y = kT39.c[p][1], z = kT39.c[p][2];
+      const double cgc = x * x * gd[0][0] + y * y * gd[1][1] + z * z * gd[2][2] +
+                         2.0 * (x * y * gd[0][1] + x * z * gd[0][2] + y * z * gd[1][2]);
+      const double sp = 2.0 * J * kT39.w[p] * (1.0 + 0.5 * (cgc / T0 - trg));
+#pragma unroll
+      for (int i = 0; i < 3; i++) Pc[i] += am * (K[p * 3 + i] + K[(p + kH39) * 3 + i]) * sp;
+    }
+    for (int i = 0; i < 3; i++) Pt[i] = Hm[i][0] * Pc[0] + Hm[i][1] * Pc[1] + Hm[i][2] * Pc[2];
+    for (int it = 0; it < 100; it++) {
+      double Ut[3], a[3], diff = 0.0, fm = 0.0;
+      for (int i = 0; i < 3; i++) Ut[i] = 0.5 * Phi[i] / J;
+      map39(Ut, [&](int k) { return QM[(k - Rec39::QM) / 16][(k - Rec39::QM) % 16]; }, a);
+      for (int i = 0; i < 3; i++) {
+        const double pn = Pt[i] - 0.5 * J * a[i];
+        diff = maxnan(diff, fabs(pn - Phi[i]));
+        fm = maxnan(fm, fabs(pn));
+        Phi[i] = pn;
+      }
+      if (diff <= 1e-15 * (fm > J ? fm : J)) break;
+    }
+    for (int i = 0; i < 3; i++) o[(Rec39::FR + i) * 32] = Phi[i] / J;
+  }
+}
+
+// One cell's arrived populations as pair sums and differences (s[0] = N_0)
+// and what the collision makes of them. ld(k): record value k.
+struct Cell39 {
+  double s[kH39 + 1], t[kH39 + 1];
+  double m, U[3], Phi[3];
+};
+
+// m, U and the force: the chord iteration Phi <- H (Pc - m/2 Q(U~)) from m F_rest,
+// converged when the change is at most tol max(m, |Phi|)
+template <typename LD>
+__device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_iter) {
+  double m = q.s[0], mu[3] = {0.0, 0.0, 0.0}, Pc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int p = 1; p <= kH39; p++) {
+    m += q.s[p];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const int ci = Lat<39>::c(p, i);
+      if (ci == 1) mu[i] += q.t[p];
+      else if (ci == -1) mu[i] -= q.t[p];
+      else if (ci != 0) mu[i] = fma((double)ci, q.t[p], mu[i]);
+      Pc[i] = fma(ld(Rec39::LK + 6 * (p - 1) + i), q.s[p], Pc[i]);
+      Pc[i] = fma(ld(Rec39::LK + 6 * (p - 1) + 3 + i), q.t[p], Pc[i]);
+    }
+  }
+  q.m = m;
+  const double im = 1.0 / m, h2m = 0.5 * im, hm = 0.5 * m;
+#pragma unroll
+  for (int i = 0; i < 3; i++) q.U[i] = mu[i] * im;
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    Pc[i] = fma(m, ld(Rec39::BC + i), Pc[i]);
+    // m/2 (PO1 + LO) U = 1/2 (PO1 + LO) (m U)
+    double v = 0.0;
+#pragma unroll
+    for (int l = 0; l < 3; l++) v = fma(ld(Rec39::PO1 + 3 * i + l), mu[l], v);
+    Pc[i] = fma(-0.5, v, Pc[i]);
+  }
+  double Pt[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    Pt[i] = ld(Rec39::HM + 3 * i) * Pc[0] + ld(Rec39::HM + 3 * i + 1) * Pc[1] + ld(Rec39::HM + 3 * i + 2) * Pc[2];
+    q.Phi[i] = m * ld(Rec39::FR + i);
+  }
+#pragma unroll 1
+  for (int it = 0; it < max_iter; it++) {
+    double Ut[3], a[3], diff = 0.0, pm = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; i++) Ut[i] = fma(q.Phi[i], h2m, q.U[i]);
+    map39(Ut, ld, a);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const double pn = fma(-hm, a[i], Pt[i]);
+      diff = maxnan(diff, fabs(pn - q.Phi[i]));
+      pm = maxnan(pm, fabs(pn));
+      q.Phi[i] = pn;
+    }
+    if (diff <= tol * (m > pm ? m : pm)) return true;
+  }
+  return false;
+}
+
+// Even and odd parts of the equilibrium bracket over the pairs, folded by the kind
+// of pair. Even: y0 + c.Y.c for a symmetric Y. Odd: c.u + k C:ccc for
+// symmetric C; with b^i = k C^iii, q^ji = 3 k C^jji, d = 6 k C^012,
+//   axis of length L:   L (u_i + L^2 b_i),
+//   corner (s0 s1 s2):  sum_i s_i (u_i + b_i + sum_{j != i} q_ji) + s0 s1 s2 d,
+//   (2 s_i, 2 s_j):     sum of s_i (2 u_i + 8 (b_i + q_ji)) over both axes.
+struct Odd39 {
+  double u[3], b[3], a[3], e[3][3], d;
+  // e[i][j]: the part of axis i in the plane of axes i and j
+  __device__ __forceinline__ Odd39(const double (&uu)[3], const double (&kC)[10]) {
+    double qj[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      u[i] = uu[i];
+      b[i] = kC[sym3(i, i, i)];
+      a[i] = u[i] + b[i];
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        if (j == i) continue;
+        qj[j][i] = 3.0 * kC[sym3(j, j, i)];
+        a[i] += qj[j][i];
+        e[i][j] = fma(8.0, b[i] + qj[j][i], 2.0 * u[i]);
+      }
+    }
+    d = 6.0 * kC[sym3(0, 1, 2)];
+  }
+  __device__ __forceinline__ double operator()(int p) const {
+    const int L = q39_len(p), nz = q39_nnz(p);
+    double r = 0.0;
+    if (nz == 1) {
+#pragma unroll
+      for (int i = 0; i < 3; i++)
+        if (Lat<39>::c(p, i) != 0) r = L == 1 ? u[i] + b[i] : (double)L * fma((double)(L * L), b[i], u[i]);
+      return r;   // the positive half's axis vectors point along +i
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const int ci = Lat<39>::c(p, i);
+      if (ci == 0) continue;
+      double v = a[i];
+      if (nz == 2) {
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+          if (j != i && Lat<39>::c(p, j) != 0) v = e[i][j];
+      }
+      r = ci > 0 ? r + v : r - v;
+    }
+    if (nz == 3) r = Lat<39>::c(p, 0) * Lat<39>::c(p, 1) * Lat<39>::c(p, 2) > 0 ? r + d : r - d;
+    return r;
+  }
+};
+__device__ __forceinline__ double even39(int p, double y0, const double (&Y)[6]) {
+  const int L = q39_len(p);
+  double r = 0.0;
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    if (Lat<39>::c(p, i) != 0) r += Y[sym<3>(i, i)];
+#pragma unroll
+    for (int j = i + 1; j < 3; j++) {
+      const int cc = Lat<39>::c(p, i) * Lat<39>::c(p, j);
+      if (cc > 0) r = fma(2.0, Y[sym<3>(i, j)], r);
+      if (cc < 0) r = fma(-2.0, Y[sym<3>(i, j)], r);
+    }
+  }
+  return L == 1 ? y0 + r : fma((double)(L * L), r, y0);
+}
+
+// B (packed) and C / (6 T0^3), u = U / T0 - V / (2 T0^2) of Eq. 33 (V^i = C^ijj)
+__device__ __forceinline__ void herm39_packed(const double (&gd)[6], const double U[3], const double Ut[3],
+                                              double (&B)[6], double (&kC)[10], double (&u)[3]) {
+  const double T0 = kT0_39;
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = i; j < 3; j++) B[sym<3>(i, j)] = fma(gd[sym<3>(i, j)], T0, Ut[i] * Ut[j]);
+  const double k = 1.0 / (6.0 * T0 * T0 * T0), kt = k * T0;
+  double du[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) du[i] = Ut[i] - U[i];
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = i; j < 3; j++)
+#pragma unroll
+      for (int l = j; l < 3; l++) {
+        double v = gd[sym<3>(i, j)] * Ut[l];
+        v = fma(gd[sym<3>(j, l)], Ut[i], v);
+        v = fma(gd[sym<3>(i, l)], Ut[j], v);
+        if (i == j) v += du[l];
+        if (j == l) v += du[i];
+        if (i == l) v += du[j];
+        kC[sym3(i, j, l)] = fma(k, (Ut[i] * Ut[j]) * Ut[l], kt * v);
+      }
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    const double v = kC[sym3(i, 0, 0)] + kC[sym3(i, 1, 1)] + kC[sym3(i, 2, 2)];
+    u[i] = fma(-3.0 * T0, v, U[i] / T0);
+  }
+}
+
+template <bool ODD>
+__device__ __forceinline__ void pull39(const Q39Args &A, int64_t c, const int64_t ic[3], Cell39 &q) {
+  q.s[0] = A.f[c];
+  q.t[0] = 0.0;
+#pragma unroll
+  for (int p = 1; p <= kH39; p++) {
+    const double a = A.f[src39<ODD>(A, c, ic, p)], b = A.f[src39<ODD>(A, c, ic, p + kH39)];
+    q.s[p] = a + b;
+    q.t[p] = a - b;
+  }
+}
+
+// One time step with the polynomial force map. Bounded by the FP64 pipe (two
+// lanes per clock and SM): about 850 FP64 operations per cell update, against 3,000 per
+// evaluation of the map direction by direction. 64^3 cells: 0.80 ms a step (330
+// MLUPS; 5.9 ms direction by direction), 168 registers, three blocks per SM.
+template <bool ODD>
+__global__ void __launch_bounds__(kQ39Threads, 3) k_step39_rec(const Q39Args A) {
+  const int64_t c = (int64_t)blockIdx.x * kQ39Threads + threadIdx.x;
+  if (c >= A.ncell) return;
+  int64_t ic[3];
+  coords(A, c, ic);
+  const double *rec = A.rec + rec39(c);
+  auto ld = [&](int k) { return __ldg(rec + k * 32); };
+  Cell39 q;
+  pull39<ODD>(A, c, ic, q);
+  if (!force39(q, ld, A.tol, A.max_iter)) atomicOr(A.err, ERR_NOCONV);
+  const double T0 = kT0_39, itau = 1.0 / A.tau;
+  double Ut[3], gd[6], B[6], kC[10], u[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++) Ut[i] = fma(q.Phi[i], 0.5 / q.m, q.U[i]);
+#pragma unroll
+  for (int i = 0; i < 6; i++) gd[i] = ld(Rec39::GD + i);
+  herm39_packed(gd, q.U, Ut, B, kC, u);
+  const Odd39 xo(u, kC);
+  // P^kl = J deltaPi^kl = 2 m sum_p w_p c^k am M^l_p xo_p  (Eq. 30), its symmetric part
+  double P[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; k++)
+#pragma unroll
+    for (int l = 0; l < 3; l++) P[k][l] = 0.0;
+#pragma unroll
+  for (int p = 1; p <= kH39; p++) {
+    const double x = q39_w(p) * q39_len(p) * xo(p);
+#pragma unroll
+    for (int l = 0; l < 3; l++) {
+      const double M = ld(Rec39::LK + 6 * (p - 1) + l);
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        if (Lat<39>::c(p, k) > 0) P[k][l] = fma(M, x, P[k][l]);
+        if (Lat<39>::c(p, k) < 0) P[k][l] = fma(-M, x, P[k][l]);
+      }
+    }
+  }
+  // N'_p = (1 - 1/tau) N_p + w [y0 + c.Y.c] +- w [(m/tau) xo + c.Phi / T0], the even part
+  // (m/tau)(1 + xe) + (c.P.c / T0 - tr P) / T0 with xe = (c.B.c / T0 - tr B) / (2 T0)
+  const double mt = q.m * itau, m2 = 2.0 * q.m;
+  double Y[6], kZ[10], uz[3];
+#pragma unroll
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = i; j < 3; j++)
+      Y[sym<3>(i, j)] = (0.5 * mt * B[sym<3>(i, j)] + m2 * (i == j ? P[i][i] : 0.5 * (P[i][j] + P[j][i]))) / (T0 * T0);
+  const double y0 = mt * (1.0 - (B[0] + B[3] + B[5]) / (2.0 * T0)) - m2 * (P[0][0] + P[1][1] + P[2][2]) / T0;
+#pragma unroll
+  for (int k = 0; k < 10; k++) kZ[k] = mt * kC[k];
+#pragma unroll
+  for (int i = 0; i < 3; i++) uz[i] = fma(mt, u[i], q.Phi[i] / T0);
+  const Odd39 zo(uz, kZ);
+  const double omt = 1.0 - itau, h = 0.5 * omt;
+  A.f[c] = fma(omt, q.s[0], q39_w(0) * y0);
+#pragma unroll
+  for (int p = 1; p <= kH39; p++) {
+    const double ev = fma(h, q.s[p], q39_w(p) * even39(p, y0, Y));
+    const double od = fma(h, q.t[p], q39_w(p) * zo(p));
+    A.f[dst39<ODD>(A, c, ic, p)] = ev + od;
+    A.f[dst39<ODD>(A, c, ic, p + kH39)] = ev - od;
+  }
+}
+
 template <bool ODD>
 __global__ void __launch_bounds__(kQ39Threads) k_step39(const Q39Args A) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < A.ncell;
@@ -330,8 +810,7 @@ __global__ void __launch_bounds__(kQ39Threads) k_step39(const Q39Args A) {
     for (int a = 0; a < kQ39; a++) N[a] = A.f[src39<ODD>(A, c, ic, a)];
     double gd[3][3], G[3], rho, U[3], F[3];
     cell_metric(A, c, gd, G);
-    if (!collide39(N, A.J[c], gd, G, A.K + c * kQ39 * 3, A.chord ? A.chord + c * 12 : nullptr, A.tau, A.tol,
-                   A.max_iter, Np, rho, U, F))
+    if (!collide39(N, A.J[c], gd, G, A.K + c * kQ39 * 3, A.chord, c, A.tau, A.tol, A.max_iter, Np, rho, U, F))
       atomicOr(A.err, ERR_NOCONV);
 #pragma unroll 1
     for (int a = 0; a < kQ39; a++) A.f[dst39<ODD>(A, c, ic, a)] = Np[a];
@@ -341,16 +820,33 @@ __global__ void __launch_bounds__(kQ39Threads) k_step39(const Q39Args A) {
 __global__ void __launch_bounds__(kQ39Threads) k_init39(const Q39Args A, const double *rho, const double *u) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < A.ncell;
        c += (int64_t)gridDim.x * blockDim.x) {
-    double gd[3][3], G[3], U[3], f[kQ39];
-    cell_metric(A, c, gd, G);
+    double gd[6], U[3], B[6], kC[10], uu[3];
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int j = i; j < 3; j++) gd[sym<3>(i, j)] = A.ginv[c * 6 + sym<3>(i, j)] - (i == j ? 1.0 : 0.0);
+#pragma unroll
     for (int i = 0; i < 3; i++) {
       double s = 0.0;
+#pragma unroll
       for (int d = 0; d < 3; d++) s += u[c * 3 + d] * A.gu[(c * 3 + i) * 3 + d];  // U^i = u . g^i
       U[i] = s;
     }
-    feq39(rho[c], U, U, gd, f);
-    const double J = A.J[c];
-    for (int a = 0; a < kQ39; a++) A.f[(int64_t)a * A.ncell + c] = J * f[a];
+    herm39_packed(gd, U, U, B, kC, uu);
+    const Odd39 xo(uu, kC);
+    // N = J rho w (1 + xe +- xo)
+    const double T0 = kT0_39, m = A.J[c] * rho[c];
+    double Y[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) Y[i] = B[i] / (2.0 * T0 * T0);
+    const double y0 = 1.0 - (B[0] + B[3] + B[5]) / (2.0 * T0);
+    A.f[c] = m * (q39_w(0) * y0);
+#pragma unroll
+    for (int p = 1; p <= kH39; p++) {
+      const double ev = even39(p, y0, Y), od = xo(p), mw = m * q39_w(p);
+      A.f[(int64_t)p * A.ncell + c] = mw * (ev + od);
+      A.f[(int64_t)(p + kH39) * A.ncell + c] = mw * (ev - od);
+    }
   }
 }
 
@@ -361,49 +857,87 @@ __device__ __forceinline__ double warp_sum39(double v) {
 
 // rho [ncell], u [ncell][3], u~ [ncell][3] into out; per-block conservation
 // sums (mass, P = sum e_a N_a, M = sum 1/2 [e_a(q) + e_a(q - c_a)] N_a) into
-// partial[block][7]
-template <bool ODD>
+// partial[block][7]. M is regrouped so that a cell needs only its own tangents:
+// with p = q - c_a in its second half, M = 1/2 sum_p g_i(p) sum_a c^i_a [N_a(p) +
+// N_a(p + c_a)], and N_a(p + c_a) sits at slot a of p + c_a (even parity) or at slot
+// abar of p (odd). REC: the polynomial force map, else collide39.
+template <bool ODD, bool REC>
 __global__ void __launch_bounds__(kMomThreads) k_moments39(const Q39Args A, double *out, double *partial) {
   double acc[7] = {0, 0, 0, 0, 0, 0, 0};
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < A.ncell;
        c += (int64_t)gridDim.x * blockDim.x) {
     int64_t ic[3];
     coords(A, c, ic);
-    double N[kQ39], Np[kQ39];
+    double mass, rho, U[3], aF[3], bP[3] = {0.0, 0.0, 0.0}, bN[3] = {0.0, 0.0, 0.0};   // aF = F / (2 rho)
+    if constexpr (REC) {
+      Cell39 q;
+      pull39<ODD>(A, c, ic, q);
+      const double *rec = A.rec + rec39(c);
+      auto ld = [&](int k) { return __ldg(rec + k * 32); };
+      if (!force39(q, ld, A.tol, A.max_iter)) atomicOr(A.err, ERR_NOCONV);
+      mass = q.m;
+      rho = q.m * ld(Rec39::IJ);
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        U[i] = q.U[i];
+        aF[i] = 0.5 * q.Phi[i] / q.m;
+        bP[i] = q.U[i] * q.m;
+      }
+    } else {
+      double N[kQ39], Np[kQ39], gd[3][3], G[3], F[3];
 #pragma unroll 1
-    for (int a = 0; a < kQ39; a++) N[a] = A.f[src39<ODD>(A, c, ic, a)];
-    double gd[3][3], G[3], rho, U[3], F[3];
-    cell_metric(A, c, gd, G);
-    if (!collide39(N, A.J[c], gd, G, A.K + c * kQ39 * 3, A.chord ? A.chord + c * 12 : nullptr, A.tau, A.tol,
-                   A.max_iter, Np, rho, U, F))
-      atomicOr(A.err, ERR_NOCONV);
-    const double *gl = A.gl + c * 9;
+      for (int a = 0; a < kQ39; a++) N[a] = A.f[src39<ODD>(A, c, ic, a)];
+      cell_metric(A, c, gd, G);
+      if (!collide39(N, A.J[c], gd, G, A.K + c * kQ39 * 3, A.chord, c, A.tau, A.tol, A.max_iter, Np, rho, U, F))
+        atomicOr(A.err, ERR_NOCONV);
+      mass = 0.0;
+      for (int a = 0; a < kQ39; a++) mass += N[a];
+      for (int i = 0; i < 3; i++) {
+        aF[i] = 0.5 * (F[i] / rho);
+        for (int a = 0; a < kQ39; a++) bP[i] += kT39.c[a][i] * N[a];
+      }
+    }
+    double gl[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) gl[k] = A.gl[c * 9 + k];
     out[c] = rho;
     bool finite = isfinite(rho);
+#pragma unroll
     for (int d = 0; d < 3; d++) {
       double uu = 0.0, ut = 0.0;
+#pragma unroll
       for (int i = 0; i < 3; i++) {
-        uu += U[i] * gl[i * 3 + d];                          // u = U^i g_i (Eq. 34)
-        ut += (U[i] + 0.5 * (F[i] / rho)) * gl[i * 3 + d];   // u~ = U~^i g_i
+        uu += U[i] * gl[i * 3 + d];             // u = U^i g_i (Eq. 34)
+        ut += (U[i] + aF[i]) * gl[i * 3 + d];   // u~ = U~^i g_i
       }
       out[A.ncell + c * 3 + d] = uu;
       out[A.ncell * 4 + c * 3 + d] = ut;
       finite = finite && isfinite(uu) && isfinite(ut);
     }
     if (!finite) atomicOr(A.err, ERR_NONFINITE);
-#pragma unroll 1
-    for (int a = 0; a < kQ39; a++) {
-      acc[0] += N[a];
-      const double *gb = A.gl + nb39(A, ic, a, -1) * 9;
-      for (int d = 0; d < 3; d++) {
-        double e = 0.0, eb = 0.0;
-        for (int i = 0; i < 3; i++) {
-          e += Lat<39>::c(a, i) * gl[i * 3 + d];
-          eb += Lat<39>::c(a, i) * gb[i * 3 + d];
-        }
-        acc[1 + d] += e * N[a];
-        acc[4 + d] += 0.5 * (e + eb) * N[a];
+    // sum_a c_a N_a(p + c_a), the pair (p, pbar) at a time
+#pragma unroll
+    for (int p = 1; p <= kH39; p++) {
+      const double a = ODD ? A.f[(int64_t)(p + kH39) * A.ncell + c] : A.f[(int64_t)p * A.ncell + nb39(A, ic, p, +1)];
+      const double b = ODD ? A.f[(int64_t)p * A.ncell + c] : A.f[(int64_t)(p + kH39) * A.ncell + nb39(A, ic, p, -1)];
+      const double t = a - b;
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        const int ci = Lat<39>::c(p, i);
+        if (ci != 0) bN[i] = fma((double)ci, t, bN[i]);
       }
+    }
+    acc[0] += mass;
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+      double pp = 0.0, nn = 0.0;
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        pp += gl[i * 3 + d] * bP[i];
+        nn += gl[i * 3 + d] * bN[i];
+      }
+      acc[1 + d] += pp;
+      acc[4 + d] += 0.5 * (pp + nn);
     }
   }
   __shared__ double sh[7][kMomThreads / 32];
@@ -487,7 +1021,8 @@ Q39Args make_args(const vlb_sim *sim) {
   A.gu = m->d_gu;
   A.ginv = m->d_ginv;
   A.K = m->d_K;
-  A.chord = static_cast<const double *>(sim->d_coef);
+  A.rec = sim->nc == kRec39 ? static_cast<const double *>(sim->d_coef) : nullptr;
+  A.chord = sim->nc == kRec39 ? nullptr : static_cast<const double *>(sim->d_coef);
   A.tau = sim->p.tau;
   A.tol = sim->p.tol;
   A.max_iter = sim->p.max_iter;
@@ -514,7 +1049,11 @@ cudaError_t q39_mesh_stats(const vlb_mesh *m, double *d_partial, int64_t nblk, c
 cudaError_t q39_prepare(const vlb_sim *sim, cudaStream_t s) {
   Q39Args A = make_args(sim);
   A.chord = nullptr;
-  k_prep39<<<grid_for(A.ncell, kQ39Threads), kQ39Threads, 0, s>>>(A, static_cast<double *>(sim->d_coef));
+  double *out = static_cast<double *>(sim->d_coef);
+  if (A.rec)
+    k_prep39_rec<<<grid_for(A.ncell, kQ39Threads), kQ39Threads, 0, s>>>(A, out);
+  else
+    k_prep39<<<grid_for(A.ncell, kQ39Threads), kQ39Threads, 0, s>>>(A, out);
   return cudaGetLastError();
 }
 
@@ -526,6 +1065,14 @@ cudaError_t q39_init(const vlb_sim *sim, const double *d_rho, const double *d_u,
 
 cudaError_t q39_step(const vlb_sim *sim, int odd, cudaStream_t s) {
   const Q39Args A = make_args(sim);
+  if (A.rec) {
+    const unsigned blocks = (unsigned)((A.ncell + kQ39Threads - 1) / kQ39Threads);
+    if (odd)
+      k_step39_rec<true><<<blocks, kQ39Threads, 0, s>>>(A);
+    else
+      k_step39_rec<false><<<blocks, kQ39Threads, 0, s>>>(A);
+    return cudaGetLastError();
+  }
   if (odd)
     k_step39<true><<<grid_for(A.ncell, kQ39Threads), kQ39Threads, 0, s>>>(A);
   else
@@ -535,10 +1082,18 @@ cudaError_t q39_step(const vlb_sim *sim, int odd, cudaStream_t s) {
 
 cudaError_t q39_moments(const vlb_sim *sim, double *d_out, double *d_partial, int64_t nblk, cudaStream_t s) {
   const Q39Args A = make_args(sim);
-  if (sim->t & 1)
-    k_moments39<true><<<(unsigned)nblk, kMomThreads, 0, s>>>(A, d_out, d_partial);
-  else
-    k_moments39<false><<<(unsigned)nblk, kMomThreads, 0, s>>>(A, d_out, d_partial);
+  const unsigned n = (unsigned)nblk;
+  if (sim->t & 1) {
+    if (A.rec)
+      k_moments39<true, true><<<n, kMomThreads, 0, s>>>(A, d_out, d_partial);
+    else
+      k_moments39<true, false><<<n, kMomThreads, 0, s>>>(A, d_out, d_partial);
+  } else {
+    if (A.rec)
+      k_moments39<false, true><<<n, kMomThreads, 0, s>>>(A, d_out, d_partial);
+    else
+      k_moments39<false, false><<<n, kMomThreads, 0, s>>>(A, d_out, d_partial);
+  }
   return cudaGetLastError();
 }
 

@@ -50,7 +50,12 @@ __host__ __device__ constexpr double q39_w(int a) {
 
 // launches of the D3Q39 path (FP64 populations, periodic meshes)
 cudaError_t q39_mesh_stats(const vlb_mesh *m, double *d_partial, int64_t nblk, cudaStream_t s);
-// per-cell chord data of the force map into sim->d_coef (12 doubles per cell)
+// FP64 values per cell of the polynomial force map's record, and of the chord
+// data alone (used where the records do not fit into device memory)
+constexpr int kRec39 = 193, kChord39 = 12;
+// bytes of sim->d_coef for the records (whole groups of 32 cells)
+inline size_t q39_record_bytes(int64_t ncell) { return sizeof(double) * kRec39 * 32 * (size_t)((ncell + 31) / 32); }
+// per-cell data of the force map into sim->d_coef (sim->nc values per cell)
 cudaError_t q39_prepare(const vlb_sim *sim, cudaStream_t s);
 cudaError_t q39_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s);
 cudaError_t q39_step(const vlb_sim *sim, int odd, cudaStream_t s);
