@@ -3,6 +3,8 @@
 // A-A read of the arrived populations N_a(q, t) for either layout parity.
 #pragma once
 
+#include <type_traits>
+
 #include "vlb_internal.cuh"
 
 namespace vlb {
@@ -30,6 +32,12 @@ struct Addr {
     ic[0] = (IT)(r / g.n[1]);
     cell = (IT)c;
     init(g);
+  }
+  // the same with divisions of the index type (32 bits when IT is)
+  static __device__ __forceinline__ Addr linear(const Grid &g, IT c) {
+    using U = typename std::conditional<sizeof(IT) == 4, uint32_t, IT>::type;
+    const U n2 = (U)g.n[2], n1 = (U)g.n[1], r = (U)c / n2, i0 = r / n1;
+    return Addr(g, (IT)i0, (IT)(r - i0 * n1), (IT)((U)c - r * n2));
   }
   // from index coordinates
   __device__ __forceinline__ Addr(const Grid &g, IT i0, IT i1, IT i2) {

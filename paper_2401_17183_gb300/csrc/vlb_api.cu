@@ -346,6 +346,7 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
     s->ncoef = mesh->ncell;
   }
   const size_t es = f64 ? 8 : 4;
+  s->cellrec = !f64 && !plane && q != VLB_D3Q39;
   // 16 bytes of padding: a 16-bit population is read as the aligned 32-bit
   // word that contains it
   cudaError_t e = cudaMalloc(&s->d_f, vlb::storage_bytes(params->precision) * q * mesh->ncell + 16);
@@ -357,6 +358,9 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
       s->nc = vlb::kChord39;
       e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
     }
+  } else if (e == cudaSuccess && s->cellrec) {
+    e = cudaMalloc(&s->d_coef, vlb::cell_record_bytes(q, mesh->ncell));
+    if (e == cudaSuccess && moving) e = cudaMalloc(&s->d_uw, sizeof(float) * dim * mesh->ncell);
   } else if (e == cudaSuccess) {
     e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
   }
@@ -489,6 +493,7 @@ void vlb_destroy(vlb_sim *s) {
   if (s->stream) cudaStreamSynchronize(s->stream);
   dfree(s->d_f);
   dfree(s->d_coef);
+  dfree(s->d_uw);
   dfree(s->d_err);
   dfree(s->d_fields);
   dfree(s->d_partial);

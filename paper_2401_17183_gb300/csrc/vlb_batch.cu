@@ -70,15 +70,20 @@ BatchKernel batch_kernel(const BatchKind &k, bool odd, int shape) {
   return k.plane ? pick_kernel<19, float, true>(odd, shape) : pick_kernel<19, float, false>(odd, shape);
 }
 
-template <int Q, typename R>
+template <int Q, typename R, bool PLANE>
 size_t smem_q(int threads) {
-  return threads == 64 ? sizeof(StepSmem<Q, R, R, 64>) : sizeof(StepSmem<Q, R, R, 128>);
+  return threads == 64 ? sizeof(StepSmem<Q, R, R, 64, PLANE>) : sizeof(StepSmem<Q, R, R, 128, PLANE>);
+}
+
+template <int Q, typename R>
+size_t smem_p(int threads, bool plane) {
+  return plane ? smem_q<Q, R, true>(threads) : smem_q<Q, R, false>(threads);
 }
 
 size_t batch_smem(const BatchKind &k, int shape) {
   const int th = shape_of(k, shape).threads;
-  if (k.q == 9) return k.f64 ? smem_q<9, double>(th) : smem_q<9, float>(th);
-  return k.f64 ? smem_q<19, double>(th) : smem_q<19, float>(th);
+  if (k.q == 9) return k.f64 ? smem_p<9, double>(th, k.plane) : smem_p<9, float>(th, k.plane);
+  return k.f64 ? smem_p<19, double>(th, k.plane) : smem_p<19, float>(th, k.plane);
 }
 
 BatchKind kind_of(const vlb_batch *b) {
@@ -89,11 +94,7 @@ BatchKind kind_of(const vlb_batch *b) {
 int batch_threads(const vlb_batch *b) { return shape_of(kind_of(b), b->shape).threads; }
 
 int64_t member_tiles(const vlb_sim *s, int threads) {
-  const vlb_mesh *m = s->mesh;
-  const int dim = m->md.dim;
-  const int64_t nfast = m->md.n[dim - 1];
-  const int64_t ntf = (nfast + threads - 1) / threads;
-  return ntf * (dim == 3 ? m->md.n[0] * m->md.n[1] : m->md.n[0]);
+  return s->mesh->md.q == 9 ? make_step_args<9>(s, threads).ntiles : make_step_args<19>(s, threads).ntiles;
 }
 
 int64_t total_tiles(const vlb_batch *b) {

@@ -218,10 +218,226 @@ __device__ void build_record(double J, const double *ginv, const double *G,
 __device__ __forceinline__ float two_prod_err(float x, float y, float p) { return fmaf(x, y, -p); }
 __device__ __forceinline__ double two_prod_err(double x, double y, double p) { return fma(x, y, -p); }
 
-// packed FP32 helpers: both lanes the same value; a 16-byte or 8-byte record load
+// packed FP32 helpers: both lanes the same value
 __device__ __forceinline__ float2 bcast2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+
+// A record as the collision reads it: values by their CoefLayout index, pairs and
+// quads where they are aligned. In memory (shared, global or local):
+template <typename R>
+struct PtrRecord {
+  const R *__restrict__ p;
+  __device__ __forceinline__ R operator[](int k) const { return p[k]; }
+  __device__ __forceinline__ float4 v4(int k) const { return *reinterpret_cast<const float4 *>(p + k); }
+  __device__ __forceinline__ float2 v2(int k) const { return *reinterpret_cast<const float2 *>(p + k); }
+};
+
+// A CellLayout record in registers with the entries it leaves out, formed in FP32
+// from the link coefficients a_p = am M_p, d_p = ad D_p (see build_record):
+//   R = sum_p w a (3 c c - I) / am,  Ao = w [4 d + (6 / am) c.R'.a]  with R' = am R,
+//   PE = (3/2) (itau / am) R',  PO1, PO2, LO, LD from Ao,  TT = 12 tau sum_p w d c,
+//   A = LO/4 + (TT + LD/2)/2,  H - I = -(I + A)^-1 A,  QM = (PE, PO2) + (H - I)(PE, PO2).
+// About 450 FP32 operations per cell against the 57 values (D3Q19) they replace; PO1,
+// H - I and QM multiply U, Pc and U U, so their rounding is far below that of the
+// terms stored. Every index is a constant after unrolling: v lives in registers.
+template <int Q>
+struct CellRecord {
+  using L = CoefLayout<Q>;
+  using CL = CellLayout<Q>;
+  static constexpr int D = L::D, H = L::H, NS = L::NS, NQ = L::NQ;
+  float v[L::RR];
+  __device__ __forceinline__ float operator[](int k) const { return v[k]; }
+  __device__ __forceinline__ float4 v4(int k) const { return make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]); }
+  __device__ __forceinline__ float2 v2(int k) const { return make_float2(v[k], v[k + 1]); }
+  // cell: index within [0, ncell); k6am = 6 / am, kpe = (3/2) itau / am, ktt = 12 tau
+  __device__ __forceinline__ void load(const float4 *__restrict__ rec, int64_t cell) {
+    const float4 *p = rec + (cell >> 5) * (CL::NG * 32) + (cell & 31);
+#pragma unroll
+    for (int g = 0; g < CL::NG; g++) {
+      const float4 q = __ldcs(p + g * 32);
+      const float e[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if (CL::entry(4 * g + u) >= 0) v[CL::entry(4 * g + u)] = e[u];
+    }
+  }
+  __device__ __forceinline__ float2 a01(int p) const { return make_float2(v[L::mp(p, 0)], v[L::mp(p, 1)]); }
+  __device__ __forceinline__ float2 d01(int p) const { return make_float2(v[L::dk(p, 0)], v[L::dk(p, 1)]); }
+  __device__ __forceinline__ void form(float k6am, float kpe, float ktt) {
+    // components 0 and 1 in the two lanes, component 2 (D = 3) apart
+    float2 R0[NS], S1[D], TT[D], C2[D][D], A0[D];   // R', 3-sum of Ao c, TT, PO2, A
+    float R2[NS], S1z[D], TTz[D], C2z[D][D], A2[D];
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = k; l < D; l++) {
+        float2 r = make_float2(0.f, 0.f);
+        float rz = 0.f;
+#pragma unroll
+        for (int p = 1; p <= H; p++) {
+          const float c = lat_w<Q, float>(p) * (float)(3 * Lat<Q>::c(p, k) * Lat<Q>::c(p, l) - (k == l ? 1 : 0));
+          if (3 * Lat<Q>::c(p, k) * Lat<Q>::c(p, l) - (k == l ? 1 : 0) == 0) continue;
+          r = __ffma2_rn(bcast2(c), a01(p), r);
+          if constexpr (D == 3) rz = fmaf(c, v[L::mp(p, 2)], rz);
+        }
+        R0[sym<D>(k, l)] = r;
+        R2[sym<D>(k, l)] = rz;
+      }
+#pragma unroll
+    for (int k = 0; k < D; k++) {
+      S1[k] = TT[k] = make_float2(0.f, 0.f);
+      S1z[k] = TTz[k] = 0.f;
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        C2[k][l] = make_float2(0.f, 0.f);
+        C2z[k][l] = 0.f;
+      }
+    }
+#pragma unroll
+    for (int p = 1; p <= H; p++) {
+      // c.R'.a, component by component of a
+      float2 x = make_float2(0.f, 0.f);
+      float xz = 0.f;
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        float2 cr = make_float2(0.f, 0.f);
+        float crz = 0.f;
+#pragma unroll
+        for (int k = 0; k < D; k++) {
+          const int ck = Lat<Q>::c(p, k);
+          if (ck == 0) continue;
+          cr = __ffma2_rn(bcast2((float)ck), R0[sym<D>(k, l)], cr);
+          if constexpr (D == 3) crz = fmaf((float)ck, R2[sym<D>(k, l)], crz);
+        }
+        const float al = v[L::mp(p, l)];
+        x = __ffma2_rn(cr, bcast2(al), x);
+        if constexpr (D == 3) xz = fmaf(crz, al, xz);
+      }
+      const float w = lat_w<Q, float>(p), wk = w * k6am;
+      const float2 Ao = __ffma2_rn(bcast2(wk), x, __fmul2_rn(bcast2(4.f * w), d01(p)));
+      const float Aoz = D == 3 ? fmaf(wk, xz, (4.f * w) * v[L::dk(p, 2)]) : 0.f;
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        const int cl = Lat<Q>::c(p, l);
+        if (cl == 0) continue;
+        S1[l] = __ffma2_rn(bcast2(3.f * cl), Ao, S1[l]);
+        TT[l] = __ffma2_rn(bcast2(w * cl), d01(p), TT[l]);
+        if constexpr (D == 3) {
+          S1z[l] = fmaf(3.f * cl, Aoz, S1z[l]);
+          TTz[l] = fmaf(w * cl, v[L::dk(p, 2)], TTz[l]);
+        }
+#pragma unroll
+        for (int k = 0; k < D; k++) {
+          if (k == l) continue;
+          const float c = 4.5f * cl * (float)(3 * Lat<Q>::c(p, k) * Lat<Q>::c(p, k) - 1);
+          C2[k][l] = __ffma2_rn(bcast2(c), Ao, C2[k][l]);
+          if constexpr (D == 3) C2z[k][l] = fmaf(c, Aoz, C2z[k][l]);
+        }
+      }
+    }
+    // LO^i_j = (2/3) [sum_{k != j} PO2^i_kj GH_kk + 2 sum_{l != j} PO2^i_jl GH_jl], PO1 + LO, A
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+      float2 lo = make_float2(0.f, 0.f), ld = make_float2(0.f, 0.f);
+      float loz = 0.f, ldz = 0.f;
+#pragma unroll
+      for (int k = 0; k < D; k++) {
+        if (k == j) continue;
+        const float gkk = (2.f / 3.f) * v[L::GH + sym<D>(k, k)], gjk = (4.f / 3.f) * v[L::GH + sym<D>(j, k)];
+        lo = __ffma2_rn(C2[k][j], bcast2(gkk), __ffma2_rn(C2[j][k], bcast2(gjk), lo));
+        ld = __fadd2_rn(ld, C2[k][j]);
+        if constexpr (D == 3) {
+          loz = fmaf(C2z[k][j], gkk, fmaf(C2z[j][k], gjk, loz));
+          ldz += C2z[k][j];
+        }
+      }
+      const float2 po = __fadd2_rn(S1[j], lo);
+      v[L::PO1 + j] = po.x;
+      v[L::PO1 + D + j] = po.y;
+      if constexpr (D == 3) v[L::PO1 + 2 * D + j] = S1z[j] + loz;
+      // A = LO/4 + TT/2 + LD/4, LD = T0 sum PO2
+      A0[j] = __ffma2_rn(bcast2(0.25f), lo, __ffma2_rn(bcast2(0.5f * ktt), TT[j], __fmul2_rn(bcast2(1.f / 12.f), ld)));
+      A2[j] = fmaf(0.25f, loz, fmaf(0.5f * ktt, TTz[j], (1.f / 12.f) * ldz));
+    }
+    // H - I = -(I + A)^-1 A
+    float B[D][D], Am[D][D], Hi[D][D];
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+      Am[0][j] = A0[j].x;
+      Am[1][j] = A0[j].y;
+      if constexpr (D == 3) Am[2][j] = A2[j];
+#pragma unroll
+      for (int i = 0; i < D; i++) B[i][j] = Am[i][j] + (i == j ? 1.f : 0.f);
+    }
+    if constexpr (D == 2) {
+      const float id = -1.f / (B[0][0] * B[1][1] - B[0][1] * B[1][0]);
+      Hi[0][0] = B[1][1] * id;
+      Hi[0][1] = -B[0][1] * id;
+      Hi[1][0] = -B[1][0] * id;
+      Hi[1][1] = B[0][0] * id;
+    } else {
+      float C[D][D], det = 0.f;
+#pragma unroll
+      for (int i = 0; i < D; i++)
+#pragma unroll
+        for (int j = 0; j < D; j++) {
+          const int i1 = (i + 1) % D, i2 = (i + 2) % D, j1 = (j + 1) % D, j2 = (j + 2) % D;
+          C[i][j] = fmaf(B[i1][j1], B[i2][j2], -(B[i1][j2] * B[i2][j1]));
+        }
+#pragma unroll
+      for (int j = 0; j < D; j++) det = fmaf(B[0][j], C[0][j], det);
+      const float id = -1.f / det;
+#pragma unroll
+      for (int i = 0; i < D; i++)
+#pragma unroll
+        for (int j = 0; j < D; j++) Hi[i][j] = C[j][i] * id;
+    }
+    float2 H0[D];
+    float Hz[D];
+#pragma unroll
+    for (int j = 0; j < D; j++) {
+      float h[D];
+#pragma unroll
+      for (int i = 0; i < D; i++) {
+        h[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < D; k++) h[i] = fmaf(Hi[i][k], Am[k][j], h[i]);
+        v[L::row(L::HM, D, i, j)] = h[i];
+      }
+      H0[j] = make_float2(h[0], h[1]);
+      Hz[j] = D == 3 ? h[D - 1] : 0.f;
+    }
+    // QM = X + (H - I) X for the columns X of (PE, PO2)
+    auto column = [&](int s, float2 x, float xz) {
+      float2 y = __ffma2_rn(H0[0], bcast2(x.x), __ffma2_rn(H0[1], bcast2(x.y), x));
+      if constexpr (D == 3) {
+        y = __ffma2_rn(H0[D - 1], bcast2(xz), y);
+        v[L::row(L::QM, NQ, 2, s)] = fmaf(Hz[0], x.x, fmaf(Hz[1], x.y, fmaf(Hz[D - 1], xz, xz)));
+      }
+      v[L::row(L::QM, NQ, 0, s)] = y.x;
+      v[L::row(L::QM, NQ, 1, s)] = y.y;
+    };
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = k; l < D; l++) {
+        const float c = k == l ? kpe : 2.f * kpe;
+        column(sym<D>(k, l), __fmul2_rn(bcast2(c), R0[sym<D>(k, l)]), c * R2[sym<D>(k, l)]);
+      }
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = 0; l < D; l++)
+        if (k != l) column(NS + offd<D>(k, l), C2[k][l], C2z[k][l]);
+  }
+};
+// the factors of CellRecord::form
+struct CellFactors {
+  float k6am, kpe, ktt;
+};
+inline CellFactors cell_factors(double tau) {
+  const double itau = 1.0 / tau, am = -0.25 * (2.0 - itau);
+  return CellFactors{(float)(6.0 / am), (float)(1.5 * itau / am), (float)(12.0 * tau)};
+}
 
 // The weights times 1/T0 = 3 of the axis (a1) and diagonal (a2) directions,
 // chosen so that the identities of Eq. 10 that the momentum balance of a
@@ -285,8 +501,8 @@ struct MomentWeights<9, R> {
 // and then mn = mdev - sum_a RR_a. Every term is formed relative to its own
 // size, and the identity behind the final pass holds for whatever J it uses,
 // as long as RR, their sum and mn use the same one.
-template <int Q, typename R, bool REST, bool RREC>
-__device__ __forceinline__ void form_np(const R (&d)[Q], const R *__restrict__ rc, R m, R mdev, R mn,
+template <int Q, typename R, bool REST, bool RREC, typename RC>
+__device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R mdev, R mn,
                                         R nref, R h2m, R rho, R itau, const R (&U)[Lat<Q>::D],
                                         const R (&Phi)[Lat<Q>::D], R (&dp)[Q]) {
   using L = CoefLayout<Q>;
@@ -418,7 +634,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const R *__restrict__ r
 #pragma unroll
     for (int p = 1; p <= H; p++) {
       const R df = (lat_nnz<Q>(p) == 1 ? r6w1 : r6w2) * xo[p];
-      const float2 am01 = ld2(rc + L::mp(p, 0));
+      const float2 am01 = rc.v2(L::mp(p, 0));
 #pragma unroll
       for (int i = 0; i < D; i++) {
         const int ci = Lat<Q>::c(p, i);
@@ -528,11 +744,10 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const R *__restrict__ r
 // unit roundoff of R, and Phi is a sum of dozens of rounded terms of its own
 // size, so smaller changes are rounding noise. With FINAL, the post-collision
 // deviations are formed at the converged Phi.
-// rc points at the cell's coefficient record (global, shared or local
-// memory); itau = 1/tau. With REST, d holds e_a = N_a - o_a relative to the
+// rc is the cell's coefficient record (PtrRecord or CellRecord); itau = 1/tau. With REST, d holds e_a = N_a - o_a relative to the
 // cell's own rest state (16-bit storage, see CoefLayout), and so does dp.
-template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true>
-__device__ __forceinline__ void collide_cell(const R (&d)[Q], const R *__restrict__ rc, R nref,
+template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>>
+__device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nref,
                                              R itau, R tol, int max_iter, R (&dp)[Q],
                                              CollideState<Q, R> &st) {
   using L = CoefLayout<Q>;
@@ -598,12 +813,12 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const R *__restric
     float s2a = D == 3 ? s[D - 1] : 0.f, s2b = 0.f;
 #pragma unroll
     for (int p = 1; p <= H; p++) {
-      const float4 q = ld4(rc + L::mp(p, 0));   // am M^0, am M^1, ad D^0, ad D^1
+      const float4 q = rc.v4(L::mp(p, 0));   // am M^0, am M^1, ad D^0, ad D^1
       float2 &acc = (p & 1) ? sa : sb;
       acc = __ffma2_rn(make_float2(q.x, q.y), bcast2(sp[p]), acc);
       acc = __ffma2_rn(make_float2(q.z, q.w), bcast2(tp[p]), acc);
       if constexpr (D == 3) {
-        const float2 r2 = ld2(rc + L::mp(p, 2));   // am M^2, ad D^2
+        const float2 r2 = rc.v2(L::mp(p, 2));   // am M^2, ad D^2
         float &a2 = (p & 1) ? s2a : s2b;
         a2 = fmaf(r2.x, sp[p], a2);
         a2 = fmaf(r2.y, tp[p], a2);
@@ -632,7 +847,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const R *__restric
   if constexpr (sizeof(R) == 4) {
     float2 x = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < D; j++) x = __ffma2_rn(ld2(rc + L::row(L::HM, D, 0, j)), bcast2(Pc[j]), x);
+    for (int j = 0; j < D; j++) x = __ffma2_rn(rc.v2(L::row(L::HM, D, 0, j)), bcast2(Pc[j]), x);
     const float2 p01 = __fadd2_rn(make_float2(Pc[0], Pc[1]), x);
     Pt[0] = p01.x;
     Pt[1] = p01.y;
@@ -682,17 +897,17 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const R *__restric
 #pragma unroll
       for (int s2 = 0; s2 < NQ; s2 += 2) {
         if (s2 + 1 < NQ) {
-          const float4 q = ld4(rc + L::QM + 2 * s2);
+          const float4 q = rc.v4(L::QM + 2 * s2);
           a01a = __ffma2_rn(make_float2(q.x, q.y), bcast2(mono[s2]), a01a);
           a01b = __ffma2_rn(make_float2(q.z, q.w), bcast2(mono[s2 + 1]), a01b);
         } else {
-          a01a = __ffma2_rn(ld2(rc + L::QM + 2 * s2), bcast2(mono[s2]), a01a);
+          a01a = __ffma2_rn(rc.v2(L::QM + 2 * s2), bcast2(mono[s2]), a01a);
         }
       }
       if constexpr (D == 3) {
 #pragma unroll
         for (int s4 = 0; s4 < NQ; s4 += 4) {
-          const float4 q = ld4(rc + L::row(L::QM, NQ, 2, s4));
+          const float4 q = rc.v4(L::row(L::QM, NQ, 2, s4));
           a2a = fmaf(q.x, mono[s4], a2a);
           a2b = fmaf(q.y, mono[s4 + 1], a2b);
           a2a = fmaf(q.z, mono[s4 + 2], a2a);
@@ -728,7 +943,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const R *__restric
     }
   }
   st.iters = it;
-  if (FINAL) form_np<Q, R, REST, RREC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
+  if (FINAL) form_np<Q, R, REST, RREC, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
 }

@@ -318,6 +318,8 @@ struct PackArgs {
   double wall_omega[3][2][3];
   int32_t ref_rest;  // fill the storage-reference offsets (16-bit storage, plane mode)
   double nref;
+  int32_t cellrec;   // CellLayout records (FP32, one per cell), wall velocities to uw (if not NULL)
+  float *uw;
 };
 
 template <int Q, typename R>
@@ -349,7 +351,7 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
     }
     CollideState<Q, double> cs;
     // chord iteration from F = 0 (the record's FR is still zero here)
-    collide_cell<Q, double, false>(N, rec, 0.0, 1.0 / a.tau, 1e-15, 400, Np, cs);
+    collide_cell<Q, double, false>(N, PtrRecord<double>{rec}, 0.0, 1.0 / a.tau, 1e-15, 400, Np, cs);
     for (int i = 0; i < D; i++) rec[L::FR + i] = cs.conv ? cs.F[i] : 0.0;
   }
   // the local rest state for the final pass: deviations from the uniform
@@ -403,15 +405,28 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
       }
     }
   }
-  // a per-cell record ends at RR (see CoefLayout::stride)
-  R *out = coef + r * a.stride;
-  for (int k = 0; k < a.stride; k++) out[k] = k < L::NC ? static_cast<R>(rec[k]) : R(0);
   // reference-state part of J F as a hi/lo pair
-  for (int i = 0; i < D; i++) {
-    const R hi = static_cast<R>(rec[L::KW + i]);
-    out[L::KW + i] = hi;
-    out[L::KWL + i] = static_cast<R>(rec[L::KW + i] - static_cast<double>(hi));
+  for (int i = 0; i < D; i++) rec[L::KWL + i] = rec[L::KW + i] - static_cast<double>(static_cast<R>(rec[L::KW + i]));
+  R *out = coef + r * a.stride;
+  bool cellrec = false;
+  if constexpr (sizeof(R) == 4) {
+    cellrec = a.cellrec != 0;
+    if (cellrec) {
+      using CL = CellLayout<Q>;
+      float4 *o = reinterpret_cast<float4 *>(coef) + (r >> 5) * (CL::NG * 32) + (r & 31);
+#pragma unroll
+      for (int g = 0; g < CL::NG; g++) {
+        float e[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) e[u] = CL::entry(4 * g + u) >= 0 ? (float)rec[CL::entry(4 * g + u)] : 0.0f;
+        o[g * 32] = make_float4(e[0], e[1], e[2], e[3]);
+      }
+    }
   }
+  // a per-cell record ends at RR (see CoefLayout::stride)
+  if (!cellrec)
+    for (int k = 0; k < a.stride; k++) out[k] = k < L::NC ? static_cast<R>(rec[k]) : R(0);
+  if (cellrec && !a.uw) return;
   // wall velocity: rigid motion of the adjacent wall, at the point halfway to the ghost node
   const Addr<Q> ad(a.g, c);
   double uw[3] = {0.0, 0.0, 0.0};
@@ -436,7 +451,12 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
     }
     break;
   }
-  for (int i = 0; i < D; i++) out[L::UW + i] = static_cast<R>(uw[i]);
+  for (int i = 0; i < D; i++) {
+    if (cellrec)
+      a.uw[r * D + i] = (float)uw[i];
+    else
+      out[L::UW + i] = static_cast<R>(uw[i]);
+  }
 }
 
 template <int Q>
@@ -456,6 +476,8 @@ static cudaError_t pack_q(const vlb_sim *sim, cudaStream_t s) {
   a.tau = sim->p.tau;
   a.ref_rest = sim->ref_rest;
   a.nref = sim->nref;
+  a.cellrec = sim->cellrec;
+  a.uw = sim->d_uw;
   for (int d = 0; d < 3; d++) a.body[d] = sim->p.body_force[d];
   for (int ax = 0; ax < 3; ax++)
     for (int sd = 0; sd < 2; sd++)

@@ -198,6 +198,39 @@ struct CoefLayout {
   }
 };
 
+// FP32 record of one cell (one record per cell): the entries of CoefLayout from
+// which the others follow -- J, 1/J, (g - I)/2, G, KW and its low part, FR, CE and
+// the link coefficients, NV values in NG groups of four. PO1, HM and QM are formed
+// again by the step (CellRecord in vlb_collide.cuh): with a record per cell the step is
+// bound by reading them, 544 bytes per D3Q19 cell whole and 320 so. Group g of
+// cell c lies at ((c / 32) NG + g) 32 + c % 32 in 16-byte units, so that a
+// warp's read of a group is 512 consecutive bytes. The wall velocity, read in the
+// wall cells of moving walls only, lies apart.
+template <int Q>
+struct CellLayout {
+  using L = CoefLayout<Q>;
+  static constexpr int D = L::D, H = L::H, NS = L::NS;
+  static constexpr int LINK = 2 * H * D;                 // values of the link coefficients
+  static constexpr int HEAD = 2 + NS + 5 * D;            // J, IJ, GH, BODY, KW, KWL, FR, CE
+  static constexpr int NV = LINK + HEAD;
+  static constexpr int NG = (NV + 3) / 4;
+  // entry of CoefLayout that value k holds (-1: padding); the links first
+  __host__ __device__ static constexpr int entry(int k) {
+    return k < LINK ? L::MPD + k
+           : k == LINK ? (int)L::J
+           : k == LINK + 1 ? (int)L::IJ
+           : k < LINK + 2 + NS ? L::GH + (k - LINK - 2)
+           : k < LINK + 2 + NS + 4 * D ? L::BODY + (k - LINK - 2 - NS)   // BODY, KW, KWL, FR
+           : k < NV ? L::CE + (k - LINK - 2 - NS - 4 * D)
+                    : -1;
+  }
+  static_assert(L::KW == L::BODY + D && L::KWL == L::KW + D && L::FR == L::KWL + D && L::CE == L::FR + D,
+                "BODY, KW, KWL, FR and CE follow one another");
+};
+inline size_t cell_record_bytes(int q, int64_t ncell) {
+  return (size_t)((ncell + 31) / 32) * 32 * 16 * (q == 9 ? CellLayout<9>::NG : CellLayout<19>::NG);
+}
+
 constexpr double kT0 = 1.0 / 3.0;
 
 // max that propagates NaN from either side (a NaN residual never converges);
@@ -431,8 +464,10 @@ struct vlb_sim {
   void *d_f = nullptr;        // populations [q][ncell]
   void *d_coef = nullptr;     // coefficient records, record r at r * nc elements
   int64_t ncoef = 0;
-  int32_t nc = 0;
+  int32_t nc = 0;             // values of a coefficient record
   int32_t plane = 0;
+  int32_t cellrec = 0;        // FP32, one record per cell: CellLayout, else CoefLayout
+  float *d_uw = nullptr;      // with cellrec and moving walls: wall velocities [ncell][dim]
   int64_t t = 0;
   double nref = 0.0;          // populations are stored as N_a - w_a nref, nref = rho_0 J_ref
   int32_t ref_rest = 0;       // 16-bit storage relative to the local rest state

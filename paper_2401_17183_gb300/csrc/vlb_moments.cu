@@ -26,6 +26,7 @@ struct MomArgs {
   int32_t has_rot[3];
   int32_t periodic[3];
   double tau;
+  CellFactors cf;   // FP32 records per cell (CellLayout)
   RefCtx ref;
   int *err;
 };
@@ -94,12 +95,23 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
   }
   // the cell's (or column's) coefficient record, stored in MT
   const IT c0 = a.plane ? c - ad.ic[D - 1] : c;   // the fastest axis has stride 1
-  const MT *rec = static_cast<const MT *>(a.coef) + (int64_t)(a.plane ? c0 / (IT)a.nfast : c) * a.rs;
   MT Np[Q];
   CollideState<Q, MT> st;
   // chord iteration from the record's rest-state start value
-  collide_cell<Q, MT, false>(dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau),
-                             static_cast<MT>(a.tol), 200, Np, st);
+  auto solve = [&](const auto &rec) {
+    collide_cell<Q, MT, false>(dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau),
+                               static_cast<MT>(a.tol), 200, Np, st);
+  };
+  if constexpr (sizeof(MT) == 4) {
+    if (!a.plane) {
+      CellRecord<Q> rec;
+      rec.load(static_cast<const float4 *>(a.coef), (int64_t)c);
+      rec.form(a.cf.k6am, a.cf.kpe, a.cf.ktt);
+      solve(rec);
+    }
+  }
+  if (sizeof(MT) == 8 || a.plane)
+    solve(PtrRecord<MT>{static_cast<const MT *>(a.coef) + (int64_t)(a.plane ? c0 / (IT)a.nfast : c) * a.rs});
   if (!st.conv) atomicOr(a.err, ERR_NOCONV);
   // the output mapping in the simulation's arithmetic (U and F are MT already)
   MT gl[D][D];
@@ -149,6 +161,7 @@ static cudaError_t moments_t(const vlb_sim *sim, double *d_out, int64_t nblk, cu
     for (int k = 0; k < 9; k++) a.rot[d][k] = m->md.rot[d][k];
   }
   a.tau = sim->p.tau;
+  a.cf = cell_factors(a.tau);
   a.ref = make_ref(sim);
   a.err = sim->d_err;
   using MT = typename std::conditional<std::is_same<S, double>::value, double, float>::type;

@@ -68,9 +68,17 @@ struct StepArgs {
   // of 16-bit storage), when every offset fits in 32 bits (else unused):
   // read by the kernel as constants, not formed per cell and direction
   int32_t soff[19], soffw[19];
+  // one record per cell (!plane): tiles are T consecutive cells of the whole mesh, whatever
+  // rows they lie in (ntf = ntiles, nA = nB = 1, full_tiles: the slots are aligned for
+  // 16-byte copies), and FP32 records are CellLayout's
+  CellFactors cf;
+  const float *uw;        // wall velocities of moving walls [ncell][dim]
+  int64_t coef_bytes;     // size of the records
 };
 
 constexpr int kStepThreads = 128;
+// tile width of a mesh with one record per cell that would leave SMs without a block
+constexpr int kSmallTile = 32;
 
 // asynchronous global -> shared copies of one element (4 or 8 bytes)
 template <int BYTES>
@@ -134,12 +142,16 @@ __host__ __device__ constexpr bool slow_move(int a) {
 
 // resident blocks per SM the register budget is cut for: 3 for FP32
 // storage (168 registers, no spills; 4 blocks at 128 registers ran 0.4%
-// slower, 5 at 102 registers 18% slower), 4 for 16-bit storage (128
-// registers; 3% faster than 3 blocks on even steps, 0.3% faster over both
-// parities), 2 for FP64
-template <typename R, typename S = R, bool ODD = false>
+// slower, 5 at 102 registers 18% slower), 4 for 16-bit storage in plane mode
+// (128 registers; 3% faster than 3 blocks on even steps, 0.3% faster over both
+// parities; a record per cell needs the registers for itself), 2 for FP64
+template <typename R, typename S = R, bool PLANE = true>
 constexpr int step_min_blocks() {
-  return sizeof(R) == 4 ? (sizeof(S) == 2 ? 4 : 3) : 2;
+  return sizeof(R) == 4 ? (sizeof(S) == 2 && PLANE ? 4 : 3) : 2;
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // pipeline depth: tiles whose copies are in flight while one is collided
@@ -150,9 +162,9 @@ constexpr int kStages = 3;
 // is staged as the aligned 32-bit word that holds it (asynchronous copies move
 // 4, 8 or 16 bytes), with one bit per direction saying which half it is.
 // T is the tile width (threads per block).
-template <int Q, typename S, typename R, int T = kStepThreads>
+template <int Q, typename S, typename R, int T = kStepThreads, bool PLANE = true>
 struct StepSmem {
-  static constexpr int RS = CoefLayout<Q>::template stride<R, true>();
+  static constexpr int RS = PLANE ? CoefLayout<Q>::template stride<R, true>() : 4;
   static constexpr bool H16 = sizeof(S) == 2;
   using PopT = typename std::conditional<H16, uint32_t, S>::type;
   alignas(16) R rec[kStages][RS];
@@ -202,12 +214,26 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
   // 16-byte pieces of the record that the kernel reads
   constexpr int RCHUNK = (REFOFS ? RS : L::SREST) * (int)sizeof(R) / 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  StepSmem<Q, S, R, T> &sm = *reinterpret_cast<StepSmem<Q, S, R, T> *>(smem_raw);
+  using Smem = StepSmem<Q, S, R, T, PLANE>;
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
+  constexpr bool CELLREC = !PLANE && sizeof(R) == 4;
+  using CL = CellLayout<Q>;
   S *__restrict__ f = static_cast<S *>(a.f);
   const R *__restrict__ coef = static_cast<const R *>(a.coef);
   const IT ps = (IT)a.ncell;
-  const IT nfast = (IT)(D == 3 ? a.g.n[2] : a.g.n[1]);
+  // cells along which a tile is cut: the fastest axis, or the whole mesh
+  const IT nfast = PLANE ? (IT)(D == 3 ? a.g.n[2] : a.g.n[1]) : ps;
   const int tid = threadIdx.x;
+  auto cell_addr = [&](const TileCursor &c, IT ifast) {
+    if constexpr (PLANE)
+      return tile_addr<Q, IT>(a.g, c, ifast);
+    else
+      return Addr<Q, IT>::linear(a.g, ifast);
+  };
+  // does the block copy a tile's row segments in 16-byte pieces (even steps)?
+  auto row_tile = [&](const TileCursor &c) {
+    return !ODD && a.full_tiles && (PLANE || (IT)c.tf * T + T <= nfast);
+  };
 
   // pieces of 16 bytes in one direction's row segment of a tile
   constexpr int PER_ROW = T * (int)sizeof(S) / 16;
@@ -245,11 +271,11 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
   // (thread tid takes pieces tid, tid + 128, ...).
   auto prefetch = [&](const TileCursor &c, int st) {
     const IT ifast = (IT)c.tf * T + (IT)tid;
-    bool rows = false;
+    const bool rows = row_tile(c);
     if constexpr (!ODD) {
-      if (a.full_tiles) {
-        rows = true;
-        const IT cell0 = tile_addr<Q, IT>(a.g, c, (IT)c.tf * T).cell;
+      if (rows) {
+        IT cell0 = (IT)c.tf * T;
+        if constexpr (PLANE) cell0 = tile_addr<Q, IT>(a.g, c, cell0).cell;
 #pragma unroll
         for (int k = tid; k < Q * PER_ROW; k += T) {
           const int av = k / PER_ROW, j = k - av * PER_ROW;
@@ -259,7 +285,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       }
     }
     if (!rows && ifast < nfast) {
-      const Addr<Q, IT> ad = tile_addr<Q, IT>(a.g, c, ifast);
+      const Addr<Q, IT> ad = cell_addr(c, ifast);
       if constexpr (H16 && HPAR) {
         // the same neighbour arithmetic on 32-bit words: the slow-axis moves
         // are even, the fastest-axis move is the cell's own word difference
@@ -306,6 +332,14 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
         cp_async<16>(reinterpret_cast<unsigned char *>(&sm.rec[st][0]) + 16 * k,
                      reinterpret_cast<const unsigned char *>(coef + rec * RS) + 16 * k);
     }
+    // the tile's records, one after another, towards L2
+    if constexpr (CELLREC) {
+      if (tid == 0) {
+        const int64_t o = (int64_t)c.tf * (T * CL::NG * 16), n = a.coef_bytes - o;
+        prefetch_l2(reinterpret_cast<const unsigned char *>(coef) + o,
+                    (uint32_t)(n < T * CL::NG * 16 ? n : T * CL::NG * 16));
+      }
+    }
   };
 
   // prologue: tiles t0 .. t0 + kStages - 2, one copy group each
@@ -335,16 +369,24 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
 
     const IT ifast = (IT)cur.tf * T + (IT)tid;
     if (ifast < nfast) {
-      const Addr<Q, IT> ad = tile_addr<Q, IT>(a.g, cur, ifast);
+      const Addr<Q, IT> ad = cell_addr(cur, ifast);
       const IT cell = ad.cell;
       // ---- pull (read side of Eq. 22): deviations d_a = N_a - w_a n_ref
       // ---- coefficients: in plane mode one record per column of the fastest
-      // axis, shared by the tile and staged in shared memory; else one per cell
-      const R *__restrict__ rc = PLANE ? &sm.rec[st][0] : coef + (int64_t)cell * RS;
+      // axis, shared by the tile and staged in shared memory; else one per
+      // cell (FP32: loaded into registers and completed there)
+      using RC = typename std::conditional<CELLREC, CellRecord<Q>, PtrRecord<R>>::type;
+      RC rc;
+      if constexpr (CELLREC) {
+        rc.load(reinterpret_cast<const float4 *>(coef), (int64_t)cell);
+        rc.form(a.cf.k6am, a.cf.kpe, a.cf.ktt);
+      } else {
+        rc.p = PLANE ? &sm.rec[st][0] : coef + (int64_t)cell * RS;
+      }
 
       R N[Q];
       if constexpr (H16) {
-        if (!ODD && a.full_tiles) {
+        if (row_tile(cur)) {
           // the tile's row segments, 16 bits per cell
 #pragma unroll
           for (int av = 0; av < Q; av++)
@@ -404,7 +446,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       R Np[Q];
       CollideState<Q, R> cst;
       // (with one record per cell the rest state is formed, not read)
-      collide_cell<Q, R, true, REFOFS, PLANE>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
+      collide_cell<Q, R, true, REFOFS, PLANE, RC>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
                                      arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
       if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
 
@@ -415,7 +457,10 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
         R uw[D], zero[D], gd[L::NS];
 #pragma unroll
         for (int i = 0; i < D; i++) {
-          uw[i] = rc[L::UW + i];
+          if constexpr (CELLREC)
+            uw[i] = a.uw[(int64_t)cell * D + i];
+          else
+            uw[i] = rc[L::UW + i];
           zero[i] = R(0);
         }
 #pragma unroll
@@ -471,13 +516,14 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
 }
 
 // One mesh: block b walks the tiles [b per_block, (b + 1) per_block).
-template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT>
-__global__ void __launch_bounds__(kStepThreads, step_min_blocks<R, S, ODD>())
+template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT,
+          int T = kStepThreads>
+__global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE>() * (kStepThreads / T))
     k_step(const __grid_constant__ StepArgs a) {
   const int64_t t0 = (int64_t)blockIdx.x * a.per_block;
   const int64_t t1 = t0 + a.per_block < a.ntiles ? t0 + a.per_block : a.ntiles;
   if (t0 >= t1) return;
-  step_tiles<Q, S, R, ODD, PLANE, REFOFS, HPAR, IT>(a, t0, t1);
+  step_tiles<Q, S, R, ODD, PLANE, REFOFS, HPAR, IT, T>(a, t0, t1);
 }
 
 // Many meshes in one launch: block b takes the run of tiles items[b] of mesh
@@ -525,12 +571,21 @@ inline StepArgs make_step_args(const vlb_sim *sim, int T = kStepThreads) {
         if (sim->p.wall_u[ax][sd][d] != 0.0 || sim->p.wall_omega[ax][sd][d] != 0.0) a.moving = 1;
   const int dim = m->md.dim;
   const int64_t nfast = dim == 3 ? m->md.n[2] : m->md.n[1];
-  a.ntf = (int32_t)((nfast + T - 1) / T);
-  a.nA = (int32_t)(dim == 3 ? m->md.n[0] : 1);
-  a.nB = (int32_t)(dim == 3 ? m->md.n[1] : m->md.n[0]);
-  a.ntiles = (int64_t)a.ntf * a.nA * a.nB;
   a.per_block = 0;
-  a.full_tiles = nfast % T == 0 ? 1 : 0;
+  if (sim->plane) {
+    a.ntf = (int32_t)((nfast + T - 1) / T);
+    a.nA = (int32_t)(dim == 3 ? m->md.n[0] : 1);
+    a.nB = (int32_t)(dim == 3 ? m->md.n[1] : m->md.n[0]);
+    a.full_tiles = nfast % T == 0 ? 1 : 0;
+  } else {
+    a.ntf = (int32_t)((m->ncell + T - 1) / T);
+    a.nA = a.nB = 1;
+    a.full_tiles = m->ncell * storage_bytes(sim->p.precision) % 16 == 0 ? 1 : 0;
+  }
+  a.ntiles = (int64_t)a.ntf * a.nA * a.nB;
+  a.cf = cell_factors(sim->p.tau);
+  a.uw = sim->d_uw;
+  a.coef_bytes = sim->cellrec ? (int64_t)cell_record_bytes(m->md.q, m->ncell) : 0;
   const bool i32 = (int64_t)Q * m->ncell < ((int64_t)1 << 31);
   for (int k = 0; k < 19; k++) {
     a.soff[k] = (i32 && k < Q) ? (int32_t)(k * m->ncell) : 0;
@@ -561,30 +616,43 @@ static int resident_blocks(const void *kern, size_t smem, int threads = kStepThr
 template <int Q, typename S, typename R>
 cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
-  StepArgs a = make_step_args<Q>(sim);
+  // one record per cell on a mesh of at most one full tile per SM: tiles of one
+  // warp, so that every SM has work (2,048 D2Q9 cells, FP32: 3.2 -> 2.9 us a step)
+  const bool small = !sim->plane && m->ncell <= (int64_t)kStepThreads * 152;
+  StepArgs a = make_step_args<Q>(sim, small ? kSmallTile : kStepThreads);
   // 32-bit indexing when every population offset fits
   const bool i32 = (int64_t)Q * m->ncell < ((int64_t)1 << 31);
   if (a.ntiles == 0) return cudaSuccess;
-  const size_t smem = sizeof(StepSmem<Q, S, R>);
-  auto go = [&](void (*kern)(StepArgs)) {
-    const int64_t nblk_max = resident_blocks(reinterpret_cast<const void *>(kern), smem);
+  auto go = [&](void (*kern)(StepArgs), size_t smem, int threads) {
+    const int64_t nblk_max = resident_blocks(reinterpret_cast<const void *>(kern), smem, threads);
     a.per_block = (a.ntiles + nblk_max - 1) / nblk_max;
     const int64_t nblk = (a.ntiles + a.per_block - 1) / a.per_block;
-    kern<<<(unsigned)nblk, kStepThreads, smem, s>>>(a);
+    kern<<<(unsigned)nblk, (unsigned)threads, smem, s>>>(a);
   };
   auto pick = [&](auto plane_tag, auto ref_tag, auto par_tag) {
     constexpr bool P = decltype(plane_tag)::value, RO = decltype(ref_tag)::value;
     constexpr bool HP = decltype(par_tag)::value;
+    constexpr size_t smem = sizeof(StepSmem<Q, S, R, kStepThreads, P>);
+    if constexpr (!P) {
+      constexpr size_t smem_s = sizeof(StepSmem<Q, S, R, kSmallTile, P>);
+      if (small && i32) {
+        if (odd)
+          go(k_step<Q, S, R, true, P, RO, HP, int32_t, kSmallTile>, smem_s, kSmallTile);
+        else
+          go(k_step<Q, S, R, false, P, RO, HP, int32_t, kSmallTile>, smem_s, kSmallTile);
+        return;
+      }
+    }
     if (i32) {
       if (odd)
-        go(k_step<Q, S, R, true, P, RO, HP, int32_t>);
+        go(k_step<Q, S, R, true, P, RO, HP, int32_t>, smem, kStepThreads);
       else
-        go(k_step<Q, S, R, false, P, RO, HP, int32_t>);
+        go(k_step<Q, S, R, false, P, RO, HP, int32_t>, smem, kStepThreads);
     } else {
       if (odd)
-        go(k_step<Q, S, R, true, P, RO, HP, int64_t>);
+        go(k_step<Q, S, R, true, P, RO, HP, int64_t>, smem, kStepThreads);
       else
-        go(k_step<Q, S, R, false, P, RO, HP, int64_t>);
+        go(k_step<Q, S, R, false, P, RO, HP, int64_t>, smem, kStepThreads);
     }
   };
   const std::true_type yes;
