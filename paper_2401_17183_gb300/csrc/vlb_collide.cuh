@@ -260,6 +260,16 @@ struct CellRecord {
         if (CL::entry(4 * g + u) >= 0) v[CL::entry(4 * g + u)] = e[u];
     }
   }
+  // the values as if just read: a loop that keeps the record may not move
+  // arithmetic on it out of its body, where products and sums would be contracted
+  // differently from the step kernel's
+  __device__ __forceinline__ void opaque() {
+#pragma unroll
+    for (int k = 0; k < L::RR; k++)
+      if (k <= L::IJ || (k >= L::MPD && k < L::MPD + 2 * H * D) || (k >= L::HM && k < L::HM + D * D) ||
+          (k >= L::QM && k < L::QM + D * NQ))
+        asm volatile("" : "+f"(v[k]));
+  }
   __device__ __forceinline__ float2 a01(int p) const { return make_float2(v[L::mp(p, 0)], v[L::mp(p, 1)]); }
   __device__ __forceinline__ float2 d01(int p) const { return make_float2(v[L::dk(p, 0)], v[L::dk(p, 1)]); }
   __device__ __forceinline__ void form(float k6am, float kpe, float ktt) {
@@ -626,7 +636,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   for (int i = 0; i < D; i++)
 #pragma unroll
     for (int j = 0; j < D; j++) dP[i][j] = R(0);
-  if constexpr (sizeof(R) == 4) {
+  {
     // columns 0 and 1 in the two lanes of packed FP32 instructions
     float2 P01[D];
 #pragma unroll
@@ -648,21 +658,6 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
     for (int i = 0; i < D; i++) {
       dP[i][0] = P01[i].x;
       dP[i][1] = P01[i].y;
-    }
-  } else {
-#pragma unroll
-    for (int p = 1; p <= H; p++) {
-      const R df = (lat_nnz<Q>(p) == 1 ? r6w1 : r6w2) * xo[p];
-#pragma unroll
-      for (int j = 0; j < D; j++) {
-        const R amM = rc[L::mp(p, j)];
-#pragma unroll
-        for (int i = 0; i < D; i++) {
-          const int ci = Lat<Q>::c(p, i);
-          if (ci > 0) dP[i][j] = fmar(amM, df, dP[i][j]);
-          if (ci < 0) dP[i][j] = fmar(-amM, df, dP[i][j]);
-        }
-      }
     }
   }
   R tr = dP[0][0];
@@ -702,7 +697,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
     const R wm = axis ? wm1 : wm2;
     const R rw = rw_at(p);
     // odd part of J f^eq over 3 w: m xo on diagonals, m O on axis pairs
-    if constexpr (sizeof(R) == 4) {
+    {
       // the pair in the two lanes of packed FP32 instructions (same roundings)
       const float2 dd = make_float2(d[p], d[p + H]);
       const float2 bs = __ffma2_rn(bcast2(-rw), bcast2(mn), REST ? dd : __fadd2_rn(dd, bcast2(-rr_at(p))));
@@ -719,20 +714,287 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
                                   __fadd2_rn(bcast2(Ep), make_float2(Op, -Op)));
       dp[p] = r.x;
       dp[p + H] = r.y;
-    } else {
-      R neqp, neqm;
-      const R r0 = REST ? R(0) : rr_at(p);
-      const R bp = fmar(-rw, mn, d[p] - r0), bm = fmar(-rw, mn, d[p + H] - r0);
-      if (axis) {
-        const R o = sl > 0 ? Oax[l] : -Oax[l];
-        neqp = fmar(-m, o, fmar(-wm, xe[p], bp));
-        neqm = fmar(m, o, fmar(-wm, xe[p], bm));
-      } else {
-        neqp = bp - wm * (xe[p] + xo[p]);
-        neqm = bm - wm * (xe[p] - xo[p]);
+    }
+  }
+}
+
+// x as FP32 by integer operations, truncated (a conversion instruction would
+// take a turn of the FP64 pipe); below the FP32 range 0, above it NaN
+__device__ __forceinline__ float trunc_f32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), mag = hi & 0x7fffffffu;
+  const uint32_t b = ((mag - 0x38000000u) << 3) | (lo >> 29);
+  return __uint_as_float((mag < 0x38100000u ? 0u : mag >= 0x47f00000u ? 0x7fc00000u : b) | (hi & 0x80000000u));
+}
+
+// The whole local collision in FP64 (see collide_cell). GB300 runs an FP64
+// instruction of a warp in 64 cycles of its quarter SM, so only the FP64 operations
+// count, about 480 per D3Q19 cell here (920 when the FP32 form was used in FP64):
+//  - the chord iteration starts from Pt = H Pc with three evaluations of the
+//    polynomial in FP32: its value is of the order of curvature times U^2, so FP32 leaves
+//    an error of about 1e-13 m, which one evaluation in FP64 reduces by the map's
+//    contraction. It is accepted when its change is at most tol max(m, |Phi|), or when a
+//    bound on the contraction times the change is below that by a factor 64 (the
+//    next change, and the error left, are then smaller still). Below four iterations
+//    allowed: the plain iteration from the rest state's force.
+//  - the test reads the sizes by integer operations on the high words;
+//  - N' is formed from the pair sums and differences, even and odd part once per pair:
+//      even: (1 - 1/tau) s/2 + w [y0 + c.Y.c],  odd: (1 - 1/tau) t/2 + w [(m/tau) xo + 3 c.Phi],
+//    Y = (9/2)(m/tau) B + 9 P, P = J deltaPi (Eq. 30) symmetrised,
+//    y0 = (mdev - (3/2) m tr B)/tau - 3 tr P.
+// D3Q19 channel, 64^3: 383 -> 219 us a step, the FP64 pipe over 90% busy.
+template <int Q, bool FINAL, typename RC>
+__device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, double nref, double itau, double tol,
+                                            int max_iter, double (&dp)[Q], CollideState<Q, double> &st) {
+  using L = CoefLayout<Q>;
+  constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS, NQ = L::NQ;
+  double s[H + 1], t[H + 1], mu[D], Pc[D], Pt[D], mdev = d[0];
+#pragma unroll
+  for (int i = 0; i < D; i++) mu[i] = Pc[i] = 0.0;
+#pragma unroll
+  for (int p = 1; p <= H; p++) {
+    s[p] = d[p] + d[p + H];
+    t[p] = d[p] - d[p + H];
+    mdev += s[p];
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      const int ci = Lat<Q>::c(p, i);
+      if (ci > 0) mu[i] += t[p];
+      if (ci < 0) mu[i] -= t[p];
+      Pc[i] = fma(rc[L::mp(p, i)], s[p], Pc[i]);
+      Pc[i] = fma(rc[L::dk(p, i)], t[p], Pc[i]);
+    }
+  }
+  const double m = nref + mdev, im = 1.0 / m, h2m = 0.5 * im, hm = 0.5 * m;
+  const double kf = fma(0.5 * itau, mdev, nref);
+  st.rho = m * rc[L::IJ];
+  double hmu[D];
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+    st.U[i] = mu[i] * im;
+    hmu[i] = -0.5 * mu[i];
+  }
+  // Pc = sum_p (am M s + ad D t) + m G - (n_ref + mdev itau/2) KW - m/2 (CE + (PO1 + LO) U)
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+    double v = fma(m, rc[L::BODY + i], Pc[i]);
+    v = fma(-hm, rc[L::CE + i], v);
+#pragma unroll
+    for (int l = 0; l < D; l++) v = fma(rc[L::PO1 + i * D + l], hmu[l], v);
+    Pc[i] = fma(-kf, rc[L::KW + i], v);
+  }
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+    Pt[i] = Pc[i];
+#pragma unroll
+    for (int j = 0; j < D; j++) Pt[i] = fma(rc[L::row(L::HM, D, i, j)], Pc[j], Pt[i]);
+  }
+  double Phi[D];
+  float lip = 1.0e30f;   // bound on the contraction of one evaluation
+  int it = 0;
+  const float mf = trunc_f32(m);
+  if (max_iter >= 4) {
+    float qf[D][NQ], Uf[D], Pf[D], df[D], l2 = 0.f, l3 = 0.f, um = 0.f;
+    const float hf = trunc_f32(h2m), hmf = 0.5f * mf;
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      Uf[i] = trunc_f32(st.U[i]);
+      Pf[i] = trunc_f32(Pt[i]);
+      df[i] = 0.f;
+#pragma unroll
+      for (int k = 0; k < NQ; k++) {
+        qf[i][k] = trunc_f32(rc[L::row(L::QM, NQ, i, k)]);
+        if (k < NS)
+          l2 += fabsf(qf[i][k]);
+        else
+          l3 += fabsf(qf[i][k]);
       }
-      dp[p] = d[p] - itau * neqp + (Ep + Op);
-      dp[p + H] = d[p + H] - itau * neqm + (Ep - Op);
+    }
+#pragma unroll
+    for (int r = 0; r < 3; r++) {
+      float x[D], mono[NQ];
+#pragma unroll
+      for (int i = 0; i < D; i++) {
+        x[i] = fmaf(Pf[i] + df[i], hf, Uf[i]);
+        um = fmaxf(um, fabsf(x[i]));
+      }
+#pragma unroll
+      for (int k = 0; k < D; k++)
+#pragma unroll
+        for (int l = 0; l < D; l++) {
+          if (k <= l) mono[sym<D>(k, l)] = x[k] * x[l];
+          if (k != l) mono[NS + offd<D>(k, l)] = (x[k] * x[k]) * x[l];
+        }
+#pragma unroll
+      for (int i = 0; i < D; i++) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < NQ; k++) v = fmaf(qf[i][k], mono[k], v);
+        df[i] = -hmf * v;
+      }
+    }
+    it = 3;
+    // |d Phi_new| <= m/2 |dQ/dU~| |d Phi| / (2 m) <= (l2 2 um + l3 3 um^2) / 4, with room for
+    // U~ to lie outside the FP32 iterates
+    um *= 1.01f;
+    lip = fmaf(0.5f * l2, um, 0.75f * l3 * um * um);
+#pragma unroll
+    for (int i = 0; i < D; i++) Phi[i] = Pt[i] + (double)df[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < D; i++) Phi[i] = m * rc[L::FR + i];
+  }
+  st.conv = false;
+  const float tolf = (float)tol, epsf = (float)(64.0 / 9007199254740992.0);
+#pragma unroll 1
+  while (it < max_iter) {
+    double Ut[D], mono[NQ];
+    float diff = 0.f, pmax = 0.f;
+#pragma unroll
+    for (int i = 0; i < D; i++) Ut[i] = fma(Phi[i], h2m, st.U[i]);
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = k; l < D; l++) mono[sym<D>(k, l)] = Ut[k] * Ut[l];
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = 0; l < D; l++)
+        if (k != l) mono[NS + offd<D>(k, l)] = mono[sym<D>(k, k)] * Ut[l];
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      // two partial sums: the chain of a small mesh is bound by latency
+      double a = rc[L::row(L::QM, NQ, i, 0)] * mono[0], b = rc[L::row(L::QM, NQ, i, 1)] * mono[1];
+#pragma unroll
+      for (int k = 2; k < NQ; k++) {
+        if (k & 1)
+          b = fma(rc[L::row(L::QM, NQ, i, k)], mono[k], b);
+        else
+          a = fma(rc[L::row(L::QM, NQ, i, k)], mono[k], a);
+      }
+      const double pn = fma(-hm, a + b, Pt[i]);
+      diff = maxnan(diff, fabsf(trunc_f32(pn - Phi[i])));
+      pmax = maxnan(pmax, fabsf(trunc_f32(pn)));
+      Phi[i] = pn;
+    }
+    it++;
+    const float scale = fmaxf(tolf * maxnan(mf, pmax), epsf * pmax);
+    if (diff <= scale || 64.f * lip * diff <= scale) {
+      st.conv = true;
+      break;
+    }
+  }
+  st.iters = it;
+#pragma unroll
+  for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
+  if constexpr (FINAL) {
+    double Ut[D], B[NS], C2[D][D], Sc[D], T0[D], T[D][D], tb = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; i++) Ut[i] = fma(Phi[i], h2m, st.U[i]);
+    // 3 B = (g - I) + 3 U~U~ (T0 = 1/3); (3/2) C^kkl = (1/2)[gd_kk U~^l + (U~^l - U^l) + 2 gd_kl U~^k]
+    // + (3/2)(U~^k)^2 U~^l, with GH = gd / 2
+    double U3[D], du[D];
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      U3[i] = 3.0 * Ut[i];
+      du[i] = Phi[i] * (0.5 * h2m);   // (U~ - U) / 2
+    }
+#pragma unroll
+    for (int i = 0; i < D; i++)
+#pragma unroll
+      for (int j = i; j < D; j++) B[sym<D>(i, j)] = fma(U3[i], Ut[j], 2.0 * rc[L::GH + sym<D>(i, j)]);
+#pragma unroll
+    for (int i = 0; i < D; i++) tb += B[sym<D>(i, i)];
+    // per axis l: xo/3 of an axis direction is T0_l = U^l - sum_k C2^kl, of a diagonal
+    // c^l T_lk + c^k T_kl with T_lk = T0_l + 3 C2^kl
+#pragma unroll
+    for (int l = 0; l < D; l++) {
+      Sc[l] = 0.0;
+#pragma unroll
+      for (int k = 0; k < D; k++) {
+        if (k == l) continue;
+        // gd_kk/2 + (3/2) U~k^2 = B_kk / 2
+        C2[k][l] = fma(0.5 * B[sym<D>(k, k)], Ut[l], fma(rc[L::GH + sym<D>(k, l)], Ut[k] + Ut[k], du[l]));
+        Sc[l] += C2[k][l];
+      }
+      T0[l] = st.U[l] - Sc[l];
+    }
+#pragma unroll
+    for (int l = 0; l < D; l++)
+#pragma unroll
+      for (int k = 0; k < D; k++)
+        if (k != l) T[l][k] = fma(3.0, C2[k][l], T0[l]);
+    // P^kl = J deltaPi^kl = 2 m sum_p w c^k am M^l xo = sum_p (6 m w) c^k am M^l (xo / 3)
+    double P[D][D];
+#pragma unroll
+    for (int i = 0; i < D; i++)
+#pragma unroll
+      for (int j = 0; j < D; j++) P[i][j] = 0.0;
+    auto xo3 = [&](int p) {
+      const int l = nz_axis<Q>(p, 0), k = nz_axis<Q>(p, 1);
+      const int sl = Lat<Q>::c(p, l);
+      if (k < 0) return sl > 0 ? T0[l] : -T0[l];
+      const double a = sl > 0 ? T[l][k] : -T[l][k];
+      return Lat<Q>::c(p, k) > 0 ? a + T[k][l] : a - T[k][l];
+    };
+    // the axis weight is 2 (D3Q19) or 4 (D2Q9) times the diagonal one
+    constexpr double wr = D == 3 ? 2.0 : 4.0;
+    const double w2 = lat_w<Q, double>(H);
+#pragma unroll
+    for (int p = 1; p <= H; p++) {
+      const double x = lat_nnz<Q>(p) == 1 ? wr * xo3(p) : xo3(p);
+#pragma unroll
+      for (int j = 0; j < D; j++) {
+        const double M = rc[L::mp(p, j)];
+#pragma unroll
+        for (int i = 0; i < D; i++) {
+          const int ci = Lat<Q>::c(p, i);
+          if (ci > 0) P[i][j] = fma(M, x, P[i][j]);
+          if (ci < 0) P[i][j] = fma(-M, x, P[i][j]);
+        }
+      }
+    }
+    // everything times w2: Y = w2 [(9/2)(m/tau) B + 9 P], B = (3 B) / 3
+    const double mt = m * itau, yb = (1.5 * w2) * mt, yp = (54.0 * w2 * w2) * m;
+    double Y[NS], trP = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      trP += P[i][i];
+#pragma unroll
+      for (int j = i; j < D; j++)
+        Y[sym<D>(i, j)] = fma(yb, B[sym<D>(i, j)], i == j ? yp * P[i][i] : (0.5 * yp) * (P[i][j] + P[j][i]));
+    }
+    // y0 = w2 [(mdev - m (3 tr B) / 2) / tau - 3 tr P]
+    const double y0 = fma(-((18.0 * w2 * w2) * m), trP, w2 * itau * fma(-hm, tb, mdev));
+    // (the weights of the odd part are MomentWeights': no momentum is made by rounding them)
+    using MW = MomentWeights<Q, double>;
+    const double omt = 1.0 - itau, h = 0.5 * omt, zm = MW::a2 * mt;
+    double Z0[D], Z[D][D];
+#pragma unroll
+    for (int l = 0; l < D; l++) {
+      Z0[l] = fma(mt, fma(MW::a1, st.U[l], -(MW::b1 * Sc[l])), MW::a1 * Phi[l]);
+#pragma unroll
+      for (int k = 0; k < D; k++)
+        if (k != l) Z[l][k] = fma(zm, T[l][k], MW::a2 * Phi[l]);
+    }
+    dp[0] = fma(omt, d[0], (lat_w<Q, double>(0) / w2) * y0);
+#pragma unroll
+    for (int p = 1; p <= H; p++) {
+      const int l = nz_axis<Q>(p, 0), k = nz_axis<Q>(p, 1);
+      const int sl = Lat<Q>::c(p, l);
+      double e, o;
+      if (k < 0) {
+        e = wr * (y0 + Y[sym<D>(l, l)]);
+        o = sl > 0 ? Z0[l] : -Z0[l];
+      } else {
+        const int sk = Lat<Q>::c(p, k);
+        const double sd = y0 + (Y[sym<D>(l, l)] + Y[sym<D>(k, k)]);
+        e = fma((double)(2 * sl * sk), Y[sym<D>(l, k)], sd);
+        const double a = sl > 0 ? Z[l][k] : -Z[l][k];
+        o = sk > 0 ? a + Z[k][l] : a - Z[k][l];
+      }
+      const double ev = fma(h, s[p], e), od = fma(h, t[p], o);
+      dp[p] = ev + od;
+      dp[p + H] = ev - od;
     }
   }
 }
@@ -746,10 +1008,11 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
 // deviations are formed at the converged Phi.
 // rc is the cell's coefficient record (PtrRecord or CellRecord); itau = 1/tau. With REST, d holds e_a = N_a - o_a relative to the
 // cell's own rest state (16-bit storage, see CoefLayout), and so does dp.
-template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>>
-__device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nref,
+template <int Q, typename R, bool FINAL, bool REST, bool RREC, typename RC>
+__device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nref,
                                              R itau, R tol, int max_iter, R (&dp)[Q],
                                              CollideState<Q, R> &st) {
+  static_assert(sizeof(R) == 4, "FP64 goes through collide_f64");
   using L = CoefLayout<Q>;
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS, NQ = L::NQ;
   static_assert(D == 2 || NQ % 4 == 0, "row 2 of the chord step is read in 16-byte quads");
@@ -806,7 +1069,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
     s[i] = m * rc[L::BODY + i] - err - R(0.5) * itau * mdev * kw;
     if constexpr (REST) s[i] += rc[L::SR + i];
   }
-  if constexpr (sizeof(R) == 4) {
+  {
     // components 0 and 1 in the two lanes of packed FP32 instructions, two
     // partial sums each
     float2 sa = make_float2(s[0], s[1]), sb = make_float2(0.f, 0.f);
@@ -828,11 +1091,6 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
     s[0] = st01.x;
     s[1] = st01.y;
     if constexpr (D == 3) s[D - 1] = s2a + s2b;
-  } else {
-#pragma unroll
-    for (int i = 0; i < D; i++)
-#pragma unroll
-      for (int p = 1; p <= H; p++) s[i] = fmar(rc[L::dk(p, i)], tp[p], fmar(rc[L::mp(p, i)], sp[p], s[i]));
   }
   // Pc = Pb - 1/2 m (CE + (PO1 + LO) U), then Pt = H Pc = Pc + (H - I) Pc
   R Pc[D];
@@ -844,7 +1102,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
     Pc[i] = (s[i] - hm * u) - pr[i];
   }
   R Pt[D];
-  if constexpr (sizeof(R) == 4) {
+  {
     float2 x = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < D; j++) x = __ffma2_rn(rc.v2(L::row(L::HM, D, 0, j)), bcast2(Pc[j]), x);
@@ -857,18 +1115,14 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
       for (int j = 0; j < D; j++) y = fmar(rc[L::row(L::HM, D, 2, j)], Pc[j], y);
       Pt[D - 1] = Pc[D - 1] + y;
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < D; i++) {
-      R y = R(0);
-#pragma unroll
-      for (int j = 0; j < D; j++) y = fmar(rc[L::row(L::HM, D, i, j)], Pc[j], y);
-      Pt[i] = Pc[i] + y;
-    }
   }
+  // Start at Pt = H Pc, the fixed point without the polynomial part: it is off by that
+  // part, of the order of curvature times U^2 (the rest state's force, the start
+  // when only a few evaluations are allowed, by curvature times U), so that one
+  // evaluation less reaches the same residual.
   R Phi[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) Phi[i] = m * rc[L::FR + i];
+  for (int i = 0; i < D; i++) Phi[i] = max_iter >= 4 ? Pt[i] : m * rc[L::FR + i];
   st.conv = false;
   int it = 0;
   while (it < max_iter) {
@@ -889,7 +1143,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
       for (int l = 0; l < D; l++)
         if (k != l) mono[NS + offd<D>(k, l)] = sq[k] * Ut[l];
     R a[D];
-    if constexpr (sizeof(R) == 4) {
+    {
       // rows 0 and 1 in the two lanes of packed FP32 instructions, two partial
       // sums per row
       float2 a01a = make_float2(0.f, 0.f), a01b = make_float2(0.f, 0.f);
@@ -918,14 +1172,6 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
       a[0] = a01.x;
       a[1] = a01.y;
       if constexpr (D == 3) a[D - 1] = a2a + a2b;
-    } else {
-#pragma unroll
-      for (int i = 0; i < D; i++) {
-        R x = R(0);
-#pragma unroll
-        for (int s2 = 0; s2 < NQ; s2++) x = fmar(rc[L::row(L::QM, NQ, i, s2)], mono[s2], x);
-        a[i] = x;
-      }
     }
     it++;
     // converged when the change is at most max(tol max(m, |Phi|), 64 eps |Phi|)
@@ -946,6 +1192,18 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
   if (FINAL) form_np<Q, R, REST, RREC, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
+}
+
+// the local collision in the arithmetic type R
+template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>>
+__device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nref, R itau, R tol, int max_iter,
+                                             R (&dp)[Q], CollideState<Q, R> &st) {
+  if constexpr (sizeof(R) == 8) {
+    static_assert(!REST, "FP64 populations are stored relative to the uniform reference");
+    collide_f64<Q, FINAL, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+  } else {
+    collide_f32<Q, R, FINAL, REST, RREC, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+  }
 }
 
 }  // namespace vlb
