@@ -159,16 +159,49 @@ __device__ __noinline__ bool dual(int dim, const double gl[3][3], double &J, dou
 }
 
 // ------------------------------------------------------------------ precompute
+// Tangents, J, co-tangents and g^ij of every cell. A cell away from every end of
+// an axis reads its 2 D + 1 node positions directly; the others go through position().
 template <int Q>
-__global__ void k_geometry(const MeshDev m, Grid g, int64_t ncell, double *J_out, double *gl_out,
-                           double *gu_out, double *ginv_out, double *K_out, int *err) {
+__global__ void __launch_bounds__(128) k_tangents(const MeshDev m, Grid g, int64_t ncell, double *J_out, double *gl_out,
+                                                  double *gu_out, double *ginv_out, int *err) {
   constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2;
   const int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= ncell) return;
-  const Addr<Q> ad(g, cell);
-  const int64_t q[3] = {ad.ic[0], ad.ic[1], ad.ic[2]};
+  const Addr<19> ad(g, cell);   // (index coordinates only)
+  bool inner = true;
+#pragma unroll
+  for (int i = 0; i < D; i++) inner = inner && ad.ic[i] > 0 && ad.ic[i] < g.n[i] - 1;
   double gl[3][3], gu[3][3], J = 0.0;
-  bool ok = tangents(m, q, gl);
+  bool ok = true;
+  if (inner) {
+    const double dx = m.dx > 0.0 ? m.dx : 1.0;
+    const double *x = m.x + cell * D;
+    double x0[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int d = 0; d < D; d++) x0[d] = x[d];
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+      for (int d = 0; d < 3; d++) gl[i][d] = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      double Dp[3] = {0.0, 0.0, 0.0}, Dm[3] = {0.0, 0.0, 0.0}, df[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int d = 0; d < D; d++) {
+        Dp[d] = x[g.s[i] * D + d] - x0[d];
+        Dm[d] = x[-g.s[i] * D + d] - x0[d];
+        df[d] = Dp[d] - Dm[d];
+      }
+      const double nd = nrm(df);
+      if (!(nd > 0.0)) ok = false;
+      const double beta = (nrm(Dp) + nrm(Dm)) / nd;
+#pragma unroll
+      for (int d = 0; d < D; d++) gl[i][d] = beta * df[d] / (2.0 * dx);
+    }
+  } else {
+    const int64_t q[3] = {ad.ic[0], ad.ic[1], ad.ic[2]};
+    ok = tangents(m, q, gl);
+  }
   ok = ok && dual(D, gl, J, gu);
   if (!ok) {
     atomicOr(err, ERR_GEOM);
@@ -186,42 +219,78 @@ __global__ void k_geometry(const MeshDev m, Grid g, int64_t ncell, double *J_out
       for (int d = 0; d < 3; d++) s += gu[i][d] * gu[j][d];  // g^ij = g^i . g^j (Eq. 8)
       ginv_out[cell * NS + sym<D>(i, j)] = s;
     }
-  for (int i = 0; i < D; i++) K_out[(cell * Q + 0) * D + i] = 0.0;
-  // K^i_a = sum_j c^j_a [g_j(q + c_a) - g_j(q)] . g^i(q) = sum_j c^j_a Theta^i_j(q + c_a, q) (Eq. 11)
-#pragma unroll 1
-  for (int a = 1; a < Q; a++) {
-    double Kv[3] = {0.0, 0.0, 0.0};
-    // links that cross a wall: zero, or from the ghost-node tangents
-    if (!ad.crosses(a, 1) || m.wall_links == VLB_WALL_LINKS_GHOST) {
-      int64_t p[3] = {q[0], q[1], q[2]};
-      for (int d = 0; d < D; d++) p[d] += Lat<Q>::c(a, d);
-      double gp[3][3];
-      if (!tangents(m, p, gp)) atomicOr(err, ERR_GEOM);
-      double de[3] = {0.0, 0.0, 0.0};
-      for (int j = 0; j < D; j++) {
-        const int cj = Lat<Q>::c(a, j);
-        if (cj == 0) continue;
-        for (int d = 0; d < 3; d++) de[d] += cj * (gp[j][d] - gl[j][d]);
-      }
-      for (int i = 0; i < D; i++) Kv[i] = de[0] * gu[i][0] + de[1] * gu[i][1] + de[2] * gu[i][2];
-    }
-    for (int i = 0; i < D; i++) K_out[(cell * Q + a) * D + i] = Kv[i];
-  }
 }
 
-cudaError_t launch_geometry(const vlb_mesh *m, int *d_err, cudaStream_t s) {
-  const int threads = 128;
-  const int64_t blocks = (m->ncell + threads - 1) / threads;
+// K^i_a = sum_j c^j_a [g_j(q + c_a) - g_j(q)] . g^i(q) = sum_j c^j_a Theta^i_j(q + c_a, q) (Eq. 11), one
+// thread per cell and direction, from the stored tangents (links off the mesh: from
+// the positions of the image or ghost nodes). Forming the tangents again at every
+// neighbour (19 times per cell, each from seven positions) had made the precompute
+// 7.0 ms on 492 K general D3Q19 cells; 0.64 ms (tangents) and 1.26 ms (links) so.
+template <int Q>
+__global__ void __launch_bounds__(256) k_links(const MeshDev m, Grid g, int64_t ncell, const double *gl,
+                                               const double *gu, double *K_out, int *err) {
+  constexpr int D = Lat<Q>::D;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= ncell * Q) return;
+  const int64_t cell = t / Q;
+  const int a = (int)(t - cell * Q);
+  int64_t q[3];
+  {
+    int64_t r = cell;
+    q[2] = r % g.n[2];
+    r /= g.n[2];
+    q[1] = r % g.n[1];
+    q[0] = r / g.n[1];
+  }
+  int c[3] = {0, 0, 0};
+  int64_t p[3] = {q[0], q[1], q[2]};
+  bool wall = false, out = false;   // the link leaves through a wall, or at all
+  for (int d = 0; d < D; d++) {
+    c[d] = Lat<Q>::c(a, d);
+    p[d] += c[d];
+    if (p[d] >= 0 && p[d] < g.n[d]) continue;
+    out = true;
+    wall = wall || g.wall[d];
+  }
+  double Kv[3] = {0.0, 0.0, 0.0};
+  // links that cross a wall: zero, or from the ghost-node tangents
+  if (a != 0 && (!wall || m.wall_links == VLB_WALL_LINKS_GHOST)) {
+    double gp[3][3], de[3] = {0.0, 0.0, 0.0};
+    if (out) {
+      if (!tangents(m, p, gp)) atomicOr(err, ERR_GEOM);
+    } else {
+      const double *o = gl + ((p[0] * g.n[1] + p[1]) * g.n[2] + p[2]) * D * D;
+      for (int j = 0; j < D; j++)
+        for (int d = 0; d < 3; d++) gp[j][d] = d < D ? o[j * D + d] : 0.0;
+    }
+    for (int j = 0; j < D; j++) {
+      if (c[j] == 0) continue;
+      for (int d = 0; d < D; d++) de[d] += c[j] * (gp[j][d] - gl[(cell * D + j) * D + d]);
+    }
+    for (int i = 0; i < D; i++) {
+      double v = 0.0;
+      for (int d = 0; d < D; d++) v += de[d] * gu[(cell * D + i) * D + d];
+      Kv[i] = v;
+    }
+  }
+  for (int i = 0; i < D; i++) K_out[t * D + i] = Kv[i];
+}
+
+template <int Q>
+static void launch_geometry_q(const vlb_mesh *m, int *d_err, cudaStream_t s) {
   const Grid g = make_grid(m);
+  k_tangents<Q><<<(unsigned)((m->ncell + 127) / 128), 128, 0, s>>>(m->md, g, m->ncell, m->d_J, m->d_gl, m->d_gu,
+                                                                    m->d_ginv, d_err);
+  k_links<Q><<<(unsigned)((m->ncell * Q + 255) / 256), 256, 0, s>>>(m->md, g, m->ncell, m->d_gl, m->d_gu, m->d_K,
+                                                                     d_err);
+}
+cudaError_t launch_geometry(const vlb_mesh *m, int *d_err, cudaStream_t s) {
   if (m->md.q == 9)
-    k_geometry<9><<<(unsigned)blocks, threads, 0, s>>>(m->md, g, m->ncell, m->d_J, m->d_gl,
-                                                       m->d_gu, m->d_ginv, m->d_K, d_err);
+    launch_geometry_q<9>(m, d_err, s);
   else if (m->md.q == 39)
-    k_geometry<39><<<(unsigned)blocks, threads, 0, s>>>(m->md, g, m->ncell, m->d_J, m->d_gl,
-                                                        m->d_gu, m->d_ginv, m->d_K, d_err);
+    launch_geometry_q<39>(m, d_err, s);
   else
-    k_geometry<19><<<(unsigned)blocks, threads, 0, s>>>(m->md, g, m->ncell, m->d_J, m->d_gl,
-                                                        m->d_gu, m->d_ginv, m->d_K, d_err);
+    launch_geometry_q<19>(m, d_err, s);
   return cudaGetLastError();
 }
 
@@ -284,7 +353,8 @@ __global__ void k_plane_check(const double *J, const double *ginv, const double 
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
   const int64_t c0 = (c / nfast) * nfast;
-  if (c0 == c) return;
+  // (a mesh that varies is known to at once: the rest need not be read)
+  if (c0 == c || *(volatile int *)flag) return;
   bool same = close12(J[c], J[c0]);
   for (int i = 0; i < NS; i++) same = same && close12(ginv[c * NS + i], ginv[c0 * NS + i]);
   for (int i = 0; i < D * D; i++) same = same && close12(gu[c * D * D + i], gu[c0 * D * D + i]);
@@ -318,9 +388,39 @@ struct PackArgs {
   double wall_omega[3][2][3];
   int32_t ref_rest;  // fill the storage-reference offsets (16-bit storage, plane mode)
   double nref;
-  int32_t cellrec;   // CellLayout records (FP32, one per cell), wall velocities to uw (if not NULL)
-  float *uw;
+  CellFactors cf;    // CellLayout records
+  float *uw;         // their wall velocities (NULL: no moving walls)
 };
+
+// wall velocity of a cell: rigid motion of the adjacent wall, at the point halfway
+// to the ghost node (zero away from walls)
+template <int Q>
+__device__ void wall_velocity(const PackArgs &a, int64_t c, double (&uw)[3]) {
+  constexpr int D = Lat<Q>::D;
+  const Addr<Q> ad(a.g, c);
+  uw[0] = uw[1] = uw[2] = 0.0;
+  for (int ax = 0; ax < D; ax++) {
+    if (!(ad.lo[ax] || ad.hi[ax])) continue;
+    const int side = ad.lo[ax] ? 0 : 1;
+    int64_t q[3] = {ad.ic[0], ad.ic[1], ad.ic[2]}, gq[3] = {ad.ic[0], ad.ic[1], ad.ic[2]};
+    gq[ax] += side ? 1 : -1;
+    double x0[3], xg[3], xw[3], u[3];
+    position(a.md, q, x0);
+    position(a.md, gq, xg);
+    for (int d = 0; d < 3; d++) xw[d] = 0.5 * (x0[d] + xg[d]);
+    const double *om = a.wall_omega[ax][side];
+    u[0] = om[1] * xw[2] - om[2] * xw[1];
+    u[1] = om[2] * xw[0] - om[0] * xw[2];
+    u[2] = om[0] * xw[1] - om[1] * xw[0];
+    for (int d = 0; d < 3; d++) u[d] += a.wall_u[ax][side][d];
+    for (int i = 0; i < D; i++) {
+      double s = 0.0;
+      for (int d = 0; d < D; d++) s += u[d] * a.gu[(c * D + i) * D + d];
+      uw[i] = s;
+    }
+    break;
+  }
+}
 
 template <int Q, typename R>
 __global__ void k_pack_coef(const PackArgs a, R *coef) {
@@ -408,55 +508,97 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
   // reference-state part of J F as a hi/lo pair
   for (int i = 0; i < D; i++) rec[L::KWL + i] = rec[L::KW + i] - static_cast<double>(static_cast<R>(rec[L::KW + i]));
   R *out = coef + r * a.stride;
-  bool cellrec = false;
-  if constexpr (sizeof(R) == 4) {
-    cellrec = a.cellrec != 0;
-    if (cellrec) {
-      using CL = CellLayout<Q>;
-      float4 *o = reinterpret_cast<float4 *>(coef) + (r >> 5) * (CL::NG * 32) + (r & 31);
-#pragma unroll
-      for (int g = 0; g < CL::NG; g++) {
-        float e[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) e[u] = CL::entry(4 * g + u) >= 0 ? (float)rec[CL::entry(4 * g + u)] : 0.0f;
-        o[g * 32] = make_float4(e[0], e[1], e[2], e[3]);
-      }
-    }
-  }
   // a per-cell record ends at RR (see CoefLayout::stride)
-  if (!cellrec)
-    for (int k = 0; k < a.stride; k++) out[k] = k < L::NC ? static_cast<R>(rec[k]) : R(0);
-  if (cellrec && !a.uw) return;
-  // wall velocity: rigid motion of the adjacent wall, at the point halfway to the ghost node
-  const Addr<Q> ad(a.g, c);
-  double uw[3] = {0.0, 0.0, 0.0};
-  for (int ax = 0; ax < D; ax++) {
-    if (!(ad.lo[ax] || ad.hi[ax])) continue;
-    const int side = ad.lo[ax] ? 0 : 1;
-    int64_t q[3] = {ad.ic[0], ad.ic[1], ad.ic[2]}, gq[3] = {ad.ic[0], ad.ic[1], ad.ic[2]};
-    gq[ax] += side ? 1 : -1;
-    double x0[3], xg[3], xw[3], u[3];
-    position(a.md, q, x0);
-    position(a.md, gq, xg);
-    for (int d = 0; d < 3; d++) xw[d] = 0.5 * (x0[d] + xg[d]);
-    const double *om = a.wall_omega[ax][side];
-    u[0] = om[1] * xw[2] - om[2] * xw[1];
-    u[1] = om[2] * xw[0] - om[0] * xw[2];
-    u[2] = om[0] * xw[1] - om[1] * xw[0];
-    for (int d = 0; d < 3; d++) u[d] += a.wall_u[ax][side][d];
-    for (int i = 0; i < D; i++) {
-      double s = 0.0;
-      for (int d = 0; d < D; d++) s += u[d] * a.gu[(c * D + i) * D + d];
-      uw[i] = s;
+  for (int k = 0; k < a.stride; k++) out[k] = k < L::NC ? static_cast<R>(rec[k]) : R(0);
+  double uw[3];
+  wall_velocity<Q>(a, c, uw);
+  for (int i = 0; i < D; i++) out[L::UW + i] = static_cast<R>(uw[i]);
+}
+
+// CellLayout records (FP32, one per cell): the entries kept are sums over the
+// links formed in FP64 (about 250 operations; the whole record takes ten times that)
+// and rounded; the rest state's force, the start value of the chord iteration, is
+// solved in FP32 on the finished record. 492 K D3Q19 cells: 2.24 -> 0.33 ms.
+template <int Q>
+__global__ void __launch_bounds__(128) k_pack_cells(const PackArgs a, float4 *coef) {
+  constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
+  using L = CoefLayout<Q>;
+  using CL = CellLayout<Q>;
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= a.nrec) return;
+  const double itau = 1.0 / a.tau, J = a.J[c];
+  CellRecord<Q> r;
+  double gd[NS], tr = 0.0, kw[D], ce[D];
+#pragma unroll
+  for (int i = 0; i < D; i++)
+#pragma unroll
+    for (int j = i; j < D; j++) {
+      gd[sym<D>(i, j)] = a.ginv[c * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0);
+      r.v[L::GH + sym<D>(i, j)] = (float)(0.5 * gd[sym<D>(i, j)]);
     }
-    break;
-  }
+#pragma unroll
   for (int i = 0; i < D; i++) {
-    if (cellrec)
-      a.uw[r * D + i] = (float)uw[i];
-    else
-      out[L::UW + i] = static_cast<R>(uw[i]);
+    tr += gd[sym<D>(i, i)];
+    kw[i] = ce[i] = 0.0;
+    double s = 0.0;
+#pragma unroll
+    for (int d = 0; d < D; d++) s += a.body[d] * a.gu[(c * D + i) * D + d];  // G^i = G . g^i
+    r.v[L::BODY + i] = (float)s;
   }
+  const double *K = a.K + c * Q * D;
+  float N[Q], Np[Q];
+  const double am = -0.25 * (2.0 - itau), ad = 0.25 * itau;
+#pragma unroll
+  for (int p = 1; p <= H; p++) {
+    const double w = lat_w<Q, double>(p);
+    double cgc = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        const int cc = Lat<Q>::c(p, k) * Lat<Q>::c(p, l);
+        if (cc != 0) cgc += cc * gd[sym<D>(k, l)];
+      }
+    // CE^i = T0 sum_kl PE^i_kl gd_kl = itau/2 sum_p w (3 c.gd.c - tr gd) M^i_p; the rest
+    // state's populations J w (1 + (3 c.gd.c - tr gd) / 2)
+    const double h = w * (3.0 * cgc - tr);
+    N[p] = N[p + H] = (float)(J * (w + 0.5 * h));
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      const double kp = K[p * D + i], km = K[(p + H) * D + i], M = kp + km;
+      kw[i] += w * M;
+      ce[i] += h * M;
+      r.v[L::mp(p, i)] = (float)(am * M);
+      r.v[L::dk(p, i)] = (float)(ad * (kp - km));
+    }
+  }
+  N[0] = (float)(J * lat_w<Q, double>(0) * (1.0 - 0.5 * tr));
+  r.v[L::J] = (float)J;
+  r.v[L::IJ] = (float)(1.0 / J);
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+    r.v[L::KW + i] = (float)kw[i];
+    r.v[L::KWL + i] = (float)(kw[i] - (double)(float)kw[i]);
+    r.v[L::CE + i] = (float)(0.5 * itau * ce[i]);
+    r.v[L::FR + i] = 0.0f;
+  }
+  r.form(a.cf.k6am, a.cf.kpe, a.cf.ktt);
+  CollideState<Q, float> cs;
+  collide_cell<Q, float, false>(N, r, 0.0f, (float)itau, 1e-6f, 100, Np, cs);
+#pragma unroll
+  for (int i = 0; i < D; i++) r.v[L::FR + i] = cs.conv ? cs.F[i] : 0.0f;
+  float4 *o = coef + (c >> 5) * (CL::NG * 32) + (c & 31);
+#pragma unroll
+  for (int g = 0; g < CL::NG; g++) {
+    float e[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) e[u] = CL::entry(4 * g + u) >= 0 ? r.v[CL::entry(4 * g + u)] : 0.0f;
+    o[g * 32] = make_float4(e[0], e[1], e[2], e[3]);
+  }
+  if (!a.uw) return;
+  double uw[3];
+  wall_velocity<Q>(a, c, uw);
+  for (int i = 0; i < D; i++) a.uw[c * D + i] = (float)uw[i];
 }
 
 template <int Q>
@@ -476,7 +618,7 @@ static cudaError_t pack_q(const vlb_sim *sim, cudaStream_t s) {
   a.tau = sim->p.tau;
   a.ref_rest = sim->ref_rest;
   a.nref = sim->nref;
-  a.cellrec = sim->cellrec;
+  a.cf = cell_factors(a.tau);
   a.uw = sim->d_uw;
   for (int d = 0; d < 3; d++) a.body[d] = sim->p.body_force[d];
   for (int ax = 0; ax < 3; ax++)
@@ -487,7 +629,9 @@ static cudaError_t pack_q(const vlb_sim *sim, cudaStream_t s) {
       }
   const int threads = 128;
   const int64_t blocks = (a.nrec + threads - 1) / threads;
-  if (arith_f64(sim->p.precision))
+  if (sim->cellrec)
+    k_pack_cells<Q><<<(unsigned)blocks, threads, 0, s>>>(a, (float4 *)sim->d_coef);
+  else if (arith_f64(sim->p.precision))
     k_pack_coef<Q, double><<<(unsigned)blocks, threads, 0, s>>>(a, (double *)sim->d_coef);
   else
     k_pack_coef<Q, float><<<(unsigned)blocks, threads, 0, s>>>(a, (float *)sim->d_coef);
