@@ -643,10 +643,10 @@ cudaError_t launch_pack_coef(const vlb_sim *sim, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ initial state
-// N_a = J f^eq_a(rho, U, U~ = U), U^i = u . g^i (Eqs. 14, 33), normal layout
-template <int Q, typename S>
+// N_a = J f^eq_a(rho, U, U~ = U), U^i = u . g^i (Eqs. 14, 33), normal layout; FP64 storage
+template <int Q>
 __global__ void k_init(const double *J, const double *gu, const double *ginv, const double *rho,
-                       const double *u, int64_t ncell, RefCtx ref, S *f) {
+                       const double *u, int64_t ncell, double nref, double *f) {
   constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
@@ -662,14 +662,14 @@ __global__ void k_init(const double *J, const double *gu, const double *ginv, co
   EqParts<Q, double> e;
   eq_parts<Q, double>(gd, U, zero, e);
   const double r = rho[c], Jc = J[c];
-  // stored relative to the storage reference of each location
-  f[c] = store_s<S>(Jc * r * lat_w<Q, double>(0) * eq_even<Q, double>(e, 0) - ref_at<Q>(ref, 0, c));
+  // stored relative to w_a n_ref
+  f[c] = Jc * r * lat_w<Q, double>(0) * eq_even<Q, double>(e, 0) - lat_w<Q, double>(0) * nref;
 #pragma unroll
   for (int p = 1; p <= H; p++) {
     const double E = eq_even<Q, double>(e, p), O = eq_odd<Q, double>(e, U, p);
-    const double w = lat_w<Q, double>(p), rw = Jc * r * w;
-    f[p * ncell + c] = store_s<S>(rw * (E + O) - ref_at<Q>(ref, p, c));
-    f[(p + H) * ncell + c] = store_s<S>(rw * (E - O) - ref_at<Q>(ref, p + H, c));
+    const double w = lat_w<Q, double>(p), rw = Jc * r * w, wn = w * nref;
+    f[p * ncell + c] = rw * (E + O) - wn;
+    f[(p + H) * ncell + c] = rw * (E - O) - wn;
   }
 }
 
@@ -731,6 +731,76 @@ __global__ void k_init_f32(const double *J, const double *gu, const double *ginv
   }
 }
 
+// The initial state of 16-bit storage relative to the rest state of Eq. 33 on the
+// location's column (plane mode): with J f^eq_a = J rho w_a (1 + x_a) and the reference
+// o_a = fl(J w_a (1 + x^0_a)) rounded to FP32 (rest_ref),
+//   N_a - o_a = J w_a [(rho - 1)(1 + x^0_a) + rho (x_a - x^0_a)] + (J w_a (1 + x^0_a) - o_a).
+// The rest state and its rounding are formed in FP64 once per pair (60 operations), the
+// flow's part, x - x^0 from U U and the odd part, in FP32. Forming every population
+// and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells; INIT_REST
+template <int Q, typename S>
+__global__ void __launch_bounds__(128) k_init_rest(const double *J, const double *gu, const double *ginv,
+                                                   const double *rho, const double *u, int64_t ncell, int64_t nfast,
+                                                   S *f) {
+  constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= ncell) return;
+  const int64_t c0 = ncell < ((int64_t)1 << 31) ? (int64_t)((uint32_t)c / (uint32_t)nfast) * nfast : c / nfast * nfast;
+  float U[D], gd[NS], zero[D];
+  double g[NS], tr = 0.0;
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+    float v = 0.0f;
+#pragma unroll
+    for (int d = 0; d < D; d++) v = fmaf((float)u[c * D + d], (float)gu[(c0 * D + i) * D + d], v);
+    U[i] = v;
+    zero[i] = 0.0f;
+  }
+#pragma unroll
+  for (int i = 0; i < D; i++)
+#pragma unroll
+    for (int j = i; j < D; j++) {
+      g[sym<D>(i, j)] = ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0);
+      gd[sym<D>(i, j)] = (float)g[sym<D>(i, j)];
+      if (i == j) tr += g[sym<D>(i, j)];
+    }
+  EqParts<Q, float> e;
+  eq_parts<Q, float>(gd, U, zero, e);
+  // the even part without the rest state's: B = U U
+  EqParts<Q, float> q = e;
+  q.trB = 0.0f;
+#pragma unroll
+  for (int i = 0; i < D; i++) {
+#pragma unroll
+    for (int j = 0; j < D; j++) q.B[i][j] = U[i] * U[j];
+    q.trB += q.B[i][i];
+  }
+  const double Jc = J[c0];
+  const float r1 = (float)(rho[c] - 1.0), r = (float)rho[c], Jf = (float)Jc;
+#pragma unroll
+  for (int p = 0; p <= H; p++) {
+    double cgc = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        const int cc = Lat<Q>::c(p, k) * Lat<Q>::c(p, l);
+        if (cc > 0) cgc += g[sym<D>(k, l)];
+        if (cc < 0) cgc -= g[sym<D>(k, l)];
+      }
+    const double o = Jc * (lat_w<Q, double>(p) * (1.0 + 0.5 * (3.0 * cgc - tr)));
+    const float of = (float)o, lo = (float)(o - (double)of);
+    const float jw = Jf * lat_w<Q, float>(p), xe = eq_even_x<Q>(q, p);
+    if (p == 0) {
+      f[c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe, lo)));
+    } else {
+      const float xo = eq_odd<Q, float>(e, U, p);
+      f[p * ncell + c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe + xo, lo)));
+      f[(p + H) * ncell + c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe - xo, lo)));
+    }
+  }
+}
+
 cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
   const int threads = 128;
@@ -739,9 +809,19 @@ cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d
   return with_storage(sim->p.precision, [&](auto tag) {
     using S = typename decltype(tag)::type;
     if constexpr (!std::is_same<S, double>::value) {
-      // FP32 arithmetic for the uniform reference (the rest reference of
-      // 16-bit storage keeps the FP64 form)
-      if (!ref.rest) {
+      // FP32 arithmetic
+      if constexpr (sizeof(S) == 2) {
+        if (ref.rest) {
+          if (m->md.q == 9)
+            k_init_rest<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
+                                                                   ref.nfast, (S *)sim->d_f);
+          else
+            k_init_rest<19, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
+                                                                    ref.nfast, (S *)sim->d_f);
+          return cudaGetLastError();
+        }
+      }
+      {
         if (m->md.q == 9)
           k_init_f32<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
                                                                 ref.nref, (S *)sim->d_f);
@@ -751,13 +831,15 @@ cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d
         return cudaGetLastError();
       }
     }
-    if (m->md.q == 9)
-      k_init<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
-                                                        ref, (S *)sim->d_f);
-    else
-      k_init<19, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
-                                                         ref, (S *)sim->d_f);
-    return cudaGetLastError();
+    else {
+      if (m->md.q == 9)
+        k_init<9><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref.nref,
+                                                       (double *)sim->d_f);
+      else
+        k_init<19><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref.nref,
+                                                        (double *)sim->d_f);
+      return cudaGetLastError();
+    }
   });
 }
 

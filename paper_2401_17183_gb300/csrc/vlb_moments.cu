@@ -65,7 +65,11 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *out) {
 // One cell per thread; IT is the index type (32-bit when every population
 // offset fits). In plane mode the tangents, like the coefficient record, are
 // those of the column (its first cell).
-template <int Q, typename S, bool ODD, typename MT, typename IT>
+// REST (16-bit storage relative to the rest state, plane mode): the collision
+// works on the stored values relative to the own column's rest state, as the
+// step does, with the record's column differences; forming every location's
+// reference in FP64 instead took 0.49 ms on 128^3 cells, MOM_REST
+template <int Q, typename S, bool ODD, typename MT, typename IT, bool REST>
 __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double *out) {
   constexpr int D = Lat<Q>::D;
   const S *f = static_cast<const S *>(a.f);
@@ -75,34 +79,39 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
   const IT n2 = (IT)a.g.n[2], n1 = (IT)a.g.n[1];
   const IT r = c / n2, i2 = c - r * n2, i0 = r / n1, i1 = r - i0 * n1;
   const Addr<Q, IT> ad(a.g, i0, i1, i2);
-  // the arrived populations as deviations from the uniform reference w_a n_ref,
-  // in MT: the stored value itself, plus (16-bit storage relative to the rest
-  // state) the location's offset from the uniform reference
+  // the arrived populations in MT, as stored: deviations from the uniform reference
+  // w_a n_ref, or (REST) from the rest state of the column that holds them
   MT dv[Q];
 #pragma unroll
   for (int av = 0; av < Q; av++) {
     int slot;
     IT loc;
     arrived_loc<Q, ODD, IT>(ad, av, slot, loc);
-    const S v = f[(IT)slot * (IT)a.ncell + loc];
-    if constexpr (sizeof(MT) == 8) {
-      dv[av] = load_s<double>(v) + (ref_at<Q>(a.ref, slot, (int64_t)loc) - lat_w<Q, double>(slot) * a.nref);
-    } else {
-      dv[av] = load_s<MT>(v);
-      if (a.ref.rest)
-        dv[av] += static_cast<MT>(ref_at<Q>(a.ref, slot, (int64_t)loc) - lat_w<Q, double>(slot) * a.nref);
-    }
+    dv[av] = load_s<MT>(f[(IT)slot * (IT)a.ncell + loc]);
   }
   // the cell's (or column's) coefficient record, stored in MT
   const IT c0 = a.plane ? c - ad.ic[D - 1] : c;   // the fastest axis has stride 1
+  if constexpr (REST && ODD) {
+    using L = CoefLayout<Q>;
+    const MT *rc = static_cast<const MT *>(a.coef) + (int64_t)(c0 / (IT)a.nfast) * a.rs;
+#pragma unroll
+    for (int av = 1; av < Q; av++) {
+      bool slow = false;
+#pragma unroll
+      for (int d = 0; d < D - 1; d++) slow = slow || Lat<Q>::c(av, d) != 0;
+      // (the differences are zero where a slow-axis wall sends the link back; a
+      // fastest-axis wall does so at the ends of a row only)
+      if (slow && !ad.crosses(av, -1)) dv[av] += rc[L::DIN + av];
+    }
+  }
   MT Np[Q];
   CollideState<Q, MT> st;
   // chord iteration from the record's rest-state start value
   auto solve = [&](const auto &rec) {
-    collide_cell<Q, MT, false>(dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau),
-                               static_cast<MT>(a.tol), 200, Np, st);
+    collide_cell<Q, MT, false, REST>(dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau),
+                                     static_cast<MT>(a.tol), 200, Np, st);
   };
-  if constexpr (sizeof(MT) == 4) {
+  if constexpr (sizeof(MT) == 4 && !REST) {
     if (!a.plane) {
       CellRecord<Q> rec;
       rec.load(static_cast<const float4 *>(a.coef), (int64_t)c);
@@ -168,16 +177,26 @@ static cudaError_t moments_t(const vlb_sim *sim, double *d_out, int64_t nblk, cu
   const int64_t blocks = (m->ncell + kMomThreads - 1) / kMomThreads;
   const bool i32 = (int64_t)Q * m->ncell + kMomThreads < ((int64_t)1 << 31);
   const bool odd = sim->t & 1;
-  if (i32) {
-    if (odd)
-      k_moments<Q, S, true, MT, int32_t><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
+  auto go = [&](auto odd_tag, auto rest_tag) {
+    constexpr bool O = decltype(odd_tag)::value, RE = decltype(rest_tag)::value;
+    if (i32)
+      k_moments<Q, S, O, MT, int32_t, RE><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
     else
-      k_moments<Q, S, false, MT, int32_t><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
+      k_moments<Q, S, O, MT, int64_t, RE><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
+  };
+  auto parity = [&](auto rest_tag) {
+    if (odd)
+      go(std::true_type(), rest_tag);
+    else
+      go(std::false_type(), rest_tag);
+  };
+  if constexpr (sizeof(S) == 2) {
+    if (a.ref.rest)
+      parity(std::true_type());
+    else
+      parity(std::false_type());
   } else {
-    if (odd)
-      k_moments<Q, S, true, MT, int64_t><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
-    else
-      k_moments<Q, S, false, MT, int64_t><<<(unsigned)blocks, kMomThreads, 0, s>>>(a, d_out);
+    parity(std::false_type());
   }
   (void)nblk;
   return cudaGetLastError();
@@ -245,6 +264,11 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
   const float bp = s - hi;
   lo += (hi - (s - bp)) + (x - bp);
   hi = s;
+}
+
+// a pair's sum; a sum that is not finite is hi alone
+__device__ __forceinline__ double pair_sum(float hi, float lo) {
+  return (double)hi + (isfinite(lo) ? (double)lo : 0.0);
 }
 
 // N_a at a storage location, absolute (stored deviation plus its reference)
@@ -518,6 +542,80 @@ __global__ void __launch_bounds__(kMomThreads) k_totals_cells(const TotArgs a, d
   block_sum<7>(acc, partial + (int64_t)blockIdx.x * 7);
 }
 
+// The same sums for FP32 or 16-bit storage relative to the uniform reference on a
+// mesh without rotations. The stored deviations are added without rounding error
+// as hi + lo pairs in FP32 (TwoSum: six FP32 operations, a fortieth of an FP64 addition's
+// time here), and only B^i, their products with the tangents and the sums over cells
+// are FP64 (31 K D2Q9 cells: 17.4 -> 11.5 us; 492 K D3Q19 cells: 240 -> 94 us). The reference's part of B^i, n_ref sum_a c^i_a w_a (1 + [p + c_a inside] + [p - c_a
+// behind a wall]), vanishes away from walls.
+template <int Q, typename S, bool ODD>
+__global__ void __launch_bounds__(kMomThreads) k_totals_cells_f32(const TotArgs a, double *partial) {
+  constexpr int D = Lat<Q>::D;
+  const S *f = static_cast<const S *>(a.f);
+  double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < a.ncell;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    const Addr<Q> ad(a.g, c);
+    float mh = load_s<float>(f[c]), ml = 0.f, ph[D], pl[D], nh[D], nl[D];
+    double wm[D];   // the reference's part of the second half of M
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      ph[i] = pl[i] = nh[i] = nl[i] = 0.f;
+      wm[i] = 0.0;
+    }
+    const bool wall = ad.wall_cell();
+#pragma unroll
+    for (int av = 1; av < Q; av++) {
+      int slot;
+      int64_t loc;
+      arrived_loc<Q, ODD, int64_t>(ad, av, slot, loc);
+      const float v = load_s<float>(f[(int64_t)slot * a.ncell + loc]);
+      two_sum_acc(mh, ml, v);
+      // N_a(p + c_a), none behind a wall; N_a(p) once more when p - c_a is behind one
+      float n = 0.f;
+      bool in = true;
+      if (!wall || !ad.crosses(av, 1))
+        n = load_s<float>(ODD ? f[(int64_t)lat_opp<Q>(av) * a.ncell + c] : f[(int64_t)av * a.ncell + ad.nb(av, 1)]);
+      else
+        in = false;
+      const bool back = wall && ad.crosses(av, -1);
+#pragma unroll
+      for (int i = 0; i < D; i++) {
+        const int ci = Lat<Q>::c(av, i);
+        if (ci == 0) continue;
+        const float sv = ci > 0 ? v : -v;
+        two_sum_acc(ph[i], pl[i], sv);
+        two_sum_acc(nh[i], nl[i], ci > 0 ? n : -n);
+        if (wall) {
+          if (back) two_sum_acc(nh[i], nl[i], sv);
+          wm[i] += ci * lat_w<Q, double>(av) * ((in ? 1 : 0) + (back ? 1 : 0));
+        }
+      }
+    }
+    acc[0] += pair_sum(mh, ml) + a.ref.nref;   // the weights sum to one
+    double BP[D], BM[D];
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      BP[i] = pair_sum(ph[i], pl[i]);
+      BM[i] = BP[i] + pair_sum(nh[i], nl[i]);
+      if (wall) BM[i] += wm[i] * a.ref.nref;
+    }
+#pragma unroll
+    for (int d = 0; d < D; d++) {
+      double p = 0.0, m = 0.0;
+#pragma unroll
+      for (int i = 0; i < D; i++) {
+        const double g = a.gl[(c * D + i) * D + d];
+        p += g * BP[i];
+        m += g * BM[i];
+      }
+      acc[1 + d] += p;
+      acc[4 + d] += 0.5 * m;
+    }
+  }
+  block_sum<7>(acc, partial + (int64_t)blockIdx.x * 7);
+}
+
 template <int Q, typename S>
 static cudaError_t totals_t(const vlb_sim *sim, double *d_partial, int64_t nblk_max, int64_t *nblk,
                             cudaStream_t s) {
@@ -547,6 +645,15 @@ static cudaError_t totals_t(const vlb_sim *sim, double *d_partial, int64_t nblk_
       k_totals_plane<Q, S, false><<<(unsigned)*nblk, kMomThreads, 0, s>>>(a, d_partial);
   } else {
     *nblk = std::min<int64_t>(nblk_max, (a.ncell + kMomThreads - 1) / kMomThreads);
+    if constexpr (sizeof(S) < 8) {
+      if (!a.ref.rest && !a.has_rot[0] && !a.has_rot[1] && !a.has_rot[2]) {
+        if (odd)
+          k_totals_cells_f32<Q, S, true><<<(unsigned)*nblk, kMomThreads, 0, s>>>(a, d_partial);
+        else
+          k_totals_cells_f32<Q, S, false><<<(unsigned)*nblk, kMomThreads, 0, s>>>(a, d_partial);
+        return cudaGetLastError();
+      }
+    }
     if (odd)
       k_totals_cells<Q, S, true><<<(unsigned)*nblk, kMomThreads, 0, s>>>(a, d_partial);
     else
