@@ -55,6 +55,7 @@ int check_kernel_flags(int *d_err, cudaStream_t s) {
   CU(cudaMemcpyAsync(&h, d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
   if (h & vlb::ERR_GEOM) return fail(VLB_EGEOM, "degenerate mesh cell (J <= 0 or D_i = D_-i)");
+  if (h & vlb::ERR_BARRIER) return fail(VLB_ECUDA, "a multi-step launch gave up waiting for its other blocks");
   if (h & vlb::ERR_NOCONV)
     return fail(VLB_ENOCONV, "local fixed-point solve for F hit its iteration cap");
   if (h & vlb::ERR_NONFINITE) return fail(VLB_ENONFINITE, "non-finite moment");
@@ -364,7 +365,7 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
   } else if (e == cudaSuccess) {
     e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
   }
-  if (e == cudaSuccess) e = cudaMalloc(&s->d_err, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&s->d_err, sizeof(int) * vlb::kErrWords);
   if (e != cudaSuccess) {
     vlb_destroy(s);
     return fail(VLB_ENOMEM, "simulation device allocation: %s", cudaGetErrorString(e));
@@ -395,11 +396,20 @@ int vlb_reset(vlb_sim *s, const double *rho, const double *u) {
 int vlb_step(vlb_sim *s, int64_t nsteps) {
   if (!s) return fail(VLB_EINVAL, "NULL sim");
   if (nsteps < 0) return fail(VLB_EINVAL, "nsteps < 0");
-  for (int64_t k = 0; k < nsteps; k++) {
+  for (int64_t k = 0; k < nsteps;) {
+    int64_t done = 0;
+    const cudaError_t es = vlb::launch_steps_small(s, nsteps - k, &done, s->stream);
+    if (es != cudaSuccess) return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(es));
+    if (done > 0) {
+      s->t += done;
+      k += done;
+      continue;
+    }
     cudaError_t e = s->mesh->md.q == VLB_D3Q39 ? vlb::q39_step(s, (int)(s->t & 1), s->stream)
                                                : vlb::launch_step(s, (int)(s->t & 1), s->stream);
     if (e != cudaSuccess) return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(e));
     s->t++;
+    k++;
   }
   return VLB_OK;
 }

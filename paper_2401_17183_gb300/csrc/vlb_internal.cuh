@@ -529,7 +529,12 @@ inline RefCtx make_ref(const vlb_sim *sim) {
 }
 
 // error flags raised by kernels
-enum : int { ERR_NOCONV = 1, ERR_NONFINITE = 2, ERR_GEOM = 4 };
+enum : int { ERR_NOCONV = 1, ERR_NONFINITE = 2, ERR_GEOM = 4, ERR_BARRIER = 8 };
+// a simulation's d_err: the error flags, and apart from them the barrier
+// counter of the multi-step kernel
+constexpr int kErrWords = 64, kBarrierWord = 32;
+// steps of one multi-step launch, and the largest mesh it is tried for
+constexpr int64_t kSmallSteps = 1024, kSmallCells = 65536;
 
 // launchers (each returns a cudaError_t from the launch)
 cudaError_t launch_geometry(const vlb_mesh *m, int *d_err, cudaStream_t s);
@@ -538,6 +543,8 @@ cudaError_t launch_plane_check(const vlb_mesh *m, int *d_flag, cudaStream_t s);
 cudaError_t launch_pack_coef(const vlb_sim *sim, cudaStream_t s);
 cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s);
 cudaError_t launch_step(const vlb_sim *sim, int odd, cudaStream_t s);
+// up to nsteps steps of a small mesh in one launch; *done: how many (0: none, not small)
+cudaError_t launch_steps_small(const vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s);
 cudaError_t launch_moments(const vlb_sim *sim, double *d_out, int64_t nblk, cudaStream_t s);
 // conservation totals (mass, P, M) of a D2Q9/D3Q19 simulation into d_totals[7]
 // through per-block partial sums in d_partial (room for nblk_max x 7 doubles)

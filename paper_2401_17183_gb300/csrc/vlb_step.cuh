@@ -33,6 +33,7 @@
 // contains it and the thread remembers which half it is.
 #pragma once
 
+#include <algorithm>
 #include <mutex>
 #include <tuple>
 #include <type_traits>
@@ -594,22 +595,26 @@ inline StepArgs make_step_args(const vlb_sim *sim, int T = kStepThreads) {
   return a;
 }
 
-// blocks the persistent kernel can keep resident on the current device
-// (queried once per kernel and device)
+// blocks a kernel can keep resident on the current device (queried once per
+// kernel, dynamic shared memory and device)
 static int resident_blocks(const void *kern, size_t smem, int threads = kStepThreads) {
   static std::mutex mu;
-  static std::vector<std::tuple<const void *, int, int>> cache;
+  static std::vector<std::tuple<const void *, size_t, int, int>> cache;
   int dev = 0;
   cudaGetDevice(&dev);
   std::lock_guard<std::mutex> lock(mu);
+  size_t most = 48 * 1024;   // the largest size the kernel's limit allows so far
   for (const auto &e : cache)
-    if (std::get<0>(e) == kern && std::get<1>(e) == dev) return std::get<2>(e);
+    if (std::get<0>(e) == kern && std::get<2>(e) == dev) {
+      if (std::get<1>(e) == smem) return std::get<3>(e);
+      most = std::max(most, std::get<1>(e));
+    }
   int nb = 0, nsm = 0;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > most) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int total = (nb > 0 ? nb : 1) * (nsm > 0 ? nsm : 1);
-  cache.emplace_back(kern, dev, total);
+  cache.emplace_back(kern, smem, dev, total);
   return total;
 }
 
