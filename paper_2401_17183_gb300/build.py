@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libvlb.so")
-SOURCES = ["vlb_api.cu", "vlb_geometry.cu", "vlb_step.cu", "vlb_step16.cu",
+SOURCES = ["vlb_api.cu", "vlb_geometry.cu", "vlb_step.cu", "vlb_step_f32.cu", "vlb_step_f16.cu", "vlb_step_bf16.cu",
            "vlb_batch.cu",
            "vlb_moments.cu", "vlb_noalloc.cu", "vlb_nn.cu", "vlb_q39.cu",
            "vlb_small.cu"]

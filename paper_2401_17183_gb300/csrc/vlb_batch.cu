@@ -72,7 +72,7 @@ BatchKernel batch_kernel(const BatchKind &k, bool odd, int shape) {
 
 template <int Q, typename R, bool PLANE>
 size_t smem_q(int threads) {
-  return threads == 64 ? sizeof(StepSmem<Q, R, R, 64, PLANE>) : sizeof(StepSmem<Q, R, R, 128, PLANE>);
+  return threads == 64 ? step_smem<Q, R, R, 64, PLANE, false>(1) : step_smem<Q, R, R, 128, PLANE, false>(1);
 }
 
 template <int Q, typename R>
