@@ -25,6 +25,7 @@
 // come from the mesh's FP64 geometry, so the relations of Eqs. 27 and 30 read
 //   sum_j c^j_a Theta^i_j(q - c_a, q) = -K^i_abar.
 #include "vlb_addr.cuh"
+#include "vlb_collide.cuh"
 #include "vlb_q39.cuh"
 
 namespace vlb {
@@ -61,7 +62,7 @@ struct Q39Args {
   // NULL before q39_prepare has filled them
   const double *chord;
   double body[3];
-  double tau, tol;
+  double tau, itau, tol;
   int32_t max_iter;
   int *err;
 };
@@ -561,11 +562,14 @@ __global__ void __launch_bounds__(kQ39Threads) k_prep39_rec(const Q39Args A, dou
 // and what the collision makes of them. ld(k): record value k.
 struct Cell39 {
   double s[kH39 + 1], t[kH39 + 1];
-  double m, U[3], Phi[3];
+  double m, h2m, U[3], Phi[3];   // h2m = 1 / (2 m)
 };
+constexpr double kIT0_39 = 1.5;   // 1 / T0, exactly (a division takes some 15 FP64 operations)
 
-// m, U and the force: the chord iteration Phi <- H (Pc - m/2 Q(U~)) from m F_rest,
-// converged when the change is at most tol max(m, |Phi|)
+// m, U and the force: the chord iteration Phi <- H (Pc - m/2 Q(U~)), started, tested
+// and accepted as in FP64 D3Q19 cells (collide_f64): three evaluations in FP32 from
+// Pt = H Pc, then FP64 ones until the change, or a bound on the next one, is at most
+// tol max(m, |Phi|); below four iterations allowed from m F_rest
 template <typename LD>
 __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_iter) {
   double m = q.s[0], mu[3] = {0.0, 0.0, 0.0}, Pc[3] = {0.0, 0.0, 0.0};
@@ -584,6 +588,7 @@ __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_it
   }
   q.m = m;
   const double im = 1.0 / m, h2m = 0.5 * im, hm = 0.5 * m;
+  q.h2m = h2m;
 #pragma unroll
   for (int i = 0; i < 3; i++) q.U[i] = mu[i] * im;
 #pragma unroll
@@ -597,94 +602,150 @@ __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_it
   }
   double Pt[3];
 #pragma unroll
-  for (int i = 0; i < 3; i++) {
-    Pt[i] = ld(Rec39::HM + 3 * i) * Pc[0] + ld(Rec39::HM + 3 * i + 1) * Pc[1] + ld(Rec39::HM + 3 * i + 2) * Pc[2];
-    q.Phi[i] = m * ld(Rec39::FR + i);
+  for (int i = 0; i < 3; i++)
+    Pt[i] = fma(ld(Rec39::HM + 3 * i), Pc[0],
+                fma(ld(Rec39::HM + 3 * i + 1), Pc[1], ld(Rec39::HM + 3 * i + 2) * Pc[2]));
+  const float mf = trunc_f32(m), tolf = (float)tol;
+  float lip = 1.0e30f;
+  int it = 0;
+  if (max_iter >= 4) {
+    float Uf[3], Pf[3], df[3] = {0.f, 0.f, 0.f}, l2 = 0.f, l3 = 0.f, um = 0.f;
+    const float hf = trunc_f32(h2m), hmf = 0.5f * mf;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      Uf[i] = trunc_f32(q.U[i]);
+      Pf[i] = trunc_f32(Pt[i]);
+    }
+#pragma unroll 1
+    for (int r = 0; r < 3; r++) {
+      float x[3];
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        x[i] = fmaf(Pf[i] + df[i], hf, Uf[i]);
+        um = fmaxf(um, fabsf(x[i]));
+      }
+      const float xx = x[0] * x[0], yy = x[1] * x[1], zz = x[2] * x[2];
+      const float mono[16] = {xx, x[0] * x[1], x[0] * x[2], yy, x[1] * x[2], zz,
+                              xx * x[0], xx * x[1], xx * x[2], x[0] * yy, (x[0] * x[1]) * x[2], x[0] * zz,
+                              yy * x[1], yy * x[2], x[1] * zz, zz * x[2]};
+      l2 = l3 = 0.f;
+#pragma unroll
+      for (int i = 0; i < 3; i++) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; k++) {
+          const float c = trunc_f32(ld(Rec39::QM + 16 * i + k));
+          v = fmaf(c, mono[k], v);
+          if (k < 6)
+            l2 += fabsf(c);
+          else
+            l3 += fabsf(c);
+        }
+        df[i] = -hmf * v;
+      }
+    }
+    it = 3;
+    um *= 1.01f;
+    lip = fmaf(0.5f * l2, um, 0.75f * l3 * um * um);
+#pragma unroll
+    for (int i = 0; i < 3; i++) q.Phi[i] = Pt[i] + (double)df[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 3; i++) q.Phi[i] = m * ld(Rec39::FR + i);
   }
 #pragma unroll 1
-  for (int it = 0; it < max_iter; it++) {
-    double Ut[3], a[3], diff = 0.0, pm = 0.0;
+  while (it < max_iter) {
+    double Ut[3], a[3];
+    float diff = 0.f, pm = 0.f;
 #pragma unroll
     for (int i = 0; i < 3; i++) Ut[i] = fma(q.Phi[i], h2m, q.U[i]);
     map39(Ut, ld, a);
 #pragma unroll
     for (int i = 0; i < 3; i++) {
       const double pn = fma(-hm, a[i], Pt[i]);
-      diff = maxnan(diff, fabs(pn - q.Phi[i]));
-      pm = maxnan(pm, fabs(pn));
+      diff = maxnan(diff, fabsf(trunc_f32(pn - q.Phi[i])));
+      pm = maxnan(pm, fabsf(trunc_f32(pn)));
       q.Phi[i] = pn;
     }
-    if (diff <= tol * (m > pm ? m : pm)) return true;
+    it++;
+    const float scale = tolf * maxnan(mf, pm);
+    if (diff <= scale || 64.f * lip * diff <= scale) return true;
   }
   return false;
 }
 
 // Even and odd parts of the equilibrium bracket over the pairs, folded by the kind
-// of pair. Even: y0 + c.Y.c for a symmetric Y. Odd: c.u + k C:ccc for
-// symmetric C; with b^i = k C^iii, q^ji = 3 k C^jji, d = 6 k C^012,
-//   axis of length L:   L (u_i + L^2 b_i),
-//   corner (s0 s1 s2):  sum_i s_i (u_i + b_i + sum_{j != i} q_ji) + s0 s1 s2 d,
-//   (2 s_i, 2 s_j):     sum of s_i (2 u_i + 8 (b_i + q_ji)) over both axes.
+// of pair, with the sums that several pairs share formed once. Even: y0 + c.Y.c for a
+// symmetric Y. Odd: c.u + k C:ccc for symmetric C; with b^i = k C^iii, q^ji = 3 k C^jji,
+// d = 6 k C^012,
+//   axis of length L:  L u_i + L^3 b_i,
+//   corner (1 s1 s2):  a_0 + s1 a_1 + s2 a_2 + s1 s2 d,  a_i = u_i + b_i + sum_{j != i} q_ji,
+//   (2 s_i, 2 s_j):    s_i e_ij + s_j e_ji,  e_ij = 2 u_i + 8 (b_i + q_ji).
+// (Every axis vector of the positive half points along +i, every corner has c^0 = 1.)
+__host__ __device__ constexpr int q39_axis(int p, int k) {   // k-th non-zero axis of pair p
+  int n = 0;
+  for (int i = 0; i < 3; i++)
+    if (Lat<39>::c(p, i) != 0) {
+      if (n == k) return i;
+      n++;
+    }
+  return -1;
+}
 struct Odd39 {
-  double u[3], b[3], a[3], e[3][3], d;
-  // e[i][j]: the part of axis i in the plane of axes i and j
+  double u2[3], u[3], b[3], ap, am, a2, e[3][3], d;
   __device__ __forceinline__ Odd39(const double (&uu)[3], const double (&kC)[10]) {
-    double qj[3][3];
+    double a[3];
 #pragma unroll
     for (int i = 0; i < 3; i++) {
       u[i] = uu[i];
+      u2[i] = uu[i] + uu[i];
       b[i] = kC[sym3(i, i, i)];
       a[i] = u[i] + b[i];
 #pragma unroll
       for (int j = 0; j < 3; j++) {
         if (j == i) continue;
-        qj[j][i] = 3.0 * kC[sym3(j, j, i)];
-        a[i] += qj[j][i];
-        e[i][j] = fma(8.0, b[i] + qj[j][i], 2.0 * u[i]);
+        const double q = kC[sym3(j, j, i)];
+        a[i] = fma(3.0, q, a[i]);
+        e[i][j] = fma(8.0, fma(3.0, q, b[i]), u2[i]);
       }
     }
+    ap = a[0] + a[1];
+    am = a[0] - a[1];
+    a2 = a[2];
     d = 6.0 * kC[sym3(0, 1, 2)];
   }
   __device__ __forceinline__ double operator()(int p) const {
-    const int L = q39_len(p), nz = q39_nnz(p);
-    double r = 0.0;
-    if (nz == 1) {
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-        if (Lat<39>::c(p, i) != 0) r = L == 1 ? u[i] + b[i] : (double)L * fma((double)(L * L), b[i], u[i]);
-      return r;   // the positive half's axis vectors point along +i
+    const int L = q39_len(p), nz = q39_nnz(p), i = q39_axis(p, 0), j = q39_axis(p, 1);
+    if (nz == 1) return L == 1 ? u[i] + b[i] : L == 2 ? fma(8.0, b[i], u2[i]) : fma(27.0, b[i], u2[i] + u[i]);
+    if (nz == 3) {
+      const int s1 = Lat<39>::c(p, 1), s2 = Lat<39>::c(p, 2);
+      const double t = s1 > 0 ? ap : am, v = s2 > 0 ? t + a2 : t - a2;
+      return s1 * s2 > 0 ? v + d : v - d;
     }
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-      const int ci = Lat<39>::c(p, i);
-      if (ci == 0) continue;
-      double v = a[i];
-      if (nz == 2) {
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-          if (j != i && Lat<39>::c(p, j) != 0) v = e[i][j];
-      }
-      r = ci > 0 ? r + v : r - v;
-    }
-    if (nz == 3) r = Lat<39>::c(p, 0) * Lat<39>::c(p, 1) * Lat<39>::c(p, 2) > 0 ? r + d : r - d;
-    return r;
+    const double v = Lat<39>::c(p, i) > 0 ? e[i][j] : -e[i][j];
+    return Lat<39>::c(p, j) > 0 ? v + e[j][i] : v - e[j][i];
   }
 };
-__device__ __forceinline__ double even39(int p, double y0, const double (&Y)[6]) {
-  const int L = q39_len(p);
-  double r = 0.0;
+struct Even39 {
+  double y0, Y[6], corner, plane[3];   // plane[k]: the two axes other than k
+  __device__ __forceinline__ Even39(double y, const double (&Yv)[6]) {
+    y0 = y;
 #pragma unroll
-  for (int i = 0; i < 3; i++) {
-    if (Lat<39>::c(p, i) != 0) r += Y[sym<3>(i, i)];
-#pragma unroll
-    for (int j = i + 1; j < 3; j++) {
-      const int cc = Lat<39>::c(p, i) * Lat<39>::c(p, j);
-      if (cc > 0) r = fma(2.0, Y[sym<3>(i, j)], r);
-      if (cc < 0) r = fma(-2.0, Y[sym<3>(i, j)], r);
-    }
+    for (int k = 0; k < 6; k++) Y[k] = Yv[k];
+    const double s01 = Y[sym<3>(0, 0)] + Y[sym<3>(1, 1)];
+    corner = y0 + (s01 + Y[sym<3>(2, 2)]);
+    plane[2] = fma(4.0, s01, y0);
+    plane[1] = fma(4.0, Y[sym<3>(0, 0)] + Y[sym<3>(2, 2)], y0);
+    plane[0] = fma(4.0, Y[sym<3>(1, 1)] + Y[sym<3>(2, 2)], y0);
   }
-  return L == 1 ? y0 + r : fma((double)(L * L), r, y0);
-}
+  __device__ __forceinline__ double operator()(int p) const {
+    const int L = q39_len(p), nz = q39_nnz(p), i = q39_axis(p, 0), j = q39_axis(p, 1);
+    if (nz == 1) return L == 1 ? y0 + Y[sym<3>(i, i)] : fma((double)(L * L), Y[sym<3>(i, i)], y0);
+    if (nz == 2) return fma(2.0 * Lat<39>::c(p, i) * Lat<39>::c(p, j), Y[sym<3>(i, j)], plane[3 - i - j]);
+    const double s1 = Lat<39>::c(p, 1), s2 = Lat<39>::c(p, 2);
+    return fma(2.0 * s1, Y[sym<3>(0, 1)], fma(2.0 * s2, Y[sym<3>(0, 2)], fma(2.0 * s1 * s2, Y[sym<3>(1, 2)], corner)));
+  }
+};
 
 // B (packed) and C / (6 T0^3), u = U / T0 - V / (2 T0^2) of Eq. 33 (V^i = C^ijj)
 __device__ __forceinline__ void herm39_packed(const double (&gd)[6], const double U[3], const double Ut[3],
@@ -715,7 +776,7 @@ __device__ __forceinline__ void herm39_packed(const double (&gd)[6], const doubl
 #pragma unroll
   for (int i = 0; i < 3; i++) {
     const double v = kC[sym3(i, 0, 0)] + kC[sym3(i, 1, 1)] + kC[sym3(i, 2, 2)];
-    u[i] = fma(-3.0 * T0, v, U[i] / T0);
+    u[i] = fma(-3.0 * T0, v, U[i] * kIT0_39);
   }
 }
 
@@ -732,9 +793,11 @@ __device__ __forceinline__ void pull39(const Q39Args &A, int64_t c, const int64_
 }
 
 // One time step with the polynomial force map. Bounded by the FP64 pipe (two
-// lanes per clock and SM): about 850 FP64 operations per cell update, against 3,000 per
-// evaluation of the map direction by direction. 64^3 cells: 0.80 ms a step (330
-// MLUPS; 5.9 ms direction by direction), 168 registers, three blocks per SM.
+// lanes per clock and SM): about 900 FP64 operations per cell update, against 3,000 per
+// evaluation of the map direction by direction. 64^3 cells: 0.42 ms a step (620
+// MLUPS), 168 registers, three blocks per SM; 5.9 ms direction by direction, 0.80 ms with
+// all evaluations of the map in FP64 and divisions by T0, 0.66 ms with the first three
+// in FP32 (see force39), 0.42 ms with the shared sums of Odd39 and Even39.
 template <bool ODD>
 __global__ void __launch_bounds__(kQ39Threads, 3) k_step39_rec(const Q39Args A) {
   const int64_t c = (int64_t)blockIdx.x * kQ39Threads + threadIdx.x;
@@ -746,10 +809,10 @@ __global__ void __launch_bounds__(kQ39Threads, 3) k_step39_rec(const Q39Args A) 
   Cell39 q;
   pull39<ODD>(A, c, ic, q);
   if (!force39(q, ld, A.tol, A.max_iter)) atomicOr(A.err, ERR_NOCONV);
-  const double T0 = kT0_39, itau = 1.0 / A.tau;
+  const double itau = A.itau;
   double Ut[3], gd[6], B[6], kC[10], u[3];
 #pragma unroll
-  for (int i = 0; i < 3; i++) Ut[i] = fma(q.Phi[i], 0.5 / q.m, q.U[i]);
+  for (int i = 0; i < 3; i++) Ut[i] = fma(q.Phi[i], q.h2m, q.U[i]);
 #pragma unroll
   for (int i = 0; i < 6; i++) gd[i] = ld(Rec39::GD + i);
   herm39_packed(gd, q.U, Ut, B, kC, u);
@@ -768,8 +831,10 @@ __global__ void __launch_bounds__(kQ39Threads, 3) k_step39_rec(const Q39Args A) 
       const double M = ld(Rec39::LK + 6 * (p - 1) + l);
 #pragma unroll
       for (int k = 0; k < 3; k++) {
-        if (Lat<39>::c(p, k) > 0) P[k][l] = fma(M, x, P[k][l]);
-        if (Lat<39>::c(p, k) < 0) P[k][l] = fma(-M, x, P[k][l]);
+        // (pair k + 1 is the first with a component along k)
+        if (p == k + 1) P[k][l] = M * x;
+        else if (Lat<39>::c(p, k) > 0) P[k][l] = fma(M, x, P[k][l]);
+        else if (Lat<39>::c(p, k) < 0) P[k][l] = fma(-M, x, P[k][l]);
       }
     }
   }
@@ -781,18 +846,19 @@ __global__ void __launch_bounds__(kQ39Threads, 3) k_step39_rec(const Q39Args A) 
   for (int i = 0; i < 3; i++)
 #pragma unroll
     for (int j = i; j < 3; j++)
-      Y[sym<3>(i, j)] = (0.5 * mt * B[sym<3>(i, j)] + m2 * (i == j ? P[i][i] : 0.5 * (P[i][j] + P[j][i]))) / (T0 * T0);
-  const double y0 = mt * (1.0 - (B[0] + B[3] + B[5]) / (2.0 * T0)) - m2 * (P[0][0] + P[1][1] + P[2][2]) / T0;
+      Y[sym<3>(i, j)] = (0.5 * mt * B[sym<3>(i, j)] + m2 * (i == j ? P[i][i] : 0.5 * (P[i][j] + P[j][i]))) * (kIT0_39 * kIT0_39);
+  const double y0 = mt * (1.0 - (0.5 * kIT0_39) * (B[0] + B[3] + B[5])) - (kIT0_39 * m2) * (P[0][0] + P[1][1] + P[2][2]);
 #pragma unroll
   for (int k = 0; k < 10; k++) kZ[k] = mt * kC[k];
 #pragma unroll
-  for (int i = 0; i < 3; i++) uz[i] = fma(mt, u[i], q.Phi[i] / T0);
+  for (int i = 0; i < 3; i++) uz[i] = fma(mt, u[i], q.Phi[i] * kIT0_39);
   const Odd39 zo(uz, kZ);
+  const Even39 ze(y0, Y);
   const double omt = 1.0 - itau, h = 0.5 * omt;
   A.f[c] = fma(omt, q.s[0], q39_w(0) * y0);
 #pragma unroll
   for (int p = 1; p <= kH39; p++) {
-    const double ev = fma(h, q.s[p], q39_w(p) * even39(p, y0, Y));
+    const double ev = fma(h, q.s[p], q39_w(p) * ze(p));
     const double od = fma(h, q.t[p], q39_w(p) * zo(p));
     A.f[dst39<ODD>(A, c, ic, p)] = ev + od;
     A.f[dst39<ODD>(A, c, ic, p + kH39)] = ev - od;
@@ -835,15 +901,16 @@ __global__ void __launch_bounds__(kQ39Threads) k_init39(const Q39Args A, const d
     herm39_packed(gd, U, U, B, kC, uu);
     const Odd39 xo(uu, kC);
     // N = J rho w (1 + xe +- xo)
-    const double T0 = kT0_39, m = A.J[c] * rho[c];
+    const double m = A.J[c] * rho[c];
     double Y[6];
 #pragma unroll
-    for (int i = 0; i < 6; i++) Y[i] = B[i] / (2.0 * T0 * T0);
-    const double y0 = 1.0 - (B[0] + B[3] + B[5]) / (2.0 * T0);
+    for (int i = 0; i < 6; i++) Y[i] = B[i] * (0.5 * kIT0_39 * kIT0_39);
+    const double y0 = 1.0 - (0.5 * kIT0_39) * (B[0] + B[3] + B[5]);
+    const Even39 xe(y0, Y);
     A.f[c] = m * (q39_w(0) * y0);
 #pragma unroll
     for (int p = 1; p <= kH39; p++) {
-      const double ev = even39(p, y0, Y), od = xo(p), mw = m * q39_w(p);
+      const double ev = xe(p), od = xo(p), mw = m * q39_w(p);
       A.f[(int64_t)p * A.ncell + c] = mw * (ev + od);
       A.f[(int64_t)(p + kH39) * A.ncell + c] = mw * (ev - od);
     }
@@ -880,7 +947,7 @@ __global__ void __launch_bounds__(kMomThreads) k_moments39(const Q39Args A, doub
 #pragma unroll
       for (int i = 0; i < 3; i++) {
         U[i] = q.U[i];
-        aF[i] = 0.5 * q.Phi[i] / q.m;
+        aF[i] = q.Phi[i] * q.h2m;
         bP[i] = q.U[i] * q.m;
       }
     } else {
@@ -1024,6 +1091,7 @@ Q39Args make_args(const vlb_sim *sim) {
   A.rec = sim->nc == kRec39 ? static_cast<const double *>(sim->d_coef) : nullptr;
   A.chord = sim->nc == kRec39 ? nullptr : static_cast<const double *>(sim->d_coef);
   A.tau = sim->p.tau;
+  A.itau = 1.0 / A.tau;
   A.tol = sim->p.tol;
   A.max_iter = sim->p.max_iter;
   A.err = sim->d_err;
