@@ -212,7 +212,8 @@ int vlb_mesh_create(const vlb_mesh_desc *desc, vlb_mesh **out) {
   m->stats.feq_rest_min = v[2];
   m->stats.ginv_diag_min = v[3];
   m->stats.ginv_diag_max = -v[4];
-  m->stats.invariant_fast_axis = hflag ? 0 : 1;
+  m->stats.invariant_fast_axis = hflag & 1 ? 0 : 1;
+  m->extruded = q == VLB_D3Q19 && hflag == 0 ? 1 : 0;
   m->stats.ncell = nc;
   rc = cleanup(VLB_OK);
   *out = m;

@@ -55,6 +55,23 @@ struct CollideState {
   bool conv;
 };
 
+// Extruded meshes (EXT; D3Q19, plane records): the first two coordinates of a cell's
+// position do not depend on the fastest axis and the third on nothing else (vlb_mesh::
+// extruded). Then K^2_a = 0, g^02 = g^12 = 0, and K_a depends on (c^0_a, c^1_a) alone, so that
+//  - the nine pairs have four sets of link coefficients: pairs 1, 6 and 7 share those of
+//    pair 1, pairs 2, 8 and 9 those of pair 2, pair 3 has none;
+//  - component 2 of Phi is m G^2, outside the iteration (row and column 2 of H - I and
+//    of PO1, row 2 of the map and CE^2, KW^2 are zero);
+//  - of the map's twelve monomials, those odd in U~^2 have coefficient zero.
+// The steps are bound by issue (FP32, 16 bits) and by the FP64 pipe: 100 steps with reset and
+// moments of D3Q19 channels, FP64 64^3 22.2 -> 17.0 ms, FP16 128^3 9.0 -> 8.1 ms, FP32 75 x 67
+// x 101 2.9 -> 2.6 ms.
+template <bool EXT, int D>
+__device__ constexpr bool map_mono(int s) {   // has monomial s of a chord step a coefficient?
+  return !EXT || !(s == sym<D>(0, 2) || s == sym<D>(1, 2) || s == D * (D + 1) / 2 + offd<D>(0, 2) ||
+                   s == D * (D + 1) / 2 + offd<D>(1, 2));
+}
+
 // D x D inverse (D = 2 or 3) by cofactors, FP64
 template <int D>
 __device__ void inverse_small(const double (&A)[D][D], double (&X)[D][D]) {
@@ -511,7 +528,7 @@ struct MomentWeights<9, R> {
 // and then mn = mdev - sum_a RR_a. Every term is formed relative to its own
 // size, and the identity behind the final pass holds for whatever J it uses,
 // as long as RR, their sum and mn use the same one.
-template <int Q, typename R, bool REST, bool RREC, typename RC>
+template <int Q, typename R, bool REST, bool RREC, bool EXT, typename RC>
 __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R mdev, R mn,
                                         R nref, R h2m, R rho, R itau, const R (&U)[Lat<Q>::D],
                                         const R (&Phi)[Lat<Q>::D], R (&dp)[Q]) {
@@ -589,7 +606,9 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
 #pragma unroll
     for (int l = 0; l < D; l++) {
       if (k == l) continue;
-      C2h[k][l] = fmar(gh[sym<D>(k, k)], Ut[l], fmar(gh[sym<D>(k, l)], Ut2x[k], fmar(U2[k], Ut[l], v[l])));
+      R t = fmar(U2[k], Ut[l], v[l]);
+      if (!EXT || (k < 2 && l < 2)) t = fmar(gh[sym<D>(k, l)], Ut2x[k], t);
+      C2h[k][l] = fmar(gh[sym<D>(k, k)], Ut[l], t);
     }
   using MW = MomentWeights<Q, R>;
   R Oax[D];   // axis pairs: a1 U^l - b1 sum_{k != l} C2h^kl
@@ -636,7 +655,23 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   for (int i = 0; i < D; i++)
 #pragma unroll
     for (int j = 0; j < D; j++) dP[i][j] = R(0);
-  {
+  if constexpr (EXT) {
+    // pairs with the same coefficients together: xo of pairs 6 and 7 is T_02 +- T_20, of
+    // pairs 8 and 9 T_12 +- T_21, and the axis weight twice the diagonal one. In units of
+    // 2 r6w2 (taken into a9 below); column 2 is zero.
+    const float2 m4 = rc.v2(L::mp(4, 0)), m5 = rc.v2(L::mp(5, 0)), mx = rc.v2(L::mp(1, 0)), my = rc.v2(L::mp(2, 0));
+    const float2 t4 = __fmul2_rn(m4, bcast2(0.5f * xo[4]));
+    const float x5 = 0.5f * xo[5];
+    const float2 P0 = __ffma2_rn(mx, bcast2(T0[0] + T[0][2]), __ffma2_rn(m5, bcast2(x5), t4));
+    const float2 P1 = __ffma2_rn(my, bcast2(T0[1] + T[1][2]), __ffma2_rn(m5, bcast2(-x5), t4));
+    const float2 P2 = __ffma2_rn(my, bcast2(T[2][1]), __fmul2_rn(mx, bcast2(T[2][0])));
+    dP[0][0] = P0.x;
+    dP[0][1] = P0.y;
+    dP[1][0] = P1.x;
+    dP[1][1] = P1.y;
+    dP[2][0] = P2.x;
+    dP[2][1] = P2.y;
+  } else {
     // columns 0 and 1 in the two lanes of packed FP32 instructions
     float2 P01[D];
 #pragma unroll
@@ -662,8 +697,8 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   }
   R tr = dP[0][0];
 #pragma unroll
-  for (int i = 1; i < D; i++) tr += dP[i][i];
-  const R J = rc[L::J];
+  for (int i = 1; i < (EXT ? 2 : D); i++) tr += dP[i][i];
+  const R J = EXT ? rc[L::J] * (R(2) * r6w2) : rc[L::J];   // J times the unit of dP
   // E_p = 9 w J c.dP.c - 3 w J tr dP; O_p = 3 w c.Phi (Eq. 31, 1/T0 = 3)
   const R a9_1 = (R(9) * lat_w<Q, R>(1)) * J, a9_2 = (R(9) * lat_w<Q, R>(Lat<Q>::H)) * J;
   const R tr3 = tr * R(1.0 / 3.0);
@@ -682,17 +717,18 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
     const bool axis = k < 0;
     R cPc, cF;
     if (axis) {
-      cPc = dP[l][l];
+      cPc = EXT && l == 2 ? R(0) : dP[l][l];
       cF = sl > 0 ? Phi[l] : -Phi[l];
     } else {
       const int sk = Lat<Q>::c(p, k);
-      const R so = dP[l][k] + dP[k][l];
-      const R sd = dP[l][l] + dP[k][k];
+      const bool flat = EXT && k == 2;
+      const R so = flat ? dP[k][l] : dP[l][k] + dP[k][l];
+      const R sd = flat ? dP[l][l] : dP[l][l] + dP[k][k];
       cPc = sl * sk > 0 ? sd + so : sd - so;
       const R f = sl > 0 ? Phi[l] : -Phi[l];
       cF = sk > 0 ? f + Phi[k] : f - Phi[k];
     }
-    const R Ep = fmar(axis ? a9_1 : a9_2, cPc, -(axis ? b3_1 : b3_2));
+    const R Ep = EXT && axis && l == 2 ? -b3_1 : fmar(axis ? a9_1 : a9_2, cPc, -(axis ? b3_1 : b3_2));
     const R Op = (axis ? MW::a1 : MW::a2) * cF;
     const R wm = axis ? wm1 : wm2;
     const R rw = rw_at(p);
@@ -742,11 +778,13 @@ __device__ __forceinline__ float trunc_f32(double x) {
 //    Y = (9/2)(m/tau) B + 9 P, P = J deltaPi (Eq. 30) symmetrised,
 //    y0 = (mdev - (3/2) m tr B)/tau - 3 tr P.
 // D3Q19 channel, 64^3: 383 -> 219 us a step, the FP64 pipe over 90% busy.
-template <int Q, bool FINAL, typename RC>
+template <int Q, bool FINAL, bool EXT, typename RC>
 __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, double nref, double itau, double tol,
                                             int max_iter, double (&dp)[Q], CollideState<Q, double> &st) {
   using L = CoefLayout<Q>;
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS, NQ = L::NQ;
+  static_assert(!EXT || Q == 19, "extruded meshes are D3Q19's");
+  constexpr int DI = EXT ? 2 : D;   // components of Phi that are iterated
   double s[H + 1], t[H + 1], mu[D], Pc[D], Pt[D], mdev = d[0];
 #pragma unroll
   for (int i = 0; i < D; i++) mu[i] = Pc[i] = 0.0;
@@ -754,6 +792,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
   for (int p = 1; p <= H; p++) {
     s[p] = d[p] + d[p + H];
     t[p] = d[p] - d[p + H];
+    if constexpr (EXT) continue;
     mdev += s[p];
 #pragma unroll
     for (int i = 0; i < D; i++) {
@@ -762,6 +801,23 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       if (ci < 0) mu[i] -= t[p];
       Pc[i] = fma(rc[L::mp(p, i)], s[p], Pc[i]);
       Pc[i] = fma(rc[L::dk(p, i)], t[p], Pc[i]);
+    }
+  }
+  if constexpr (EXT) {
+    const double sg[4] = {s[1] + (s[6] + s[7]), s[2] + (s[8] + s[9]), s[4], s[5]};
+    const double tg[4] = {t[1] + (t[6] + t[7]), t[2] + (t[8] + t[9]), t[4], t[5]};
+    mdev += s[3] + ((sg[0] + sg[1]) + (sg[2] + sg[3]));
+    mu[0] = tg[0] + (tg[2] + tg[3]);
+    mu[1] = tg[1] + (tg[2] - tg[3]);
+    mu[2] = t[3] + ((t[6] - t[7]) + (t[8] - t[9]));
+#pragma unroll
+    for (int g = 0; g < 4; g++) {
+      const int p = g < 2 ? g + 1 : g + 2;
+#pragma unroll
+      for (int i = 0; i < 2; i++) {
+        Pc[i] = fma(rc[L::mp(p, i)], sg[g], Pc[i]);
+        Pc[i] = fma(rc[L::dk(p, i)], tg[g], Pc[i]);
+      }
     }
   }
   const double m = nref + mdev, im = 1.0 / m, h2m = 0.5 * im, hm = 0.5 * m;
@@ -775,19 +831,20 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
   }
   // Pc = sum_p (am M s + ad D t) + m G - (n_ref + mdev itau/2) KW - m/2 (CE + (PO1 + LO) U)
 #pragma unroll
-  for (int i = 0; i < D; i++) {
+  for (int i = 0; i < DI; i++) {
     double v = fma(m, rc[L::BODY + i], Pc[i]);
     v = fma(-hm, rc[L::CE + i], v);
 #pragma unroll
-    for (int l = 0; l < D; l++) v = fma(rc[L::PO1 + i * D + l], hmu[l], v);
+    for (int l = 0; l < DI; l++) v = fma(rc[L::PO1 + i * D + l], hmu[l], v);
     Pc[i] = fma(-kf, rc[L::KW + i], v);
   }
 #pragma unroll
-  for (int i = 0; i < D; i++) {
+  for (int i = 0; i < DI; i++) {
     Pt[i] = Pc[i];
 #pragma unroll
-    for (int j = 0; j < D; j++) Pt[i] = fma(rc[L::row(L::HM, D, i, j)], Pc[j], Pt[i]);
+    for (int j = 0; j < DI; j++) Pt[i] = fma(rc[L::row(L::HM, D, i, j)], Pc[j], Pt[i]);
   }
+  if constexpr (EXT) Pt[2] = m * rc[L::BODY + 2];
   double Phi[D];
   float lip = 1.0e30f;   // bound on the contraction of one evaluation
   int it = 0;
@@ -802,6 +859,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       df[i] = 0.f;
 #pragma unroll
       for (int k = 0; k < NQ; k++) {
+        if (i >= DI || !map_mono<EXT, D>(k)) continue;
         qf[i][k] = trunc_f32(rc[L::row(L::QM, NQ, i, k)]);
         if (k < NS)
           l2 += fabsf(qf[i][k]);
@@ -825,10 +883,11 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
           if (k != l) mono[NS + offd<D>(k, l)] = (x[k] * x[k]) * x[l];
         }
 #pragma unroll
-      for (int i = 0; i < D; i++) {
+      for (int i = 0; i < DI; i++) {
         float v = 0.f;
 #pragma unroll
-        for (int k = 0; k < NQ; k++) v = fmaf(qf[i][k], mono[k], v);
+        for (int k = 0; k < NQ; k++)
+          if (map_mono<EXT, D>(k)) v = fmaf(qf[i][k], mono[k], v);
         df[i] = -hmf * v;
       }
     }
@@ -838,17 +897,18 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     um *= 1.01f;
     lip = fmaf(0.5f * l2, um, 0.75f * l3 * um * um);
 #pragma unroll
-    for (int i = 0; i < D; i++) Phi[i] = Pt[i] + (double)df[i];
+    for (int i = 0; i < DI; i++) Phi[i] = Pt[i] + (double)df[i];
   } else {
 #pragma unroll
-    for (int i = 0; i < D; i++) Phi[i] = m * rc[L::FR + i];
+    for (int i = 0; i < DI; i++) Phi[i] = m * rc[L::FR + i];
   }
+  if constexpr (EXT) Phi[2] = Pt[2];
   st.conv = false;
   const float tolf = (float)tol, epsf = (float)(64.0 / 9007199254740992.0);
 #pragma unroll 1
   while (it < max_iter) {
     double Ut[D], mono[NQ];
-    float diff = 0.f, pmax = 0.f;
+    float diff = 0.f, pmax = EXT ? fabsf(trunc_f32(Phi[D - 1])) : 0.f;
 #pragma unroll
     for (int i = 0; i < D; i++) Ut[i] = fma(Phi[i], h2m, st.U[i]);
 #pragma unroll
@@ -861,11 +921,12 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       for (int l = 0; l < D; l++)
         if (k != l) mono[NS + offd<D>(k, l)] = mono[sym<D>(k, k)] * Ut[l];
 #pragma unroll
-    for (int i = 0; i < D; i++) {
+    for (int i = 0; i < DI; i++) {
       // two partial sums: the chain of a small mesh is bound by latency
       double a = rc[L::row(L::QM, NQ, i, 0)] * mono[0], b = rc[L::row(L::QM, NQ, i, 1)] * mono[1];
 #pragma unroll
       for (int k = 2; k < NQ; k++) {
+        if (!map_mono<EXT, D>(k)) continue;
         if (k & 1)
           b = fma(rc[L::row(L::QM, NQ, i, k)], mono[k], b);
         else
@@ -901,7 +962,9 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
 #pragma unroll
     for (int i = 0; i < D; i++)
 #pragma unroll
-      for (int j = i; j < D; j++) B[sym<D>(i, j)] = fma(U3[i], Ut[j], 2.0 * rc[L::GH + sym<D>(i, j)]);
+      for (int j = i; j < D; j++)
+        B[sym<D>(i, j)] =
+            EXT && i < 2 && j == 2 ? U3[i] * Ut[j] : fma(U3[i], Ut[j], 2.0 * rc[L::GH + sym<D>(i, j)]);
 #pragma unroll
     for (int i = 0; i < D; i++) tb += B[sym<D>(i, i)];
     // per axis l: xo/3 of an axis direction is T0_l = U^l - sum_k C2^kl, of a diagonal
@@ -913,7 +976,8 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       for (int k = 0; k < D; k++) {
         if (k == l) continue;
         // gd_kk/2 + (3/2) U~k^2 = B_kk / 2
-        C2[k][l] = fma(0.5 * B[sym<D>(k, k)], Ut[l], fma(rc[L::GH + sym<D>(k, l)], Ut[k] + Ut[k], du[l]));
+        const double x = EXT && (k == 2 || l == 2) ? du[l] : fma(rc[L::GH + sym<D>(k, l)], Ut[k] + Ut[k], du[l]);
+        C2[k][l] = fma(0.5 * B[sym<D>(k, k)], Ut[l], x);
         Sc[l] += C2[k][l];
       }
       T0[l] = st.U[l] - Sc[l];
@@ -939,8 +1003,19 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     // the axis weight is 2 (D3Q19) or 4 (D2Q9) times the diagonal one
     constexpr double wr = D == 3 ? 2.0 : 4.0;
     const double w2 = lat_w<Q, double>(H);
+    if constexpr (EXT) {
+      // pairs with the same coefficients together (see form_np), in units of 2
+      const double x4 = 0.5 * xo3(4), x5 = 0.5 * xo3(5);
 #pragma unroll
-    for (int p = 1; p <= H; p++) {
+      for (int j = 0; j < 2; j++) {
+        const double t4 = rc[L::mp(4, j)] * x4;
+        P[0][j] = fma(rc[L::mp(1, j)], T0[0] + T[0][2], fma(rc[L::mp(5, j)], x5, t4));
+        P[1][j] = fma(rc[L::mp(2, j)], T0[1] + T[1][2], fma(rc[L::mp(5, j)], -x5, t4));
+        P[2][j] = fma(rc[L::mp(2, j)], T[2][1], rc[L::mp(1, j)] * T[2][0]);
+      }
+    }
+#pragma unroll
+    for (int p = 1; p <= (EXT ? 0 : H); p++) {
       const double x = lat_nnz<Q>(p) == 1 ? wr * xo3(p) : xo3(p);
 #pragma unroll
       for (int j = 0; j < D; j++) {
@@ -954,17 +1029,22 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       }
     }
     // everything times w2: Y = w2 [(9/2)(m/tau) B + 9 P], B = (3 B) / 3
-    const double mt = m * itau, yb = (1.5 * w2) * mt, yp = (54.0 * w2 * w2) * m;
+    constexpr double pu = EXT ? 2.0 : 1.0;   // the unit of P
+    const double mt = m * itau, yb = (1.5 * w2) * mt, yp = (54.0 * w2 * w2 * pu) * m;
     double Y[NS], trP = 0.0;
 #pragma unroll
     for (int i = 0; i < D; i++) {
-      trP += P[i][i];
+      if (i < DI) trP = i == 0 ? P[0][0] : trP + P[i][i];
 #pragma unroll
-      for (int j = i; j < D; j++)
-        Y[sym<D>(i, j)] = fma(yb, B[sym<D>(i, j)], i == j ? yp * P[i][i] : (0.5 * yp) * (P[i][j] + P[j][i]));
+      for (int j = i; j < D; j++) {
+        if (EXT && j == 2)
+          Y[sym<D>(i, j)] = i == 2 ? yb * B[sym<D>(i, j)] : fma(0.5 * yp, P[j][i], yb * B[sym<D>(i, j)]);
+        else
+          Y[sym<D>(i, j)] = fma(yb, B[sym<D>(i, j)], i == j ? yp * P[i][i] : (0.5 * yp) * (P[i][j] + P[j][i]));
+      }
     }
     // y0 = w2 [(mdev - m (3 tr B) / 2) / tau - 3 tr P]
-    const double y0 = fma(-((18.0 * w2 * w2) * m), trP, w2 * itau * fma(-hm, tb, mdev));
+    const double y0 = fma(-((18.0 * w2 * w2 * pu) * m), trP, w2 * itau * fma(-hm, tb, mdev));
     // (the weights of the odd part are MomentWeights': no momentum is made by rounding them)
     using MW = MomentWeights<Q, double>;
     const double omt = 1.0 - itau, h = 0.5 * omt, zm = MW::a2 * mt;
@@ -1008,7 +1088,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
 // deviations are formed at the converged Phi.
 // rc is the cell's coefficient record (PtrRecord or CellRecord); itau = 1/tau. With REST, d holds e_a = N_a - o_a relative to the
 // cell's own rest state (16-bit storage, see CoefLayout), and so does dp.
-template <int Q, typename R, bool FINAL, bool REST, bool RREC, typename RC>
+template <int Q, typename R, bool FINAL, bool REST, bool RREC, bool EXT, typename RC>
 __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nref,
                                              R itau, R tol, int max_iter, R (&dp)[Q],
                                              CollideState<Q, R> &st) {
@@ -1016,6 +1096,8 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   using L = CoefLayout<Q>;
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS, NQ = L::NQ;
   static_assert(D == 2 || NQ % 4 == 0, "row 2 of the chord step is read in 16-byte quads");
+  static_assert(!EXT || Q == 19, "extruded meshes are D3Q19's");
+  constexpr int DI = EXT ? 2 : D;   // components of Phi that are iterated
   const R epsn = sizeof(R) == 4 ? R(64.0 / 16777216.0) : R(64.0 / 9007199254740992.0);
   // pair sums s_p = d_p + d_pbar and differences t_p = d_p - d_pbar
   // (with REST: of e_a; the rest state's part of the s_p enters through SR)
@@ -1025,7 +1107,20 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   for (int p = 1; p <= H; p++) {
     sp[p] = d[p] + d[p + H];
     tp[p] = d[p] - d[p + H];
-    mdev += sp[p];
+    if constexpr (!EXT) mdev += sp[p];
+  }
+  // sums over the pairs that share link coefficients
+  R sg[4], tg[4];
+  if constexpr (EXT) {
+    sg[0] = sp[1] + (sp[6] + sp[7]);
+    sg[1] = sp[2] + (sp[8] + sp[9]);
+    tg[0] = tp[1] + (tp[6] + tp[7]);
+    tg[1] = tp[2] + (tp[8] + tp[9]);
+    sg[2] = sp[4];
+    sg[3] = sp[5];
+    tg[2] = tp[4];
+    tg[3] = tp[5];
+    mdev += sp[3] + ((sg[0] + sg[1]) + (sg[2] + sg[3]));
   }
   // m - J, the mass of the flow
   R mn;
@@ -1044,11 +1139,17 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
 #pragma unroll
   for (int i = 0; i < D; i++) {
     R s = R(0);
+    if constexpr (EXT) {
+      s = i == 0   ? tg[0] + (tg[2] + tg[3])
+          : i == 1 ? tg[1] + (tg[2] - tg[3])
+                   : tp[3] + ((tp[6] - tp[7]) + (tp[8] - tp[9]));
+    } else {
 #pragma unroll
-    for (int p = 1; p <= H; p++) {
-      const int ci = Lat<Q>::c(p, i);
-      if (ci > 0) s += tp[p];
-      if (ci < 0) s -= tp[p];
+      for (int p = 1; p <= H; p++) {
+        const int ci = Lat<Q>::c(p, i);
+        if (ci > 0) s += tp[p];
+        if (ci < 0) s -= tp[p];
+      }
     }
     st.U[i] = s * im;
   }
@@ -1062,7 +1163,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   // whose two weights the record's link coefficients already carry.
   R s[D], pr[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) {
+  for (int i = 0; i < DI; i++) {
     const R kw = rc[L::KW + i];
     pr[i] = nref * kw;
     const R err = two_prod_err(nref, kw, pr[i]) + nref * rc[L::KWL + i];
@@ -1073,14 +1174,16 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     // components 0 and 1 in the two lanes of packed FP32 instructions, two
     // partial sums each
     float2 sa = make_float2(s[0], s[1]), sb = make_float2(0.f, 0.f);
-    float s2a = D == 3 ? s[D - 1] : 0.f, s2b = 0.f;
+    float s2a = D == 3 && !EXT ? s[D - 1] : 0.f, s2b = 0.f;
 #pragma unroll
-    for (int p = 1; p <= H; p++) {
+    for (int k = 1; k <= (EXT ? 4 : H); k++) {
+      const int p = EXT && k > 2 ? k + 1 : k;
+      const R sk = EXT ? sg[(k - 1) & 3] : sp[p], tk = EXT ? tg[(k - 1) & 3] : tp[p];
       const float4 q = rc.v4(L::mp(p, 0));   // am M^0, am M^1, ad D^0, ad D^1
-      float2 &acc = (p & 1) ? sa : sb;
-      acc = __ffma2_rn(make_float2(q.x, q.y), bcast2(sp[p]), acc);
-      acc = __ffma2_rn(make_float2(q.z, q.w), bcast2(tp[p]), acc);
-      if constexpr (D == 3) {
+      float2 &acc = (k & 1) ? sa : sb;
+      acc = __ffma2_rn(make_float2(q.x, q.y), bcast2(sk), acc);
+      acc = __ffma2_rn(make_float2(q.z, q.w), bcast2(tk), acc);
+      if constexpr (D == 3 && !EXT) {
         const float2 r2 = rc.v2(L::mp(p, 2));   // am M^2, ad D^2
         float &a2 = (p & 1) ? s2a : s2b;
         a2 = fmaf(r2.x, sp[p], a2);
@@ -1090,26 +1193,28 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     const float2 st01 = __fadd2_rn(sa, sb);
     s[0] = st01.x;
     s[1] = st01.y;
-    if constexpr (D == 3) s[D - 1] = s2a + s2b;
+    if constexpr (D == 3 && !EXT) s[D - 1] = s2a + s2b;
   }
   // Pc = Pb - 1/2 m (CE + (PO1 + LO) U), then Pt = H Pc = Pc + (H - I) Pc
   R Pc[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) {
+  for (int i = 0; i < DI; i++) {
     R u = rc[L::CE + i];
 #pragma unroll
-    for (int l = 0; l < D; l++) u = fmar(rc[L::PO1 + i * D + l], st.U[l], u);
+    for (int l = 0; l < DI; l++) u = fmar(rc[L::PO1 + i * D + l], st.U[l], u);
     Pc[i] = (s[i] - hm * u) - pr[i];
   }
   R Pt[D];
   {
     float2 x = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < D; j++) x = __ffma2_rn(rc.v2(L::row(L::HM, D, 0, j)), bcast2(Pc[j]), x);
+    for (int j = 0; j < DI; j++) x = __ffma2_rn(rc.v2(L::row(L::HM, D, 0, j)), bcast2(Pc[j]), x);
     const float2 p01 = __fadd2_rn(make_float2(Pc[0], Pc[1]), x);
     Pt[0] = p01.x;
     Pt[1] = p01.y;
-    if constexpr (D == 3) {
+    if constexpr (EXT) {
+      Pt[2] = m * rc[L::BODY + 2];
+    } else if constexpr (D == 3) {
       R y = R(0);
 #pragma unroll
       for (int j = 0; j < D; j++) y = fmar(rc[L::row(L::HM, D, 2, j)], Pc[j], y);
@@ -1122,7 +1227,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   // evaluation less reaches the same residual.
   R Phi[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) Phi[i] = max_iter >= 4 ? Pt[i] : m * rc[L::FR + i];
+  for (int i = 0; i < D; i++) Phi[i] = max_iter >= 4 || i >= DI ? Pt[i] : m * rc[L::FR + i];
   st.conv = false;
   int it = 0;
   while (it < max_iter) {
@@ -1150,6 +1255,15 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
       float a2a = 0.f, a2b = 0.f;
 #pragma unroll
       for (int s2 = 0; s2 < NQ; s2 += 2) {
+        if constexpr (EXT) {
+          if (!map_mono<EXT, D>(s2) || !map_mono<EXT, D>(s2 + 1)) {
+            // one monomial of the two (extruded meshes: never none)
+            const int s1 = map_mono<EXT, D>(s2) ? s2 : s2 + 1;
+            float2 &acc = (s2 & 2) ? a01a : a01b;
+            acc = __ffma2_rn(rc.v2(L::QM + 2 * s1), bcast2(mono[s1]), acc);
+            continue;
+          }
+        }
         if (s2 + 1 < NQ) {
           const float4 q = rc.v4(L::QM + 2 * s2);
           a01a = __ffma2_rn(make_float2(q.x, q.y), bcast2(mono[s2]), a01a);
@@ -1158,7 +1272,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
           a01a = __ffma2_rn(rc.v2(L::QM + 2 * s2), bcast2(mono[s2]), a01a);
         }
       }
-      if constexpr (D == 3) {
+      if constexpr (D == 3 && !EXT) {
 #pragma unroll
         for (int s4 = 0; s4 < NQ; s4 += 4) {
           const float4 q = rc.v4(L::row(L::QM, NQ, 2, s4));
@@ -1171,13 +1285,13 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
       const float2 a01 = __fadd2_rn(a01a, a01b);
       a[0] = a01.x;
       a[1] = a01.y;
-      if constexpr (D == 3) a[D - 1] = a2a + a2b;
+      if constexpr (D == 3 && !EXT) a[D - 1] = a2a + a2b;
     }
     it++;
     // converged when the change is at most max(tol max(m, |Phi|), 64 eps |Phi|)
-    R diff = R(0), pmax = R(0);
+    R diff = R(0), pmax = EXT ? absr(Phi[D - 1]) : R(0);
 #pragma unroll
-    for (int i = 0; i < D; i++) {
+    for (int i = 0; i < DI; i++) {
       const R pn = fmar(-hm, a[i], Pt[i]);
       diff = maxnan(diff, absr(pn - Phi[i]));
       pmax = maxnan(pmax, absr(Phi[i]));
@@ -1189,20 +1303,21 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     }
   }
   st.iters = it;
-  if (FINAL) form_np<Q, R, REST, RREC, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
+  if (FINAL) form_np<Q, R, REST, RREC, EXT, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
 }
 
 // the local collision in the arithmetic type R
-template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>>
+template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>,
+          bool EXT = false>
 __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nref, R itau, R tol, int max_iter,
                                              R (&dp)[Q], CollideState<Q, R> &st) {
   if constexpr (sizeof(R) == 8) {
     static_assert(!REST, "FP64 populations are stored relative to the uniform reference");
-    collide_f64<Q, FINAL, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+    collide_f64<Q, FINAL, EXT, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   } else {
-    collide_f32<Q, R, FINAL, REST, RREC, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+    collide_f32<Q, R, FINAL, REST, RREC, EXT, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   }
 }
 

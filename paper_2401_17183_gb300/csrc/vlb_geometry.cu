@@ -341,7 +341,9 @@ cudaError_t launch_mesh_stats(const vlb_mesh *m, double *d_partial, int64_t nblk
 }
 
 // plane check: does every cell's geometry equal that of the first cell of its
-// column along the fastest axis (to 1e-12 relative)?
+// column along the fastest axis (to 1e-12 relative)? Flag bit 0: no. Bit 1: the columns are
+// not those of an extruded mesh (D3Q19; see collide_f32), to the rounding of FP64:
+// g^02 = g^12 = 0, K^2_a = 0, and K_a is that of the pair with c^2_a = 0.
 __device__ __forceinline__ bool close12(double a, double b) {
   return fabs(a - b) <= 1e-12 * (1.0 + fabs(b));
 }
@@ -354,7 +356,25 @@ __global__ void k_plane_check(const double *J, const double *ginv, const double 
   if (c >= ncell) return;
   const int64_t c0 = (c / nfast) * nfast;
   // (a mesh that varies is known to at once: the rest need not be read)
-  if (c0 == c || *(volatile int *)flag) return;
+  if (*(volatile int *)flag & 1) return;
+  if (c0 == c) {
+    if constexpr (Q == 19) {
+      const double *k = K + c * Q * D, tiny = 1e-15;
+      bool ext = fabs(ginv[c * NS + sym<D>(0, 2)]) <= tiny && fabs(ginv[c * NS + sym<D>(1, 2)]) <= tiny;
+      for (int a = 1; a < Q; a++) {
+        int b = 0;   // the direction with the same c^0, c^1 and c^2 = 0
+        for (int e = 1; e < Q; e++)
+          if (Lat<Q>::c(e, 0) == Lat<Q>::c(a, 0) && Lat<Q>::c(e, 1) == Lat<Q>::c(a, 1) && Lat<Q>::c(e, 2) == 0) b = e;
+        for (int i = 0; i < 2; i++) {
+          const double r = b > 0 ? k[b * D + i] : 0.0;
+          ext = ext && fabs(k[a * D + i] - r) <= tiny * (1.0 + fabs(r));
+        }
+        ext = ext && fabs(k[a * D + 2]) <= tiny;
+      }
+      if (!ext) atomicOr(flag, 2);
+    }
+    return;
+  }
   bool same = close12(J[c], J[c0]);
   for (int i = 0; i < NS; i++) same = same && close12(ginv[c * NS + i], ginv[c0 * NS + i]);
   for (int i = 0; i < D * D; i++) same = same && close12(gu[c * D * D + i], gu[c0 * D * D + i]);

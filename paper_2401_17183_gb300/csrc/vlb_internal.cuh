@@ -455,6 +455,7 @@ struct vlb_mesh {
   double *d_K = nullptr;     // [ncell][q][dim]
   vlb_mesh_stats stats;
   int device = 0;
+  int32_t extruded = 0;      // D3Q19, invariant fastest axis: see collide_f32 in vlb_collide.cuh
 };
 
 struct vlb_sim {

@@ -14,8 +14,11 @@ cudaError_t launch_steps_small(const vlb_sim *sim, int64_t nsteps, int64_t *done
   auto go = [&](auto qt, auto tag) {
     constexpr int Q = decltype(qt)::value;
     using R = typename decltype(tag)::type;
-    return sim->plane ? launch_small_t<Q, R, true>(sim, nsteps, done, s)
-                      : launch_small_t<Q, R, false>(sim, nsteps, done, s);
+    if constexpr (Q == 19) {
+      if (sim->plane && m->extruded) return launch_small_t<Q, R, true, true>(sim, nsteps, done, s);
+    }
+    return sim->plane ? launch_small_t<Q, R, true, false>(sim, nsteps, done, s)
+                      : launch_small_t<Q, R, false, false>(sim, nsteps, done, s);
   };
   auto lat = [&](auto tag) {
     return q == 9 ? go(std::integral_constant<int, 9>(), tag) : go(std::integral_constant<int, 19>(), tag);

@@ -47,7 +47,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target) {
 
 // one cell's step: pull, collide, push (see step_tiles); populations are read
 // past L1, which other SMs' writes do not reach
-template <int Q, typename R, bool ODD, bool PLANE, typename RC>
+template <int Q, typename R, bool ODD, bool PLANE, bool EXT, typename RC>
 __device__ __forceinline__ void small_cell(const StepArgs &a, const Addr<Q, int32_t> &ad, const RC &rc) {
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H;
   using L = CoefLayout<Q>;
@@ -60,7 +60,7 @@ __device__ __forceinline__ void small_cell(const StepArgs &a, const Addr<Q, int3
     N[av] = __ldcg(f + (own ? a.soff[av] + cell : a.soff[lat_opp<Q>(av)] + ad.nb(av, -1)));
   }
   CollideState<Q, R> cst;
-  collide_cell<Q, R, true, false, PLANE, RC>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
+  collide_cell<Q, R, true, false, PLANE, RC, EXT>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
                                              arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
   if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
   if (a.moving && ad.wall_cell()) {
@@ -111,7 +111,7 @@ struct SmallRecords {
 
 // CLUSTER: all blocks form one thread-block cluster, whose barrier the hardware
 // keeps; else they count themselves in global memory.
-template <int Q, typename R, bool PLANE, int T, int MINB, bool CLUSTER>
+template <int Q, typename R, bool PLANE, bool EXT, int T, int MINB, bool CLUSTER>
 __global__ void __launch_bounds__(T, MINB)
     k_steps_small(const __grid_constant__ StepArgs a, int32_t first, int32_t nsteps, unsigned *count) {
   constexpr bool CELLREC = !PLANE && sizeof(R) == 4;
@@ -143,9 +143,9 @@ __global__ void __launch_bounds__(T, MINB)
     if constexpr (CELLREC) rc.opaque();
     if (live) {
       if ((first + k) & 1)
-        small_cell<Q, R, true, PLANE, RC>(a, ad, rc);
+        small_cell<Q, R, true, PLANE, EXT, RC>(a, ad, rc);
       else
-        small_cell<Q, R, false, PLANE, RC>(a, ad, rc);
+        small_cell<Q, R, false, PLANE, EXT, RC>(a, ad, rc);
     }
     if constexpr (CLUSTER) {
       __syncwarp();
@@ -201,11 +201,11 @@ static bool cluster_fits(const void *kern, int nblk, int threads, size_t smem) {
 }
 
 // One cluster over the whole mesh, T cells per block; *done = 0 when it does not fit.
-template <int Q, typename R, bool PLANE, int T>
+template <int Q, typename R, bool PLANE, bool EXT, int T>
 cudaError_t launch_cluster_t(const vlb_sim *sim, int32_t first, int32_t n, int64_t *done, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
   const size_t smem = SmallRecords<Q, R, PLANE>::bytes(T, m->md.n[m->md.dim - 1]);
-  auto kern = k_steps_small<Q, R, PLANE, T, 1, true>;
+  auto kern = k_steps_small<Q, R, PLANE, EXT, T, 1, true>;
   const int64_t nblk = (m->ncell + T - 1) / T;
   if (nblk > kClusterMax || !cluster_fits(reinterpret_cast<const void *>(kern), (int)nblk, T, smem)) return cudaSuccess;
   StepArgs a = make_step_args<Q>(sim, T);
@@ -227,7 +227,7 @@ cudaError_t launch_cluster_t(const vlb_sim *sim, int32_t first, int32_t n, int64
 
 // Advances the simulation by up to `nsteps` steps in one launch if its cells fit on the
 // device at once; *done is the number of steps launched (0: take the step kernel).
-template <int Q, typename R, bool PLANE>
+template <int Q, typename R, bool PLANE, bool EXT>
 cudaError_t launch_small_t(const vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s) {
   constexpr int T = small_threads<R>();
   constexpr int MINB = sizeof(R) == 8 ? 8 : Q == 9 ? 4 : 3;
@@ -239,13 +239,13 @@ cudaError_t launch_small_t(const vlb_sim *sim, int64_t nsteps, int64_t *done, cu
     // 1.29 us a step, against 2.43 with the counter in global memory; 4,096 cells 1.72)
     cudaError_t e = cudaSuccess;
     if (m->ncell <= kClusterMax * 128)
-      e = launch_cluster_t<Q, R, PLANE, 128>(sim, first, n, done, s);
+      e = launch_cluster_t<Q, R, PLANE, EXT, 128>(sim, first, n, done, s);
     else if (m->ncell <= kClusterMax * 256)
-      e = launch_cluster_t<Q, R, PLANE, 256>(sim, first, n, done, s);
+      e = launch_cluster_t<Q, R, PLANE, EXT, 256>(sim, first, n, done, s);
     if (e != cudaSuccess || *done > 0) return e;
   }
   const size_t smem = SmallRecords<Q, R, PLANE>::bytes(T, m->md.n[m->md.dim - 1]);
-  auto kern = k_steps_small<Q, R, PLANE, T, MINB, false>;
+  auto kern = k_steps_small<Q, R, PLANE, EXT, T, MINB, false>;
   const int64_t nblk = (m->ncell + T - 1) / T;
   if (smem > 96 * 1024 || nblk > resident_blocks(reinterpret_cast<const void *>(kern), smem, T)) return cudaSuccess;
   StepArgs a = make_step_args<Q>(sim, T);

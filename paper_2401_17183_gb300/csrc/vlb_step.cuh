@@ -78,6 +78,7 @@ struct StepArgs {
   // plane records, linear tiles: records staged per tile at most (0: tiles
   // along the fastest axis)
   int32_t nrec;
+  int32_t ext;   // plane records of an extruded mesh
 };
 
 constexpr int kStepThreads = 128;
@@ -218,8 +219,9 @@ __device__ __forceinline__ __nv_bfloat16 s16_from_bits<__nv_bfloat16>(unsigned s
 // the fastest axis, so that rows that are not whole tiles leave no idle threads; a tile then
 // meets several columns, and each thread reads its own column's record. (Records per
 // cell are always taken so.)
+// EXT (PLANE): extruded mesh (see collide_f32).
 template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT,
-          int T = kStepThreads, bool TAB = true, bool LIN = false>
+          int T = kStepThreads, bool TAB = true, bool LIN = false, bool EXT = false>
 __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, const int64_t t1) {
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H;
   static_assert(Q <= 19, "the slot-offset table holds 19 directions");
@@ -482,7 +484,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       R Np[Q];
       CollideState<Q, R> cst;
       // (with one record per cell the rest state is formed, not read)
-      collide_cell<Q, R, true, REFOFS, PLANE, RC>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
+      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
                                      arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
       if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
 
@@ -553,13 +555,13 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
 
 // One mesh: block b walks the tiles [b per_block, (b + 1) per_block).
 template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT,
-          int T = kStepThreads, bool LIN = false>
+          int T = kStepThreads, bool LIN = false, bool EXT = false>
 __global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE>() * (kStepThreads / T))
     k_step(const __grid_constant__ StepArgs a) {
   const int64_t t0 = (int64_t)blockIdx.x * a.per_block;
   const int64_t t1 = t0 + a.per_block < a.ntiles ? t0 + a.per_block : a.ntiles;
   if (t0 >= t1) return;
-  step_tiles<Q, S, R, ODD, PLANE, REFOFS, HPAR, IT, T, true, LIN>(a, t0, t1);
+  step_tiles<Q, S, R, ODD, PLANE, REFOFS, HPAR, IT, T, true, LIN, EXT>(a, t0, t1);
 }
 
 // Many meshes in one launch: block b takes the run of tiles items[b] of mesh
@@ -577,7 +579,14 @@ __global__ void __launch_bounds__(T, MINB)
     k_step_batch(const StepArgs *__restrict__ args, const BatchItem *__restrict__ items) {
   const BatchItem it = items[blockIdx.x];
   // the arguments sit in global memory here: slot offsets are formed, not read
-  step_tiles<Q, S, R, ODD, PLANE, false, false, IT, T, false>(args[it.sim], it.t0, it.t1);
+  const StepArgs &a = args[it.sim];
+  if constexpr (Q == 19 && PLANE) {
+    if (a.ext) {   // as the member's own steps
+      step_tiles<Q, S, R, ODD, PLANE, false, false, IT, T, false, false, true>(a, it.t0, it.t1);
+      return;
+    }
+  }
+  step_tiles<Q, S, R, ODD, PLANE, false, false, IT, T, false>(a, it.t0, it.t1);
 }
 
 // Arguments of one simulation's step kernel for tiles of T cells (per_block
@@ -609,6 +618,7 @@ inline StepArgs make_step_args(const vlb_sim *sim, int T = kStepThreads, bool li
   const int dim = m->md.dim;
   const int64_t nfast = dim == 3 ? m->md.n[2] : m->md.n[1];
   a.per_block = 0;
+  a.ext = sim->plane && m->extruded ? 1 : 0;
   a.nrec = lin ? (int32_t)((T - 1) / nfast + 2) : 0;
   if (sim->plane && !lin) {
     a.ntf = (int32_t)((nfast + T - 1) / T);
@@ -676,17 +686,17 @@ cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
     const int64_t nblk = (a.ntiles + a.per_block - 1) / a.per_block;
     kern<<<(unsigned)nblk, (unsigned)threads, smem, s>>>(a);
   };
-  auto pick = [&](auto plane_tag, auto ref_tag, auto par_tag) {
+  auto pick_ext = [&](auto plane_tag, auto ref_tag, auto par_tag, auto ext_tag) {
     constexpr bool P = decltype(plane_tag)::value, RO = decltype(ref_tag)::value;
-    constexpr bool HP = decltype(par_tag)::value;
+    constexpr bool HP = decltype(par_tag)::value, E = decltype(ext_tag)::value;
     constexpr size_t smem = step_smem<Q, S, R, kStepThreads, P, RO>(1);
     if constexpr (P) {
       if (lin) {
         const size_t smem_l = step_smem<Q, S, R, kStepThreads, P, RO>(a.nrec);
         if (odd)
-          go(k_step<Q, S, R, true, P, RO, HP, int32_t, kStepThreads, true>, smem_l, kStepThreads);
+          go(k_step<Q, S, R, true, P, RO, HP, int32_t, kStepThreads, true, E>, smem_l, kStepThreads);
         else
-          go(k_step<Q, S, R, false, P, RO, HP, int32_t, kStepThreads, true>, smem_l, kStepThreads);
+          go(k_step<Q, S, R, false, P, RO, HP, int32_t, kStepThreads, true, E>, smem_l, kStepThreads);
         return;
       }
     }
@@ -702,18 +712,30 @@ cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
     }
     if (i32) {
       if (odd)
-        go(k_step<Q, S, R, true, P, RO, HP, int32_t>, smem, kStepThreads);
+        go(k_step<Q, S, R, true, P, RO, HP, int32_t, kStepThreads, false, E>, smem, kStepThreads);
       else
-        go(k_step<Q, S, R, false, P, RO, HP, int32_t>, smem, kStepThreads);
+        go(k_step<Q, S, R, false, P, RO, HP, int32_t, kStepThreads, false, E>, smem, kStepThreads);
     } else {
       if (odd)
-        go(k_step<Q, S, R, true, P, RO, HP, int64_t>, smem, kStepThreads);
+        go(k_step<Q, S, R, true, P, RO, HP, int64_t, kStepThreads, false, E>, smem, kStepThreads);
       else
-        go(k_step<Q, S, R, false, P, RO, HP, int64_t>, smem, kStepThreads);
+        go(k_step<Q, S, R, false, P, RO, HP, int64_t, kStepThreads, false, E>, smem, kStepThreads);
     }
   };
   const std::true_type yes;
   const std::false_type no;
+  // extruded meshes: every storage but 16 bits relative to the uniform reference, which
+  // meshes with plane records have little use for
+  auto pick = [&](auto plane_tag, auto ref_tag, auto par_tag) {
+    constexpr bool P = decltype(plane_tag)::value, RO = decltype(ref_tag)::value;
+    if constexpr (Q == 19 && P && (RO || sizeof(S) > 2)) {
+      if (a.ext) {
+        pick_ext(plane_tag, ref_tag, par_tag, yes);
+        return;
+      }
+    }
+    pick_ext(plane_tag, ref_tag, par_tag, no);
+  };
   if constexpr (sizeof(S) == 2) {
     // the half of a 16-bit value follows from the cell parity when both the
     // cell count and the fastest axis are even
