@@ -149,9 +149,13 @@ __host__ __device__ constexpr bool slow_move(int a) {
 // storage (168 registers, no spills; 4 blocks at 128 registers ran 0.4%
 // slower, 5 at 102 registers 18% slower), 4 for 16-bit storage in plane mode
 // (128 registers; 3% faster than 3 blocks on even steps, 0.3% faster over both
-// parities; a record per cell needs the registers for itself), 2 for FP64
-template <typename R, typename S = R, bool PLANE = true>
+// parities; a record per cell needs the registers for itself), 2 for FP64. Extruded meshes
+// need fewer registers: 16-bit storage 6 blocks (80 registers; 128^3, FP16: 4 blocks 61.3 us a
+// step, 5 blocks 61.4, 6 blocks 59.5); FP32 3 (four fit: 20.7 us a step at 75 x 67 x 101, cut
+// for 4 blocks 21.4, for 5 21.6)
+template <typename R, typename S = R, bool PLANE = true, bool EXT = false>
 constexpr int step_min_blocks() {
+  if (EXT && sizeof(S) == 2) return 6;
   return sizeof(R) == 4 ? (sizeof(S) == 2 && PLANE ? 4 : 3) : 2;
 }
 
@@ -556,7 +560,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
 // One mesh: block b walks the tiles [b per_block, (b + 1) per_block).
 template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT,
           int T = kStepThreads, bool LIN = false, bool EXT = false>
-__global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE>() * (kStepThreads / T))
+__global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE, EXT>() * (kStepThreads / T))
     k_step(const __grid_constant__ StepArgs a) {
   const int64_t t0 = (int64_t)blockIdx.x * a.per_block;
   const int64_t t1 = t0 + a.per_block < a.ntiles ? t0 + a.per_block : a.ntiles;
