@@ -18,7 +18,7 @@ SOURCES = ["vlb_api.cu", "vlb_geometry.cu", "vlb_step.cu", "vlb_step_f32.cu", "v
            "vlb_batch.cu",
            "vlb_moments.cu", "vlb_noalloc.cu", "vlb_nn.cu", "vlb_q39.cu",
            "vlb_small.cu"]
-HEADERS = ["vlb_internal.cuh", "vlb_collide.cuh", "vlb_addr.cuh", "vlb_step.cuh", "vlb_q39.cuh",
+HEADERS = ["vlb_chain.cuh", "vlb_internal.cuh", "vlb_collide.cuh", "vlb_addr.cuh", "vlb_step.cuh", "vlb_q39.cuh",
            "vlb_nn_tc.cuh", "vlb_small.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/vlb.h"
+#include "vlb_chain.cuh"
 
 namespace vlb {
 

@@ -232,6 +232,7 @@ struct Pair<__nv_bfloat16> {
 // -> 6 us for 16 MB written at width 64, 32 x 64, batch 32). Grid (C, B).
 template <typename T>
 __global__ void k_pool(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int H, int W) {
+  vlb::chain_begin();
   const int Ho = H / 2, Wo = W / 2, c = blockIdx.x, b = blockIdx.y;
   const T *p = in + (int64_t)b * ibs + (int64_t)c * H * W;
   T *o = out + (int64_t)b * obs + (int64_t)c * Ho * Wo;
@@ -259,6 +260,7 @@ __global__ void k_pool_bwd(const float *__restrict__ gout, int64_t gobs, float *
 // values per store. Grid (C, B).
 template <typename T>
 __global__ void k_up(const T *__restrict__ in, int64_t ibs, T *__restrict__ out, int64_t obs, int h, int w) {
+  vlb::chain_begin();
   const int c = blockIdx.x, b = blockIdx.y;
   const T *p = in + (int64_t)b * ibs + (int64_t)c * h * w;
   typename Pair<T>::V *o = reinterpret_cast<typename Pair<T>::V *>(out + (int64_t)b * obs + (int64_t)c * 4 * h * w);
@@ -278,6 +280,7 @@ template <typename T, typename TW, int NCO>
 __global__ void __launch_bounds__(128) k_head(const T *__restrict__ in, int64_t ibs, const TW *__restrict__ w,
                                               const float *__restrict__ bias, float *__restrict__ out, int64_t obs,
                                               int C, int Co, int HW) {
+  vlb::chain_begin();
   const int b = blockIdx.y, o0 = blockIdx.z * NCO, p = (blockIdx.x * 128 + threadIdx.x) * 2;
   if (p >= HW) return;
   const T *ib = in + (int64_t)b * ibs + p;
@@ -325,6 +328,7 @@ __global__ void k_convert(const float *__restrict__ in, TO *__restrict__ out, in
 template <typename TO>
 __global__ void k_convert_into(const float *__restrict__ src, int64_t sbs, TO *__restrict__ dst, int64_t dbs,
                                int64_t CHW, int B) {
+  vlb::chain_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= CHW * B) return;
   const int64_t b = i / CHW, r = i % CHW;
@@ -457,6 +461,13 @@ inline int pick_nb(const vlb_nn *n, int co, int64_t tiles, int most) {
   return nb;
 }
 
+// A launch chained to the kernel before it (every kernel launched so begins with
+// chain_begin): one pass is 17 launches, its gradients another 45, of 5 to 30 us each.
+template <typename... P, typename... A>
+cudaError_t chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A &&...args) {
+  return vlb::launch_chained(kern, grid, block, smem, (cudaStream_t)0, std::forward<A>(args)...);
+}
+
 template <int NB, bool RELU, bool EVENW>
 cudaError_t launch_conv_mma(const vlb_nn *n, const NNLayer &l, const nn::bf16 *in, int64_t ibs, const nn::bf16 *wp,
                             const float *bias, nn::bf16 *out, int64_t obs, int B) {
@@ -465,7 +476,7 @@ cudaError_t launch_conv_mma(const vlb_nn *n, const NNLayer &l, const nn::bf16 *i
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((int64_t)l.h * l.w / nn::kTcM), (unsigned)(l.cout / NB), (unsigned)B);
-  kern<<<grid, 128, smem>>>(in, ibs, l.cin, wp, l.cout, bias, out, obs, l.h, l.w, n->d_err);
+  chain(kern, grid, dim3(128), smem, in, ibs, l.cin, wp, l.cout, bias, out, obs, l.h, l.w, n->d_err);
   return cudaGetLastError();
 }
 template <bool RELU>
@@ -494,7 +505,8 @@ cudaError_t launch_dgrad(const vlb_nn *n, const NNLayer &l, int64_t plane, int64
   auto kern = nn::k_dgrad_mma<NB>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, nst * stage);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((unsigned)tiles, (unsigned)(l.cin / NB)), 192, nst * stage>>>(n->planes, plane, npos, l.cout, wp, l.cin,
+  chain(kern, dim3((unsigned)tiles, (unsigned)(l.cin / NB)), dim3(192), nst * stage, n->planes, plane, npos, l.cout,
+        wp, l.cin,
                                                                             out, obs, l.h, l.w, B, nst, n->d_err);
   return cudaGetLastError();
 }
@@ -507,7 +519,7 @@ cudaError_t launch_wgrad_t(const NNLayer &l, const nn::bf16 *in, int64_t ibs, co
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)(l.cout / CB * ngrp), (unsigned)nsplit);
-  kern<<<grid, 256, smem>>>(in, ibs, l.cin, g, npos, plane, l.cout, dwp, l.h, l.w, B, ngrp, err);
+  chain(kern, grid, dim3(256), smem, in, ibs, l.cin, g, npos, plane, l.cout, dwp, l.h, l.w, B, ngrp, err);
   return cudaGetLastError();
 }
 template <int CB>
@@ -554,10 +566,12 @@ int conv(const vlb_nn *n, const NNLayer &l, const T *in, int64_t ibs, const void
     const int HW = l.h * l.w;
     const dim3 hg((unsigned)((HW + 255) / 256), (unsigned)B, (unsigned)((l.cout + NCO - 1) / NCO));
     if (bf)
-      nn::k_head<T, __nv_bfloat16, NCO><<<hg, 128>>>(in, ibs, (const __nv_bfloat16 *)w, bias, (float *)out, obs, l.cin,
+      chain(nn::k_head<T, __nv_bfloat16, NCO>, hg, dim3(128), 0, in, ibs, (const __nv_bfloat16 *)w, bias,
+            (float *)out, obs, l.cin,
                                                     l.cout, HW);
     else
-      nn::k_head<T, float, NCO><<<hg, 128>>>(in, ibs, (const float *)w, bias, (float *)out, obs, l.cin, l.cout, HW);
+      chain(nn::k_head<T, float, NCO>, hg, dim3(128), 0, in, ibs, (const float *)w, bias, (float *)out, obs, l.cin,
+            l.cout, HW);
   }
   NN_CU(cudaGetLastError());
   return VLB_OK;
@@ -640,24 +654,28 @@ int forward_t(vlb_nn *n, const float *d_x, float *d_y, int B) {
   const auto &L = n->L;
   // input in the storage type
   const int64_t chw = (int64_t)n->ci * H * W;
-  nn::k_convert_into<T><<<nn::nblk(chw * B), 256>>>(d_x, chw, A + n->x_in.off, n->x_in.bs, chw, B);
+  chain(nn::k_convert_into<T>, dim3(nn::nblk(chw * B)), dim3(256), 0, d_x, chw, A + n->x_in.off, n->x_in.bs, chw, B);
   NN_CU(cudaGetLastError());
   NN_TRY(conv<T>(n, L[0], A + n->x_in.off, n->x_in.bs, wp(L[0]), n->p + L[0].boff, A + n->e1.off, n->e1.bs, true, B));
   NN_TRY(conv<T>(n, L[1], A + n->e1.off, n->e1.bs, wp(L[1]), n->p + L[1].boff, A + n->s1.off, n->s1.bs, true, B));
-  nn::k_pool<T><<<dim3((unsigned)w, (unsigned)B), 256>>>(A + n->s1.off, n->s1.bs, A + n->p1.off, n->p1.bs, H, W);
+  chain(nn::k_pool<T>, dim3((unsigned)w, (unsigned)B), dim3(256), 0, A + n->s1.off, n->s1.bs, A + n->p1.off,
+        n->p1.bs, H, W);
   NN_CU(cudaGetLastError());
   NN_TRY(conv<T>(n, L[2], A + n->p1.off, n->p1.bs, wp(L[2]), n->p + L[2].boff, A + n->e2.off, n->e2.bs, true, B));
   NN_TRY(conv<T>(n, L[3], A + n->e2.off, n->e2.bs, wp(L[3]), n->p + L[3].boff, A + n->s2.off, n->s2.bs, true, B));
-  nn::k_pool<T><<<dim3((unsigned)(2 * w), (unsigned)B), 128>>>(A + n->s2.off, n->s2.bs, A + n->p2.off, n->p2.bs, H2, W2);
+  chain(nn::k_pool<T>, dim3((unsigned)(2 * w), (unsigned)B), dim3(128), 0, A + n->s2.off, n->s2.bs, A + n->p2.off,
+        n->p2.bs, H2, W2);
   NN_CU(cudaGetLastError());
   NN_TRY(conv<T>(n, L[4], A + n->p2.off, n->p2.bs, wp(L[4]), n->p + L[4].boff, A + n->e3.off, n->e3.bs, true, B));
   NN_TRY(conv<T>(n, L[5], A + n->e3.off, n->e3.bs, wp(L[5]), n->p + L[5].boff, A + n->b3.off, n->b3.bs, true, B));
   // c2 = [up(b3), s2]: s2 already sits in its slice
-  nn::k_up<T><<<dim3((unsigned)(4 * w), (unsigned)B), 128>>>(A + n->b3.off, n->b3.bs, A + n->c2.off, n->c2.bs, H4, W4);
+  chain(nn::k_up<T>, dim3((unsigned)(4 * w), (unsigned)B), dim3(128), 0, A + n->b3.off, n->b3.bs, A + n->c2.off,
+        n->c2.bs, H4, W4);
   NN_CU(cudaGetLastError());
   NN_TRY(conv<T>(n, L[6], A + n->c2.off, n->c2.bs, wp(L[6]), n->p + L[6].boff, A + n->d2.off, n->d2.bs, true, B));
   NN_TRY(conv<T>(n, L[7], A + n->d2.off, n->d2.bs, wp(L[7]), n->p + L[7].boff, A + n->t2.off, n->t2.bs, true, B));
-  nn::k_up<T><<<dim3((unsigned)(2 * w), (unsigned)B), 256>>>(A + n->t2.off, n->t2.bs, A + n->c1.off, n->c1.bs, H2, W2);
+  chain(nn::k_up<T>, dim3((unsigned)(2 * w), (unsigned)B), dim3(256), 0, A + n->t2.off, n->t2.bs, A + n->c1.off,
+        n->c1.bs, H2, W2);
   NN_CU(cudaGetLastError());
   NN_TRY(conv<T>(n, L[8], A + n->c1.off, n->c1.bs, wp(L[8]), n->p + L[8].boff, A + n->d1.off, n->d1.bs, true, B));
   NN_TRY(conv<T>(n, L[9], A + n->d1.off, n->d1.bs, wp(L[9]), n->p + L[9].boff, A + n->t1.off, n->t1.bs, true, B));
@@ -700,7 +718,8 @@ int layer_backward(vlb_nn *n, int li, View in, View out, const GradSrc &src, con
         const dim3 grid((unsigned)blocks, (unsigned)(l.cout / 8));
         const T *act = A + out.off;
         auto launch = [&](auto kern) {
-          kern<<<grid, 128>>>(G + src.g.off, src.g.bs, G + src.gp.off, src.gp.bs, act, out.bs, n->planes, plane,
+          chain(kern, grid, dim3(128), 0, G + src.g.off, src.g.bs, G + src.gp.off, src.gp.bs, act, out.bs, n->planes,
+                plane,
                               (int)npos, n->bsum, l.h, l.w, B);
         };
         if (src.mode == 0)
@@ -726,7 +745,8 @@ int layer_backward(vlb_nn *n, int li, View in, View out, const GradSrc &src, con
         case 64: NN_CU(launch_wgrad<64>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
         default: NN_CU(launch_wgrad<128>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
       }
-      nn::k_sum_parts<<<nn::nblk(nw + l.cout), 256>>>(n->dwp, ns * nn::wg_groups(cb), nw, n->bsum, blocks, l.cout,
+      chain(nn::k_sum_parts, dim3(nn::nblk(nw + l.cout)), dim3(256), 0, n->dwp, ns * nn::wg_groups(cb), nw, n->bsum,
+            blocks, l.cout,
                                                       n->g + l.woff);
       NN_CU(cudaGetLastError());
       if (gin) {
@@ -760,7 +780,7 @@ template <int NCO>
 void launch_head_bwd(vlb_nn *n, const float *d_dy, int64_t ybs, int B) {
   const NNLayer &l = n->L[10];
   const int64_t npos = nn::Padded{l.h, l.w, B}.positions();
-  nn::k_head_bwd<NCO><<<dim3((unsigned)plane_blocks(n, l.cin, npos), (unsigned)(l.cin / 8)), 128>>>(
+  chain(nn::k_head_bwd<NCO>, dim3((unsigned)plane_blocks(n, l.cin, npos), (unsigned)(l.cin / 8)), dim3(128), 0, 
       d_dy, ybs, (const __nv_bfloat16 *)n->pc + l.woff, (const __nv_bfloat16 *)n->act + n->t1.off, n->t1.bs, n->planes,
       npos * l.cin, (int)npos, n->bsum, n->hp, l.h, l.w, B);
 }
@@ -782,7 +802,8 @@ int backward_t(vlb_nn *n, const float *d_dy, int B) {
     }
     NN_CU(cudaGetLastError());
     const int64_t nw = (int64_t)n->co * L[10].cin + n->co;
-    nn::k_sum_parts<<<nn::nblk(nw), 256>>>(n->hp, plane_blocks(n, L[10].cin, nn::Padded{n->H, n->W, B}.positions()), nw,
+    chain(nn::k_sum_parts, dim3(nn::nblk(nw)), dim3(256), 0, n->hp, plane_blocks(n, L[10].cin, nn::Padded{n->H, n->W,
+          B}.positions()), nw,
                                            nullptr, 0, 0, n->g + L[10].woff);
     NN_CU(cudaGetLastError());
   } else {

@@ -21,6 +21,8 @@
 
 #include <type_traits>
 
+#include "vlb_chain.cuh"
+
 namespace nn {
 
 using bf16 = __nv_bfloat16;
@@ -165,6 +167,7 @@ template <int NB, bool RELU, bool EVENW>
 __global__ void __launch_bounds__(128) k_conv3_mma(const bf16 *__restrict__ in, int64_t ibs, int C,
                                                    const bf16 *__restrict__ wp, int Co, const float *__restrict__ bias,
                                                    bf16 *__restrict__ out, int64_t obs, int H, int W, int *err) {
+  vlb::chain_begin();
   static_assert(NB % 16 == 0 && NB >= 16 && NB <= 256, "MMA N for M = 128");
   constexpr int TCOLS = NB <= 32 ? 32 : NB <= 64 ? 64 : NB <= 128 ? 128 : 256;
   constexpr int BBytes = kTcKG * NB * 16;
@@ -336,6 +339,7 @@ template <int NB>
 __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g, int64_t plane, int64_t npos, int C,
                                                       const bf16 *__restrict__ wp, int rows, float *__restrict__ out,
                                                       int64_t obs, int H, int W, int B, int nstage, int *err) {
+  vlb::chain_begin();
   static_assert(NB % 16 == 0 && NB <= 64, "three accumulators in 256 tensor-memory columns");
   constexpr int TCOLS = dg_cols(NB);
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -504,6 +508,7 @@ __global__ void __launch_bounds__(256, 1) k_wgrad_mma(const bf16 *__restrict__ i
                                                       const bf16 *__restrict__ g, int64_t npos, int64_t gplane, int Co,
                                                       float *__restrict__ dwp, int H, int W, int B, int ngrp,
                                                       int *err) {
+  vlb::chain_begin();
   constexpr int NSET = wg_sets(CB), NG = wg_groups(CB), COLS = NBK * 72;
   constexpr int stage = NSET * kWgA + NBK * kWgB;
   constexpr int units = NBK * 128, UPT = (units + 255) / 256;
@@ -743,6 +748,7 @@ __global__ void __launch_bounds__(128) k_mask_split(const float *__restrict__ g,
                                                     const bf16 *__restrict__ act, int64_t abs_,
                                                     bf16 *__restrict__ planes, int64_t plane, int npos,
                                                     float *__restrict__ bsum, int H, int W, int B) {
+  vlb::chain_begin();
   const int c0 = blockIdx.y * 8, C = gridDim.y * 8, HW = H * W;
   float s[8];
 #pragma unroll
@@ -787,6 +793,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(const float *__restrict__ dy, 
                                                   const bf16 *__restrict__ act, int64_t abs_, bf16 *__restrict__ planes,
                                                   int64_t plane, int npos, float *__restrict__ bsum,
                                                   float *__restrict__ hp, int H, int W, int B) {
+  vlb::chain_begin();
   const int c0 = blockIdx.y * 8, C = gridDim.y * 8, HW = H * W;
   float wv[NCO][8], sums[9 * NCO + 8];   // dw [NCO][8], db [NCO], masked gradient [8]
 #pragma unroll
@@ -843,6 +850,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(const float *__restrict__ dy, 
 // lie one after the other. Fixed order.
 __global__ void k_sum_parts(const float *__restrict__ src, int nsplit, int64_t n, const float *__restrict__ bsum,
                             int nsamp, int nbias, float *__restrict__ dst) {
+  vlb::chain_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n + nbias) return;
   const float *q = i < n ? src + i : bsum + (i - n);
