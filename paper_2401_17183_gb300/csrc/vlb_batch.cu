@@ -7,6 +7,7 @@
 // by timing (vlb_batch_tune). The per-cell work is that of vlb_step, so a
 // batch reproduces the members' individual steps bit for bit. Whole runs of
 // 32 steps replay a CUDA graph of 32 kernel nodes (alternating A-A parity).
+#include <algorithm>
 #include <new>
 
 #include "vlb_step.cuh"
@@ -107,8 +108,10 @@ int64_t total_tiles(const vlb_batch *b) {
 // blocks the batch kernel keeps resident on the device
 int64_t batch_resident(const vlb_batch *b) {
   const BatchKind k = kind_of(b);
-  return resident_blocks(reinterpret_cast<const void *>(batch_kernel(k, false, b->shape)),
-                         batch_smem(k, b->shape), batch_threads(b));
+  const size_t smem = batch_smem(k, b->shape);
+  // (both parities: asking also lifts a kernel's shared-memory limit)
+  return std::min(resident_blocks(reinterpret_cast<const void *>(batch_kernel(k, false, b->shape)), smem, batch_threads(b)),
+                  resident_blocks(reinterpret_cast<const void *>(batch_kernel(k, true, b->shape)), smem, batch_threads(b)));
 }
 
 // switch to block shape `shape`: the members' kernel arguments (their tile
