@@ -1088,7 +1088,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
 // deviations are formed at the converged Phi.
 // rc is the cell's coefficient record (PtrRecord or CellRecord); itau = 1/tau. With REST, d holds e_a = N_a - o_a relative to the
 // cell's own rest state (16-bit storage, see CoefLayout), and so does dp.
-template <int Q, typename R, bool FINAL, bool REST, bool RREC, bool EXT, typename RC>
+template <int Q, typename R, bool FINAL, bool REST, bool RREC, bool EXT, bool FR0, typename RC>
 __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nref,
                                              R itau, R tol, int max_iter, R (&dp)[Q],
                                              CollideState<Q, R> &st) {
@@ -1224,10 +1224,12 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   // Start at Pt = H Pc, the fixed point without the polynomial part: it is off by that
   // part, of the order of curvature times U^2 (the rest state's force, the start
   // when only a few evaluations are allowed, by curvature times U), so that one
-  // evaluation less reaches the same residual.
+  // evaluation less reaches the same residual. FR0 starts there in any case: 16-bit storage
+  // relative to the uniform reference rounds large values, so that its rounding noise is
+  // 1 to 30% of the velocity, and another rounding in FP32 another noise of that size.
   R Phi[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) Phi[i] = max_iter >= 4 || i >= DI ? Pt[i] : m * rc[L::FR + i];
+  for (int i = 0; i < D; i++) Phi[i] = (max_iter >= 4 && !FR0) || i >= DI ? Pt[i] : m * rc[L::FR + i];
   st.conv = false;
   int it = 0;
   while (it < max_iter) {
@@ -1310,14 +1312,14 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
 
 // the local collision in the arithmetic type R
 template <int Q, typename R, bool FINAL, bool REST = false, bool RREC = true, typename RC = PtrRecord<R>,
-          bool EXT = false>
+          bool EXT = false, bool FR0 = false>
 __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nref, R itau, R tol, int max_iter,
                                              R (&dp)[Q], CollideState<Q, R> &st) {
   if constexpr (sizeof(R) == 8) {
     static_assert(!REST, "FP64 populations are stored relative to the uniform reference");
     collide_f64<Q, FINAL, EXT, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   } else {
-    collide_f32<Q, R, FINAL, REST, RREC, EXT, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+    collide_f32<Q, R, FINAL, REST, RREC, EXT, FR0, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   }
 }
 
