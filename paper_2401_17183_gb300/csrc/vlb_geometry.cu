@@ -757,7 +757,7 @@ __global__ void k_init_f32(const double *J, const double *gu, const double *ginv
 //   N_a - o_a = J w_a [(rho - 1)(1 + x^0_a) + rho (x_a - x^0_a)] + (J w_a (1 + x^0_a) - o_a).
 // The rest state and its rounding are formed in FP64 once per pair (60 operations), the
 // flow's part, x - x^0 from U U and the odd part, in FP32. Forming every population
-// and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells; INIT_REST
+// and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells; 0.48 so
 template <int Q, typename S>
 __global__ void __launch_bounds__(128) k_init_rest(const double *J, const double *gu, const double *ginv,
                                                    const double *rho, const double *u, int64_t ncell, int64_t nfast,

@@ -19,7 +19,10 @@
 // populations of its cell in tile k + 2 into shared memory with asynchronous
 // copies while it collides its cell in tile k (three stages); on even steps of
 // full tiles, where every direction reads the tile's own row segment, the
-// block copies the Q segments in 16-byte pieces instead. The DRAM latency
+// block copies the Q segments in 16-byte pieces instead; on odd steps (FP32 and 16 bits, no
+// walls on the fastest axis) it copies the segments of the neighbouring rows so, with one
+// more piece where the direction moves along the row, and the threads read them one value
+// to the side. The DRAM latency
 // of the reads is thereby hidden behind the arithmetic of a tile without
 // holding the loads in registers. In plane mode the tile's shared coefficient
 // record travels in the same copy group, in 16-byte pieces; one block barrier
@@ -174,7 +177,9 @@ template <int Q, typename S, typename R, int T = kStepThreads>
 struct StepSmem {
   static constexpr bool H16 = sizeof(S) == 2;
   using PopT = typename std::conditional<H16, uint32_t, S>::type;
-  alignas(16) PopT pop[kStages][Q][T];
+  // (on odd steps of whole rows, a direction's segment has a 16-byte piece on either side)
+  static constexpr int W = H16 ? T : T + 32 / (int)sizeof(S);
+  alignas(16) PopT pop[kStages][Q][W];
   alignas(16) uint32_t half_hi[H16 ? kStages : 1][T];
 };
 // The plane records follow: per stage, those of the columns that a tile meets, each the
@@ -262,8 +267,14 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
     return !ODD && a.full_tiles && (ROWS || (IT)c.tf * T + T <= nfast);
   };
 
-  // pieces of 16 bytes in one direction's row segment of a tile
-  constexpr int PER_ROW = T * (int)sizeof(S) / 16;
+  // pieces of 16 bytes in one direction's row segment of a tile, values in a piece
+  constexpr int PER_ROW = T * (int)sizeof(S) / 16, PIECE = 16 / (int)sizeof(S);
+  // does the block copy the neighbouring rows' segments on odd steps? (uniform; PER_ROW
+  // lanes of a warp copy a direction.) A 4-byte copy per thread and direction kept the
+  // shared-memory queue full: D3Q19 256^3, FP32 485 -> 448 us a step over both parities;
+  // 128^3, FP16 57.5 -> 55.5. FP64 steps are bound by their arithmetic and keep it.
+  constexpr bool ODDROWS = ODD && ROWS && T == 128 && sizeof(S) <= 4;
+  const bool odd_rows = ODDROWS && a.full_tiles && !a.g.wall[D - 1];
 
   // offset of slot k in elements (soff) and in 32-bit words of 16-bit
   // storage (soffw)
@@ -311,7 +322,55 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
         }
       }
     }
-    if (!rows && ifast < nfast) {
+    if constexpr (ODDROWS) {
+      if (odd_rows) {
+        const IT f0 = (IT)c.tf * T;
+        const Addr<Q, IT> ad = tile_addr<Q, IT>(a.g, c, f0);
+        // the pieces before and behind the segment (periodic wrap)
+        const IT pre = f0 == 0 ? nfast - PIECE : (IT)-PIECE, post = f0 + T == nfast ? T - nfast : (IT)T;
+        // where direction av's segment begins: slot abar of the row of q - c_a, or the own
+        // row's slot a when a slow axis' wall sends it back
+        auto segment = [&](int av) -> IT {
+          if (av == 0 || ad.crosses(av, -1)) return soff(av) + ad.cell;
+          IT r = soff(lat_opp<Q>(av)) + ad.cell;
+#pragma unroll
+          for (int d = 0; d < D - 1; d++) {
+            if (Lat<Q>::c(av, d) > 0) r += ad.dm[d];
+            if (Lat<Q>::c(av, d) < 0) r += ad.dp[d];
+          }
+          return r;
+        };
+        const int lane = tid & 31;
+        // warp W copies directions W, W + 4, ...
+        auto copy = [&](auto wt) {
+          constexpr int W = decltype(wt)::value, PAIR = 32 / PER_ROW;   // directions at once
+          const int half = PAIR == 2 ? lane >> 4 : 0, j = PAIR == 2 ? lane & 15 : lane;
+#pragma unroll
+          for (int av = W; av < Q; av += 4 * PAIR) {
+            const int av2 = av + 4 < Q ? av + 4 : av;
+            const IT s1 = segment(av), s2 = PAIR == 2 ? segment(av2) : s1;
+            unsigned char *const d1 = reinterpret_cast<unsigned char *>(&sm.pop[st][av][0]);
+            unsigned char *const d2 = reinterpret_cast<unsigned char *>(&sm.pop[st][av2][0]);
+            if (PAIR == 1 || half == 0 || av + 4 < Q)
+              cp_async<16>((half ? d2 : d1) + 16 + 16 * j, f + (half ? s2 : s1) + PIECE * j);
+            auto edge = [&](int e, IT seg, unsigned char *dst) {
+              const int cz = Lat<Q>::c(e, D - 1);
+              if (cz > 0) cp_async<16>(dst, f + seg + pre);
+              if (cz < 0) cp_async<16>(dst + 16 + T * sizeof(S), f + seg + post);
+            };
+            if (lane == 0) edge(av, s1, d1);
+            if (PAIR == 2 && av + 4 < Q && lane == 16) edge(av2, s2, d2);
+          }
+        };
+        switch (tid >> 5) {
+          case 0: copy(std::integral_constant<int, 0>()); break;
+          case 1: copy(std::integral_constant<int, 1>()); break;
+          case 2: copy(std::integral_constant<int, 2>()); break;
+          default: copy(std::integral_constant<int, 3>());
+        }
+      }
+    }
+    if (!rows && !odd_rows && ifast < nfast) {
       const Addr<Q, IT> ad = cell_addr(c, ifast);
       if constexpr (H16 && HPAR) {
         // the same neighbour arithmetic on 32-bit words: the slow-axis moves
@@ -427,7 +486,26 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       }
 
       R N[Q];
-      if constexpr (H16) {
+      // odd steps of whole rows: the value one to the side the population comes from
+      auto take_rows = [&](auto inner_tag) {
+        [[maybe_unused]] constexpr bool INNER = decltype(inner_tag)::value;
+#pragma unroll
+        for (int av = 0; av < Q; av++) {
+          const bool moved = INNER || !ad.crosses(av, -1);
+          const int k = PIECE + tid - (moved ? Lat<Q>::c(av, D - 1) : 0);
+          if constexpr (H16)
+            N[av] = load_s<R>(s16_from_bits<S>(reinterpret_cast<const unsigned short *>(&sm.pop[st][av][0])[k]));
+          else
+            N[av] = static_cast<R>(sm.pop[st][av][k]);
+        }
+      };
+      if (ODDROWS && odd_rows) {
+        // (a tile away from the slow axes' walls, uniform over the block)
+        if (ad.wall_cell())
+          take_rows(walls_no);
+        else
+          take_rows(walls_yes);
+      } else if constexpr (H16) {
         if (row_tile(cur)) {
           // the tile's row segments, 16 bits per cell
 #pragma unroll
@@ -464,6 +542,11 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
           else
             unpack(std::false_type());
         }
+      } else {
+#pragma unroll
+        for (int av = 0; av < Q; av++) N[av] = static_cast<R>(sm.pop[st][av][tid]);
+      }
+      if constexpr (H16) {
         if constexpr (REFOFS && ODD) {
           // relative to the own column's rest state: a population read from a
           // neighbouring column carries that column's storage reference. The
@@ -479,9 +562,6 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
               N[av] = cz == 0 ? N[av] + dv : fmar(dv, cz > 0 ? mlo : mhi, N[av]);
             }
         }
-      } else {
-#pragma unroll
-        for (int av = 0; av < Q; av++) N[av] = static_cast<R>(sm.pop[st][av][tid]);
       }
 
       // ---- collide (section 2.2)

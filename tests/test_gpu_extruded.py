@@ -90,3 +90,27 @@ def test_batch_of_extruded_and_other_members(V, prec):
         s.step(35)
         t.sync()
         assert np.array_equal(s.get_state(), t.get_state())
+
+
+@pytest.mark.parametrize("prec", ["VLB_F32", "VLB_F16", "VLB_BF16"])
+@pytest.mark.parametrize("kind", ["spacing", "sheared"])
+@pytest.mark.parametrize("n2,copies", [(64, 2), (96, 4)])
+def test_rows_of_whole_tiles_repeat_a_narrower_mesh(V, prec, kind, n2, copies):
+    """A flow that repeats along the fastest axis, on rows of whole tiles (the
+    block copies the neighbouring rows' segments on odd steps, with wrap-around
+    pieces at their ends and, in 16 bits, values one half-word to the side)
+    and on rows of one period (copied value by value): the same populations."""
+    precision = getattr(V, prec)
+    got = []
+    for k in (1, copies):
+        mesh = _mesh(11, 9, n2 * k, kind)
+        rho, u = W.noise_fields(_mesh(11, 9, n2, kind), amp=0.01, seed=5)
+        rho = np.tile(rho.reshape(99, n2), (1, k)).reshape(-1)
+        u = np.tile(u.reshape(99, n2, 3), (1, k, 1)).reshape(-1, 3)
+        g = V.Sim(V.Mesh(mesh), _params(True), rho, u, precision=precision,
+                  reference=V.VLB_REF_UNIFORM if prec == "VLB_F32" else V.VLB_REF_REST)
+        for _ in range(13):
+            g.step(1)
+        got.append(g.get_state().reshape(19, 99, k, n2))
+    for k in range(copies):
+        assert np.array_equal(got[1][:, :, k], got[0][:, :, 0])
