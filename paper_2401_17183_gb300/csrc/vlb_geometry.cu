@@ -755,19 +755,46 @@ __global__ void k_init_f32(const double *J, const double *gu, const double *ginv
 // location's column (plane mode): with J f^eq_a = J rho w_a (1 + x_a) and the reference
 // o_a = fl(J w_a (1 + x^0_a)) rounded to FP32 (rest_ref),
 //   N_a - o_a = J w_a [(rho - 1)(1 + x^0_a) + rho (x_a - x^0_a)] + (J w_a (1 + x^0_a) - o_a).
-// The rest state and its rounding are formed in FP64 once per pair (60 operations), the
-// flow's part, x - x^0 from U U and the odd part, in FP32. Forming every population
-// and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells; 0.48 so
+// The rest state and its rounding are formed in FP64 once per pair and column (60 operations;
+// by a thread each, into shared memory, for the columns that a block of 128 consecutive
+// cells meets), the flow's part, x - x^0 from U U and the odd part, in FP32. Forming every
+// population and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells, the rest
+// state once per pair and cell 0.48 (100 steps with reset and moments 7.6 ms, 7.2 so).
+constexpr int kInitThreads = 128;
 template <int Q, typename S>
-__global__ void __launch_bounds__(128) k_init_rest(const double *J, const double *gu, const double *ginv,
+__global__ void __launch_bounds__(kInitThreads) k_init_rest(const double *J, const double *gu, const double *ginv,
                                                    const double *rho, const double *u, int64_t ncell, int64_t nfast,
                                                    S *f) {
   constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // o_a rounded and its remainder, per column of the block
+  extern __shared__ float2 so[];
+  const int64_t b0 = (int64_t)blockIdx.x * kInitThreads, b1 = b0 + kInitThreads < ncell ? b0 + kInitThreads : ncell;
+  const int64_t r0 = b0 / nfast;
+  const int ncol = (int)((b1 - 1) / nfast - r0) + 1;
+  for (int k = threadIdx.x; k < ncol * (H + 1); k += kInitThreads) {
+    const int p = k % (H + 1);
+    const int64_t c0 = (r0 + k / (H + 1)) * nfast;
+    double tr = 0.0, cgc = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; i++)
+#pragma unroll
+      for (int j = 0; j < D; j++) {
+        const double g = ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0);
+        const int cc = Lat<Q>::c(p, i) * Lat<Q>::c(p, j);
+        if (i == j) tr += g;
+        if (cc > 0) cgc += g;
+        if (cc < 0) cgc -= g;
+      }
+    const double o = J[c0] * (lat_w<Q, double>(p) * (1.0 + 0.5 * (3.0 * cgc - tr)));
+    so[k] = make_float2((float)o, (float)(o - (double)(float)o));
+  }
+  __syncthreads();
+  const int64_t c = b0 + threadIdx.x;
   if (c >= ncell) return;
-  const int64_t c0 = ncell < ((int64_t)1 << 31) ? (int64_t)((uint32_t)c / (uint32_t)nfast) * nfast : c / nfast * nfast;
+  const int64_t row = ncell < ((int64_t)1 << 31) ? (int64_t)((uint32_t)c / (uint32_t)nfast) : c / nfast;
+  const int64_t c0 = row * nfast;
+  const float2 *const oc = so + (int)(row - r0) * (H + 1);
   float U[D], gd[NS], zero[D];
-  double g[NS], tr = 0.0;
 #pragma unroll
   for (int i = 0; i < D; i++) {
     float v = 0.0f;
@@ -779,11 +806,8 @@ __global__ void __launch_bounds__(128) k_init_rest(const double *J, const double
 #pragma unroll
   for (int i = 0; i < D; i++)
 #pragma unroll
-    for (int j = i; j < D; j++) {
-      g[sym<D>(i, j)] = ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0);
-      gd[sym<D>(i, j)] = (float)g[sym<D>(i, j)];
-      if (i == j) tr += g[sym<D>(i, j)];
-    }
+    for (int j = i; j < D; j++)
+      gd[sym<D>(i, j)] = (float)(ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0));
   EqParts<Q, float> e;
   eq_parts<Q, float>(gd, U, zero, e);
   // the even part without the rest state's: B = U U
@@ -795,21 +819,10 @@ __global__ void __launch_bounds__(128) k_init_rest(const double *J, const double
     for (int j = 0; j < D; j++) q.B[i][j] = U[i] * U[j];
     q.trB += q.B[i][i];
   }
-  const double Jc = J[c0];
-  const float r1 = (float)(rho[c] - 1.0), r = (float)rho[c], Jf = (float)Jc;
+  const float r1 = (float)(rho[c] - 1.0), r = (float)rho[c], Jf = (float)J[c0];
 #pragma unroll
   for (int p = 0; p <= H; p++) {
-    double cgc = 0.0;
-#pragma unroll
-    for (int k = 0; k < D; k++)
-#pragma unroll
-      for (int l = 0; l < D; l++) {
-        const int cc = Lat<Q>::c(p, k) * Lat<Q>::c(p, l);
-        if (cc > 0) cgc += g[sym<D>(k, l)];
-        if (cc < 0) cgc -= g[sym<D>(k, l)];
-      }
-    const double o = Jc * (lat_w<Q, double>(p) * (1.0 + 0.5 * (3.0 * cgc - tr)));
-    const float of = (float)o, lo = (float)(o - (double)of);
+    const float of = oc[p].x, lo = oc[p].y;
     const float jw = Jf * lat_w<Q, float>(p), xe = eq_even_x<Q>(q, p);
     if (p == 0) {
       f[c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe, lo)));
@@ -832,11 +845,14 @@ cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d
       // FP32 arithmetic
       if constexpr (sizeof(S) == 2) {
         if (ref.rest) {
+          static_assert(kInitThreads == 128, "blocks of k_init_rest");
+          // columns that a block meets at most: 129 of one cell each, 10 KB
+          const size_t smem = sizeof(float2) * (m->md.q / 2 + 1) * (size_t)((kInitThreads - 1) / ref.nfast + 2);
           if (m->md.q == 9)
-            k_init_rest<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
+            k_init_rest<9, S><<<(unsigned)blocks, threads, smem, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
                                                                    ref.nfast, (S *)sim->d_f);
           else
-            k_init_rest<19, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
+            k_init_rest<19, S><<<(unsigned)blocks, threads, smem, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
                                                                     ref.nfast, (S *)sim->d_f);
           return cudaGetLastError();
         }
