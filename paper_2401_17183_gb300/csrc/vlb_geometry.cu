@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(256) k_links(const MeshDev m, Grid g, int64_t 
       for (int d = 0; d < D; d++) de[d] += c[j] * (gp[j][d] - gl[(cell * D + j) * D + d]);
     }
     for (int i = 0; i < D; i++) {
-      double v = 0.0;
-      for (int d = 0; d < D; d++) v += de[d] * gu[(cell * D + i) * D + d];
-      Kv[i] = v;
+      // (one expression: how its products and sums are contracted shows in the last bit)
+      const double *r = gu + (cell * D + i) * D;
+      Kv[i] = de[0] * r[0] + de[1] * r[1] + de[2] * (D == 3 ? r[D - 1] : 0.0);
     }
   }
   for (int i = 0; i < D; i++) K_out[t * D + i] = Kv[i];

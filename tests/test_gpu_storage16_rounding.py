@@ -1,0 +1,66 @@
+"""Runs with 16-bit population storage, bit for bit. Every step rounds each
+population to 16 bits, and a last bit of the FP32 or FP64 arithmetic before it
+decides which way: another order of a sum gives another sequence of roundings,
+1e-4 to 1e-2 of the velocity away after a hundred steps, although neither is
+more exact. So the geometry's link sums, the initial state, the step and the
+moments of such runs are pinned by digests of their values."""
+import zlib
+
+import numpy as np
+import pytest
+
+from paper_2401_17183_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+MESHES = {
+    "even_rows": lambda: W.channel_mesh(16, 12, 8, stretch=0.7, bump=0.05),
+    "odd_rows": lambda: W.channel_mesh(9, 7, 37, stretch=0.5, bump=0.02),
+    "whole_tiles": lambda: W.channel_mesh(11, 9, 128, stretch=0.5, bump=0.02),
+    "general": lambda: W.channel_bump3d_mesh(12, 10, 16, stretch=0.7, bump=0.05),
+    "channel2d": lambda: W.channel2d_mesh(31, 40, stretch=0.5),
+}
+
+
+def _mesh(name):
+    """The mesh with its positions rounded to 2^-20, so that no host's sin or tanh shows."""
+    mesh = dict(MESHES[name]())
+    mesh["x"] = np.round(np.asarray(mesh["x"], dtype=np.float64) * 2.0 ** 20) / 2.0 ** 20
+    return mesh
+
+
+@pytest.fixture(scope="module")
+def V():
+    from paper_2401_17183_gb300 import build as B
+    B.build()
+    from paper_2401_17183_gb300 import vlb
+    vlb.load()
+    return vlb
+
+
+def _digest(*arrays):
+    crc = 0
+    for a in arrays:
+        crc = zlib.crc32(np.ascontiguousarray(a, dtype=np.float64).tobytes(), crc)
+    return "%08x" % crc
+
+
+def _run(V, mesh, prec, mode, ref):
+    """A simulation, and the same flow's initial state as the FP64 path gives it."""
+    force = (1e-5, -4e-6, 6e-6) if mesh["dim"] == 3 else (2e-6, 1e-5, 0)
+    rho, u = W.noise_fields(mesh, amp=0.01, seed=5)
+    vm, prm = V.Mesh(mesh), W.params(0.8, body_force=force)
+    s = V.Sim(vm, prm, rho, u, precision=getattr(V, "VLB_" + prec), coef_mode=getattr(V, "VLB_COEF_" + mode),
+              reference=getattr(V, "VLB_REF_" + ref))
+    return s, V.Sim(vm, prm, rho, u).get_state()
+
+
+LINK_SUMS = {
+    "channel2d": "5c538014", "even_rows": "a2332909", "general": "d1ec4710", "odd_rows": "4a8a0037",
+    "whole_tiles": "51a7261e",
+}
+
+
+@pytest.mark.parametrize("name", sorted(MESHES))
+def test_link_sums(V, name):
+    assert _digest(V.Mesh(_mesh(name)).geometry()["K"]) == LINK_SUMS[name]
