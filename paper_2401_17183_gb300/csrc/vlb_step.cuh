@@ -153,12 +153,10 @@ __host__ __device__ constexpr bool slow_move(int a) {
 // slower, 5 at 102 registers 18% slower), 4 for 16-bit storage in plane mode
 // (128 registers; 3% faster than 3 blocks on even steps, 0.3% faster over both
 // parities; a record per cell needs the registers for itself), 2 for FP64. Extruded meshes
-// need fewer registers: 16-bit storage 6 blocks (80 registers; 128^3, FP16: 4 blocks 61.3 us a
-// step, 5 blocks 61.4, 6 blocks 59.5); FP32 3 (four fit: 20.7 us a step at 75 x 67 x 101, cut
+// need fewer registers; FP32 stays at 3 (four fit: 20.7 us a step at 75 x 67 x 101, cut
 // for 4 blocks 21.4, for 5 21.6)
-template <typename R, typename S = R, bool PLANE = true, bool EXT = false>
+template <typename R, typename S = R, bool PLANE = true>
 constexpr int step_min_blocks() {
-  if (EXT && sizeof(S) == 2) return 6;
   return sizeof(R) == 4 ? (sizeof(S) == 2 && PLANE ? 4 : 3) : 2;
 }
 
@@ -568,7 +566,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       R Np[Q];
       CollideState<Q, R> cst;
       // (with one record per cell the rest state is formed, not read)
-      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16 && PLANE && !REFOFS>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
+      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16 && PLANE>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
                                      arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
       if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
 
@@ -640,7 +638,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
 // One mesh: block b walks the tiles [b per_block, (b + 1) per_block).
 template <int Q, typename S, typename R, bool ODD, bool PLANE, bool REFOFS, bool HPAR, typename IT,
           int T = kStepThreads, bool LIN = false, bool EXT = false>
-__global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE, EXT>() * (kStepThreads / T))
+__global__ void __launch_bounds__(T, step_min_blocks<R, S, PLANE>() * (kStepThreads / T))
     k_step(const __grid_constant__ StepArgs a) {
   // (D3Q19 507 K cells, FP32: 21.2 -> 18.8 us a step; 128^3, FP16: 59.5 -> 57.5)
   chain_begin();
@@ -811,11 +809,11 @@ cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
   };
   const std::true_type yes;
   const std::false_type no;
-  // extruded meshes: every storage but 16 bits relative to the uniform reference, which
-  // meshes with plane records have little use for
+  // extruded meshes: FP32 and FP64 storage (16-bit storage keeps the sums of the general form,
+  // see FR0 in collide_f32)
   auto pick = [&](auto plane_tag, auto ref_tag, auto par_tag) {
-    constexpr bool P = decltype(plane_tag)::value, RO = decltype(ref_tag)::value;
-    if constexpr (Q == 19 && P && (RO || sizeof(S) > 2)) {
+    constexpr bool P = decltype(plane_tag)::value;
+    if constexpr (Q == 19 && P && sizeof(S) > 2) {
       if (a.ext) {
         pick_ext(plane_tag, ref_tag, par_tag, yes);
         return;

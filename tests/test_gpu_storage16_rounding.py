@@ -64,3 +64,34 @@ LINK_SUMS = {
 @pytest.mark.parametrize("name", sorted(MESHES))
 def test_link_sums(V, name):
     assert _digest(V.Mesh(_mesh(name)).geometry()["K"]) == LINK_SUMS[name]
+
+
+PLANE = [(m, p, "AUTO", r) for m in ("even_rows", "odd_rows", "whole_tiles", "channel2d") for p in ("F16", "BF16")
+         for r in ("REST", "UNIFORM")]
+STEPS = {
+    "even_rows-F16-AUTO-REST": "0bd544d8", "even_rows-F16-AUTO-UNIFORM": "8589fcc8",
+    "even_rows-BF16-AUTO-REST": "32f09459", "even_rows-BF16-AUTO-UNIFORM": "e0160812",
+    "odd_rows-F16-AUTO-REST": "6cd6f8a7", "odd_rows-F16-AUTO-UNIFORM": "4a8e93b9",
+    "odd_rows-BF16-AUTO-REST": "2681e163", "odd_rows-BF16-AUTO-UNIFORM": "c25ef3f7",
+    "whole_tiles-F16-AUTO-REST": "b57a875d", "whole_tiles-F16-AUTO-UNIFORM": "d5477769",
+    "whole_tiles-BF16-AUTO-REST": "3321055e", "whole_tiles-BF16-AUTO-UNIFORM": "942b356d",
+    "channel2d-F16-AUTO-REST": "d68da9c7", "channel2d-F16-AUTO-UNIFORM": "f9221850",
+    "channel2d-BF16-AUTO-REST": "b811683f", "channel2d-BF16-AUTO-UNIFORM": "7bc9ad7d",
+}
+
+
+def _step_digest(V, case):
+    name, prec, mode, ref = case
+    s, N = _run(V, _mesh(name), prec, mode, ref)
+    s.set_state(N)
+    states = []
+    for n in (1, 1, 19):
+        for _ in range(n):
+            s.step(1)
+        states.append(s.get_state())
+    return _digest(*states)
+
+
+@pytest.mark.parametrize("case", PLANE, ids="-".join)
+def test_steps(V, case):
+    assert _step_digest(V, case) == STEPS["-".join(case)]
