@@ -366,6 +366,7 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
   } else if (e == cudaSuccess) {
     e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
   }
+  if (e == cudaSuccess && s->ref_rest) e = cudaMalloc(&s->d_ro, sizeof(float) * (q / 2 + 1) * s->ncoef);
   if (e == cudaSuccess) e = cudaMalloc(&s->d_err, sizeof(int) * vlb::kErrWords);
   if (e != cudaSuccess) {
     vlb_destroy(s);
@@ -505,6 +506,7 @@ void vlb_destroy(vlb_sim *s) {
   dfree(s->d_f);
   dfree(s->d_coef);
   dfree(s->d_uw);
+  dfree(s->d_ro);
   dfree(s->d_err);
   dfree(s->d_fields);
   dfree(s->d_partial);

@@ -410,6 +410,7 @@ struct PackArgs {
   double nref;
   CellFactors cf;    // CellLayout records
   float *uw;         // their wall velocities (NULL: no moving walls)
+  float *ro;         // (ref_rest) the storage reference per column and pair
 };
 
 // wall velocity of a cell: rigid motion of the adjacent wall, at the point halfway
@@ -501,6 +502,7 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
     for (int av = 0; av < Q; av++) {
       own[av] = rest_ref<Q>(a.J[c], a.ginv + c * NS, av);
       osum += own[av];
+      if (av <= H) a.ro[r * (H + 1) + av] = (float)own[av];   // (an FP32 value already)
     }
     rec[L::MDV] = osum - a.nref;   // the weights sum to one
     rec[L::MNV] = osum - a.J[c];
@@ -640,6 +642,7 @@ static cudaError_t pack_q(const vlb_sim *sim, cudaStream_t s) {
   a.nref = sim->nref;
   a.cf = cell_factors(a.tau);
   a.uw = sim->d_uw;
+  a.ro = sim->d_ro;
   for (int d = 0; d < 3; d++) a.body[d] = sim->p.body_force[d];
   for (int ax = 0; ax < 3; ax++)
     for (int sd = 0; sd < 2; sd++)
@@ -663,10 +666,14 @@ cudaError_t launch_pack_coef(const vlb_sim *sim, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ initial state
-// N_a = J f^eq_a(rho, U, U~ = U), U^i = u . g^i (Eqs. 14, 33), normal layout; FP64 storage
-template <int Q>
+// N_a = J f^eq_a(rho, U, U~ = U), U^i = u . g^i (Eqs. 14, 33), normal layout, in FP64: for FP64
+// storage and for 16-bit storage relative to the rest state, whose stored value is what is left of
+// N_a after the reference o_a. Bound by the FP64 pipe (some 400 operations a D3Q19 cell); o_a is
+// read (RefCtx::o) rather than formed per population, which had doubled them: 128^3 cells, FP16:
+// 2.06 -> 0.83 ms.
+template <int Q, typename S>
 __global__ void k_init(const double *J, const double *gu, const double *ginv, const double *rho,
-                       const double *u, int64_t ncell, double nref, double *f) {
+                       const double *u, int64_t ncell, RefCtx ref, S *f) {
   constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncell) return;
@@ -682,14 +689,14 @@ __global__ void k_init(const double *J, const double *gu, const double *ginv, co
   EqParts<Q, double> e;
   eq_parts<Q, double>(gd, U, zero, e);
   const double r = rho[c], Jc = J[c];
-  // stored relative to w_a n_ref
-  f[c] = Jc * r * lat_w<Q, double>(0) * eq_even<Q, double>(e, 0) - lat_w<Q, double>(0) * nref;
+  // stored relative to the storage reference of each location
+  f[c] = store_s<S>(Jc * r * lat_w<Q, double>(0) * eq_even<Q, double>(e, 0) - ref_at<Q>(ref, 0, c));
 #pragma unroll
   for (int p = 1; p <= H; p++) {
     const double E = eq_even<Q, double>(e, p), O = eq_odd<Q, double>(e, U, p);
-    const double w = lat_w<Q, double>(p), rw = Jc * r * w, wn = w * nref;
-    f[p * ncell + c] = rw * (E + O) - wn;
-    f[(p + H) * ncell + c] = rw * (E - O) - wn;
+    const double w = lat_w<Q, double>(p), rw = Jc * r * w, o = ref_at<Q>(ref, p, c);
+    f[p * ncell + c] = store_s<S>(rw * (E + O) - o);
+    f[(p + H) * ncell + c] = store_s<S>(rw * (E - O) - o);
   }
 }
 
@@ -751,89 +758,6 @@ __global__ void k_init_f32(const double *J, const double *gu, const double *ginv
   }
 }
 
-// The initial state of 16-bit storage relative to the rest state of Eq. 33 on the
-// location's column (plane mode): with J f^eq_a = J rho w_a (1 + x_a) and the reference
-// o_a = fl(J w_a (1 + x^0_a)) rounded to FP32 (rest_ref),
-//   N_a - o_a = J w_a [(rho - 1)(1 + x^0_a) + rho (x_a - x^0_a)] + (J w_a (1 + x^0_a) - o_a).
-// The rest state and its rounding are formed in FP64 once per pair and column (60 operations;
-// by a thread each, into shared memory, for the columns that a block of 128 consecutive
-// cells meets), the flow's part, x - x^0 from U U and the odd part, in FP32. Forming every
-// population and, per direction, its reference in FP64 took 2.06 ms on 128^3 cells, the rest
-// state once per pair and cell 0.48 (100 steps with reset and moments 7.6 ms, 7.2 so).
-constexpr int kInitThreads = 128;
-template <int Q, typename S>
-__global__ void __launch_bounds__(kInitThreads) k_init_rest(const double *J, const double *gu, const double *ginv,
-                                                   const double *rho, const double *u, int64_t ncell, int64_t nfast,
-                                                   S *f) {
-  constexpr int D = Lat<Q>::D, NS = D * (D + 1) / 2, H = Lat<Q>::H;
-  // o_a rounded and its remainder, per column of the block
-  extern __shared__ float2 so[];
-  const int64_t b0 = (int64_t)blockIdx.x * kInitThreads, b1 = b0 + kInitThreads < ncell ? b0 + kInitThreads : ncell;
-  const int64_t r0 = b0 / nfast;
-  const int ncol = (int)((b1 - 1) / nfast - r0) + 1;
-  for (int k = threadIdx.x; k < ncol * (H + 1); k += kInitThreads) {
-    const int p = k % (H + 1);
-    const int64_t c0 = (r0 + k / (H + 1)) * nfast;
-    double tr = 0.0, cgc = 0.0;
-#pragma unroll
-    for (int i = 0; i < D; i++)
-#pragma unroll
-      for (int j = 0; j < D; j++) {
-        const double g = ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0);
-        const int cc = Lat<Q>::c(p, i) * Lat<Q>::c(p, j);
-        if (i == j) tr += g;
-        if (cc > 0) cgc += g;
-        if (cc < 0) cgc -= g;
-      }
-    const double o = J[c0] * (lat_w<Q, double>(p) * (1.0 + 0.5 * (3.0 * cgc - tr)));
-    so[k] = make_float2((float)o, (float)(o - (double)(float)o));
-  }
-  __syncthreads();
-  const int64_t c = b0 + threadIdx.x;
-  if (c >= ncell) return;
-  const int64_t row = ncell < ((int64_t)1 << 31) ? (int64_t)((uint32_t)c / (uint32_t)nfast) : c / nfast;
-  const int64_t c0 = row * nfast;
-  const float2 *const oc = so + (int)(row - r0) * (H + 1);
-  float U[D], gd[NS], zero[D];
-#pragma unroll
-  for (int i = 0; i < D; i++) {
-    float v = 0.0f;
-#pragma unroll
-    for (int d = 0; d < D; d++) v = fmaf((float)u[c * D + d], (float)gu[(c0 * D + i) * D + d], v);
-    U[i] = v;
-    zero[i] = 0.0f;
-  }
-#pragma unroll
-  for (int i = 0; i < D; i++)
-#pragma unroll
-    for (int j = i; j < D; j++)
-      gd[sym<D>(i, j)] = (float)(ginv[c0 * NS + sym<D>(i, j)] - (i == j ? 1.0 : 0.0));
-  EqParts<Q, float> e;
-  eq_parts<Q, float>(gd, U, zero, e);
-  // the even part without the rest state's: B = U U
-  EqParts<Q, float> q = e;
-  q.trB = 0.0f;
-#pragma unroll
-  for (int i = 0; i < D; i++) {
-#pragma unroll
-    for (int j = 0; j < D; j++) q.B[i][j] = U[i] * U[j];
-    q.trB += q.B[i][i];
-  }
-  const float r1 = (float)(rho[c] - 1.0), r = (float)rho[c], Jf = (float)J[c0];
-#pragma unroll
-  for (int p = 0; p <= H; p++) {
-    const float of = oc[p].x, lo = oc[p].y;
-    const float jw = Jf * lat_w<Q, float>(p), xe = eq_even_x<Q>(q, p);
-    if (p == 0) {
-      f[c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe, lo)));
-    } else {
-      const float xo = eq_odd<Q, float>(e, U, p);
-      f[p * ncell + c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe + xo, lo)));
-      f[(p + H) * ncell + c] = store_s<S>(fmaf(r1, of, fmaf(jw * r, xe - xo, lo)));
-    }
-  }
-}
-
 cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
   const int threads = 128;
@@ -842,22 +766,9 @@ cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d
   return with_storage(sim->p.precision, [&](auto tag) {
     using S = typename decltype(tag)::type;
     if constexpr (!std::is_same<S, double>::value) {
-      // FP32 arithmetic
-      if constexpr (sizeof(S) == 2) {
-        if (ref.rest) {
-          static_assert(kInitThreads == 128, "blocks of k_init_rest");
-          // columns that a block meets at most: 129 of one cell each, 10 KB
-          const size_t smem = sizeof(float2) * (m->md.q / 2 + 1) * (size_t)((kInitThreads - 1) / ref.nfast + 2);
-          if (m->md.q == 9)
-            k_init_rest<9, S><<<(unsigned)blocks, threads, smem, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
-                                                                   ref.nfast, (S *)sim->d_f);
-          else
-            k_init_rest<19, S><<<(unsigned)blocks, threads, smem, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
-                                                                    ref.nfast, (S *)sim->d_f);
-          return cudaGetLastError();
-        }
-      }
-      {
+      // FP32 arithmetic for the uniform reference (the rest reference of 16-bit storage keeps
+      // the FP64 form: what is stored is a small difference, rounded to 16 bits)
+      if (!ref.rest) {
         if (m->md.q == 9)
           k_init_f32<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell,
                                                                 ref.nref, (S *)sim->d_f);
@@ -867,15 +778,15 @@ cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d
         return cudaGetLastError();
       }
     }
-    else {
+    if constexpr (!std::is_same<S, float>::value) {
       if (m->md.q == 9)
-        k_init<9><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref.nref,
-                                                       (double *)sim->d_f);
+        k_init<9, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref,
+                                                          (S *)sim->d_f);
       else
-        k_init<19><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref.nref,
-                                                        (double *)sim->d_f);
-      return cudaGetLastError();
+        k_init<19, S><<<(unsigned)blocks, threads, 0, s>>>(m->d_J, m->d_gu, m->d_ginv, d_rho, d_u, m->ncell, ref,
+                                                           (S *)sim->d_f);
     }
+    return cudaGetLastError();
   });
 }
 

@@ -415,17 +415,15 @@ __device__ __forceinline__ double rest_ref(double J, const double *ginv, int a) 
 struct RefCtx {
   int32_t rest;          // VLB_REF_REST in use
   double nref;           // uniform reference
-  const double *J;       // FP64 geometry (rest)
-  const double *ginv;
+  const float *o;        // (rest) rest_ref per column and pair [ncoef][H + 1]
   int64_t nfast;         // plane mode: a column's geometry is that of its first cell
 };
 
 template <int Q>
 __device__ __forceinline__ double ref_at(const RefCtx &r, int slot, int64_t cell) {
   if (!r.rest) return lat_w<Q, double>(slot) * r.nref;
-  constexpr int NS = Lat<Q>::D * (Lat<Q>::D + 1) / 2;
-  const int64_t c0 = (cell / r.nfast) * r.nfast;
-  return rest_ref<Q>(r.J[c0], r.ginv + c0 * NS, slot);
+  constexpr int H = Lat<Q>::H;
+  return r.o[(cell / r.nfast) * (H + 1) + (slot <= H ? slot : slot - H)];
 }
 
 // --------------------------------------------------------------------------
@@ -470,6 +468,7 @@ struct vlb_sim {
   int32_t plane = 0;
   int32_t cellrec = 0;        // FP32, one record per cell: CellLayout, else CoefLayout
   float *d_uw = nullptr;      // with cellrec and moving walls: wall velocities [ncell][dim]
+  float *d_ro = nullptr;      // with ref_rest: the storage reference per column and pair (RefCtx::o)
   int64_t t = 0;
   double nref = 0.0;          // populations are stored as N_a - w_a nref, nref = rho_0 J_ref
   int32_t ref_rest = 0;       // 16-bit storage relative to the local rest state
@@ -524,8 +523,7 @@ inline RefCtx make_ref(const vlb_sim *sim) {
   RefCtx r;
   r.rest = sim->ref_rest;
   r.nref = sim->nref;
-  r.J = sim->mesh->d_J;
-  r.ginv = sim->mesh->d_ginv;
+  r.o = sim->d_ro;
   r.nfast = sim->plane ? sim->mesh->md.n[sim->mesh->md.dim - 1] : 1;
   return r;
 }

@@ -95,3 +95,22 @@ def _step_digest(V, case):
 @pytest.mark.parametrize("case", PLANE, ids="-".join)
 def test_steps(V, case):
     assert _step_digest(V, case) == STEPS["-".join(case)]
+
+
+INITIAL = {
+    "even_rows-F16-AUTO-REST": "c11e6111", "even_rows-F16-AUTO-UNIFORM": "a61eaeeb",
+    "even_rows-BF16-AUTO-REST": "9c1d1680", "even_rows-BF16-AUTO-UNIFORM": "fa6fdaf4",
+    "odd_rows-F16-AUTO-REST": "202c6631", "odd_rows-F16-AUTO-UNIFORM": "54361136",
+    "odd_rows-BF16-AUTO-REST": "8a10b247", "odd_rows-BF16-AUTO-UNIFORM": "7cf77f39",
+    "whole_tiles-F16-AUTO-REST": "2a16aa7a", "whole_tiles-F16-AUTO-UNIFORM": "f526ed1d",
+    "whole_tiles-BF16-AUTO-REST": "e7813a84", "whole_tiles-BF16-AUTO-UNIFORM": "e4b8a683",
+    "channel2d-F16-AUTO-REST": "204812f6", "channel2d-F16-AUTO-UNIFORM": "84e64455",
+    "channel2d-BF16-AUTO-REST": "8790d7b7", "channel2d-BF16-AUTO-UNIFORM": "bcadea85",
+}
+
+
+@pytest.mark.parametrize("case", PLANE, ids="-".join)
+def test_initial_state(V, case):
+    name, prec, mode, ref = case
+    s, _ = _run(V, _mesh(name), prec, mode, ref)
+    assert _digest(s.get_state()) == INITIAL["-".join(case)]
