@@ -65,10 +65,10 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *out) {
 // One cell per thread; IT is the index type (32-bit when every population
 // offset fits). In plane mode the tangents, like the coefficient record, are
 // those of the column (its first cell).
-// REST (16-bit storage relative to the rest state, plane mode): the collision
-// works on the stored values relative to the own column's rest state, as the
-// step does, with the record's column differences; forming every location's
-// reference in FP64 instead took 0.49 ms on 128^3 cells, 0.11 so
+// REST (16-bit storage relative to the rest state, plane mode): each location's
+// offset from the uniform reference is one FP64 difference of its stored reference
+// (RefCtx::o), rounded once; forming that reference too, 19 times a cell, took
+// 0.49 ms on 128^3 cells, 0.21 (even) to 0.30 (odd) so
 template <int Q, typename S, bool ODD, typename MT, typename IT, bool REST>
 __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double *out) {
   constexpr int D = Lat<Q>::D;
@@ -79,37 +79,39 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
   const IT n2 = (IT)a.g.n[2], n1 = (IT)a.g.n[1];
   const IT r = c / n2, i2 = c - r * n2, i0 = r / n1, i1 = r - i0 * n1;
   const Addr<Q, IT> ad(a.g, i0, i1, i2);
-  // the arrived populations in MT, as stored: deviations from the uniform reference
-  // w_a n_ref, or (REST) from the rest state of the column that holds them
+  // the cell's (or column's) coefficient record, stored in MT
+  const IT c0 = a.plane ? c - ad.ic[D - 1] : c;   // the fastest axis has stride 1
+  // the arrived populations in MT as deviations from the uniform reference w_a n_ref:
+  // the stored value, plus (REST) the offset of the reference of the column that holds it
   MT dv[Q];
+  const IT col = a.plane ? c0 / (IT)a.nfast : c;
 #pragma unroll
   for (int av = 0; av < Q; av++) {
     int slot;
     IT loc;
     arrived_loc<Q, ODD, IT>(ad, av, slot, loc);
     dv[av] = load_s<MT>(f[(IT)slot * (IT)a.ncell + loc]);
-  }
-  // the cell's (or column's) coefficient record, stored in MT
-  const IT c0 = a.plane ? c - ad.ic[D - 1] : c;   // the fastest axis has stride 1
-  if constexpr (REST && ODD) {
-    using L = CoefLayout<Q>;
-    const MT *rc = static_cast<const MT *>(a.coef) + (int64_t)(c0 / (IT)a.nfast) * a.rs;
+    if constexpr (REST) {
+      constexpr int H = Lat<Q>::H;
+      IT lc = col;
+      if (ODD && av != 0 && !ad.crosses(av, -1)) {
 #pragma unroll
-    for (int av = 1; av < Q; av++) {
-      bool slow = false;
-#pragma unroll
-      for (int d = 0; d < D - 1; d++) slow = slow || Lat<Q>::c(av, d) != 0;
-      // (the differences are zero where a slow-axis wall sends the link back; a
-      // fastest-axis wall does so at the ends of a row only)
-      if (slow && !ad.crosses(av, -1)) dv[av] += rc[L::DIN + av];
+        for (int d = 0; d < D - 1; d++) {
+          if (Lat<Q>::c(av, d) > 0) lc += ad.dm[d] / (IT)a.nfast;
+          if (Lat<Q>::c(av, d) < 0) lc += ad.dp[d] / (IT)a.nfast;
+        }
+      }
+      const double o = a.ref.o[(int64_t)lc * (H + 1) + (av <= H ? av : av - H)];
+      dv[av] += static_cast<MT>(o - lat_w<Q, double>(slot) * a.nref);
     }
   }
   MT Np[Q];
   CollideState<Q, MT> st;
   // chord iteration from the record's rest-state start value
   auto solve = [&](const auto &rec) {
-    collide_cell<Q, MT, false, REST>(dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau),
-                                     static_cast<MT>(a.tol), 200, Np, st);
+    using RC = typename std::decay<decltype(rec)>::type;
+    collide_cell<Q, MT, false, false, true, RC, false, sizeof(S) == 2>(
+        dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau), static_cast<MT>(a.tol), 200, Np, st);
   };
   if constexpr (sizeof(MT) == 4 && !REST) {
     if (!a.plane) {
@@ -120,7 +122,7 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
     }
   }
   if (sizeof(MT) == 8 || a.plane)
-    solve(PtrRecord<MT>{static_cast<const MT *>(a.coef) + (int64_t)(a.plane ? c0 / (IT)a.nfast : c) * a.rs});
+    solve(PtrRecord<MT>{static_cast<const MT *>(a.coef) + (int64_t)col * a.rs});
   if (!st.conv) atomicOr(a.err, ERR_NOCONV);
   // the output mapping in the simulation's arithmetic (U and F are MT already)
   MT gl[D][D];

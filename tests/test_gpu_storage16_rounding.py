@@ -114,3 +114,32 @@ def test_initial_state(V, case):
     name, prec, mode, ref = case
     s, _ = _run(V, _mesh(name), prec, mode, ref)
     assert _digest(s.get_state()) == INITIAL["-".join(case)]
+
+
+MOMENTS = {
+    "even_rows-F16-AUTO-REST": "d5af4d01", "even_rows-F16-AUTO-UNIFORM": "8d691d28",
+    "even_rows-BF16-AUTO-REST": "89466f16", "even_rows-BF16-AUTO-UNIFORM": "1b099365",
+    "odd_rows-F16-AUTO-REST": "2f09d30c", "odd_rows-F16-AUTO-UNIFORM": "14dcef6f",
+    "odd_rows-BF16-AUTO-REST": "8ed0ac40", "odd_rows-BF16-AUTO-UNIFORM": "6ad3dddf",
+    "whole_tiles-F16-AUTO-REST": "6ede362d", "whole_tiles-F16-AUTO-UNIFORM": "f17179c4",
+    "whole_tiles-BF16-AUTO-REST": "0ac4eb9d", "whole_tiles-BF16-AUTO-UNIFORM": "f92f426b",
+    "channel2d-F16-AUTO-REST": "04ea3ebd", "channel2d-F16-AUTO-UNIFORM": "1d546fc5",
+    "channel2d-BF16-AUTO-REST": "ba2f99f5", "channel2d-BF16-AUTO-UNIFORM": "d97f521a",
+}
+
+
+def _moments_digest(V, case):
+    name, prec, mode, ref = case
+    s, N = _run(V, _mesh(name), prec, mode, ref)
+    s.set_state(N)
+    out = []
+    for n in (1, 1, 19):      # both parities
+        s.step(n)
+        m = s.moments()
+        out += [m["rho"], m["u"], m["u_tilde"]]
+    return _digest(*out)
+
+
+@pytest.mark.parametrize("case", PLANE, ids="-".join)
+def test_moments(V, case):
+    assert _moments_digest(V, case) == MOMENTS["-".join(case)]
