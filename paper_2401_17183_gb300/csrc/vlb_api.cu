@@ -348,7 +348,7 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
     s->ncoef = mesh->ncell;
   }
   const size_t es = f64 ? 8 : 4;
-  s->cellrec = !f64 && !plane && q != VLB_D3Q39;
+  s->cellrec = params->precision == VLB_F32 && !plane && q != VLB_D3Q39;
   // 16 bytes of padding: a 16-bit population is read as the aligned 32-bit
   // word that contains it
   cudaError_t e = cudaMalloc(&s->d_f, vlb::storage_bytes(params->precision) * q * mesh->ncell + 16);

@@ -199,7 +199,7 @@ struct CoefLayout {
   }
 };
 
-// FP32 record of one cell (one record per cell): the entries of CoefLayout from
+// Record of one cell of FP32 populations (one record per cell): the entries of CoefLayout from
 // which the others follow -- J, 1/J, (g - I)/2, G, KW and its low part, FR, CE and
 // the link coefficients, NV values in NG groups of four. PO1, HM and QM are formed
 // again by the step (CellRecord in vlb_collide.cuh): with a record per cell the step is

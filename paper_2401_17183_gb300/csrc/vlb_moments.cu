@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
     collide_cell<Q, MT, false, false, true, RC, false, sizeof(S) == 2>(
         dv, rec, static_cast<MT>(a.nref), static_cast<MT>(1.0 / a.tau), static_cast<MT>(a.tol), 200, Np, st);
   };
-  if constexpr (sizeof(MT) == 4 && !REST) {
+  if constexpr (sizeof(S) == 4) {
     if (!a.plane) {
       CellRecord<Q> rec;
       rec.load(static_cast<const float4 *>(a.coef), (int64_t)c);
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kMomThreads) k_moments(const MomArgs a, double
       solve(rec);
     }
   }
-  if (sizeof(MT) == 8 || a.plane)
+  if (sizeof(S) != 4 || a.plane)
     solve(PtrRecord<MT>{static_cast<const MT *>(a.coef) + (int64_t)col * a.rs});
   if (!st.conv) atomicOr(a.err, ERR_NOCONV);
   // the output mapping in the simulation's arithmetic (U and F are MT already)

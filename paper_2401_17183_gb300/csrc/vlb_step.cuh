@@ -246,7 +246,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
   Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
   R *const srec = reinterpret_cast<R *>(smem_raw + sizeof(Smem));
   const int nrec = ROWS ? 1 : a.nrec;
-  constexpr bool CELLREC = !PLANE && sizeof(R) == 4;
+  constexpr bool CELLREC = !PLANE && sizeof(S) == 4;
   using CL = CellLayout<Q>;
   S *__restrict__ f = static_cast<S *>(a.f);
   const R *__restrict__ coef = static_cast<const R *>(a.coef);
@@ -566,7 +566,7 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       R Np[Q];
       CollideState<Q, R> cst;
       // (with one record per cell the rest state is formed, not read)
-      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16 && PLANE>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
+      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
                                      arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
       if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
 

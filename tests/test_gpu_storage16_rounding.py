@@ -143,3 +143,16 @@ def _moments_digest(V, case):
 @pytest.mark.parametrize("case", PLANE, ids="-".join)
 def test_moments(V, case):
     assert _moments_digest(V, case) == MOMENTS["-".join(case)]
+
+
+GENERAL = [(m, p, "FULL", "UNIFORM") for m in ("odd_rows", "general", "channel2d") for p in ("F16", "BF16")]
+RECORD_PER_CELL = {
+    "odd_rows-F16-FULL-UNIFORM": ["f4136f97", "13a2aa24"], "odd_rows-BF16-FULL-UNIFORM": ["7c7c1d94", "7dde50ed"],
+    "general-F16-FULL-UNIFORM": ["430a5077", "5e41db62"], "general-BF16-FULL-UNIFORM": ["984d3000", "a580c551"],
+    "channel2d-F16-FULL-UNIFORM": ["5cfdf266", "ab0ec671"], "channel2d-BF16-FULL-UNIFORM": ["d7a804c9", "9b2f1d0c"],
+}
+
+
+@pytest.mark.parametrize("case", GENERAL, ids="-".join)
+def test_one_record_per_cell(V, case):
+    assert [_step_digest(V, case), _moments_digest(V, case)] == RECORD_PER_CELL["-".join(case)]
