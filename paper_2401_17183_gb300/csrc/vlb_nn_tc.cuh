@@ -77,12 +77,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     if (t - t0 > kTcWaitNs) return false;
   }
 }
+// the same by a whole warp, whose lanes get one answer and go on together: what follows a wait
+// may be an instruction of the whole warp (.sync.aligned), also where the time limit ends some
+// lanes' wait and not others'
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
 __device__ __forceinline__ void cp16(uint32_t sdst, const void *gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sdst), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp16_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // 16 tensor-memory columns of the warp's 32 lanes
 __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
       "tcgen05.wait::ld.sync.aligned;\n"
@@ -101,6 +108,7 @@ __device__ __forceinline__ uint32_t tc_begin(uint64_t *bar, uint32_t *tslot) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 32) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -363,6 +371,7 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tslot)), "r"(TCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -376,7 +385,7 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
     int j = 0;
     for (; j < nch; j++) {
       const int s = j % nstage, use = j / nstage;
-      if (use > 0 && !mbar_wait(smem_u32(&empty[s]), (use - 1) & 1)) {
+      if (use > 0 && !mbar_wait_warp(smem_u32(&empty[s]), (use - 1) & 1)) {
         ok = false;
         break;
       }
@@ -394,12 +403,12 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
     }
     // copies that nothing has waited for (after a failure) land before the block ends
     for (int i = j > nstage ? j - nstage : 0; i < j; i++)
-      if (!mbar_wait(smem_u32(&full[i % nstage]), (i / nstage) & 1)) ok = false;
+      if (!mbar_wait_warp(smem_u32(&full[i % nstage]), (i / nstage) & 1)) ok = false;
   } else if (warp == 5) {
     for (int j = 0; j < nch; j++) {
       const int s = j % nstage, d = j & 1;
-      if (!mbar_wait(smem_u32(&full[s]), (j / nstage) & 1) ||
-          (j >= 2 && !mbar_wait(smem_u32(&dempty[d]), ((j >> 1) - 1) & 1))) {
+      if (!mbar_wait_warp(smem_u32(&full[s]), (j / nstage) & 1) ||
+          (j >= 2 && !mbar_wait_warp(smem_u32(&dempty[d]), ((j >> 1) - 1) & 1))) {
         ok = false;
         break;
       }
@@ -421,7 +430,7 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
     if (!ok && lane == 0) umma_commit(smem_u32(&dfin));
     __syncwarp();
     // every MMA is done before the block ends
-    if (!mbar_wait(smem_u32(&dfin), 0)) ok = false;
+    if (!mbar_wait_warp(smem_u32(&dfin), 0)) ok = false;
   } else {
     float acc[NB];
 #pragma unroll
@@ -438,7 +447,7 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
     };
     for (int j = 0; j < nch && ok; j++) {
       const int d = j & 1;
-      if (!mbar_wait(smem_u32(&dfull[d]), (j >> 1) & 1)) {
+      if (!mbar_wait_warp(smem_u32(&dfull[d]), (j >> 1) & 1)) {
         ok = false;
         break;
       }
@@ -447,8 +456,7 @@ __global__ void __launch_bounds__(192, 2) k_dgrad_mma(const bf16 *__restrict__ g
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&dempty[d])) : "memory");
     }
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&dfin), 0));
+    if (ok) ok = mbar_wait_warp(smem_u32(&dfin), 0);
     if (ok) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       add(ta + 2 * NB);
@@ -492,6 +500,7 @@ __host__ __device__ constexpr int wg_groups(int cb) { return kTcM / cb < 3 ? kTc
 
 // 24 tensor-memory columns of the warp's 32 lanes
 __device__ __forceinline__ void tmem_ld24(uint32_t addr, uint32_t (&r)[24]) {
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%24];\n"
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%25];\n"
