@@ -440,10 +440,12 @@ inline bool tc_shape(const vlb_nn *n, const NNLayer &l) {
   const bool pow2 = l.cout >= 16 && l.cout <= 256 && (l.cout & (l.cout - 1)) == 0;
   return n->storage == VLB_NN_BF16 && l.k == 3 && pow2 && ((int64_t)l.h * l.w) % nn::kTcM == 0 && l.cin % 8 == 0;
 }
+// longest rows of the input gradient's tiles
+constexpr int kDgMaxRow = 256;
 // its backward pass: pixel groups of 8 within a row, the positions a tap
 // reaches within a block's shared memory, positions in 32 bits
 inline bool tc_bwd_shape(const vlb_nn *n, const NNLayer &l) {
-  return tc_shape(n, l) && l.w % 8 == 0 && l.w <= 256 &&
+  return tc_shape(n, l) && l.w % 8 == 0 && l.w <= kDgMaxRow &&
          (int64_t)n->maxb * (l.h + 1) * (l.w + 1) < ((int64_t)1 << 30);
 }
 
@@ -495,19 +497,24 @@ cudaError_t conv_mma(const vlb_nn *n, const NNLayer &l, const nn::bf16 *in, int6
   }
 }
 
+// shared memory of a block of which an SM holds two
+constexpr int kDgTwoBlocks = 112 * 1024;
 template <int NB>
 cudaError_t launch_dgrad(const vlb_nn *n, const NNLayer &l, int64_t plane, int64_t npos, const nn::bf16 *wp, float *out,
                          int64_t obs, int B, int tiles) {
   const int stage = nn::dg_stage_bytes(NB, l.w);
   // two blocks per SM where two stages of each fit
-  int nst = 112 * 1024 / stage;
+  int nst = kDgTwoBlocks / stage;
   nst = nst < 2 ? 2 : nst > nn::kDgMaxStages ? nn::kDgMaxStages : nst;
   auto kern = nn::k_dgrad_mma<NB>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, nst * stage);
+  // the limit belongs to the kernel, not to this launch: every call sets the same one, that of
+  // the widest rows, or a thread with narrower rows would lower it under another's launch
+  constexpr int widest = 2 * nn::dg_stage_bytes(NB, kDgMaxRow), most = widest > kDgTwoBlocks ? widest : kDgTwoBlocks;
+  static_assert(most <= 227 * 1024, "shared memory of a block");
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
   chain(kern, dim3((unsigned)tiles, (unsigned)(l.cin / NB)), dim3(192), nst * stage, n->planes, plane, npos, l.cout,
-        wp, l.cin,
-                                                                            out, obs, l.h, l.w, B, nst, n->d_err);
+        wp, l.cin, out, obs, l.h, l.w, B, nst, n->d_err);
   return cudaGetLastError();
 }
 

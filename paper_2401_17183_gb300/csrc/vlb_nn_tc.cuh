@@ -332,7 +332,7 @@ struct Padded {
 // grid (tiles, rows / NB), block 192. C a multiple of 16.
 constexpr int kDgMaxStages = 4;
 __host__ __device__ constexpr int dg_cols(int nb) { return 3 * nb <= 64 ? 64 : 3 * nb <= 128 ? 128 : 256; }
-inline int dg_stage_bytes(int nb, int W) { return 6 * (132 + 2 * W) * 16 + 18 * nb * 16; }
+constexpr int dg_stage_bytes(int nb, int W) { return 6 * (132 + 2 * W) * 16 + 18 * nb * 16; }
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
