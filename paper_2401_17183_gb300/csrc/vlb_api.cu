@@ -353,9 +353,14 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
   // word that contains it
   cudaError_t e = cudaMalloc(&s->d_f, vlb::storage_bytes(params->precision) * q * mesh->ncell + 16);
   if (e == cudaSuccess && q == VLB_D3Q39) {
-    e = cudaMalloc(&s->d_coef, vlb::q39_record_bytes(mesh->ncell));
+    // the records where they leave room for what the simulation allocates later (staging of the
+    // state, 39 values a cell, and the fields, 7); else the chord data alone, a
+    // sixteenth of the memory, and the map direction by direction
+    const size_t rec = vlb::q39_record_bytes(mesh->ncell), later = es * (39 + 7) * mesh->ncell + (1 << 20);
+    size_t room = 0, total = 0;
+    e = cudaMemGetInfo(&room, &total);
+    if (e == cudaSuccess) e = room < rec + later ? cudaErrorMemoryAllocation : cudaMalloc(&s->d_coef, rec);
     if (e == cudaErrorMemoryAllocation) {
-      // no room for the records: the chord data alone, and the map direction by direction
       cudaGetLastError();
       s->nc = vlb::kChord39;
       e = cudaMalloc(&s->d_coef, es * s->nc * s->ncoef);
@@ -497,6 +502,18 @@ int vlb_sim_layout(const vlb_sim *s, int32_t *coef_per_cell, int32_t *plane_mode
   if (coef_per_cell) *coef_per_cell = s->nc;
   if (plane_mode) *plane_mode = s->plane;
   if (records) *records = s->ncoef;
+  return VLB_OK;
+}
+
+// (for tests, not in vlb.h) has a D3Q39 simulation take the form without records
+int vlb_internal_q39_compact(vlb_sim *s) {
+  if (!s || s->mesh->md.q != VLB_D3Q39) return fail(VLB_EINVAL, "not a D3Q39 simulation");
+  if (s->nc == vlb::kChord39) return VLB_OK;
+  CU(cudaStreamSynchronize(s->stream));
+  dfree(s->d_coef);
+  s->nc = vlb::kChord39;
+  CU(cudaMalloc(&s->d_coef, sizeof(double) * s->nc * s->ncoef));
+  CU(vlb::q39_prepare(s, s->stream));
   return VLB_OK;
 }
 
