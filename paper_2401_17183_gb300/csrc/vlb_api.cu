@@ -415,6 +415,7 @@ int vlb_step(vlb_sim *s, int64_t nsteps) {
     cudaError_t e = s->mesh->md.q == VLB_D3Q39 ? vlb::q39_step(s, (int)(s->t & 1), s->stream)
                                                : vlb::launch_step(s, (int)(s->t & 1), s->stream);
     if (e != cudaSuccess) return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(e));
+    s->path = vlb::PATH_STEP;
     s->t++;
     k++;
   }
@@ -504,6 +505,9 @@ int vlb_sim_layout(const vlb_sim *s, int32_t *coef_per_cell, int32_t *plane_mode
   if (records) *records = s->ncoef;
   return VLB_OK;
 }
+
+// (for tests, not in vlb.h) how the last launch of vlb_step advanced the simulation (PATH_*)
+int vlb_internal_step_path(const vlb_sim *s) { return s ? s->path : 0; }
 
 // (for tests, not in vlb.h) has a D3Q39 simulation take the form without records
 int vlb_internal_q39_compact(vlb_sim *s) {

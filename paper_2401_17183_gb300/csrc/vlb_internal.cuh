@@ -470,6 +470,7 @@ struct vlb_sim {
   float *d_uw = nullptr;      // with cellrec and moving walls: wall velocities [ncell][dim]
   float *d_ro = nullptr;      // with ref_rest: the storage reference per column and pair (RefCtx::o)
   int64_t t = 0;
+  int32_t path = 0;           // PATH_*: how the last launch of vlb_step advanced it
   double nref = 0.0;          // populations are stored as N_a - w_a nref, nref = rho_0 J_ref
   int32_t ref_rest = 0;       // 16-bit storage relative to the local rest state
   int *d_err = nullptr;       // sticky kernel error flags
@@ -535,6 +536,8 @@ enum : int { ERR_NOCONV = 1, ERR_NONFINITE = 2, ERR_GEOM = 4, ERR_BARRIER = 8 };
 constexpr int kErrWords = 64, kBarrierWord = 32;
 // steps of one multi-step launch, and the largest mesh it is tried for
 constexpr int64_t kSmallSteps = 1024, kSmallCells = 65536;
+// launches of vlb_step: one step, or several as one cluster or as a cooperative launch
+enum : int32_t { PATH_STEP = 1, PATH_CLUSTER = 2, PATH_COOPERATIVE = 3 };
 
 // launchers (each returns a cudaError_t from the launch)
 cudaError_t launch_geometry(const vlb_mesh *m, int *d_err, cudaStream_t s);
@@ -543,8 +546,9 @@ cudaError_t launch_plane_check(const vlb_mesh *m, int *d_flag, cudaStream_t s);
 cudaError_t launch_pack_coef(const vlb_sim *sim, cudaStream_t s);
 cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s);
 cudaError_t launch_step(const vlb_sim *sim, int odd, cudaStream_t s);
-// up to nsteps steps of a small mesh in one launch; *done: how many (0: none, not small)
-cudaError_t launch_steps_small(const vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s);
+// up to nsteps steps of a small mesh in one launch; *done: how many (0: none, not small), and
+// sim->path then
+cudaError_t launch_steps_small(vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s);
 cudaError_t launch_moments(const vlb_sim *sim, double *d_out, int64_t nblk, cudaStream_t s);
 // conservation totals (mass, P, M) of a D2Q9/D3Q19 simulation into d_totals[7]
 // through per-block partial sums in d_partial (room for nblk_max x 7 doubles)

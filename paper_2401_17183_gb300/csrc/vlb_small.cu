@@ -3,7 +3,7 @@
 
 namespace vlb {
 
-cudaError_t launch_steps_small(const vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s) {
+cudaError_t launch_steps_small(vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s) {
   *done = 0;
   const vlb_mesh *m = sim->mesh;
   const int q = m->md.q;

@@ -202,7 +202,7 @@ static bool cluster_fits(const void *kern, int nblk, int threads, size_t smem) {
 
 // One cluster over the whole mesh, T cells per block; *done = 0 when it does not fit.
 template <int Q, typename R, bool PLANE, bool EXT, int T>
-cudaError_t launch_cluster_t(const vlb_sim *sim, int32_t first, int32_t n, int64_t *done, cudaStream_t s) {
+cudaError_t launch_cluster_t(vlb_sim *sim, int32_t first, int32_t n, int64_t *done, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
   const size_t smem = SmallRecords<Q, R, PLANE>::bytes(T, m->md.n[m->md.dim - 1]);
   auto kern = k_steps_small<Q, R, PLANE, EXT, T, 1, true>;
@@ -221,14 +221,14 @@ cudaError_t launch_cluster_t(const vlb_sim *sim, int32_t first, int32_t n, int64
   cfg.attrs = at;
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a, first, n, (unsigned *)nullptr);
-  if (e == cudaSuccess) *done = n;
+  if (e == cudaSuccess) *done = n, sim->path = PATH_CLUSTER;
   return e;
 }
 
 // Advances the simulation by up to `nsteps` steps in one launch if its cells fit on the
 // device at once; *done is the number of steps launched (0: take the step kernel).
 template <int Q, typename R, bool PLANE, bool EXT>
-cudaError_t launch_small_t(const vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s) {
+cudaError_t launch_small_t(vlb_sim *sim, int64_t nsteps, int64_t *done, cudaStream_t s) {
   constexpr int T = small_threads<R>();
   constexpr int MINB = sizeof(R) == 8 ? 8 : Q == 9 ? 4 : 3;
   const vlb_mesh *m = sim->mesh;
@@ -254,7 +254,7 @@ cudaError_t launch_small_t(const vlb_sim *sim, int64_t nsteps, int64_t *done, cu
   cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
   e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3((unsigned)nblk), dim3(T), args, smem, s);
-  if (e == cudaSuccess) *done = n;
+  if (e == cudaSuccess) *done = n, sim->path = PATH_COOPERATIVE;
   return e;
 }
 
