@@ -45,11 +45,6 @@ sys.path.insert(0, ROOT)
 BYTES_PER_CELL = {("19", "f32"): 2 * 19 * 4, ("19", "f64"): 2 * 19 * 8, ("9", "f32"): 2 * 9 * 4,
                   ("9", "f64"): 2 * 9 * 8, ("19", "f16"): 2 * 19 * 2, ("19", "bf16"): 2 * 19 * 2}
 STEP_SOURCES = ["vlb_step.cu", "vlb_step.cuh", "vlb_collide.cuh", "vlb_addr.cuh", "vlb_internal.cuh"]
-# the coefficient record values the D3Q19 FP32 step kernel reads per cell
-# with one record per cell (CoefLayout<19>::RR: everything before the rest
-# state, which that mode forms from J and g^ij; the wall velocity after it is
-# read in moving-wall cells only)
-RECORD_FLOATS_READ = 136
 
 
 def args_parse():
@@ -334,13 +329,13 @@ def general_mesh_leg(a, stream):
     value = ncell * a.general_steps / (ms / 1e3) / 1e6
     peak, peak_kind = measured_peak_hbm()
     # bytes the kernel moves per cell update: populations read and written, and
-    # the part of the cell's coefficient record it reads
-    rec_bytes = 4 * RECORD_FLOATS_READ
+    # the cell's coefficient record, all of which it reads (whole groups of 32 cells)
+    rec_bytes = lay["record_bytes"] / (-(-ncell // 32) * 32)
     per_launch = ms / 1e3 / a.general_steps
     out = {"workload": "channel_bump3d_d3q19_%d^3_fp32_full_records" % n, "cells": ncell,
            "value": value, "unit": "MLUPS", "steps": a.general_steps,
            "ms_per_step": ms / a.general_steps, "coef_mode": "plane" if lay["plane"] else "full",
-           "record_floats_stored": lay["coef_per_cell"], "record_bytes_read_per_cell": rec_bytes,
+           "record_floats_stored": rec_bytes / 4, "record_bytes_read_per_cell": rec_bytes,
            "roofline": {"bound": "hbm", "peak": peak, "unit": "GB/s", "peak_kind": peak_kind,
                         "achieved_populations": 152 * ncell / per_launch / 1e9,
                         "frac_populations": 152 * ncell / per_launch / 1e9 / peak,

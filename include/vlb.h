@@ -203,10 +203,16 @@ int vlb_set_state(vlb_sim *sim, const double *N);
 
 /* Steps taken since vlb_init / vlb_reset / vlb_set_state. */
 int64_t vlb_time(const vlb_sim *sim);
-/* Bytes per cell of the coefficient record and whether it is one per column
- * (plane mode); for reporting. */
+/* For reporting: the values of one coefficient record as the collision works
+ * with it, whether records are one per column (plane mode), and how many there
+ * are. D3Q39: the values stored per cell (193, or 12 where device memory does
+ * not hold those). */
 int vlb_sim_layout(const vlb_sim *sim, int32_t *coef_per_cell, int32_t *plane_mode,
                    int64_t *coef_records);
+/* Bytes of device memory that the coefficient records take. With one record
+ * per cell, VLB_F32 stores only the values that the step does not form from
+ * others: 80 of D3Q19's 136, 320 bytes per cell. */
+int vlb_sim_record_bytes(const vlb_sim *sim, int64_t *bytes);
 
 void vlb_destroy(vlb_sim *sim);
 const char *vlb_last_error(void);

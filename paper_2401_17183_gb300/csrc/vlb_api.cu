@@ -506,6 +506,16 @@ int vlb_sim_layout(const vlb_sim *s, int32_t *coef_per_cell, int32_t *plane_mode
   return VLB_OK;
 }
 
+int vlb_sim_record_bytes(const vlb_sim *s, int64_t *bytes) {
+  if (!s || !bytes) return fail(VLB_EINVAL, "NULL argument");
+  const int64_t nc = s->mesh->ncell;
+  const int q = s->mesh->md.q;
+  *bytes = q == VLB_D3Q39 && s->nc == vlb::kRec39 ? (int64_t)vlb::q39_record_bytes(nc)
+           : s->cellrec                            ? (int64_t)vlb::cell_record_bytes(q, nc)
+                        : (vlb::arith_f64(s->p.precision) ? 8 : 4) * (int64_t)s->nc * s->ncoef;
+  return VLB_OK;
+}
+
 // (for tests, not in vlb.h) how the last launch of vlb_step advanced the simulation (PATH_*)
 int vlb_internal_step_path(const vlb_sim *s) { return s ? s->path : 0; }
 

@@ -462,9 +462,10 @@ struct vlb_sim {
   vlb_params p;
   cudaStream_t stream = nullptr;
   void *d_f = nullptr;        // populations [q][ncell]
-  void *d_coef = nullptr;     // coefficient records, record r at r * nc elements
+  void *d_coef = nullptr;     // coefficient records: record r at r * nc elements, or CellLayout's
+                              // (cellrec), or D3Q39's in groups of 32 cells (Rec39)
   int64_t ncoef = 0;
-  int32_t nc = 0;             // values of a coefficient record
+  int32_t nc = 0;             // values of a coefficient record (CoefLayout's; D3Q39: stored)
   int32_t plane = 0;
   int32_t cellrec = 0;        // FP32, one record per cell: CellLayout, else CoefLayout
   float *d_uw = nullptr;      // with cellrec and moving walls: wall velocities [ncell][dim]

@@ -79,6 +79,7 @@ def load():
         "vlb_time": ([vp], C.c_int64),
         "vlb_sim_layout": ([vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                             C.POINTER(C.c_int64)], C.c_int),
+        "vlb_sim_record_bytes": ([vp, C.POINTER(C.c_int64)], C.c_int),
         "vlb_destroy": ([vp], None),
         "vlb_last_error": ([], C.c_char_p),
         "vlb_totals_noalloc": ([vp, vp], C.c_int),
@@ -266,7 +267,9 @@ class Sim:
     def layout(self):
         a, b, c = C.c_int32(), C.c_int32(), C.c_int64()
         _check(load().vlb_sim_layout(self.h, C.byref(a), C.byref(b), C.byref(c)), "vlb_sim_layout")
-        return {"coef_per_cell": a.value, "plane": bool(b.value), "records": c.value}
+        d = C.c_int64()
+        _check(load().vlb_sim_record_bytes(self.h, C.byref(d)), "vlb_sim_record_bytes")
+        return {"coef_per_cell": a.value, "plane": bool(b.value), "records": c.value, "record_bytes": d.value}
 
     def close(self):
         if getattr(self, "h", None):
