@@ -754,13 +754,29 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   }
 }
 
-// x as FP32 by integer operations, truncated (a conversion instruction would
-// take a turn of the FP64 pipe); below the FP32 range 0, above it NaN
-__device__ __forceinline__ float trunc_f32(double x) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), mag = hi & 0x7fffffffu;
-  const uint32_t b = ((mag - 0x38000000u) << 3) | (lo >> 29);
-  return __uint_as_float((mag < 0x38100000u ? 0u : mag >= 0x47f00000u ? 0x7fc00000u : b) | (hi & 0x80000000u));
+// x 2^-e as FP32 by integer operations, truncated (a conversion instruction would take a turn of
+// the FP64 pipe); below the FP32 range 0, above it NaN. unit: kUnit1 + e 2^20.
+constexpr int32_t kUnit1 = 0x38000000;
+__device__ __forceinline__ float trunc_f32(double x, int32_t unit = kUnit1) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int32_t t = (int32_t)(hi & 0x7fffffffu) - unit;
+  const uint32_t b = ((uint32_t)t << 3) | (lo >> 29);
+  return __uint_as_float((t < 0x00100000 ? 0u : t >= 0x0ff00000 ? 0x7fc00000u : b) | (hi & 0x80000000u));
 }
+// The FP32 part of an FP64 force solve measures m and Phi in units of the power of two below
+// |m|, so that it does what it does at m = 1 for every density (in FP32's own range a density
+// of 1e39 was NaN). An exact scaling, by integer operations alone.
+struct Unit64 {
+  int32_t m, inv;   // units for trunc_f32: of m and Phi, and of 1 / m
+  double one;       // the power of two
+  __device__ __forceinline__ explicit Unit64(double v) {
+    int32_t e = __double2hiint(v) & 0x7ff00000;
+    e = min(max(e, 0x08000000), 0x77000000);   // (2^-895 to 2^881)
+    m = kUnit1 + (e - 0x3ff00000);
+    inv = kUnit1 - (e - 0x3ff00000);
+    one = __hiloint2double(e, 0);
+  }
+};
 
 // The whole local collision in FP64 (see collide_cell). GB300 runs an FP64
 // instruction of a warp in 64 cycles of its quarter SM, so only the FP64 operations
@@ -848,14 +864,15 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
   double Phi[D];
   float lip = 1.0e30f;   // bound on the contraction of one evaluation
   int it = 0;
-  const float mf = trunc_f32(m);
+  const Unit64 un(m);
+  const float mf = trunc_f32(m, un.m);
   if (max_iter >= 4) {
     float qf[D][NQ], Uf[D], Pf[D], df[D], l2 = 0.f, l3 = 0.f, um = 0.f;
-    const float hf = trunc_f32(h2m), hmf = 0.5f * mf;
+    const float hf = trunc_f32(h2m, un.inv), hmf = 0.5f * mf;
 #pragma unroll
     for (int i = 0; i < D; i++) {
       Uf[i] = trunc_f32(st.U[i]);
-      Pf[i] = trunc_f32(Pt[i]);
+      Pf[i] = trunc_f32(Pt[i], un.m);
       df[i] = 0.f;
 #pragma unroll
       for (int k = 0; k < NQ; k++) {
@@ -897,7 +914,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     um *= 1.01f;
     lip = fmaf(0.5f * l2, um, 0.75f * l3 * um * um);
 #pragma unroll
-    for (int i = 0; i < DI; i++) Phi[i] = Pt[i] + (double)df[i];
+    for (int i = 0; i < DI; i++) Phi[i] = fma((double)df[i], un.one, Pt[i]);
   } else {
 #pragma unroll
     for (int i = 0; i < DI; i++) Phi[i] = m * rc[L::FR + i];
@@ -908,7 +925,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
 #pragma unroll 1
   while (it < max_iter) {
     double Ut[D], mono[NQ];
-    float diff = 0.f, pmax = EXT ? fabsf(trunc_f32(Phi[D - 1])) : 0.f;
+    float diff = 0.f, pmax = EXT ? fabsf(trunc_f32(Phi[D - 1], un.m)) : 0.f;
 #pragma unroll
     for (int i = 0; i < D; i++) Ut[i] = fma(Phi[i], h2m, st.U[i]);
 #pragma unroll
@@ -933,8 +950,8 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
           a = fma(rc[L::row(L::QM, NQ, i, k)], mono[k], a);
       }
       const double pn = fma(-hm, a + b, Pt[i]);
-      diff = maxnan(diff, fabsf(trunc_f32(pn - Phi[i])));
-      pmax = maxnan(pmax, fabsf(trunc_f32(pn)));
+      diff = maxnan(diff, fabsf(trunc_f32(pn - Phi[i], un.m)));
+      pmax = maxnan(pmax, fabsf(trunc_f32(pn, un.m)));
       Phi[i] = pn;
     }
     it++;

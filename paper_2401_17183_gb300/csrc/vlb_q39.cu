@@ -605,16 +605,17 @@ __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_it
   for (int i = 0; i < 3; i++)
     Pt[i] = fma(ld(Rec39::HM + 3 * i), Pc[0],
                 fma(ld(Rec39::HM + 3 * i + 1), Pc[1], ld(Rec39::HM + 3 * i + 2) * Pc[2]));
-  const float mf = trunc_f32(m), tolf = (float)tol;
+  const Unit64 un(m);
+  const float mf = trunc_f32(m, un.m), tolf = (float)tol;
   float lip = 1.0e30f;
   int it = 0;
   if (max_iter >= 4) {
     float Uf[3], Pf[3], df[3] = {0.f, 0.f, 0.f}, l2 = 0.f, l3 = 0.f, um = 0.f;
-    const float hf = trunc_f32(h2m), hmf = 0.5f * mf;
+    const float hf = trunc_f32(h2m, un.inv), hmf = 0.5f * mf;
 #pragma unroll
     for (int i = 0; i < 3; i++) {
       Uf[i] = trunc_f32(q.U[i]);
-      Pf[i] = trunc_f32(Pt[i]);
+      Pf[i] = trunc_f32(Pt[i], un.m);
     }
 #pragma unroll 1
     for (int r = 0; r < 3; r++) {
@@ -648,7 +649,7 @@ __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_it
     um *= 1.01f;
     lip = fmaf(0.5f * l2, um, 0.75f * l3 * um * um);
 #pragma unroll
-    for (int i = 0; i < 3; i++) q.Phi[i] = Pt[i] + (double)df[i];
+    for (int i = 0; i < 3; i++) q.Phi[i] = fma((double)df[i], un.one, Pt[i]);
   } else {
 #pragma unroll
     for (int i = 0; i < 3; i++) q.Phi[i] = m * ld(Rec39::FR + i);
@@ -663,8 +664,8 @@ __device__ __forceinline__ bool force39(Cell39 &q, LD ld, double tol, int max_it
 #pragma unroll
     for (int i = 0; i < 3; i++) {
       const double pn = fma(-hm, a[i], Pt[i]);
-      diff = maxnan(diff, fabsf(trunc_f32(pn - q.Phi[i])));
-      pm = maxnan(pm, fabsf(trunc_f32(pn)));
+      diff = maxnan(diff, fabsf(trunc_f32(pn - q.Phi[i], un.m)));
+      pm = maxnan(pm, fabsf(trunc_f32(pn, un.m)));
       q.Phi[i] = pn;
     }
     it++;
