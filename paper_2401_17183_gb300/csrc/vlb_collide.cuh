@@ -785,8 +785,8 @@ struct Unit64 {
 //    polynomial in FP32: its value is of the order of curvature times U^2, so FP32 leaves
 //    an error of about 1e-13 m, which one evaluation in FP64 reduces by the map's
 //    contraction. It is accepted when its change is at most tol max(m, |Phi|), or when a
-//    bound on the contraction times the change is below that by a factor 64 (the
-//    next change, and the error left, are then smaller still). Below four iterations
+//    bound on the contraction times the change is below that by a factor 64; that next
+//    change is then added to first order, in FP32. Below four iterations
 //    allowed: the plain iteration from the rest state's force.
 //  - the test reads the sizes by integer operations on the high words;
 //  - N' is formed from the pair sums and differences, even and odd part once per pair:
@@ -837,7 +837,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     }
   }
   const double m = nref + mdev, im = 1.0 / m, h2m = 0.5 * im, hm = 0.5 * m;
-  const double kf = fma(0.5 * itau, mdev, nref);
+  const double kf = (0.5 * itau) * mdev;
   st.rho = m * rc[L::IJ];
   double hmu[D];
 #pragma unroll
@@ -845,14 +845,15 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     st.U[i] = mu[i] * im;
     hmu[i] = -0.5 * mu[i];
   }
-  // Pc = sum_p (am M s + ad D t) + m G - (n_ref + mdev itau/2) KW - m/2 (CE + (PO1 + LO) U)
+  // Pc = sum_p (am M s + ad D t) + m G - (mdev itau/2) KW - m/2 (CE + (PO1 + LO) U) - n_ref KW,
+  // the last and largest product exact
 #pragma unroll
   for (int i = 0; i < DI; i++) {
     double v = fma(m, rc[L::BODY + i], Pc[i]);
     v = fma(-hm, rc[L::CE + i], v);
 #pragma unroll
     for (int l = 0; l < DI; l++) v = fma(rc[L::PO1 + i * D + l], hmu[l], v);
-    Pc[i] = fma(-kf, rc[L::KW + i], v);
+    Pc[i] = fma(-nref, rc[L::KW + i], fma(-kf, rc[L::KW + i], v));
   }
 #pragma unroll
   for (int i = 0; i < DI; i++) {
@@ -922,6 +923,9 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
   if constexpr (EXT) Phi[2] = Pt[2];
   st.conv = false;
   const float tolf = (float)tol, epsf = (float)(64.0 / 9007199254740992.0);
+  float dl[D];
+#pragma unroll
+  for (int i = 0; i < D; i++) dl[i] = 0.f;
 #pragma unroll 1
   while (it < max_iter) {
     double Ut[D], mono[NQ];
@@ -950,7 +954,8 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
           a = fma(rc[L::row(L::QM, NQ, i, k)], mono[k], a);
       }
       const double pn = fma(-hm, a + b, Pt[i]);
-      diff = maxnan(diff, fabsf(trunc_f32(pn - Phi[i], un.m)));
+      dl[i] = trunc_f32(pn - Phi[i], un.m);
+      diff = maxnan(diff, fabsf(dl[i]));
       pmax = maxnan(pmax, fabsf(trunc_f32(pn, un.m)));
       Phi[i] = pn;
     }
@@ -962,6 +967,33 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     }
   }
   st.iters = it;
+  // What the accepted step leaves, the next change, to first order: -m/2 Q'(U~) dU~ of the last
+  // change, in FP32 (its error is 2^-22 of a change below tol / 64). Without it 6 to 15% of the
+  // populations of a step were a last bit off those of a solve to the end, now 0.2 to 1%.
+  if (st.conv) {
+    float x[D], dm[NQ];
+    const float hf = trunc_f32(h2m, un.inv), hmf = 0.5f * mf;
+#pragma unroll
+    for (int i = 0; i < D; i++) {
+      x[i] = fmaf(trunc_f32(Phi[i], un.m), hf, trunc_f32(st.U[i]));
+      dl[i] *= hf;
+    }
+#pragma unroll
+    for (int k = 0; k < D; k++)
+#pragma unroll
+      for (int l = 0; l < D; l++) {
+        if (k <= l) dm[sym<D>(k, l)] = fmaf(x[k], dl[l], dl[k] * x[l]);
+        if (k != l) dm[NS + offd<D>(k, l)] = x[k] * fmaf(x[k], dl[l], 2.f * dl[k] * x[l]);
+      }
+#pragma unroll
+    for (int i = 0; i < DI; i++) {
+      float v = 0.f;
+#pragma unroll
+      for (int k = 0; k < NQ; k++)
+        if (map_mono<EXT, D>(k)) v = fmaf(trunc_f32(rc[L::row(L::QM, NQ, i, k)]), dm[k], v);
+      Phi[i] = fma((double)(-hmf * v), un.one, Phi[i]);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
   if constexpr (FINAL) {
