@@ -326,6 +326,7 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
     plane = mesh->stats.invariant_fast_axis != 0 && mesh->md.n[dim - 1] > 1;
   }
   s->plane = plane ? 1 : 0;
+  cudaDeviceGetAttribute(&s->nsm, cudaDevAttrMultiProcessorCount, mesh->device);
   s->ncoef = plane ? mesh->ncell / mesh->md.n[dim - 1] : mesh->ncell;
   const bool f16 = params->precision == VLB_F16 || params->precision == VLB_BF16;
   if (params->reference == VLB_REF_REST && f16) {

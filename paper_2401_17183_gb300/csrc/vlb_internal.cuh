@@ -467,6 +467,7 @@ struct vlb_sim {
   int64_t ncoef = 0;
   int32_t nc = 0;             // values of a coefficient record (CoefLayout's; D3Q39: stored)
   int32_t plane = 0;
+  int32_t nsm = 152;          // SMs of the device
   int32_t cellrec = 0;        // FP32, one record per cell: CellLayout, else CoefLayout
   float *d_uw = nullptr;      // with cellrec and moving walls: wall velocities [ncell][dim]
   float *d_ro = nullptr;      // with ref_rest: the storage reference per column and pair (RefCtx::o)

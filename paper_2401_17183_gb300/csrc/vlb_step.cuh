@@ -191,7 +191,13 @@ template <int Q, typename S, typename R, int T, bool PLANE, bool REFOFS>
 constexpr size_t step_smem(int records) {
   return sizeof(StepSmem<Q, S, R, T>) + (PLANE ? sizeof(R) * kStages * staged_record<Q, R, REFOFS>() * records : 0);
 }
-// linear tiles of plane-record meshes: rows of at least this many cells
+// Linear tiles of plane-record meshes: rows of at least this many cells. us a step of 500 K
+// D3Q19 cells, tiles along the rows / linear: FP32, rows of 16 cells 52.9 / 18.6, of 40 28.7 /
+// 18.3, of 100 21.0 / 18.2; FP16 65.1 / 23.0, 36.4 / 22.5, 26.8 / 23.3; FP64 958 / 288, 481 /
+// 286, 380 / 291; D2Q9 (FP32) 39.6 / 13.6, 19.9 / 13.3, 13.1 / 13.1. At 16 a tile stages nine
+// records (FP64: 95 KB a block, two blocks per SM). Shorter rows would gain as well (8 cells, FP32:
+// 102.7 / 20.8) until their records fill an SM (FP64 at 8: 125 KB a block, at 4: 187 KB); no mesh
+// family here has them, and they keep the tiles that take any length.
 constexpr int64_t kLinearRow = 16;
 
 // a 16-bit storage value from its bit pattern
@@ -754,7 +760,7 @@ cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
   const vlb_mesh *m = sim->mesh;
   // one record per cell on a mesh of at most one full tile per SM: tiles of one
   // warp, so that every SM has work (2,048 D2Q9 cells, FP32: 3.2 -> 2.9 us a step)
-  const bool small = !sim->plane && m->ncell <= (int64_t)kStepThreads * 152;
+  const bool small = !sim->plane && m->ncell <= (int64_t)kStepThreads * sim->nsm;
   // 32-bit indexing when every population offset fits
   const bool i32 = (int64_t)Q * m->ncell < ((int64_t)1 << 31);
   // plane records and rows that are not whole tiles: linear tiles, unless the rows
