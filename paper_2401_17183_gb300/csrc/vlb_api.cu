@@ -383,6 +383,18 @@ int vlb_init(const vlb_mesh *mesh, const vlb_params *params, const double *rho, 
     vlb_destroy(s);
     return fail(VLB_ECUDA, "coefficient pack: %s", cudaGetErrorString(e));
   }
+  if (s->ref_rest && mesh->extruded) {
+    int flag = 0;
+    e = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream);
+    if (e == cudaSuccess) e = vlb::launch_zero_entries(s, s->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) {
+      vlb_destroy(s);
+      return fail(VLB_ECUDA, "record check: %s", cudaGetErrorString(e));
+    }
+    s->zero_ext = flag & vlb::ERR_ZERO_EXT ? 0 : 1;
+  }
   int rc = upload_fields(s, rho, u);
   if (rc == VLB_OK) rc = check_kernel_flags(s->d_err, s->stream);
   if (rc) {

@@ -64,8 +64,12 @@ struct CollideState {
 //    of PO1, row 2 of the map and CE^2, KW^2 are zero);
 //  - of the map's twelve monomials, those odd in U~^2 have coefficient zero.
 // The steps are bound by issue (FP32, 16 bits) and by the FP64 pipe: 100 steps with reset and
-// moments of D3Q19 channels, FP64 64^3 22.2 -> 17.0 ms, FP16 128^3 9.0 -> 8.1 ms, FP32 75 x 67
-// x 101 2.9 -> 2.6 ms.
+// moments of D3Q19 channels, FP64 64^3 22.2 -> 17.0 ms, FP32 75 x 67 x 101 2.9 -> 2.6 ms.
+// 16-bit storage (FR0) keeps the order of every sum and with it the rounding of every
+// population: where all of these entries are zero in the FP32 records (vlb_sim::zero_ext,
+// k_zero_entries) it leaves out the terms that they multiply, pair 3 and row and column 2
+// of the map among them, and a product with zero changes no sum. FP16 128^3: 69.9 -> 60.6 us
+// a step over both parities (55.4 with the sums regrouped as above, and other roundings).
 template <bool EXT, int D>
 __device__ constexpr bool map_mono(int s) {   // has monomial s of a chord step a coefficient?
   return !EXT || !(s == sym<D>(0, 2) || s == sym<D>(1, 2) || s == D * (D + 1) / 2 + offd<D>(0, 2) ||
@@ -528,12 +532,13 @@ struct MomentWeights<9, R> {
 // and then mn = mdev - sum_a RR_a. Every term is formed relative to its own
 // size, and the identity behind the final pass holds for whatever J it uses,
 // as long as RR, their sum and mn use the same one.
-template <int Q, typename R, bool REST, bool RREC, bool EXT, typename RC>
+template <int Q, typename R, bool REST, bool RREC, bool EXT, bool FR0, typename RC>
 __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R mdev, R mn,
                                         R nref, R h2m, R rho, R itau, const R (&U)[Lat<Q>::D],
                                         const R (&Phi)[Lat<Q>::D], R (&dp)[Q]) {
   using L = CoefLayout<Q>;
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS;
+  constexpr bool ZERO = EXT && FR0, GRP = EXT && !FR0;   // see map_mono
   static_assert(RREC || !REST, "rest-relative storage keeps the rest state in the record");
   R gh[NS];
 #pragma unroll
@@ -655,7 +660,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   for (int i = 0; i < D; i++)
 #pragma unroll
     for (int j = 0; j < D; j++) dP[i][j] = R(0);
-  if constexpr (EXT) {
+  if constexpr (GRP) {
     // pairs with the same coefficients together: xo of pairs 6 and 7 is T_02 +- T_20, of
     // pairs 8 and 9 T_12 +- T_21, and the axis weight twice the diagonal one. In units of
     // 2 r6w2 (taken into a9 below); column 2 is zero.
@@ -678,6 +683,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
     for (int i = 0; i < D; i++) P01[i] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int p = 1; p <= H; p++) {
+      if (ZERO && p == 3) continue;
       const R df = (lat_nnz<Q>(p) == 1 ? r6w1 : r6w2) * xo[p];
       const float2 am01 = rc.v2(L::mp(p, 0));
 #pragma unroll
@@ -686,7 +692,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
         if (ci == 0) continue;
         const R sdf = ci > 0 ? df : -df;
         P01[i] = __ffma2_rn(am01, bcast2(sdf), P01[i]);
-        if constexpr (D == 3) dP[i][2] = fmar(rc[L::mp(p, 2)], sdf, dP[i][2]);
+        if constexpr (D == 3 && !EXT) dP[i][2] = fmar(rc[L::mp(p, 2)], sdf, dP[i][2]);
       }
     }
 #pragma unroll
@@ -698,7 +704,7 @@ __device__ __forceinline__ void form_np(const R (&d)[Q], const RC &rc, R m, R md
   R tr = dP[0][0];
 #pragma unroll
   for (int i = 1; i < (EXT ? 2 : D); i++) tr += dP[i][i];
-  const R J = EXT ? rc[L::J] * (R(2) * r6w2) : rc[L::J];   // J times the unit of dP
+  const R J = GRP ? rc[L::J] * (R(2) * r6w2) : rc[L::J];   // J times the unit of dP
   // E_p = 9 w J c.dP.c - 3 w J tr dP; O_p = 3 w c.Phi (Eq. 31, 1/T0 = 3)
   const R a9_1 = (R(9) * lat_w<Q, R>(1)) * J, a9_2 = (R(9) * lat_w<Q, R>(Lat<Q>::H)) * J;
   const R tr3 = tr * R(1.0 / 3.0);
@@ -1146,6 +1152,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   constexpr int D = Lat<Q>::D, H = Lat<Q>::H, NS = L::NS, NQ = L::NQ;
   static_assert(D == 2 || NQ % 4 == 0, "row 2 of the chord step is read in 16-byte quads");
   static_assert(!EXT || Q == 19, "extruded meshes are D3Q19's");
+  constexpr bool ZERO = EXT && FR0, GRP = EXT && !FR0;   // see map_mono
   constexpr int DI = EXT ? 2 : D;   // components of Phi that are iterated
   const R epsn = sizeof(R) == 4 ? R(64.0 / 16777216.0) : R(64.0 / 9007199254740992.0);
   // pair sums s_p = d_p + d_pbar and differences t_p = d_p - d_pbar
@@ -1156,11 +1163,11 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   for (int p = 1; p <= H; p++) {
     sp[p] = d[p] + d[p + H];
     tp[p] = d[p] - d[p + H];
-    if constexpr (!EXT) mdev += sp[p];
+    if constexpr (!GRP) mdev += sp[p];
   }
   // sums over the pairs that share link coefficients
   R sg[4], tg[4];
-  if constexpr (EXT) {
+  if constexpr (GRP) {
     sg[0] = sp[1] + (sp[6] + sp[7]);
     sg[1] = sp[2] + (sp[8] + sp[9]);
     tg[0] = tp[1] + (tp[6] + tp[7]);
@@ -1188,7 +1195,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
 #pragma unroll
   for (int i = 0; i < D; i++) {
     R s = R(0);
-    if constexpr (EXT) {
+    if constexpr (GRP) {
       s = i == 0   ? tg[0] + (tg[2] + tg[3])
           : i == 1 ? tg[1] + (tg[2] - tg[3])
                    : tp[3] + ((tp[6] - tp[7]) + (tp[8] - tp[9]));
@@ -1225,9 +1232,10 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     float2 sa = make_float2(s[0], s[1]), sb = make_float2(0.f, 0.f);
     float s2a = D == 3 && !EXT ? s[D - 1] : 0.f, s2b = 0.f;
 #pragma unroll
-    for (int k = 1; k <= (EXT ? 4 : H); k++) {
-      const int p = EXT && k > 2 ? k + 1 : k;
-      const R sk = EXT ? sg[(k - 1) & 3] : sp[p], tk = EXT ? tg[(k - 1) & 3] : tp[p];
+    for (int k = 1; k <= (GRP ? 4 : H); k++) {
+      if (ZERO && k == 3) continue;
+      const int p = GRP && k > 2 ? k + 1 : k;
+      const R sk = GRP ? sg[(k - 1) & 3] : sp[p], tk = GRP ? tg[(k - 1) & 3] : tp[p];
       const float4 q = rc.v4(L::mp(p, 0));   // am M^0, am M^1, ad D^0, ad D^1
       float2 &acc = (k & 1) ? sa : sb;
       acc = __ffma2_rn(make_float2(q.x, q.y), bcast2(sk), acc);
@@ -1280,7 +1288,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
   // stored), relative to the rest state 4e-4 (FP16, 100 steps of a 128^3 channel).
   R Phi[D];
 #pragma unroll
-  for (int i = 0; i < D; i++) Phi[i] = (max_iter >= 4 && !FR0) || i >= DI ? Pt[i] : m * rc[L::FR + i];
+  for (int i = 0; i < D; i++) Phi[i] = (max_iter >= 4 && !FR0) || (GRP && i >= DI) ? Pt[i] : m * rc[L::FR + i];
   st.conv = false;
   int it = 0;
   while (it < max_iter) {
@@ -1312,7 +1320,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
           if (!map_mono<EXT, D>(s2) || !map_mono<EXT, D>(s2 + 1)) {
             // one monomial of the two (extruded meshes: never none)
             const int s1 = map_mono<EXT, D>(s2) ? s2 : s2 + 1;
-            float2 &acc = (s2 & 2) ? a01a : a01b;
+            float2 &acc = (GRP ? (s2 & 2) != 0 : (s1 & 1) == 0) ? a01a : a01b;
             acc = __ffma2_rn(rc.v2(L::QM + 2 * s1), bcast2(mono[s1]), acc);
             continue;
           }
@@ -1342,7 +1350,8 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     }
     it++;
     // converged when the change is at most max(tol max(m, |Phi|), 64 eps |Phi|)
-    R diff = R(0), pmax = EXT ? absr(Phi[D - 1]) : R(0);
+    R diff = ZERO ? absr(Pt[D - 1] - Phi[D - 1]) : R(0), pmax = EXT ? absr(Phi[D - 1]) : R(0);
+    if constexpr (ZERO) Phi[D - 1] = Pt[D - 1];
 #pragma unroll
     for (int i = 0; i < DI; i++) {
       const R pn = fmar(-hm, a[i], Pt[i]);
@@ -1356,7 +1365,7 @@ __device__ __forceinline__ void collide_f32(const R (&d)[Q], const RC &rc, R nre
     }
   }
   st.iters = it;
-  if (FINAL) form_np<Q, R, REST, RREC, EXT, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
+  if (FINAL) form_np<Q, R, REST, RREC, EXT, FR0, RC>(d, rc, m, mdev, mn, nref, h2m, st.rho, itau, st.U, Phi, dp);
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
 }

@@ -537,6 +537,53 @@ __global__ void k_pack_coef(const PackArgs a, R *coef) {
   for (int i = 0; i < D; i++) out[L::UW + i] = static_cast<R>(uw[i]);
 }
 
+// Are the entries that the collision of extruded meshes with 16-bit storage leaves out (see
+// map_mono) zero in every record? Three groups may keep what is left of FP64 sums whose terms
+// cancel, 2^-45 of their block at most (1e-16 of it on the channels here): column 2 of
+// H - I and of PO1, and the map's monomials odd in U~^2. A product with such an entry is below the
+// last FP32 bit of a sum whose terms do not cancel to 2^-20 of themselves. And H - I may
+// keep a last bit of its diagonal, which is added to one. Raises ERR_ZERO_EXT where not.
+__global__ void k_zero_entries(const float *coef, int64_t nrec, int64_t stride, int *err) {
+  using L = CoefLayout<19>;
+  constexpr int D = L::D, H = L::H, NQ = L::NQ;
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nrec) return;
+  const float *c = coef + r * stride;
+  // the largest of the zeros, of the remainders of the map and of PO1, and of those blocks
+  float zero = 0.0f, left = 0.0f, map = 0.0f, pleft = 0.0f, po = 0.0f;
+  auto see = [&](float &m, int k) { m = maxnan(m, fabsf(c[k])); };
+  for (int i = 0; i < 2; i++) {
+    see(zero, L::GH + sym<D>(i, 2));
+    for (int j = 0; j < D; j++) see(j < 2 ? po : pleft, L::PO1 + i * D + j);
+    see(zero, L::row(L::HM, D, 2, i));
+    see(zero, L::mp(3, i));
+    see(zero, L::dk(3, i));
+    for (int k = 0; k < NQ; k++) see(map_mono<true, D>(k) ? map : left, L::row(L::QM, NQ, i, k));
+  }
+  for (int j = 0; j < D; j++) see(zero, L::PO1 + 2 * D + j);
+  for (int k = 0; k < NQ; k++) see(zero, L::row(L::QM, NQ, 2, k));
+  for (int q = 1; q <= H; q++) {
+    see(zero, L::mp(q, 2));
+    see(zero, L::dk(q, 2));
+  }
+  see(zero, L::KW + 2);
+  see(zero, L::KWL + 2);
+  see(zero, L::CE + 2);
+  see(zero, L::SR + 2);
+  float col = 0.0f;
+  for (int i = 0; i < 2; i++) see(col, L::row(L::HM, D, i, 2));
+  const float tiny = 2.8421709e-14f;   // 2^-45
+  const bool ok = zero == 0.0f && left <= tiny * map && pleft <= tiny * po && col <= tiny &&
+                  fabsf(c[L::row(L::HM, D, 2, 2)]) <= 1.4901161e-8f;
+  if (!ok) atomicOr(err, ERR_ZERO_EXT);
+}
+
+cudaError_t launch_zero_entries(const vlb_sim *sim, cudaStream_t s) {
+  k_zero_entries<<<(unsigned)((sim->ncoef + 127) / 128), 128, 0, s>>>(static_cast<const float *>(sim->d_coef),
+                                                                     sim->ncoef, sim->nc, sim->d_err);
+  return cudaGetLastError();
+}
+
 // CellLayout records (FP32, one per cell): the entries kept are sums over the
 // links formed in FP64 (about 250 operations; the whole record takes ten times that)
 // and rounded; the rest state's force, the start value of the chord iteration, is

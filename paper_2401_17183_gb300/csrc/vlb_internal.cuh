@@ -474,6 +474,7 @@ struct vlb_sim {
   int64_t t = 0;
   int32_t path = 0;           // PATH_*: how the last launch of vlb_step advanced it
   double nref = 0.0;          // populations are stored as N_a - w_a nref, nref = rho_0 J_ref
+  int32_t zero_ext = 0;       // 16-bit storage, extruded mesh: the entries that follow are zero (k_zero_entries)
   int32_t ref_rest = 0;       // 16-bit storage relative to the local rest state
   int *d_err = nullptr;       // sticky kernel error flags
   double *d_fields = nullptr; // moments output staging: rho [ncell], u and u~ [ncell][dim]
@@ -532,7 +533,7 @@ inline RefCtx make_ref(const vlb_sim *sim) {
 }
 
 // error flags raised by kernels
-enum : int { ERR_NOCONV = 1, ERR_NONFINITE = 2, ERR_GEOM = 4, ERR_BARRIER = 8 };
+enum : int { ERR_NOCONV = 1, ERR_NONFINITE = 2, ERR_GEOM = 4, ERR_BARRIER = 8, ERR_ZERO_EXT = 16 };
 // a simulation's d_err: the error flags, and apart from them the barrier
 // counter of the multi-step kernel
 constexpr int kErrWords = 64, kBarrierWord = 32;
@@ -546,6 +547,8 @@ cudaError_t launch_geometry(const vlb_mesh *m, int *d_err, cudaStream_t s);
 cudaError_t launch_mesh_stats(const vlb_mesh *m, double *d_partial, int64_t nblk, cudaStream_t s);
 cudaError_t launch_plane_check(const vlb_mesh *m, int *d_flag, cudaStream_t s);
 cudaError_t launch_pack_coef(const vlb_sim *sim, cudaStream_t s);
+// raises ERR_ZERO_EXT where a record of a D3Q19 extruded mesh has other than zero (k_zero_entries)
+cudaError_t launch_zero_entries(const vlb_sim *sim, cudaStream_t s);
 cudaError_t launch_init(const vlb_sim *sim, const double *d_rho, const double *d_u, cudaStream_t s);
 cudaError_t launch_step(const vlb_sim *sim, int odd, cudaStream_t s);
 // up to nsteps steps of a small mesh in one launch; *done: how many (0: none, not small), and

@@ -81,7 +81,7 @@ struct StepArgs {
   // plane records, linear tiles: records staged per tile at most (0: tiles
   // along the fastest axis)
   int32_t nrec;
-  int32_t ext;   // plane records of an extruded mesh
+  int32_t ext;   // plane records of an extruded mesh (16-bit storage: vlb_sim::zero_ext)
 };
 
 constexpr int kStepThreads = 128;
@@ -154,7 +154,8 @@ __host__ __device__ constexpr bool slow_move(int a) {
 // (128 registers; 3% faster than 3 blocks on even steps, 0.3% faster over both
 // parities; a record per cell needs the registers for itself), 2 for FP64. Extruded meshes
 // need fewer registers; FP32 stays at 3 (four fit: 20.7 us a step at 75 x 67 x 101, cut
-// for 4 blocks 21.4, for 5 21.6)
+// for 4 blocks 21.4, for 5 21.6), 16-bit storage at 4 (FP16 128^3 and 100 x 96 x 111, cut for 4
+// blocks 60.6 and 40.5 us a step, for 5 61.1 and 38.9, for 6 60.4 and 40.8)
 template <typename R, typename S = R, bool PLANE = true>
 constexpr int step_min_blocks() {
   return sizeof(R) == 4 ? (sizeof(S) == 2 && PLANE ? 4 : 3) : 2;
@@ -708,7 +709,7 @@ inline StepArgs make_step_args(const vlb_sim *sim, int T = kStepThreads, bool li
   const int dim = m->md.dim;
   const int64_t nfast = dim == 3 ? m->md.n[2] : m->md.n[1];
   a.per_block = 0;
-  a.ext = sim->plane && m->extruded ? 1 : 0;
+  a.ext = storage_bytes(sim->p.precision) == 2 ? sim->zero_ext : sim->plane && m->extruded ? 1 : 0;
   a.nrec = lin ? (int32_t)((T - 1) / nfast + 2) : 0;
   if (sim->plane && !lin) {
     a.ntf = (int32_t)((nfast + T - 1) / T);
@@ -815,11 +816,11 @@ cudaError_t launch_step_t(const vlb_sim *sim, int odd, cudaStream_t s) {
   };
   const std::true_type yes;
   const std::false_type no;
-  // extruded meshes: FP32 and FP64 storage (16-bit storage keeps the sums of the general form,
-  // see FR0 in collide_f32)
+  // extruded meshes: every storage but 16 bits relative to the uniform reference, which meshes
+  // with plane records have little use for
   auto pick = [&](auto plane_tag, auto ref_tag, auto par_tag) {
     constexpr bool P = decltype(plane_tag)::value;
-    if constexpr (Q == 19 && P && sizeof(S) > 2) {
+    if constexpr (Q == 19 && P && (decltype(ref_tag)::value || sizeof(S) > 2)) {
       if (a.ext) {
         pick_ext(plane_tag, ref_tag, par_tag, yes);
         return;
