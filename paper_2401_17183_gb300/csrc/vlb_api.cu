@@ -413,13 +413,19 @@ int vlb_reset(vlb_sim *s, const double *rho, const double *u) {
   return VLB_OK;
 }
 
+// (the runtime keeps a failed launch's error until it is asked for: the next call would report it)
+static int step_failed(cudaError_t e) {
+  cudaGetLastError();
+  return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(e));
+}
+
 int vlb_step(vlb_sim *s, int64_t nsteps) {
   if (!s) return fail(VLB_EINVAL, "NULL sim");
   if (nsteps < 0) return fail(VLB_EINVAL, "nsteps < 0");
   for (int64_t k = 0; k < nsteps;) {
     int64_t done = 0;
     const cudaError_t es = vlb::launch_steps_small(s, nsteps - k, &done, s->stream);
-    if (es != cudaSuccess) return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(es));
+    if (es != cudaSuccess) return step_failed(es);
     if (done > 0) {
       s->t += done;
       k += done;
@@ -427,7 +433,7 @@ int vlb_step(vlb_sim *s, int64_t nsteps) {
     }
     cudaError_t e = s->mesh->md.q == VLB_D3Q39 ? vlb::q39_step(s, (int)(s->t & 1), s->stream)
                                                : vlb::launch_step(s, (int)(s->t & 1), s->stream);
-    if (e != cudaSuccess) return fail(VLB_ECUDA, "step launch: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess) return step_failed(e);
     s->path = vlb::PATH_STEP;
     s->t++;
     k++;
