@@ -27,8 +27,9 @@
  *     the legacy default stream). vlb_step is asynchronous; calls that
  *     return host data synchronise the stream first.
  *   - Errors raised inside kernels (a fixed-point solve that hit its
- *     iteration cap) are sticky: they are reported by the next call that
- *     synchronises (vlb_sync, vlb_moments, vlb_get_state).
+ *     iteration cap, a wait that ran out in vlb_step) are sticky: they are
+ *     reported by the next call that synchronises (vlb_sync, vlb_moments,
+ *     vlb_get_state).
  */
 #ifndef VLB_H
 #define VLB_H
@@ -54,7 +55,10 @@ enum vlb_status {
  * speeds up to 3. Periodic meshes only (every axis at least 3 cells, no
  * periodic rotation), FP64 populations, per-cell geometry; no batches and no
  * vlb_totals_noalloc. The paper names no velocity set with this property;
- * the weights are those of the published D3Q39 set. */
+ * the weights are those of the published D3Q39 set. A simulation keeps a
+ * record of 1,544 bytes per cell for its force map where vlb_init finds room
+ * for it beside the staging of the fields and the state, else 96 bytes per
+ * cell, at several times the time per step. */
 enum vlb_lattice_kind { VLB_D2Q9 = 9, VLB_D3Q19 = 19, VLB_D3Q39 = 39 };
 enum vlb_bc { VLB_PERIODIC = 0, VLB_WALL = 1 };
 enum vlb_precision { VLB_F64 = 0, VLB_F32 = 1, VLB_F16 = 2, VLB_BF16 = 3 };
@@ -179,7 +183,13 @@ int vlb_reset(vlb_sim *sim, const double *rho, const double *u);
 
 /* Advance nsteps time steps (Eq. 12 with Eq. 22), one fused pull-collide-push
  * kernel launch per step, alternating the two in-place A-A layouts. Returns
- * after queueing the launches. */
+ * after queueing the launches. VLB_F64 and VLB_F32 meshes of D2Q9 or D3Q19
+ * whose cells fit on the device at once (65,536 cells at most) take up to 1024
+ * steps in one launch; the populations are those of single steps, bit for bit. The
+ * blocks of such a launch wait for one another, each for at most one second
+ * a step; one that gives up raises a sticky error, which the next call that
+ * synchronises reports as VLB_ECUDA (the state is then undefined until
+ * vlb_reset or vlb_set_state). Errors: VLB_EINVAL, VLB_ECUDA. */
 int vlb_step(vlb_sim *sim, int64_t nsteps);
 
 /* Synchronise the stream and report any sticky kernel error. */

@@ -64,7 +64,9 @@ int vlb_nn_mse(vlb_nn *net, const float *d_y, const float *d_target, float *d_dy
                double *loss);
 /* Gradients of the parameters for dL/dy = d_dy, through the activations of the
  * last forward call (replaces any previous gradients). Gradients are FP32; on
- * the tensor cores each is the exact sum of three bfloat16 operands. */
+ * the tensor cores each is the exact sum of three bfloat16 operands where it is
+ * at least 2^-109 in size (below, its low bits fall under bfloat16's smallest
+ * value). */
 int vlb_nn_backward(vlb_nn *net, const float *d_dy, int32_t batch);
 int vlb_nn_get_grads(const vlb_nn *net, float *host);
 /* One Adam step (step index t >= 1) on the FP32 master parameters; the

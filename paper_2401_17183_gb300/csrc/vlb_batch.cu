@@ -4,8 +4,10 @@
 // of a single launch of k_step_batch, which reads its member's kernel
 // arguments from a device array. The block shape (tile width and the
 // resident blocks the registers are cut for) and the run length are chosen
-// by timing (vlb_batch_tune). The per-cell work is that of vlb_step, so a
-// batch reproduces the members' individual steps bit for bit. Whole runs of
+// by timing (vlb_batch_tune). The per-cell work is that of vlb_step, and a
+// batch reproduces the members' individual steps bit for bit; small members' own
+// calls of several steps run another kernel (vlb_small.cuh), whose populations the
+// tests hold to be those of the step kernel bit for bit in every form. Whole runs of
 // 32 steps replay a CUDA graph of 32 kernel nodes (alternating A-A parity).
 #include <algorithm>
 #include <new>

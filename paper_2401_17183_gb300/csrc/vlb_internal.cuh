@@ -150,7 +150,7 @@ struct CoefLayout {
   // those deviations over all Q directions, and RW + p the weight of the rest
   // state, w_p (1 + x_p). Both follow from J and g^ij; with one record per
   // cell the step recomputes them rather than streaming them (see
-  // rest_state), so a per-cell record is read up to RR only.
+  // form_np), so a per-cell record is read up to RR only.
   static constexpr int RR = round4(QM + D * NQ);
   static constexpr int RW = RR + round4(H + 2);
   // wall velocity U_w^i (read in the wall cells of moving walls only), in the
@@ -192,7 +192,8 @@ struct CoefLayout {
   // every record and group starts on a 16-byte boundary. One record per
   // column (PLANE) holds everything; one record per cell ends at RR (the rest
   // state is formed from J and g^ij, the 16-bit rest-relative block needs
-  // plane mode), which for D3Q19 FP32 is 544 bytes, 17 whole 32-byte sectors.
+  // plane mode): 136 values of D3Q19, read so by FP64 and 16-bit storage (1,088 and
+  // 544 bytes, whole 32-byte sectors). FP32 storage keeps CellLayout's 80 instead.
   template <typename R, bool PLANE = true>
   static constexpr int stride() {
     return PLANE ? round4(NC) : RR;

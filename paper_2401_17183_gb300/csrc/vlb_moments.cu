@@ -548,7 +548,9 @@ __global__ void __launch_bounds__(kMomThreads) k_totals_cells(const TotArgs a, d
 // mesh without rotations. The stored deviations are added without rounding error
 // as hi + lo pairs in FP32 (TwoSum: six FP32 operations, a fortieth of an FP64 addition's
 // time here), and only B^i, their products with the tangents and the sums over cells
-// are FP64 (31 K D2Q9 cells: 17.4 -> 11.5 us; 492 K D3Q19 cells: 240 -> 94 us). The reference's part of B^i, n_ref sum_a c^i_a w_a (1 + [p + c_a inside] + [p - c_a
+// are FP64 (31 K D2Q9 cells: 17.4 -> 11.5 us; 492 K D3Q19 cells: 240 -> 94 us). Against 113-bit sums of
+// the stored values the mass is off by 6e-17 (FP64 sums of N_a 1.7e-16) and P by 5e-18 of the
+// terms' sizes (1.6e-15). The reference's part of B^i, n_ref sum_a c^i_a w_a (1 + [p + c_a inside] + [p - c_a
 // behind a wall]), vanishes away from walls.
 template <int Q, typename S, bool ODD>
 __global__ void __launch_bounds__(kMomThreads) k_totals_cells_f32(const TotArgs a, double *partial) {

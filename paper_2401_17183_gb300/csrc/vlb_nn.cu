@@ -574,8 +574,7 @@ int conv(const vlb_nn *n, const NNLayer &l, const T *in, int64_t ibs, const void
     const dim3 hg((unsigned)((HW + 255) / 256), (unsigned)B, (unsigned)((l.cout + NCO - 1) / NCO));
     if (bf)
       chain(nn::k_head<T, __nv_bfloat16, NCO>, hg, dim3(128), 0, in, ibs, (const __nv_bfloat16 *)w, bias,
-            (float *)out, obs, l.cin,
-                                                    l.cout, HW);
+            (float *)out, obs, l.cin, l.cout, HW);
     else
       chain(nn::k_head<T, float, NCO>, hg, dim3(128), 0, in, ibs, (const float *)w, bias, (float *)out, obs, l.cin,
             l.cout, HW);
@@ -726,8 +725,7 @@ int layer_backward(vlb_nn *n, int li, View in, View out, const GradSrc &src, con
         const T *act = A + out.off;
         auto launch = [&](auto kern) {
           chain(kern, grid, dim3(128), 0, G + src.g.off, src.g.bs, G + src.gp.off, src.gp.bs, act, out.bs, n->planes,
-                plane,
-                              (int)npos, n->bsum, l.h, l.w, B);
+                plane, (int)npos, n->bsum, l.h, l.w, B);
         };
         if (src.mode == 0)
           launch(nn::k_mask_split<0>);
@@ -753,8 +751,7 @@ int layer_backward(vlb_nn *n, int li, View in, View out, const GradSrc &src, con
         default: NN_CU(launch_wgrad<128>(l, x, in.bs, n->planes, npos, plane, n->dwp, nbk, ng, ns, B, n->d_err)); break;
       }
       chain(nn::k_sum_parts, dim3(nn::nblk(nw + l.cout)), dim3(256), 0, n->dwp, ns * nn::wg_groups(cb), nw, n->bsum,
-            blocks, l.cout,
-                                                      n->g + l.woff);
+            blocks, l.cout, n->g + l.woff);
       NN_CU(cudaGetLastError());
       if (gin) {
         float *o = G + gin->off;
@@ -787,9 +784,9 @@ template <int NCO>
 void launch_head_bwd(vlb_nn *n, const float *d_dy, int64_t ybs, int B) {
   const NNLayer &l = n->L[10];
   const int64_t npos = nn::Padded{l.h, l.w, B}.positions();
-  chain(nn::k_head_bwd<NCO>, dim3((unsigned)plane_blocks(n, l.cin, npos), (unsigned)(l.cin / 8)), dim3(128), 0, 
-      d_dy, ybs, (const __nv_bfloat16 *)n->pc + l.woff, (const __nv_bfloat16 *)n->act + n->t1.off, n->t1.bs, n->planes,
-      npos * l.cin, (int)npos, n->bsum, n->hp, l.h, l.w, B);
+  chain(nn::k_head_bwd<NCO>, dim3((unsigned)plane_blocks(n, l.cin, npos), (unsigned)(l.cin / 8)), dim3(128), 0, d_dy,
+        ybs, (const __nv_bfloat16 *)n->pc + l.woff, (const __nv_bfloat16 *)n->act + n->t1.off, n->t1.bs, n->planes,
+        npos * l.cin, (int)npos, n->bsum, n->hp, l.h, l.w, B);
 }
 
 template <typename T>
@@ -809,9 +806,8 @@ int backward_t(vlb_nn *n, const float *d_dy, int B) {
     }
     NN_CU(cudaGetLastError());
     const int64_t nw = (int64_t)n->co * L[10].cin + n->co;
-    chain(nn::k_sum_parts, dim3(nn::nblk(nw)), dim3(256), 0, n->hp, plane_blocks(n, L[10].cin, nn::Padded{n->H, n->W,
-          B}.positions()), nw,
-                                           nullptr, 0, 0, n->g + L[10].woff);
+    const int blocks = plane_blocks(n, L[10].cin, nn::Padded{n->H, n->W, B}.positions());
+    chain(nn::k_sum_parts, dim3(nn::nblk(nw)), dim3(256), 0, n->hp, blocks, nw, nullptr, 0, 0, n->g + L[10].woff);
     NN_CU(cudaGetLastError());
   } else {
     NN_TRY(conv_bwd_weight<T>(n, L[10], A + n->t1.off, n->t1.bs, d_dy, ybs, B));

@@ -3,8 +3,9 @@
 // the input and gradient with respect to the weights.
 //
 // Operands are bfloat16 and accumulators FP32 in tensor memory. Gradients of
-// activations are FP32: each is split exactly into three bfloat16 planes
-// (hi + mid + lo, 24 significant bits), and since the other operand of either
+// activations are FP32: each is split into three bfloat16 planes (hi + mid + lo: all 24
+// bits of a value of 2^-109 or more; below, the last ones are less than bfloat16's smallest
+// value), and since the other operand of either
 // gradient (weights, activations) is stored in bfloat16, the sum of the three
 // planes' products is the product of the FP32 gradient.
 //

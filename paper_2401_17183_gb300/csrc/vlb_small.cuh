@@ -4,7 +4,9 @@
 // between steps, in place of a launch per step. Up to 16 blocks form one thread-block
 // cluster and meet at its hardware barrier; more are launched cooperatively, so that
 // every block is resident, and count themselves in global memory (that wait is bounded
-// all the same). The arithmetic per cell is that of the step kernel.
+// all the same). The arithmetic per cell is that of the step kernel, compiled apart: a
+// compiler might contract a product and a sum otherwise, so the tests compare the two
+// bit for bit in every form.
 #pragma once
 
 #include "vlb_step.cuh"

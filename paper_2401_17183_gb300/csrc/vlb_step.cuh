@@ -573,8 +573,9 @@ __device__ __forceinline__ void step_tiles(const StepArgs &a, const int64_t t0, 
       R Np[Q];
       CollideState<Q, R> cst;
       // (with one record per cell the rest state is formed, not read)
-      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
-                                     arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
+      collide_cell<Q, R, true, REFOFS, PLANE, RC, EXT, H16>(N, rc, arg_r<R>(a.nref, a.nref_f),
+                                                            arg_r<R>(a.itau, a.itau_f), arg_r<R>(a.tol, a.tol_f),
+                                                            a.max_iter, Np, cst);
       if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
 
       // ---- moving walls (wall cells only, one branch per cell): a reflected
