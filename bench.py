@@ -442,8 +442,8 @@ def bench_batch(a):
 
 
 def bench_d3q39(a):
-    """The 6th-order isotropic velocity set D3Q39 (FP64, pair-form
-    collision) on a periodic sine-mapped box of --n^3 cells."""
+    """The 6th-order isotropic velocity set D3Q39 (FP64, polynomial
+    force map) on a periodic sine-mapped box of --n^3 cells."""
     import torch
 
     from paper_2401_17183_gb300 import build as B
@@ -484,7 +484,7 @@ def bench_d3q39(a):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_kind": peak_kind,
                      "bytes_per_cell_update": bpc,
-                     "limiter": "FP64 arithmetic of the per-direction collision, not DRAM"},
+                     "limiter": "FP64 arithmetic of the collision, not DRAM"},
         "clocks": clocks, "gpu_launches": a.steps,
     }
     print(json.dumps(line))

@@ -163,8 +163,10 @@ __device__ __forceinline__ void a_store(const uint32_t (&w)[72], unsigned char *
 // block 128. wp: weights in pipeline-step order [ceil(C/16)][18 K groups][Co][8]
 // (k_pack_weights).
 //
-// Bounded by shared-memory bandwidth: a step of 16 channels stores the
-// 128 x 144 patch matrix (36 KB) and the nine MMAs read it with NB x 144 weights.
+// Bounded by the chain of a step: 16 channels' loads, the 128 x 144 patch matrix (36 KB)
+// stored by the threads, a barrier, and the nine MMAs that read it with NB x 144 weights; the
+// shared-memory pipes are 17 to 41% busy, the issue slots 17 to 31%, with one or two
+// blocks of four warps on an SM.
 // A thread keeps a pixel pair (rows i and 64 + i of the tile, so that a warp's
 // stores are consecutive) and 8 of the 16 channels: 9 aligned 32-bit loads per
 // channel give the 18 taps of both pixels, and byte permutes place them; the
@@ -327,7 +329,7 @@ struct Padded {
 // its sum to the accumulator's last bits, so a long chain of them drifts), mid and lo, 2^-8
 // of hi, to a third that is read once. NB = 64: 192 accumulator columns, two
 // blocks per SM. Bounded by the MMAs' shared-memory reads (A 32 + B 16 cycles for 32 of
-// arithmetic at NB = 64).
+// arithmetic at NB = 64; that pipe is 40 to 54% busy) and by waits between the roles.
 // Warm-start network (width 64, 32 x 64, batch 32): nine layers in 242 us (CUDA cores:
 // 2,900 us); the gradients' error against 64 bits 3.4e-7 (CUDA cores: 1.2e-6).
 // grid (tiles, rows / NB), block 192. C a multiple of 16.
