@@ -788,7 +788,7 @@ struct Unit64 {
 
 // The whole local collision in FP64 (see collide_cell). GB300 runs an FP64
 // instruction of a warp in 64 cycles of its quarter SM, so only the FP64 operations
-// count, about 480 per D3Q19 cell here (920 when the FP32 form was used in FP64):
+// count, about 540 per D3Q19 cell here (920 when the FP32 form was used in FP64):
 //  - the chord iteration starts from Pt = H Pc with three evaluations of the
 //    polynomial in FP32: its value is of the order of curvature times U^2, so FP32 leaves
 //    an error of about 1e-13 m, which one evaluation in FP64 reduces by the map's
@@ -797,12 +797,16 @@ struct Unit64 {
 //    change is then added to first order, in FP32. Below four iterations
 //    allowed: the plain iteration from the rest state's force.
 //  - the test reads the sizes by integer operations on the high words;
-//  - N' is formed from the pair sums and differences, even and odd part once per pair:
-//      even: (1 - 1/tau) s/2 + w [y0 + c.Y.c],  odd: (1 - 1/tau) t/2 + w [(m/tau) xo + 3 c.Phi],
-//    Y = (9/2)(m/tau) B + 9 P, P = J deltaPi (Eq. 30) symmetrised,
-//    y0 = (mdev - (3/2) m tr B)/tau - 3 tr P.
-// D3Q19 channel, 64^3: 383 -> 219 us a step, the FP64 pipe over 90% busy.
-template <int Q, bool FINAL, bool EXT, typename RC>
+//  - N' is formed once per pair and part from what differs from the cell's own rest state, n_a =
+//    J w (1 + x0) - w n_ref (RR, RW; see form_np), so that no term of the metric's size is rounded
+//    at every step:
+//      even: s/2 - (1/tau) [s/2 - RR - RW (m - J)] + w [y0 + c.Y.c],  odd: t/2 - t/(2 tau) + w [(m/tau) xo + 3 c.Phi],
+//    Y = (9/2)(m/tau) U~U~ + 9 P, P = J deltaPi (Eq. 30) symmetrised,
+//    y0 = -(3/2)(m/tau) U~.U~ - 3 tr P.
+//    (From mdev and the whole of B instead, 60 operations fewer, errors against an 80-bit run were
+//    0.9 to 1.5 times as large in N after 20 steps and up to 7 times in u; 0.99 to 1.02 so.)
+// D3Q19 channel, 64^3: 383 -> 181 us a step, the FP64 pipe 85% busy.
+template <int Q, bool FINAL, bool EXT, bool RREC, typename RC>
 __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, double nref, double itau, double tol,
                                             int max_iter, double (&dp)[Q], CollideState<Q, double> &st) {
   using L = CoefLayout<Q>;
@@ -1005,7 +1009,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
 #pragma unroll
   for (int i = 0; i < D; i++) st.F[i] = Phi[i] * rc[L::IJ];
   if constexpr (FINAL) {
-    double Ut[D], B[NS], C2[D][D], Sc[D], T0[D], T[D][D], tb = 0.0;
+    double Ut[D], B[NS], Bd[D], C2[D][D], Sc[D], T0[D], T[D][D], tb = 0.0;
 #pragma unroll
     for (int i = 0; i < D; i++) Ut[i] = fma(Phi[i], h2m, st.U[i]);
     // 3 B = (g - I) + 3 U~U~ (T0 = 1/3); (3/2) C^kkl = (1/2)[gd_kk U~^l + (U~^l - U^l) + 2 gd_kl U~^k]
@@ -1020,10 +1024,12 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
     for (int i = 0; i < D; i++)
 #pragma unroll
       for (int j = i; j < D; j++)
-        B[sym<D>(i, j)] =
-            EXT && i < 2 && j == 2 ? U3[i] * Ut[j] : fma(U3[i], Ut[j], 2.0 * rc[L::GH + sym<D>(i, j)]);
+        B[sym<D>(i, j)] = U3[i] * Ut[j];
 #pragma unroll
-    for (int i = 0; i < D; i++) tb += B[sym<D>(i, i)];
+    for (int i = 0; i < D; i++) {
+      tb += B[sym<D>(i, i)];
+      Bd[i] = fma(U3[i], Ut[i], 2.0 * rc[L::GH + sym<D>(i, i)]);
+    }
     // per axis l: xo/3 of an axis direction is T0_l = U^l - sum_k C2^kl, of a diagonal
     // c^l T_lk + c^k T_kl with T_lk = T0_l + 3 C2^kl
 #pragma unroll
@@ -1034,7 +1040,7 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
         if (k == l) continue;
         // gd_kk/2 + (3/2) U~k^2 = B_kk / 2
         const double x = EXT && (k == 2 || l == 2) ? du[l] : fma(rc[L::GH + sym<D>(k, l)], Ut[k] + Ut[k], du[l]);
-        C2[k][l] = fma(0.5 * B[sym<D>(k, k)], Ut[l], x);
+        C2[k][l] = fma(0.5 * Bd[k], Ut[l], x);
         Sc[l] += C2[k][l];
       }
       T0[l] = st.U[l] - Sc[l];
@@ -1101,10 +1107,10 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       }
     }
     // y0 = w2 [(mdev - m (3 tr B) / 2) / tau - 3 tr P]
-    const double y0 = fma(-((18.0 * w2 * w2 * pu) * m), trP, w2 * itau * fma(-hm, tb, mdev));
+    const double y0 = fma(-((18.0 * w2 * w2 * pu) * m), trP, -(w2 * itau) * (hm * tb));
     // (the weights of the odd part are MomentWeights': no momentum is made by rounding them)
     using MW = MomentWeights<Q, double>;
-    const double omt = 1.0 - itau, h = 0.5 * omt, zm = MW::a2 * mt;
+    const double zm = MW::a2 * mt, hi = -0.5 * itau;
     double Z0[D], Z[D][D];
 #pragma unroll
     for (int l = 0; l < D; l++) {
@@ -1113,7 +1119,37 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       for (int k = 0; k < D; k++)
         if (k != l) Z[l][k] = fma(zm, T[l][k], MW::a2 * Phi[l]);
     }
-    dp[0] = fma(omt, d[0], (lat_w<Q, double>(0) / w2) * y0);
+    // the rest state: RR, RW of the record, or formed from J and g^ij (see form_np)
+    double rw[RREC ? 1 : H + 1], rr[RREC ? 1 : H + 1], mn;
+    if constexpr (RREC) {
+      mn = mdev - rc[L::RR + H + 1];
+    } else {
+      const double Jc = rc[L::J], Jd = Jc - nref;
+      double tr3 = rc[L::GH + sym<D>(0, 0)], rsum = 0.0;
+#pragma unroll
+      for (int i = 1; i < D; i++) tr3 += rc[L::GH + sym<D>(i, i)];
+      tr3 *= 1.0 / 3.0;
+#pragma unroll
+      for (int q = 0; q <= H; q++) {
+        double x = -tr3;
+        if (q > 0) {
+          const int l = nz_axis<Q>(q, 0), k = nz_axis<Q>(q, 1);
+          x = rc[L::GH + sym<D>(l, l)];
+          if (k >= 0)
+            x = fma((double)(2 * Lat<Q>::c(q, l) * Lat<Q>::c(q, k)), rc[L::GH + sym<D>(l, k)],
+                    x + rc[L::GH + sym<D>(k, k)]);
+          x -= tr3;
+        }
+        const double w = lat_w<Q, double>(q);
+        rw[q] = fma(3.0 * w, x, w);
+        rr[q] = fma((3.0 * w) * Jc, x, w * Jd);
+        rsum += q == 0 ? rr[q] : 2.0 * rr[q];
+      }
+      mn = mdev - rsum;
+    }
+    auto rr_at = [&](int q) -> double { if constexpr (RREC) return rc[L::RR + q]; else return rr[q]; };
+    auto rw_at = [&](int q) -> double { if constexpr (RREC) return rc[L::RW + q]; else return rw[q]; };
+    dp[0] = d[0] + fma(-itau, fma(-rw_at(0), mn, d[0] - rr_at(0)), (lat_w<Q, double>(0) / w2) * y0);
 #pragma unroll
     for (int p = 1; p <= H; p++) {
       const int l = nz_axis<Q>(p, 0), k = nz_axis<Q>(p, 1);
@@ -1129,9 +1165,10 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
         const double a = sl > 0 ? Z[l][k] : -Z[l][k];
         o = sk > 0 ? a + Z[k][l] : a - Z[k][l];
       }
-      const double ev = fma(h, s[p], e), od = fma(h, t[p], o);
-      dp[p] = ev + od;
-      dp[p + H] = ev - od;
+      const double ne = fma(-rw_at(p), mn, fma(0.5, s[p], -rr_at(p)));
+      const double ae = fma(-itau, ne, e), ao = fma(hi, t[p], o);
+      dp[p] = d[p] + (ae + ao);
+      dp[p + H] = d[p + H] + (ae - ao);
     }
   }
 }
@@ -1379,7 +1416,7 @@ __device__ __forceinline__ void collide_cell(const R (&d)[Q], const RC &rc, R nr
                                              R (&dp)[Q], CollideState<Q, R> &st) {
   if constexpr (sizeof(R) == 8) {
     static_assert(!REST, "FP64 populations are stored relative to the uniform reference");
-    collide_f64<Q, FINAL, EXT, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
+    collide_f64<Q, FINAL, EXT, RREC, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   } else {
     collide_f32<Q, R, FINAL, REST, RREC, EXT, FR0, RC>(d, rc, nref, itau, tol, max_iter, dp, st);
   }
