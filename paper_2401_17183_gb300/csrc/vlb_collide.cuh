@@ -786,6 +786,38 @@ struct Unit64 {
   }
 };
 
+// RR, RW and the sum of the RR (see CoefLayout) of a record that ends before them, in FP64. (Written
+// so that no product can be contracted into a sum: the multi-step kernel forms them once a
+// launch, the step kernel once a cell, with the same last bits.)
+template <int Q, typename RC>
+__device__ __forceinline__ void rest_state(const RC &rc, double nref, double (&rr)[Lat<Q>::H + 1],
+                                           double (&rw)[Lat<Q>::H + 1], double &rsum) {
+  using L = CoefLayout<Q>;
+  constexpr int D = Lat<Q>::D, H = Lat<Q>::H;
+  const double Jc = rc[L::J], Jd = Jc - nref;
+  double tr = rc[L::GH + sym<D>(0, 0)];
+#pragma unroll
+  for (int i = 1; i < D; i++) tr += rc[L::GH + sym<D>(i, i)];
+  const double tr3 = __dmul_rn(tr, 1.0 / 3.0);
+  rsum = 0.0;
+#pragma unroll
+  for (int q = 0; q <= H; q++) {
+    double x = -tr3;
+    if (q > 0) {
+      const int l = nz_axis<Q>(q, 0), k = nz_axis<Q>(q, 1);
+      x = rc[L::GH + sym<D>(l, l)];
+      if (k >= 0)
+        x = fma((double)(2 * Lat<Q>::c(q, l) * Lat<Q>::c(q, k)), rc[L::GH + sym<D>(l, k)],
+                x + rc[L::GH + sym<D>(k, k)]);
+      x -= tr3;
+    }
+    const double w = lat_w<Q, double>(q);
+    rw[q] = fma(3.0 * w, x, w);
+    rr[q] = fma(__dmul_rn(3.0 * w, Jc), x, __dmul_rn(w, Jd));
+    rsum += q == 0 ? rr[q] : 2.0 * rr[q];
+  }
+}
+
 // The whole local collision in FP64 (see collide_cell). GB300 runs an FP64
 // instruction of a warp in 64 cycles of its quarter SM, so only the FP64 operations
 // count, about 540 per D3Q19 cell here (920 when the FP32 form was used in FP64):
@@ -1119,32 +1151,13 @@ __device__ __forceinline__ void collide_f64(const double (&d)[Q], const RC &rc, 
       for (int k = 0; k < D; k++)
         if (k != l) Z[l][k] = fma(zm, T[l][k], MW::a2 * Phi[l]);
     }
-    // the rest state: RR, RW of the record, or formed from J and g^ij (see form_np)
-    double rw[RREC ? 1 : H + 1], rr[RREC ? 1 : H + 1], mn;
+    // the rest state: RR, RW of the record, or formed from J and g^ij
+    double rw[H + 1], rr[H + 1], mn;
     if constexpr (RREC) {
       mn = mdev - rc[L::RR + H + 1];
     } else {
-      const double Jc = rc[L::J], Jd = Jc - nref;
-      double tr3 = rc[L::GH + sym<D>(0, 0)], rsum = 0.0;
-#pragma unroll
-      for (int i = 1; i < D; i++) tr3 += rc[L::GH + sym<D>(i, i)];
-      tr3 *= 1.0 / 3.0;
-#pragma unroll
-      for (int q = 0; q <= H; q++) {
-        double x = -tr3;
-        if (q > 0) {
-          const int l = nz_axis<Q>(q, 0), k = nz_axis<Q>(q, 1);
-          x = rc[L::GH + sym<D>(l, l)];
-          if (k >= 0)
-            x = fma((double)(2 * Lat<Q>::c(q, l) * Lat<Q>::c(q, k)), rc[L::GH + sym<D>(l, k)],
-                    x + rc[L::GH + sym<D>(k, k)]);
-          x -= tr3;
-        }
-        const double w = lat_w<Q, double>(q);
-        rw[q] = fma(3.0 * w, x, w);
-        rr[q] = fma((3.0 * w) * Jc, x, w * Jd);
-        rsum += q == 0 ? rr[q] : 2.0 * rr[q];
-      }
+      double rsum;
+      rest_state<Q>(rc, nref, rr, rw, rsum);
       mn = mdev - rsum;
     }
     auto rr_at = [&](int q) -> double { if constexpr (RREC) return rc[L::RR + q]; else return rr[q]; };

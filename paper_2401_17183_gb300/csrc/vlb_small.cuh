@@ -62,8 +62,9 @@ __device__ __forceinline__ void small_cell(const StepArgs &a, const Addr<Q, int3
     N[av] = __ldcg(f + (own ? a.soff[av] + cell : a.soff[lat_opp<Q>(av)] + ad.nb(av, -1)));
   }
   CollideState<Q, R> cst;
-  collide_cell<Q, R, true, false, PLANE, RC, EXT>(N, rc, arg_r<R>(a.nref, a.nref_f), arg_r<R>(a.itau, a.itau_f),
-                                             arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
+  collide_cell<Q, R, true, false, PLANE || sizeof(R) == 8, RC, EXT>(N, rc, arg_r<R>(a.nref, a.nref_f),
+                                                                    arg_r<R>(a.itau, a.itau_f),
+                                                                    arg_r<R>(a.tol, a.tol_f), a.max_iter, Np, cst);
   if (!cst.conv) atomicOr(a.err, ERR_NOCONV);
   if (a.moving && ad.wall_cell()) {
     R uw[D], zero[D], gd[L::NS];
@@ -97,14 +98,14 @@ __device__ __forceinline__ void small_cell(const StepArgs &a, const Addr<Q, int3
 }
 
 // records a block keeps in shared memory: of its cells' columns (plane mode), or
-// of its cells (FP64, padded by one value against bank conflicts); FP32 records per
-// cell stay in registers
+// of its cells (FP64, with the rest state formed once a launch: 64 x 64 box 10.7 -> 9.8 us
+// a step; an odd number of values against bank conflicts); FP32 records per cell stay in registers
 template <int Q, typename R, bool PLANE>
 struct SmallRecords {
   using L = CoefLayout<Q>;
   static constexpr int SRC = L::template stride<R, PLANE>();
   static constexpr int KEEP = PLANE ? L::SREST : SRC;            // values the step reads
-  static constexpr int STRIDE = PLANE ? round4(KEEP) : KEEP + 1;
+  static constexpr int STRIDE = PLANE ? round4(KEEP) : (L::RW + L::H + 1) | 1;
   static size_t bytes(int T, int64_t nfast) {
     if (!PLANE) return sizeof(R) == 8 ? sizeof(R) * STRIDE * T : 0;
     return sizeof(R) * STRIDE * (size_t)((T - 1) / nfast + 2);
@@ -139,6 +140,20 @@ __global__ void __launch_bounds__(T, MINB)
     }
     __syncthreads();
     rc.p = sm + (ad.cell / nf - r0) * SR::STRIDE;
+    if constexpr (!PLANE && sizeof(R) == 8) {   // a thread's own cell
+      using L = CoefLayout<Q>;
+      double rr[Lat<Q>::H + 1], rw[Lat<Q>::H + 1], rsum;
+      rest_state<Q>(rc, a.nref, rr, rw, rsum);
+      R *const o = sm + (ad.cell - r0) * SR::STRIDE;
+      __syncthreads();   // (threads past the last cell share its record)
+#pragma unroll
+      for (int q = 0; q <= Lat<Q>::H; q++) {
+        o[L::RR + q] = rr[q];
+        o[L::RW + q] = rw[q];
+      }
+      o[L::RR + Lat<Q>::H + 1] = rsum;
+      __syncthreads();
+    }
   }
 #pragma unroll 1
   for (int32_t k = 0; k < nsteps; k++) {
